@@ -21,18 +21,17 @@
 #include "es_3d.h"
 #include "es_3d_grid.cuh"
 #include "es_device.cuh"
+#include "es_flux64.cuh"
 #include "es_internal.h"
 
 namespace es {
 
-// node fields of the 3D path (global planes and shared-memory slots)
-enum Field3 {
-    G_RHO, G_V1, G_V2, G_V3, G_T, G_IT, G_OM, G_IOM, G_G, G_RT, G_VT1, G_VT2, G_VT3, G_V2T,
-    G_RV1, G_RV2, G_RV3, G_LNR, G_LNOM, G_LNT, G_RP, G_LNRP, G_W0,
-    F3_COUNT,
-    G_NX = F3_COUNT, G_NY, G_NZ, G_XT,     // metrics of the direction (shared memory only)
-    S3_COUNT
-};
+// node fields of the 3D path (global planes and shared-memory slots), and the direction's metrics (shared memory only)
+using SL3 = flux64::Slots<3>;
+constexpr int F3_COUNT = SL3::COUNT;
+constexpr int G_N = F3_COUNT;              // halves of the three metric components, then of J xi_t
+constexpr int G_XT = G_N + 3;
+constexpr int S3_COUNT = G_XT + 1;
 
 // field at a possibly-ghost node, ghosts by copy / wrap (monitor and filter)
 __device__ __forceinline__ double field3(const Grid3& g, const double* f, int i1, int i2, int i3) {
@@ -150,7 +149,7 @@ __global__ void k3_deriv(Grid3 g, const double* XE, double* D) {
     }
 }
 
-// J dxi_k/dx_j on direction k's grid (n_k + 6 nodes along xi_k, interior across); the direction is a template
+// Half of J dxi_k/dx_j (a face takes the mean of two nodes as a sum) on direction k's grid (n_k + 6 nodes along xi_k, interior across); the direction is a template
 // parameter (no run-time indexing of the grid's arrays)
 template <int k>
 __global__ void k3_metric(Grid3 g, const double* D, double* NKo) {
@@ -162,7 +161,7 @@ __global__ void k3_metric(Grid3 g, const double* D, double* NKo) {
     else m3 += 6;
     const size_t M = size_t(m1) * m2 * m3;
     const int l = (k + 1) % 3, m = (k + 2) % 3;
-    const double scale = g.inv_dxi[l] * g.inv_dxi[m];
+    const double scale = 0.5 * (g.inv_dxi[l] * g.inv_dxi[m]);
     const size_t stl = l == 0 ? 1 : (l == 1 ? size_t(E1) : size_t(E1) * E2);
     const size_t stm = m == 0 ? 1 : (m == 1 ? size_t(E1) : size_t(E1) * E2);
     for (size_t t = blockIdx.x * size_t(blockDim.x) + threadIdx.x; t < M; t += size_t(gridDim.x) * blockDim.x) {
@@ -189,205 +188,13 @@ __global__ void k3_metric(Grid3 g, const double* D, double* NKo) {
 __global__ void k3_nodes(Grid3 g, Gas G, const double* JU, const double* J, double* NF, DevStatus* st) {
     const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
     for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
-        const double iJ = rcp_nr(J[id]);
-        const double rho = JU[id] * iJ;
-        const double m1 = JU[N + id] * iJ, m2 = JU[2 * N + id] * iJ, m3 = JU[3 * N + id] * iJ;
-        const double E = JU[4 * N + id] * iJ;
-        const double irho = rcp_nr(rho);
-        const double v1 = m1 * irho, v2 = m2 * irho, v3 = m3 * irho;
-        const double ke = 0.5 * (v1 * v1 + v2 * v2 + v3 * v3);
-        const double T = (E * irho - ke + G.a * rho) * G.icv;
-        const double om = 1.0 - G.b * rho;
-        const double iom = rcp_nr(om);
-        const double p = rho * G.R * T * iom - G.a * rho * rho;
-        const double iT = rcp_nr(T);
-        if (!(rho > 0.0) || !(om > 0.0) || !(T > 0.0) || !(p > 0.0)) raise_error(st, ES_ERR_INADMISSIBLE, int(id));
-        const double lnr = log(rho);
-        const double lnom = G.b > 0.0 ? log(om) : 0.0;
-        const double lnT = log(T);
-        const double lnp = log(p);
-        NF[G_RHO * N + id] = rho;
-        NF[G_V1 * N + id] = v1;
-        NF[G_V2 * N + id] = v2;
-        NF[G_V3 * N + id] = v3;
-        NF[G_T * N + id] = T;
-        NF[G_IT * N + id] = iT;
-        NF[G_OM * N + id] = om;
-        NF[G_IOM * N + id] = iom;
-        NF[G_G * N + id] = G.R * iom - G.a * rho * iT;
-        NF[G_RT * N + id] = rho * iT;
-        NF[G_VT1 * N + id] = v1 * iT;
-        NF[G_VT2 * N + id] = v2 * iT;
-        NF[G_VT3 * N + id] = v3 * iT;
-        NF[G_V2T * N + id] = 2.0 * ke * iT;
-        NF[G_RV1 * N + id] = m1;
-        NF[G_RV2 * N + id] = m2;
-        NF[G_RV3 * N + id] = m3;
-        NF[G_LNR * N + id] = lnr;
-        NF[G_LNOM * N + id] = lnom;
-        NF[G_LNT * N + id] = lnT;
-        NF[G_RP * N + id] = div_nr(rho, p);
-        NF[G_LNRP * N + id] = lnr - lnp;
-        // entropy variables V = ((e + p/rho)/T - s - |v|^2/(2T), v/T, -1/T); V_1..3 = VT, V_4 = -IT
-        const double s = G.cv * lnT + G.R * (lnom - lnr);
-        NF[G_W0 * N + id] = G.cv - s - 2.0 * G.a * rho * iT + G.R * iom - ke * iT;
+        const double U[5] = {JU[id], JU[N + id], JU[2 * N + id], JU[3 * N + id], JU[4 * N + id]};
+        const bool ok = flux64::node_fields<3>(U, J[id], G, [&](int f, double v) { NF[f * N + id] = v; });
+        if (!ok) raise_error(st, ES_ERR_INADMISSIBLE, int(id));
     }
 }
 
 // ================================================================ direction flux
-// two-point EC flux of Sec. 3.1 contracted with the face-averaged metrics (n, J xi_t)
-__device__ __forceinline__ void pair_flux3(const double* S, int NB, int l, int r, double nx, double ny, double nz,
-                                           double xt, const Gas& G, double* out) {
-    const double rl = S[G_RHO * NB + l], rr = S[G_RHO * NB + r];
-    const double Tl = S[G_T * NB + l], Tr = S[G_T * NB + r];
-    const double rho_m = 0.5 * (rl + rr);
-    const double T_m = 0.5 * (Tl + Tr);
-    const double iT_m = 0.5 * (S[G_IT * NB + l] + S[G_IT * NB + r]);
-    const double ilr = inv_log_mean(rl, rr, S[G_LNR * NB + l], S[G_LNR * NB + r]);
-    const double ilT = inv_log_mean(Tl, Tr, S[G_LNT * NB + l], S[G_LNT * NB + r]);
-    const double Pinv = S[G_IOM * NB + l] * S[G_IOM * NB + r];
-    const double iTa = rcp_nr(T_m);
-    const double coef = G.R * G.b * Pinv - G.a * iTa;
-    double D = G.R * ilr + coef - G.a * iTa;
-    if (G.b > 0.0)
-        D += G.R * G.b * inv_log_mean(S[G_OM * NB + l], S[G_OM * NB + r], S[G_LNOM * NB + l], S[G_LNOM * NB + r]);
-    const double iD = rcp_nr(D);
-    const double g_m = 0.5 * (S[G_G * NB + l] + S[G_G * NB + r]);
-    const double rT_m = 0.5 * (S[G_RT * NB + l] + S[G_RT * NB + r]);
-    const double v2T_m = 0.5 * (S[G_V2T * NB + l] + S[G_V2T * NB + r]);
-    double vm[3], vT[3], rv[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        vm[c] = 0.5 * (S[(G_V1 + c) * NB + l] + S[(G_V1 + c) * NB + r]);
-        vT[c] = 0.5 * (S[(G_VT1 + c) * NB + l] + S[(G_VT1 + c) * NB + r]);
-        rv[c] = 0.5 * (S[(G_RV1 + c) * NB + l] + S[(G_RV1 + c) * NB + r]);
-    }
-    const double U1 = (rho_m * coef + g_m) * iD;
-    const double F11 = (rv[0] * coef + g_m * vm[0]) * iD;
-    const double F21 = (rv[1] * coef + g_m * vm[1]) * iD;
-    const double F31 = (rv[2] * coef + g_m * vm[2]) * iD;
-    const double P = rho_m * T_m * g_m;
-    const double B0 = 0.5 * v2T_m - G.cv * T_m * ilT + 2.0 * G.a * rT_m;
-    const double Q1 = xt * U1 + nx * F11 + ny * F21 + nz * F31;
-    const double sv = vT[0] * vm[0] + vT[1] * vm[1] + vT[2] * vm[2];
-    out[0] = Q1;
-    out[1] = vm[0] * Q1 + nx * P;
-    out[2] = vm[1] * Q1 + ny * P;
-    out[3] = vm[2] * Q1 + nz * P;
-    out[4] = div_nr(G.a * rT_m * (xt * rho_m + nx * rv[0] + ny * rv[1] + nz * rv[2]) + (sv - B0) * Q1 +
-                        P * (nx * vT[0] + ny * vT[1] + nz * vT[2]),
-                    iT_m);
-}
-
-// -1/2 Lambda T^{-1} R Y [[W]]^WENO at the face between pencil nodes l and l+1 (Sec. 3.3,
-// eq. HOstable) with the 3D rotation: theta = atan2(n_2, n_1) (0 when |(n_1, n_2)| <= 1e-12 |n|, the
-// rounding of metrics that vanish exactly),
-// phi = atan2(n_3, sqrt(n_1^2 + n_2^2)), so the rows of T's momentum block are
-// e_n = n/L, e_t1 = (-sin theta, cos theta, 0), e_t2 = (-sin phi cos theta, -sin phi sin theta, cos phi);
-// R's tangential columns are (0, 0, 1, 0, v_t1) and (0, 0, 0, 1, v_t2), scaled by sqrt(rho T).
-__device__ __forceinline__ void face_dissipation3(const double* S, int NB, int l, double nx, double ny, double nz,
-                                                  double xtf, const Gas& G, const Weno& Wc, double* out,
-                                                  DevStatus* st) {
-    const int r = l + 1;
-    const double ilr = inv_log_mean(S[G_RHO * NB + l], S[G_RHO * NB + r], S[G_LNR * NB + l], S[G_LNR * NB + r]);
-    const double rho = rcp_nr(ilr);
-    const double ilrp = inv_log_mean(S[G_RP * NB + l], S[G_RP * NB + r], S[G_LNRP * NB + l], S[G_LNRP * NB + r]);
-    const double p = rho * ilrp;
-    const double om = 1.0 - G.b * rho;
-    const double T = (p + G.a * rho * rho) * om * ilr * G.iR;
-    const double iom = rcp_nr(om);
-    const double c2 = (1.0 + G.delta) * G.R * T * iom * iom - 2.0 * G.a * rho;
-    const double dcrit = G.R * T - 2.0 * G.a * rho * om * om;
-    if (!(c2 > 0.0) || !(dcrit > 0.0) || !(om > 0.0)) raise_error(st, ES_ERR_INADMISSIBLE, 0);
-    const double c = sqrt(c2);
-    const double vm1 = 0.5 * (S[G_V1 * NB + l] + S[G_V1 * NB + r]);
-    const double vm2 = 0.5 * (S[G_V2 * NB + l] + S[G_V2 * NB + r]);
-    const double vm3 = 0.5 * (S[G_V3 * NB + l] + S[G_V3 * NB + r]);
-    const double L = sqrt(nx * nx + ny * ny + nz * nz);
-    const double r12 = sqrt(nx * nx + ny * ny);
-    double ct = 1.0, sn = 0.0;
-    if (r12 > 1e-12 * L) {
-        const double ir = rcp_nr(r12);
-        ct = nx * ir;
-        sn = ny * ir;
-    }
-    const double iL = rcp_nr(L);
-    const double cp = r12 * iL, sp = nz * iL;
-    const double en[3] = {cp * ct, cp * sn, sp};
-    const double et1[3] = {-sn, ct, 0.0};
-    const double et2[3] = {-sp * ct, -sp * sn, cp};
-    const double vn = en[0] * vm1 + en[1] * vm2 + en[2] * vm3;
-    const double vt1 = et1[0] * vm1 + et1[1] * vm2;
-    const double vt2 = et2[0] * vm1 + et2[1] * vm2 + et2[2] * vm3;
-    const double E = rho * (G.cv * T - G.a * rho) + 0.5 * rho * (vn * vn + vt1 * vt1 + vt2 * vt2);
-    const double H = (E + p) * ilr;
-    const double mid = H - c2 * om * G.idelta;
-    const double ic2 = rcp_nr(c2);
-    const double sA = sqrt(0.5 * rho * T * ic2);
-    const double sE = sqrt(div_nr(G.R * G.delta * rho * T * T * ic2, dcrit));
-    const double sT = sqrt(rho * T);
-    const double Lam = fabs(xtf + L * vn) + L * c;
-    const double Hm = H - vn * c, Hp = H + vn * c;
-
-    // W = R^T (T V) at nodes l-2 .. l+3
-    double W[6][5];
-    double aTV[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int o = 0; o < 6; ++o) {
-        const int q = l + (o - 2);
-        const double V0 = S[G_W0 * NB + q];
-        const double a1 = S[G_VT1 * NB + q], a2 = S[G_VT2 * NB + q], a3 = S[G_VT3 * NB + q];
-        const double V4 = -S[G_IT * NB + q];
-        const double V1 = en[0] * a1 + en[1] * a2 + en[2] * a3;
-        const double V2 = et1[0] * a1 + et1[1] * a2;
-        const double V3 = et2[0] * a1 + et2[1] * a2 + et2[2] * a3;
-        const double base = V0 + vt1 * V2 + vt2 * V3;
-        W[o][0] = sA * (base + (vn - c) * V1 + Hm * V4);
-        W[o][1] = sE * (base + vn * V1 + mid * V4);
-        W[o][2] = sT * (V2 + vt1 * V4);
-        W[o][3] = sT * (V3 + vt2 * V4);
-        W[o][4] = sA * (base + (vn + c) * V1 + Hp * V4);
-        if (o == 2 || o == 3) {
-            aTV[0] += fabs(V0);
-            aTV[1] += fabs(V1);
-            aTV[2] += fabs(V2);
-            aTV[3] += fabs(V3);
-            aTV[4] += fabs(V4);
-        }
-    }
-    const double avt1 = fabs(vt1), avt2 = fabs(vt2);
-    const double common = aTV[0] + avt1 * aTV[2] + avt2 * aTV[3];
-    double scl[5];
-    scl[0] = sA * (common + fabs(vn - c) * aTV[1] + fabs(Hm) * aTV[4]);
-    scl[1] = sE * (common + fabs(vn) * aTV[1] + fabs(mid) * aTV[4]);
-    // tangential waves: round-off in a velocity follows the flow's velocity scale |v_t| + c
-    scl[2] = sT * (aTV[2] + (avt1 + c) * aTV[4]);
-    scl[3] = sT * (aTV[3] + (avt2 + c) * aTV[4]);
-    scl[4] = sA * (common + fabs(vn + c) * aTV[1] + fabs(Hp) * aTV[4]);
-    double y[5];
-#pragma unroll
-    for (int m = 0; m < 5; ++m) {
-        const double wmin = mr_weno5(W[0][m], W[1][m], W[2][m], W[3][m], W[4][m], Wc);
-        const double wplu = mr_weno5(W[5][m], W[4][m], W[3][m], W[2][m], W[1][m], Wc);
-        const double jw = wplu - wmin;
-        double j = W[3][m] - W[2][m];
-        if (fabs(j) <= Wc.sign_tol * scl[m]) j = 0.0;
-        const bool keep = (jw > 0.0 && j > 0.0) || (jw < 0.0 && j < 0.0);
-        y[m] = keep ? jw : 0.0;
-    }
-    const double h = -0.5 * Lam;
-    const double y0 = sA * y[0], y1 = sE * y[1], y2 = sT * y[2], y3 = sT * y[3], y4 = sA * y[4];
-    const double i0 = y0 + y1 + y4;
-    const double i1 = (vn - c) * y0 + vn * y1 + (vn + c) * y4;
-    const double i2 = vt1 * i0 + y2;
-    const double i3 = vt2 * i0 + y3;
-    const double i4 = Hm * y0 + mid * y1 + vt1 * y2 + vt2 * y3 + Hp * y4;
-    out[0] = h * i0;
-#pragma unroll
-    for (int c3 = 0; c3 < 3; ++c3) out[1 + c3] = h * (en[c3] * i1 + et1[c3] * i2 + et2[c3] * i3);
-    out[4] = h * i4;
-}
-
 struct Dir3Params {
     Grid3 g;
     Gas gas;
@@ -466,9 +273,9 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
 #pragma unroll
         for (int f = 0; f < F3_COUNT; ++f) S[f * NB + bx] = v[f];
         if ((s < 0 || s >= nk) && end_mirrored(g.bc[K], s < 0)) {     // wall / symmetry ghost
-            S[(G_V1 + K) * NB + bx] = -S[(G_V1 + K) * NB + bx];
-            S[(G_VT1 + K) * NB + bx] = -S[(G_VT1 + K) * NB + bx];
-            S[(G_RV1 + K) * NB + bx] = -S[(G_RV1 + K) * NB + bx];
+            S[(SL3::V + K) * NB + bx] = -S[(SL3::V + K) * NB + bx];
+            S[(SL3::VT + K) * NB + bx] = -S[(SL3::VT + K) * NB + bx];
+            S[(SL3::RV + K) * NB + bx] = -S[(SL3::RV + K) * NB + bx];
         }
         // metrics: the metric grid holds s in [-3, n_K + 3); the tail of a ragged pencil is clamped
         int se = s + 3;
@@ -478,9 +285,9 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
         else { j1 = a; j2 = b; j3 = se; }
         const size_t mi = (size_t(j3) * M2 + j2) * M1 + j1;
         const double nx = P.NK[mi], ny = P.NK[M + mi], nz = P.NK[2 * M + mi];
-        S[G_NX * NB + bx] = nx;
-        S[G_NY * NB + bx] = ny;
-        S[G_NZ * NB + bx] = nz;
+        S[G_N * NB + bx] = nx;
+        S[(G_N + 1) * NB + bx] = ny;
+        S[(G_N + 2) * NB + bx] = nz;
         double xt = 0.0;
         if (P.xdot) {
             // mesh velocity at the node: wrap, odd reflection, or at a wall / symmetry end the
@@ -497,7 +304,7 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
                     xd[c] += tk.w[u] * P.xdot[c * N + idx3(g, k1, k2, k3)];
                 }
             }
-            xt = -(xd[0] * nx + xd[1] * ny + xd[2] * nz);
+            xt = -fma(xd[0], nx, fma(xd[1], ny, xd[2] * nz));
         }
         S[G_XT * NB + bx] = xt;
     }
@@ -511,12 +318,11 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
         else if (kk < 2 * LB + 3) { m = 2; q = 1 + (kk - LB - 1); }
         else { m = 3; q = kk - 2 * LB - 3; }
         const int l = line * LS + q, r = l + m;
-        const double nx = 0.5 * (S[G_NX * NB + l] + S[G_NX * NB + r]);
-        const double ny = 0.5 * (S[G_NY * NB + l] + S[G_NY * NB + r]);
-        const double nz = 0.5 * (S[G_NZ * NB + l] + S[G_NZ * NB + r]);
-        const double xt = 0.5 * (S[G_XT * NB + l] + S[G_XT * NB + r]);
+        double n[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) n[c] = S[(G_N + c) * NB + l] + S[(G_N + c) * NB + r];
         double f[5];
-        pair_flux3(S, NB, l, r, nx, ny, nz, xt, P.gas, f);
+        flux64::pair_flux<3>(S, NB, l, r, n, S[G_XT * NB + l] + S[G_XT * NB + r], P.gas, f);
 #pragma unroll
         for (int c = 0; c < 5; ++c) PB[c * NP + t] = f[c];
     }
@@ -529,7 +335,6 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
         const int pbase = line * PC::PL;
         const int base = line * LS;
         double F[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        double FJ = 0.0;
 #pragma unroll
         for (int m = 1; m <= 3; ++m) {
             const int off = m == 1 ? 0 : (m == 2 ? LB + 1 : 2 * LB + 3);
@@ -538,20 +343,19 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
                 const int qq = q - s;
                 const int pi = pbase + off + (qq - (3 - m));
 #pragma unroll
-                for (int c = 0; c < 5; ++c) F[c] += al * PB[c * NP + pi];
-                FJ += al * 0.5 * (S[G_XT * NB + base + qq] + S[G_XT * NB + base + qq + m]);
+                for (int c = 0; c < 5; ++c) F[c] = fma(c == 4 ? 4.0 * al : al, PB[c * NP + pi], F[c]);   // (a quarter of the energy)
             }
         }
+        // sum_m alpha_m sum of the pairs' mean J xi_t, collected by node
+        const double* XT = S + G_XT * NB + base + q;            // halves
+        const double a3 = ec_alpha(3), a2 = ec_alpha(2) + a3, a1 = ec_alpha(1) + a2;
+        const double FJ = fma(a1, XT[0] + XT[1], fma(a2, XT[-1] + XT[2], a3 * (XT[-2] + XT[3])));
         if (P.diss) {
             const int l = base + q;
-            const double nx = 0.5 * (S[G_NX * NB + l] + S[G_NX * NB + l + 1]);
-            const double ny = 0.5 * (S[G_NY * NB + l] + S[G_NY * NB + l + 1]);
-            const double nz = 0.5 * (S[G_NZ * NB + l] + S[G_NZ * NB + l + 1]);
-            const double xtf = 0.5 * (S[G_XT * NB + l] + S[G_XT * NB + l + 1]);
-            double d[5];
-            face_dissipation3(S, NB, l, nx, ny, nz, xtf, P.gas, P.weno, d, P.status);
+            double n[3];
 #pragma unroll
-            for (int c = 0; c < 5; ++c) F[c] += d[c];
+            for (int c = 0; c < 3; ++c) n[c] = S[(G_N + c) * NB + l] + S[(G_N + c) * NB + l + 1];
+            flux64::face_dissipation<3>(S, NB, l, 1, n, XT[0] + XT[1], P.gas, P.weno, F, P.status, 0);
         }
 #pragma unroll
         for (int c = 0; c < 5; ++c) FB[c * NFc + t] = F[c];
@@ -595,8 +399,8 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
         double acc[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            acc[c] = -(FB[c * NFc + fm + 1] - FB[c * NFc + fm]) * inv;
-            if (!P.first) acc[c] += rh[c];
+            // (explicit: every pencil shape fuses the same product)
+            acc[c] = fma(FB[c * NFc + fm] - FB[c * NFc + fm + 1], inv, rh[c]);
         }
         if (!P.last) {
 #pragma unroll
@@ -607,8 +411,8 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
             P.Jo[id] = acc[5];
         } else {
 #pragma unroll
-            for (int c = 0; c < 5; ++c) P.JUo[c * N + id] = P.ca * un[c] + P.cb * (us[c] + dt * acc[c]);
-            const double Jnew = P.ca * un[5] + P.cb * (us[5] + dt * acc[5]);
+            for (int c = 0; c < 5; ++c) P.JUo[c * N + id] = fma(P.ca, un[c], P.cb * fma(dt, acc[c], us[c]));
+            const double Jnew = fma(P.ca, un[5], P.cb * fma(dt, acc[5], us[5]));
             P.Jo[id] = Jnew;
             if (!(Jnew > 0.0)) raise_error(P.status, ES_ERR_MESH, int(id));
         }
@@ -665,9 +469,10 @@ __global__ void k3_cfl(Grid3 g, Gas G, const double* NF, const double* J, const 
     double mx = 0.0;
     for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
         const int i1 = int(id % g.n[0]), i2 = int((id / g.n[0]) % g.n[1]), i3 = int(id / (size_t(g.n[0]) * g.n[1]));
-        const double rho = NF[G_RHO * N + id], T = NF[G_T * N + id], iom = NF[G_IOM * N + id];
-        const double v[3] = {NF[G_V1 * N + id], NF[G_V2 * N + id], NF[G_V3 * N + id]};
-        const double c2 = (1.0 + G.delta) * G.R * T * (iom * iom) - 2.0 * G.a * rho;
+        // the node fields and metrics are halves
+        const double r = NF[SL3::RHO * N + id], hT = NF[SL3::T * N + id], iom = NF[SL3::IOM * N + id];
+        const double v[3] = {NF[SL3::V * N + id], NF[(SL3::V + 1) * N + id], NF[(SL3::V + 2) * N + id]};
+        const double c2 = 2.0 * (1.0 + G.delta) * G.R * hT * (iom * iom) - 4.0 * G.a * r;
         const double c = sqrt(fmax(c2, 0.0));
         const double iJ = rcp_nr(J[id]);
         const double xd[3] = {xdot ? xdot[id] : 0.0, xdot ? xdot[N + id] : 0.0, xdot ? xdot[2 * N + id] : 0.0};
@@ -677,8 +482,8 @@ __global__ void k3_cfl(Grid3 g, Gas G, const double* NF, const double* J, const 
             const size_t mi = (size_t(i3 + (k == 2 ? 3 : 0)) * m2 + i2 + (k == 1 ? 3 : 0)) * m1 + i1 + (k == 0 ? 3 : 0);
             const double n0 = NK[k][mi], n1 = NK[k][M[k] + mi], n2 = NK[k][2 * M[k] + mi];
             const double xt = -(xd[0] * n0 + xd[1] * n1 + xd[2] * n2);
-            tot += (fabs(xt + (n0 * v[0] + n1 * v[1] + n2 * v[2])) + sqrt(n0 * n0 + n1 * n1 + n2 * n2) * c) * iJ *
-                   g.inv_dxi[k];
+            tot += (fabs(xt + 2.0 * (n0 * v[0] + n1 * v[1] + n2 * v[2])) + sqrt(n0 * n0 + n1 * n1 + n2 * n2) * c) * iJ *
+                   (2.0 * g.inv_dxi[k]);
         }
         if (!(c2 > 0.0)) tot = 1e300;
         mx = fmax(mx, tot);

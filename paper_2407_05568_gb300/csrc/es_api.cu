@@ -602,6 +602,7 @@ int es_create(es_ctx** out, const es_params* p, void* stream) {
     c->weno.ig3 = gs / g3;
     c->weno.eps = p->weno_eps;
     c->weno.sign_tol = p->sign_tol;
+    weno_coefficients(c->weno);
     c->mon.kind = p->monitor;
     c->mon.kappa = p->kappa;
     if (p->monitor == ES_MONITOR_SMOOTH) {

@@ -23,46 +23,40 @@ inline void gas_reciprocals(Gas& g) {
     g.icv = 1.0 / g.cv;
 }
 
-// Reciprocal and quotient for finite, normal, nonzero divisors (all the kernels' divisors are
-// positive physical quantities or sums of them): the hardware's approximate reciprocal refined by
-// two Newton-Raphson steps, y <- y + y (1 - b y), each of which squares the relative error, and
-// for the quotient one correction q <- q + y (a - b q) (Markstein, IBM J. Res. Develop. 34(1),
-// 1990).  Checked against IEEE division on the GPU (es_selftest_division).
+// Reciprocal, quotient and reciprocal square root for finite, normal, positive arguments (the reciprocal also for
+// negative ones): all the kernels' divisors are positive physical quantities or sums of them.  The FP64 pipe
+// issues at 1/64 of the FP32 rate and bounds every kernel that uses these, so each is counted in its
+// instructions.  The hardware's approximations have relative errors below 2^-22; one third-order step
+// y <- y (1 + e + e^2), e = 1 - b y (Householder's iteration of order two for 1/y - b) leaves e^3 < 2^-65 in three
+// instructions, where two Newton steps take four.  The quotient needs only a Newton-refined reciprocal
+// (e^2 < 2^-44): its correction q <- q + y (a - b q) squares that error again (Markstein, IBM J. Res. Develop.
+// 34(1), 1990), five instructions instead of seven.  Checked against IEEE division (es_selftest_division).
 __device__ __forceinline__ double rcp_nr(double b) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    y = fma(y, fma(-b, y, 1.0), y);
-    y = fma(y, fma(-b, y, 1.0), y);
-    return y;
+    const double e = fma(-b, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 __device__ __forceinline__ double div_nr(double a, double b) {
-    const double y = rcp_nr(b);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    y = fma(y, fma(-b, y, 1.0), y);
     const double q = a * y;
     return fma(fma(-b, q, a), y, q);
+}
+// 1/sqrt(x): y <- y (1 + e/2 + 3 e^2/8), e = 1 - x y^2, the same order (five instructions; sqrt(x) = x rsqrt_nr(x)
+// is one more, against about ten of the library's correctly rounded square root)
+__device__ __forceinline__ double rsqrt_nr(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Sixth-order EC combination weights alpha_{3,m}, m = 1, 2, 3 (Sec. 3.1:
 // sum m alpha = 1, sum m^3 alpha = sum m^5 alpha = 0).
 __device__ __forceinline__ double ec_alpha(int m) {
     return m == 1 ? 1.5 : (m == 2 ? -0.3 : 1.0 / 30.0);
-}
-
-// ------------------------------------------------------------ log mean
-// Reciprocal of the logarithmic mean {a}^ln = [[a]]/[[ln a]] (Sec. 3.1), from
-// per-node logarithms.  When |f| = |a_l - a_r|/(a_l + a_r) < 1e-2 the quotient
-// of differences loses digits, so the Taylor series of artanh(f)/f is used:
-// 1/{a}^ln = 2 F(f)/(a_l + a_r), F = 1 + f^2/3 + f^4/5 + ... (six terms).
-__device__ __forceinline__ double inv_log_mean(double al, double ar, double lnl, double lnr) {
-    const double s = al + ar;
-    const double d = al - ar;
-    if (fabs(d) < 1e-2 * s) {
-        const double is = rcp_nr(s);
-        const double f = d * is;
-        const double u = f * f;
-        const double F = 1.0 + u * (1.0 / 3.0 + u * (1.0 / 5.0 + u * (1.0 / 7.0 + u * (1.0 / 9.0 + u * (1.0 / 11.0)))));
-        return 2.0 * F * is;
-    }
-    return div_nr(lnl - lnr, d);
 }
 
 // --------------------------------------------------------- MR-WENO5 (Sec. 3.3)
@@ -75,46 +69,24 @@ struct Weno {
     double ig3;            // 1/g3
     double eps;
     double sign_tol;       // relative round-off size under which a plain jump counts as zero
+    // derived (weno_coefficients): the candidates of the FP64 reconstruction as coefficients of the data's
+    // differences, and the linear weights over g3
+    double h1, h2;         // g1/g3, g2/g3
+    double q2;             // (g2/g3) p2 - (g2/g3) w0 = q2 (d_- + 2 d_+)
+    double q3[4];          // p3 - w0 = q3 . (the four differences of the stencil)
 };
 
-__device__ __forceinline__ double mr_weno5(double wm2, double wm1, double w0, double wp1, double wp2,
-                                           const Weno& c) {
-    // candidate interface values
-    const double q2 = (-wm1 + 5.0 * w0 + 2.0 * wp1) * (1.0 / 6.0);
-    const double q3 = (2.0 * wm2 - 13.0 * wm1 + 47.0 * w0 + 27.0 * wp1 - 3.0 * wp2) * (1.0 / 60.0);
-    const double p1 = w0;
-    const double p2 = (q2 - c.g12 * p1) * c.ig22;
-    const double p3 = (q3 - c.g1 * p1 - c.g2 * p2) * c.ig3;
-    // smoothness: beta_1 from the two one-sided differences
-    const double dl = w0 - wm1, dr = wp1 - w0;
-    const double b1 = fmin(dl * dl, dr * dr);
-    // beta_2: sum_alpha int (d^alpha q)^2 of the quadratic on the cell
-    const double s2a = wm1 - 2.0 * w0 + wp1, s2b = wp1 - wm1;
-    const double b2 = (13.0 / 12.0) * s2a * s2a + 0.25 * s2b * s2b;
-    // beta_3: coefficients c1..c4 of the quartic q(x) = sum c_k x^k (unit cell
-    // centred at 0) whose cell averages are w_{-2..2}; odd part from
-    // o1 = (w1 - w-1)/2, o2 = (w2 - w-2)/2, even part from the means of w_{+-1} and
-    // w_{+-2} relative to w0 (beta ignores a constant added to the data, so everything is
-    // formed from differences: no rounding of |w|-sized terms in small indicators)
-    const double o1 = 0.5 * (wp1 - wm1), o2 = 0.5 * (wp2 - wm2);
-    const double a1 = 0.5 * ((wp1 - w0) + (wm1 - w0)), a2 = 0.5 * ((wp2 - w0) + (wm2 - w0));
-    const double c3 = (o2 - 2.0 * o1) * (1.0 / 6.0);
-    const double c1 = (34.0 * o1 - 5.0 * o2) * (1.0 / 24.0);
-    const double c4 = (a2 - 4.0 * a1) * (1.0 / 12.0);
-    const double c2 = (12.0 * a1 - a2) * 0.125;
-    // int_{-1/2}^{1/2} of (q')^2 + (q'')^2 + (q''')^2 + (q'''')^2 (int x^2 = 1/12, x^4 = 1/80,
-    // x^6 = 1/448), collected by monomial: c1^2 + c1 c3/2 + 13/3 c2^2 + 3129/80 c3^2
-    // + 21/5 c2 c4 + 87617/140 c4^2
-    const double b3 = c1 * (c1 + 0.5 * c3) + c2 * ((13.0 / 3.0) * c2 + 4.2 * c4) + (3129.0 / 80.0) * c3 * c3
-                    + (87617.0 / 140.0) * c4 * c4;
-    const double t = 0.5 * (fabs(b3 - b1) + fabs(b3 - b2));
-    const double tau = t * t;
-    // w~_l = g_l (1 + tau/(beta_l + eps)); scaled by (d1 d2 d3) to need one division
-    const double d1 = b1 + c.eps, d2 = b2 + c.eps, d3 = b3 + c.eps;
-    const double n1 = c.g1 * (d1 + tau) * (d2 * d3);
-    const double n2 = c.g2 * (d2 + tau) * (d1 * d3);
-    const double n3 = c.g3 * (d3 + tau) * (d1 * d2);
-    return div_nr(n1 * p1 + n2 * p2 + n3 * p3, n1 + n2 + n3);
+// p2 = (q_2 - g12 w0)/ig22^-1 and p3 = (q_3 - g1 w0 - g2 p2)/g3 with the 3- and 5-point interface values
+// q_2 - w0 = (d1 + 2 d2)/6 and q_3 - w0 = (-2 d0 + 11 d1 + 24 d2 - 3 d3)/60
+inline void weno_coefficients(Weno& w) {
+    w.h1 = w.g1 * w.ig3;
+    w.h2 = w.g2 * w.ig3;
+    w.q2 = w.h2 * w.ig22 / 6.0;
+    const double p2 = w.g2 * w.ig22 / 6.0;
+    w.q3[0] = -2.0 / 60.0 * w.ig3;
+    w.q3[1] = (11.0 / 60.0 - p2) * w.ig3;
+    w.q3[2] = (24.0 / 60.0 - 2.0 * p2) * w.ig3;
+    w.q3[3] = -3.0 / 60.0 * w.ig3;
 }
 
 // --------------------------------------------------------- index helpers

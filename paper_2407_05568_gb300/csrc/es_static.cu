@@ -121,6 +121,7 @@ extern "C" int es_rk3_step_static(const es_params* p, double dt, double* JU, dou
     P.weno.ig3 = gs / g3;
     P.weno.eps = p->weno_eps;
     P.weno.sign_tol = p->sign_tol;
+    weno_coefficients(P.weno);
     P.diss = p->dissipation;
     P.tile = p->tile > 0 ? p->tile - 1 : 0;
     P.status = status;
