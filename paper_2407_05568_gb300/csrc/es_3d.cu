@@ -221,7 +221,8 @@ struct Pencil {
     static constexpr int PL = 3 * LB + 6;               // pairs per line
     static constexpr int NP = W * PL;
     static constexpr int NF = W * (LB + 1);             // faces
-    static constexpr size_t SMEM = sizeof(double) * (size_t(S3_COUNT) * NB + 5 * NP + 6 * NF);
+    static constexpr int NJ = W * (LB + 5);             // entropy-variable jumps between neighbours
+    static constexpr size_t SMEM = sizeof(double) * (size_t(S3_COUNT) * NB + 5 * NP + 6 * NF + 5 * NJ);
 };
 
 template <int K, int LB, int W, int NT>
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
     double* S = smem;
     double* PB = S + S3_COUNT * NB;
     double* FB = PB + 5 * NP;
+    double* JB = FB + 6 * NFc;
     const Grid3& g = P.g;
     const int tid = threadIdx.x;
     const int nk = g.n[K];
@@ -310,7 +312,8 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
     }
     __syncthreads();
 
-    // ---- C: pair fluxes F(U_q, U_{q+m}), m = 1..3, q = 3-m .. LB+2 along each line
+    // ---- C: pair fluxes F(U_q, U_{q+m}), m = 1..3, q = 3-m .. LB+2 along each line, and the entropy variables' jumps
+    // between neighbours, q = 0 .. LB+4
     for (int t = tid; t < NP; t += NT) {
         const int line = t / PC::PL, kk = t % PC::PL;
         int m, q;
@@ -325,6 +328,13 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
         flux64::pair_flux<3>(S, NB, l, r, n, S[G_XT * NB + l] + S[G_XT * NB + r], P.gas, f);
 #pragma unroll
         for (int c = 0; c < 5; ++c) PB[c * NP + t] = f[c];
+    }
+    for (int t = tid; t < PC::NJ; t += NT) {
+        const int l = t / (LB + 5) * LS + t % (LB + 5);
+        double f[5];
+        flux64::entropy_jump<3>(S, NB, l, l + 1, f);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) JB[c * PC::NJ + t] = f[c];
     }
     __syncthreads();
 
@@ -355,7 +365,8 @@ __global__ void __launch_bounds__(NT, W >= 16 ? 1 : (NT <= 96 ? 3 : 2)) k3_dir(D
             double n[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) n[c] = S[(G_N + c) * NB + l] + S[(G_N + c) * NB + l + 1];
-            flux64::face_dissipation<3>(S, NB, l, 1, n, XT[0] + XT[1], P.gas, P.weno, F, P.status, 0);
+            flux64::face_dissipation<3>(S, NB, l, 1, n, XT[0] + XT[1], P.gas, P.weno, JB, PC::NJ,
+                                        line * (LB + 5) + q, F, P.status, 0);
         }
 #pragma unroll
         for (int c = 0; c < 5; ++c) FB[c * NFc + t] = F[c];

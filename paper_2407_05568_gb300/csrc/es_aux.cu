@@ -11,6 +11,7 @@
 #include "es_bits.cuh"
 #include "es_df.cuh"
 #include "es_device.cuh"
+#include "es_log64.cuh"
 
 namespace es {
 
@@ -847,5 +848,19 @@ extern "C" int es_selftest_division(const double* a, const double* b, double* q,
     if (!a || !b || !q || !r || n <= 0) return ES_ERR_ARG;
     const int64_t blocks = (n + 255) / 256;
     es::k_selftest_division<<<int(blocks < 4096 ? blocks : 4096), 256, 0, (cudaStream_t)stream>>>(a, b, q, r, n);
+    return cudaGetLastError() == cudaSuccess ? ES_OK : ES_ERR_CUDA;
+}
+
+namespace es {
+__global__ void k_selftest_log(const double* x, double* y, int64_t n) {
+    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+        y[i] = log_tab(x[i]);
+}
+}  // namespace es
+
+extern "C" int es_selftest_log(const double* x, double* y, int64_t n, void* stream) {
+    if (!x || !y || n <= 0) return ES_ERR_ARG;
+    const int64_t blocks = (n + 255) / 256;
+    es::k_selftest_log<<<int(blocks < 4096 ? blocks : 4096), 256, 0, (cudaStream_t)stream>>>(x, y, n);
     return cudaGetLastError() == cudaSuccess ? ES_OK : ES_ERR_CUDA;
 }

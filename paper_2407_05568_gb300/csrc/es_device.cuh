@@ -74,6 +74,7 @@ struct Weno {
     double h1, h2;         // g1/g3, g2/g3
     double q2;             // (g2/g3) p2 - (g2/g3) w0 = q2 (d_- + 2 d_+)
     double q3[4];          // p3 - w0 = q3 . (the four differences of the stencil)
+    double eps4;           // eps/4
 };
 
 // p2 = (q_2 - g12 w0)/ig22^-1 and p3 = (q_3 - g1 w0 - g2 p2)/g3 with the 3- and 5-point interface values
@@ -87,6 +88,7 @@ inline void weno_coefficients(Weno& w) {
     w.q3[1] = (11.0 / 60.0 - p2) * w.ig3;
     w.q3[2] = (24.0 / 60.0 - 2.0 * p2) * w.ig3;
     w.q3[3] = -3.0 / 60.0 * w.ig3;
+    w.eps4 = 0.25 * w.eps;
 }
 
 // --------------------------------------------------------- index helpers

@@ -8,7 +8,9 @@
 //   * quantities are formed in the products that the formulas need, not in the ones the paper prints (the ratio
 //     {a}/{a}^ln instead of 1/{a}^ln, p/rho instead of p, A = J xi_t {rho} + n . {rho v} once for both of its uses);
 //   * comparisons against constants, sign tests and minima of non-negative values use the bits of the numbers, and
-//     the sign switch's round-off test is decided in FP32 bounds wherever those are clear.
+//     the sign switch's round-off test is decided in FP32 bounds wherever those are clear;
+//   * the logarithms come from a table (es_log64.cuh), and the differences of the entropy variables that every face's
+//     reconstruction starts from are formed once per pair of neighbours.
 // Every product that feeds an addition is written as fma() or __dmul_rn(), so that the compiler has no choice of which
 // product to fuse and every tile shape gives the same bits.
 // Instructions on the FP64 pipe at a 2D pair: 140 before this form, 78 now; at a 2D face: about 1000 and 600.
@@ -16,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include "es_device.cuh"
+#include "es_log64.cuh"
 
 namespace es {
 namespace flux64 {
@@ -33,7 +36,7 @@ struct Slots {
         E0,         // |v|^2/(4T) + a rho/T
         RP,         // rho/(2p)
         W0, WE,     // half of the entropy variables V_1 and V_{D+2} = -1/T
-        LNR, LNOM, LNT, LNRP,   // half of the logarithms of rho, 1 - b rho, T and (up to a constant) rho/p
+        LNR, LNOM, LNT, LNRP,   // logarithms of rho, 1 - b rho, T and rho/p
         V,          // v_k/2
         VT = V + D, // v_k/(2T), half of the entropy variables between V_1 and V_{D+2}
         RV = VT + D,// rho v_k/2
@@ -66,26 +69,26 @@ __device__ __forceinline__ float abs_f(double x) {
 
 // ------------------------------------------------------------ logarithmic mean
 // With f = (a_l - a_r)/(a_l + a_r) and u = f^2: {a}/{a}^ln = artanh(f)/f = 1 + u/3 + u^2/5 + u^3/7 + ... and its
-// reciprocal 1 - u/3 - 4 u^2/45 - 44 u^3/945 - ...  Below |f| = 1e-2 (tested on the bits of f) the next terms,
-// u^4/9 and 0.03 u^4, are under 2^-56; above it the difference of the nodes' logarithms keeps its digits.
-__device__ __forceinline__ bool series_range(double f) {
-    return (__double2hiint(f) & 0x7fffffff) < 0x3f847ae1;            // the leading bits of 1e-2
-}
-// {a}/{a}^ln from f and the halves of ln a_l, ln a_r
-__device__ __forceinline__ double mean_over_logmean(double f, double hlnl, double hlnr) {
-    if (series_range(f)) {
+// reciprocal 1 - u/3 - 4 u^2/45 - 44 u^3/945 - ...  Below |f| = 1e-2 (tested on the leading bits of f) the next terms,
+// u^4/9 and 0.03 u^4, are under 2^-56; above it [[ln a]] = 2 artanh(f) from the nodes' logarithms keeps its digits.
+// (Logarithms formed only where a face needs them cost the nodes nothing, but the tiles on a shock then took 40% longer
+// than the others, and 200^2 nodes are one wave of tiles: 202 -> 260 us per stage.)
+constexpr int F_SERIES = 0x3f847ae1;                                  // 1e-2
+// {a}/{a}^ln
+__device__ __forceinline__ double mean_over_logmean(double f, double lnl, double lnr) {
+    if ((__double2hiint(f) & 0x7fffffff) < F_SERIES) {
         const double u = f * f;
         return fma(u, fma(u, fma(u, 1.0 / 7.0, 1.0 / 5.0), 1.0 / 3.0), 1.0);
     }
-    return div_nr(hlnl - hlnr, f);
+    return div_nr(lnl - lnr, f + f);
 }
-// {a}^ln from the mean m, the halved jump hd = (a_l - a_r)/2, f = hd/m and the halves of the logarithms
-__device__ __forceinline__ double logmean(double m, double hd, double f, double hlnl, double hlnr) {
-    if (series_range(f)) {
+// {a}^ln/{a}
+__device__ __forceinline__ double logmean_over_mean(double f, double lnl, double lnr) {
+    if ((__double2hiint(f) & 0x7fffffff) < F_SERIES) {
         const double u = f * f;
-        return m * fma(u, fma(u, fma(u, -44.0 / 945.0, -4.0 / 45.0), -1.0 / 3.0), 1.0);
+        return fma(u, fma(u, fma(u, -44.0 / 945.0, -4.0 / 45.0), -1.0 / 3.0), 1.0);
     }
-    return div_nr(hd, hlnl - hlnr);
+    return div_nr(f + f, lnl - lnr);
 }
 
 // ------------------------------------------------------------ node
@@ -116,8 +119,6 @@ __device__ __forceinline__ bool node_fields(const double* JU, double J, const Ga
     const double art = __dmul_rn(G.a * r, iT);             // a rho/(2T)
     const double E0 = fma(2.0, art, hke * iT);
     const double prho = fma(2.0 * hRiom, T, -(G.a * rho));  // p/rho
-    const double hlnr = half(log(rho)), hlnT = half(log(T));
-    const double hlnom = G.b > 0.0 ? half(log(om)) : 0.0;
     st(SL::RHO, r);
     st(SL::T, half(T));
     st(SL::OM, half(om));
@@ -127,13 +128,13 @@ __device__ __forceinline__ bool node_fields(const double* JU, double J, const Ga
     st(SL::E0, E0);
     st(SL::RP, half(rcp_nr(prho)));
     // V_1 = (e + p/rho)/T - s - |v|^2/(2T) with s = cv ln T + R ln((1 - b rho)/rho)
-    const double hs = fma(G.cv, hlnT, G.R * (hlnom - hlnr));
-    st(SL::W0, (fma(0.5, G.cv, hRiom) - hs) - E0);
+    const double lnr = log_tab(rho), lnT = log_tab(T), lnom = G.b > 0.0 ? log_tab(om) : 0.0;
+    st(SL::LNR, lnr);
+    st(SL::LNOM, lnom);
+    st(SL::LNT, lnT);
+    st(SL::LNRP, -log_tab(prho));
+    st(SL::W0, fma(-0.5 * G.cv, lnT, fma(-0.5 * G.R, lnom - lnr, fma(0.5, G.cv, hRiom) - E0)));
     st(SL::WE, -half(iT));
-    st(SL::LNR, hlnr);
-    st(SL::LNOM, hlnom);
-    st(SL::LNT, hlnT);
-    st(SL::LNRP, -half(log(prho)));
 #pragma unroll
     for (int k = 0; k < D; ++k) {
         st(SL::V + k, v[k]);
@@ -172,17 +173,17 @@ __device__ __forceinline__ void pair_flux(const double* S, int NB, int l, int r,
     }
     const double iD = rcp_nr(D1);
     const double g = mean(SL::G);
-    double vm[D], vT[D];
+    double vm[D];
     double A = xt * rm, B = xt, nv = 0.0;                  // J xi_t {rho} + n . {rho v}; J xi_t + n . {v}; n . {v/T}
     double sv = fma(G.cv, FT, -mean(SL::E0));              // {v/T} . {v} - B0, B0 = {|v|^2/T}/2 - cv {T}/{T}^ln + 2a {rho/T}
 #pragma unroll
     for (int k = 0; k < D; ++k) {
+        const double vT = mean(SL::VT + k);
         vm[k] = mean(SL::V + k);
-        vT[k] = mean(SL::VT + k);
         A = fma(n[k], mean(SL::RV + k), A);
         B = fma(n[k], vm[k], B);
-        nv = k == 0 ? n[k] * vT[k] : fma(n[k], vT[k], nv);
-        sv = fma(vT[k], vm[k], sv);
+        nv = k == 0 ? n[k] * vT : fma(n[k], vT, nv);
+        sv = fma(vT, vm[k], sv);
     }
     const double Q = fma(coef, A, g * B) * iD;             // the density component
     const double P = rm * Tm * g;
@@ -193,38 +194,50 @@ __device__ __forceinline__ void pair_flux(const double* S, int NB, int l, int r,
     out[D + 1] = fma(mean(SL::ART), A, fma(sv, Q, P * nv)) * (Tl * Tr * iT);
 }
 
+// Half of the entropy variables' jump V_r - V_l
+template <int D>
+__device__ __forceinline__ void entropy_jump(const double* S, int NB, int l, int r, double* dV) {
+    using SL = Slots<D>;
+#pragma unroll
+    for (int m = 0; m < D + 2; ++m) {
+        const int f = m == 0 ? SL::W0 : (m == D + 1 ? SL::WE : SL::VT + m - 1);
+        dV[m] = S[f * NB + r] - S[f * NB + l];
+    }
+}
+
 // ------------------------------------------------------------ MR-WENO5 (Sec. 3.3)
-// One side's reconstruction as numerator and denominator of (w_{i+1/2} - w_i): d0..d3 are the differences of the five
-// stencil values w_{-2} .. w_2 in order, b1 = min(d1^2, d2^2) the first indicator.  Everything is formed from
+// One side's reconstruction as numerator and denominator of (w_{i+1/2} - w_i)/2: d0..d3 are HALF the differences of the
+// five stencil values w_{-2} .. w_2 in order, k1 = min(d1^2, d2^2) + eps/4 the first indicator.  Everything is formed from
 // differences (the indicators ignore a constant added to the data).  With S = d1 + d2, Dd = d2 - d1 (first and second
 // difference of the 3-point stencil), G = (d0 + d3) - S and E = (d3 - d0) - 3 Dd (the odd and even parts that only
 // the 5-point stencil sees): beta_2 = 13/12 Dd^2 + S^2/4 and the quartic's integrals collect to
 //   beta_3 - beta_2 = E (4405/4032 E - 11/60 Dd) + G (89/320 G - S/12),
-// the difference that tau needs, without cancellation.  Weights g_k (1 + tau/(beta_k + eps)) with a common
-// denominator, over g_3.
-__device__ __forceinline__ void weno_side(double d0, double d1, double d2, double d3, double b1, const Weno& c,
+// the difference that tau needs, without cancellation.  Halved differences make every indicator a quarter, so that
+// with k = (beta + eps)/4 and t = |k_3 - k_1| + |k_3 - k_2| the weights g (1 + tau/(beta + eps)) are g (1 + t^2/k); over
+// the common denominator k1 k2 k3 they are g (k1 k2 k3 + t^2 k k'), taken over g_3.
+__device__ __forceinline__ void weno_side(double d0, double d1, double d2, double d3, double k1, const Weno& c,
                                           double& num, double& den) {
     const double s = d1 + d2, dd = d2 - d1;
     const double g = (d0 + d3) - s;
     const double e = fma(-3.0, dd, d3 - d0);
-    const double b2 = fma(0.25 * s, s, ((13.0 / 12.0) * dd) * dd);
+    const double k2 = fma(0.25 * s, s, fma((13.0 / 12.0) * dd, dd, c.eps4));
     const double q = fma(e, fma(4405.0 / 4032.0, e, (-11.0 / 60.0) * dd), g * fma(89.0 / 320.0, g, (-1.0 / 12.0) * s));
-    const double b3 = b2 + q;
-    const double t = fabs(b3 - b1) + fabs(q);               // 2 sqrt(tau)
+    const double k3 = k2 + q;
+    const double t = fabs(k3 - k1) + fabs(q);
     const double tt = t * t;
-    const double k1 = b1 + c.eps, k2 = b2 + c.eps, k3 = b3 + c.eps;
-    const double y1 = fma(0.25, tt, k1) * (k2 * k3);
-    const double y2 = fma(0.25, tt, k2) * (k1 * k3);
-    const double y3 = fma(0.25, tt, k3) * (k1 * k2);
+    const double k12 = k1 * k2, k123 = k12 * k3;
+    const double y1 = fma(tt, k2 * k3, k123);
+    const double y2 = fma(tt, k1 * k3, k123);
+    const double y3 = fma(tt, k12, k123);
     const double p2 = c.q2 * fma(2.0, d2, d1);
     const double p3 = fma(c.q3[0], d0, fma(c.q3[1], d1, fma(c.q3[2], d2, c.q3[3] * d3)));
     num = fma(y2, p2, y3 * p3);
     den = fma(c.h1, y1, fma(c.h2, y2, y3));
 }
 
-// w^+ - w^- at the face between the third and fourth of six values, from their five differences
+// (w^+ - w^-)/2 at the face between the third and fourth of six values, from half their five differences
 __device__ __forceinline__ double weno_jump(const double* d, const Weno& c) {
-    const double s1 = d[1] * d[1], s2 = d[2] * d[2], s3 = d[3] * d[3];
+    const double s1 = fma(d[1], d[1], c.eps4), s2 = fma(d[2], d[2], c.eps4), s3 = fma(d[3], d[3], c.eps4);
     double nm, dm, np, dp;
     weno_side(d[0], d[1], d[2], d[3], min_pos(s1, s2), c, nm, dm);
     weno_side(d[4], d[3], d[2], d[1], min_pos(s2, s3), c, np, dp);   // mirrored: the numerator changes sign
@@ -284,11 +297,13 @@ __device__ __forceinline__ Frame<D> face_frame(const double* n) {
 // ------------------------------------------------------------ face dissipation
 // F += -1/2 Lambda T^{-1} R Y [[W]]^WENO at the face between nodes l and l + step (Sec. 3.3, eq. HOstable): face state
 // rho = {rho}^ln, v = {v}, p = {rho}^ln/{rho/p}^ln; n, xtf the means of the nodes' metrics and J xi_t; R = R~ S in the
-// frame of the face normal; W = R^T T V at the six stencil nodes.  The entropy variables are stored halved, so the
-// scales S are doubled and Lambda/2 halved again.
+// frame of the face normal; W = R^T T V at the six stencil nodes, from the entropy variables' jumps between neighbours
+// along the line (JB[c * NJ + jq + o] = half of V_{l+o+1} - V_{l+o}, o = -2 .. 2).  They are halved, and with them W
+// and its reconstructed jump, so Lambda/2 becomes Lambda.
 template <int D>
 __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l, int step, const double* n, double xtf,
-                                                 const Gas& G, const Weno& Wc, double* F, DevStatus* st, int gidx) {
+                                                 const Gas& G, const Weno& Wc, const double* JB, int NJ, int jq, double* F,
+                                                 DevStatus* st, int gidx) {
     using SL = Slots<D>;
     constexpr int NC = D + 2;
     const int r = l + step;
@@ -296,8 +311,8 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
     double rho, z;                                          // {rho}^ln; p/rho + a rho
     {
         const double al = at(SL::RHO, l), ar = at(SL::RHO, r);
-        const double m = al + ar, hd = al - ar;
-        rho = logmean(m, hd, hd * rcp_nr(m), at(SL::LNR, l), at(SL::LNR, r));
+        const double m = al + ar;
+        rho = m * logmean_over_mean((al - ar) * rcp_nr(m), at(SL::LNR, l), at(SL::LNR, r));
     }
     double prho;                                            // p/rho = 1/{rho/p}^ln
     {
@@ -333,9 +348,9 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
     // H = (E + p)/rho = cv T - a rho + |v|^2/2 + p/rho, cv T = R T/delta
     const double H = fma(0.5, v2, fma(RT, G.idelta, fma(-G.a, rho, prho)));
     const double hm = __dmul_rn(c2 * om, G.idelta);                  // H less the entropy wave's last entry
-    // twice the scales: S_acoustic = sqrt(rho T/2)/c, S_entropy = sqrt(rho T) sqrt(delta z/w)/c, S_shear = sqrt(rho T)
+    // the scales: S_acoustic = sqrt(rho T/2)/c, S_entropy = sqrt(rho T) sqrt(delta z/w)/c, S_shear = sqrt(rho T)
     const double rT = rho * (RT * G.iR);
-    const double sT = (2.0 * rT) * rsqrt_nr(rT);
+    const double sT = rT * rsqrt_nr(rT);
     const double sTc = sT * ic;
     const double sA = 0.70710678118654752440 * sTc;
     const double dz = G.delta * z;
@@ -343,22 +358,14 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
     const double Lam = fma(L, c, fabs(fma(L, vn, xtf)));
     const double sAc = sA * c;
 
-    // differences of W = R^T T V along the stencil nodes l-2 .. l+3; with A = V_1 + v . V_v + H V_E and
+    // half the differences of W = R^T T V along the stencil nodes l-2 .. l+3; with A = V_1 + v . V_v + H V_E and
     // B = V_n + v_n V_E: W_acoustic = S (A -+ c B), W_entropy = S (A - hm V_E), W_shear = S (V_t + v_t V_E)
     double dW[NC][5];
-    double prev[NC];
-#pragma unroll
-    for (int m = 0; m < NC; ++m) prev[m] = at(m == 0 ? SL::W0 : (m == NC - 1 ? SL::WE : SL::VT + m - 1), l - 2 * step);
 #pragma unroll
     for (int o = 0; o < 5; ++o) {
-        const int q = l + (o - 1) * step;
         double d[NC];
 #pragma unroll
-        for (int m = 0; m < NC; ++m) {
-            const double v = at(m == 0 ? SL::W0 : (m == NC - 1 ? SL::WE : SL::VT + m - 1), q);
-            d[m] = v - prev[m];
-            prev[m] = v;
-        }
+        for (int m = 0; m < NC; ++m) d[m] = JB[m * NJ + jq + o - 2];
         double rv[D];
 #pragma unroll
         for (int a = 0; a < D; ++a) {
@@ -386,7 +393,8 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
     bool zero[NC];
     unsigned open = 0u;
     {
-        const float vs = abs_f(at(SL::W0, l)) + abs_f(at(SL::W0, r)), es = abs_f(at(SL::WE, l)) + abs_f(at(SL::WE, r));
+        const float vs = abs_f(at(SL::W0, l)) + abs_f(at(SL::W0, r));
+        const float es = abs_f(at(SL::WE, l)) + abs_f(at(SL::WE, r));
         float qs = 0.0f, vsum = 0.0f;
 #pragma unroll
         for (int k = 0; k < D; ++k) {
@@ -455,7 +463,7 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
                           (__double2hiint(jw) & 0x7fffffff) <= 0x7ff00000;
         y[m] = keep ? jw : 0.0;
     }
-    const double h = -0.25 * Lam;
+    const double h = -Lam;
     const double y0 = __dmul_rn(sA, y[0]), y1 = __dmul_rn(sE, y[1]), y4 = __dmul_rn(sA, y[NC - 1]);
     const double i0 = (y0 + y4) + y1;
     const double qc = c * (y4 - y0);

@@ -49,15 +49,21 @@ struct Tile {
     // direction.
     static constexpr size_t FIELDS = sizeof(double) * size_t(Slot<DIM>::COUNT) * NB;
     static constexpr int PAIRJ = ((NP1 + NP2) * NC > 4 * NB) ? (NP1 + NP2) * NC : 4 * NB;
-    static constexpr size_t SMEM_JOINT = FIELDS + sizeof(double) * (size_t(PAIRJ) + size_t(NF1 + NF2) * (NC + 1));
+    // entropy-variable jumps between neighbours along each line (box positions q, q + 1)
+    static constexpr int NJ1 = (DIM == 2 ? BY : 1) * (BX + 5);
+    static constexpr int NJ2 = DIM == 2 ? BX * (BY + 5) : 0;
+    static constexpr size_t SMEM_JOINT =
+        FIELDS + sizeof(double) * (size_t(PAIRJ) + size_t(NF1 + NF2) * (NC + 1) + size_t(NJ1 + NJ2) * NC);
     static constexpr bool JOINT = DIM == 2 && SMEM_JOINT <= 227 * 1024;
     // pair and face buffers: per-component strides and the offset of direction 2's entries
     static constexpr int PS = JOINT ? NP1 + NP2 : NP;
     static constexpr int FS = JOINT ? NF1 + NF2 : NF;
+    static constexpr int JS = JOINT ? NJ1 + NJ2 : (NJ1 > NJ2 ? NJ1 : NJ2);
     static constexpr int POFF2 = JOINT ? NP1 : 0;
     static constexpr int FOFF2 = JOINT ? NF1 : 0;
     static constexpr int PAIR_DOUBLES = JOINT ? PAIRJ : ((NP * NC > 4 * NB) ? NP * NC : 4 * NB);   // also holds coords
-    static constexpr size_t SMEM = FIELDS + sizeof(double) * (size_t(PAIR_DOUBLES) + size_t(FS) * (NC + 1));
+    static constexpr size_t SMEM =
+        FIELDS + sizeof(double) * (size_t(PAIR_DOUBLES) + size_t(FS) * (NC + 1) + size_t(JS) * NC);
     static constexpr int THREADS = NT;
     static_assert(NT >= BX * (DIM == 2 ? BY : 1) && NT % 32 == 0, "threads cover the tile");
 };
@@ -100,7 +106,8 @@ __device__ __forceinline__ void stage_coords(const StageParams& P, int gi, int g
                 as = fma(w, fma(cdt, xdk, P.xn[k * N + id]), as);
                 ad = fma(w, xdk, ad);
             }
-        xs[k] = fma(double(k == 0 ? ti.q : tj.q), P.period[k], as);
+        const int per = k == 0 ? ti.q : tj.q;
+        xs[k] = per != 0 ? fma(double(per), P.period[k], as) : as;
         xd[k] = ad;
     }
 }
@@ -142,14 +149,24 @@ __device__ __forceinline__ void pair_item(const double* S, int NB, const DirGeo<
 #pragma unroll
     for (int c = 0; c < DIM + 2; ++c) PB[c * ps + out] = f[c];
 }
+// the entropy variables' jump between box positions q and q + 1 of a line, q = 0 .. LB+4, item t; at JB[c * js + out]
+template <int DIM, int BX, int BY>
+__device__ __forceinline__ void jump_item(const double* S, int NB, const DirGeo<DIM, BX, BY>& d, int t, double* JB,
+                                          int js, int out) {
+    const int l = d.base(t / (d.LB + 5)) + t % (d.LB + 5) * d.step;
+    double f[DIM + 2];
+    flux64::entropy_jump<DIM>(S, NB, l, l + d.step, f);
+#pragma unroll
+    for (int c = 0; c < DIM + 2; ++c) JB[c * js + out] = f[c];
+}
 
 // ---- D: face flux at q+1/2, q = 2 .. LB+2 (box coordinates), item t of direction d: the 6th-order
 // combination of the direction's pairs (which start at PB[c * ps + poff]) plus the dissipation;
 // stored at FB[c * fs + out]
 template <int DIM, int BX, int BY>
 __device__ __forceinline__ void face_item(const double* S, int NB, const DirGeo<DIM, BX, BY>& d, int t,
-                                          const StageParams& P, const double* PB, int ps, int poff, double* FB,
-                                          int fs, int out) {
+                                          const StageParams& P, const double* PB, int ps, int poff, const double* JB,
+                                          int js, int joff, double* FB, int fs, int out) {
     constexpr int NC = DIM + 2;
     const int line = t / (d.LB + 1), f = t % (d.LB + 1);
     const int q = 2 + f;
@@ -179,7 +196,8 @@ __device__ __forceinline__ void face_item(const double* S, int NB, const DirGeo<
         double n[DIM];
 #pragma unroll
         for (int c = 0; c < DIM; ++c) n[c] = S[(d.fN + c) * NB + l] + S[(d.fN + c) * NB + r];
-        flux64::face_dissipation<DIM>(S, NB, l, d.step, n, XT[0] + XT[d.step], P.gas, P.weno, F, P.status, 0);
+        flux64::face_dissipation<DIM>(S, NB, l, d.step, n, XT[0] + XT[d.step], P.gas, P.weno, JB, js,
+                                      joff + line * (d.LB + 5) + q, F, P.status, 0);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) FB[c * fs + out] = F[c];
@@ -195,6 +213,7 @@ stage_kernel_fp64(StageParams P) {
     double* S = smem;                                   // COUNT * NB
     double* PB = smem + Slot<DIM>::COUNT * NB;                   // pair buffer (also the coordinates)
     double* FB = PB + TL::PAIR_DOUBLES;                 // face buffer (NC + 1) * FS
+    double* JB = FB + (NC + 1) * TL::FS;                // entropy-variable jumps NC * JS
     const int tid = threadIdx.x;
     const int ntx = (P.n1 + BX - 1) / BX;
     const int i0 = (blockIdx.x % ntx) * BX;
@@ -275,11 +294,15 @@ stage_kernel_fp64(StageParams P) {
             const bool two = t >= TL::NP1;
             pair_item<DIM, BX, BY>(S, NB, DirGeo<DIM, BX, BY>(two ? 1 : 0), two ? t - TL::NP1 : t, G, PB, TL::PS, t);
         }
+        for (int t = tid; t < TL::NJ1 + TL::NJ2; t += TL::THREADS) {
+            const bool two = t >= TL::NJ1;
+            jump_item<DIM, BX, BY>(S, NB, DirGeo<DIM, BX, BY>(two ? 1 : 0), two ? t - TL::NJ1 : t, JB, TL::JS, t);
+        }
         __syncthreads();
         for (int t = tid; t < TL::NF1 + TL::NF2; t += TL::THREADS) {
             const bool two = t >= TL::NF1;
             face_item<DIM, BX, BY>(S, NB, DirGeo<DIM, BX, BY>(two ? 1 : 0), two ? t - TL::NF1 : t, P, PB, TL::PS,
-                                   two ? TL::POFF2 : 0, FB, TL::FS, t);
+                                   two ? TL::POFF2 : 0, JB, TL::JS, two ? TL::NJ1 : 0, FB, TL::FS, t);
         }
         __syncthreads();
         if (tid < BX * BY) {
@@ -298,9 +321,11 @@ stage_kernel_fp64(StageParams P) {
             const DirGeo<DIM, BX, BY> d(k);
             for (int t = tid; t < d.nlines * d.per_line; t += TL::THREADS)
                 pair_item<DIM, BX, BY>(S, NB, d, t, G, PB, TL::PS, t);
+            for (int t = tid; t < d.nlines * (d.LB + 5); t += TL::THREADS)
+                jump_item<DIM, BX, BY>(S, NB, d, t, JB, TL::JS, t);
             __syncthreads();
             for (int t = tid; t < d.nlines * (d.LB + 1); t += TL::THREADS)
-                face_item<DIM, BX, BY>(S, NB, d, t, P, PB, TL::PS, 0, FB, TL::FS, t);
+                face_item<DIM, BX, BY>(S, NB, d, t, P, PB, TL::PS, 0, JB, TL::JS, 0, FB, TL::FS, t);
             __syncthreads();
             if (tid < BX * (DIM == 2 ? BY : 1)) {
                 const int line = k == 0 ? ty : tx;

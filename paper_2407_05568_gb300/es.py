@@ -73,6 +73,8 @@ def lib():
         L.es_time_stage.argtypes = [vp, vp, vp, vp, i, d, i, ctypes.POINTER(d)]
         L.es_selftest_division.argtypes = [vp, vp, vp, vp, ctypes.c_int64, vp]
         L.es_selftest_division.restype = ctypes.c_int
+        L.es_selftest_log.argtypes = [vp, vp, ctypes.c_int64, vp]
+        L.es_selftest_log.restype = ctypes.c_int
         L.es_selftest_mixed_arith.argtypes = [vp, vp, vp, vp, ctypes.c_int64, vp, vp, vp, vp, vp]
         L.es_selftest_mixed_arith.restype = ctypes.c_int
         L.es_selftest_peaks.argtypes = [ctypes.POINTER(d), ctypes.POINTER(d), vp]
@@ -419,6 +421,11 @@ def es_selftest_division(a, b, q, r, stream=None):
     """q = a / b and r = 1 / b with the library's FP64 division (float64 device arrays)."""
     _nn_rc(lib().es_selftest_division(_ptr(a, F64), _ptr(b, F64), _ptr(q, F64), _ptr(r, F64), a.numel(),
                                       _stream_handle(stream)), "es_selftest_division")
+
+
+def es_selftest_log(x, y, stream=None):
+    """y = ln x with the library's FP64 logarithm (float64 device arrays, x > 0)."""
+    _nn_rc(lib().es_selftest_log(_ptr(x, F64), _ptr(y, F64), x.numel(), _stream_handle(stream)), "es_selftest_log")
 
 
 def es_selftest_mixed_arith(x, f, a, b, stream=None):
