@@ -92,10 +92,16 @@ __device__ __forceinline__ double logmean_over_mean(double f, double lnl, double
 }
 
 // ------------------------------------------------------------ node
-// Fields of a node from its density, momentum and energy; st(slot, value) stores them.  false: inadmissible
+// Fields of a node from its density, momentum and energy; st(slot, value) stores them.  `parts` (a constant, or the same
+// for a warp): which of them, so that several warps can share a node's logarithms; PLAIN leaves V_1/2 without its
+// logarithms in W0 (v1_logs adds them).  false: inadmissible
 // (rho > 0, 1 - b rho > 0, T > 0, p > 0; the condition R T - 2 a rho (1 - b rho)^2 > 0 enters at the faces).
+enum { LOG_RHO = 1, LOG_OM = 2, LOG_T = 4, LOG_RP = 8, PLAIN = 16, ALL = 32 };
+__device__ __forceinline__ double v1_logs(double w0, double lnr, double lnom, double lnT, const Gas& G) {
+    return fma(-0.5 * G.cv, lnT, fma(-0.5 * G.R, lnom - lnr, w0));
+}
 template <int D, class ST>
-__device__ __forceinline__ bool node_fields(const double* JU, double J, const Gas& G, ST st) {
+__device__ __forceinline__ bool node_fields(const double* JU, double J, const Gas& G, ST st, int parts = ALL) {
     using SL = Slots<D>;
     const double iJ = rcp_nr(J);
     const double ihJ = half(iJ);
@@ -119,27 +125,30 @@ __device__ __forceinline__ bool node_fields(const double* JU, double J, const Ga
     const double art = __dmul_rn(G.a * r, iT);             // a rho/(2T)
     const double E0 = fma(2.0, art, hke * iT);
     const double prho = fma(2.0 * hRiom, T, -(G.a * rho));  // p/rho
-    st(SL::RHO, r);
-    st(SL::T, half(T));
-    st(SL::OM, half(om));
-    st(SL::IOM, iom);
-    st(SL::G, hRiom - art);
-    st(SL::ART, art);
-    st(SL::E0, E0);
-    st(SL::RP, half(rcp_nr(prho)));
-    // V_1 = (e + p/rho)/T - s - |v|^2/(2T) with s = cv ln T + R ln((1 - b rho)/rho)
-    const double lnr = log_tab(rho), lnT = log_tab(T), lnom = G.b > 0.0 ? log_tab(om) : 0.0;
-    st(SL::LNR, lnr);
-    st(SL::LNOM, lnom);
-    st(SL::LNT, lnT);
-    st(SL::LNRP, -log_tab(prho));
-    st(SL::W0, fma(-0.5 * G.cv, lnT, fma(-0.5 * G.R, lnom - lnr, fma(0.5, G.cv, hRiom) - E0)));
-    st(SL::WE, -half(iT));
+    double lnr = 0.0, lnT = 0.0, lnom = 0.0;
+    if (parts & (LOG_RHO | ALL)) st(SL::LNR, lnr = log_tab(rho));
+    if (parts & (LOG_OM | ALL)) st(SL::LNOM, lnom = G.b > 0.0 ? log_tab(om) : 0.0);
+    if (parts & (LOG_T | ALL)) st(SL::LNT, lnT = log_tab(T));
+    if (parts & (LOG_RP | ALL)) st(SL::LNRP, -log_tab(prho));
+    if (parts & (PLAIN | ALL)) {
+        st(SL::RHO, r);
+        st(SL::T, half(T));
+        st(SL::OM, half(om));
+        st(SL::IOM, iom);
+        st(SL::G, hRiom - art);
+        st(SL::ART, art);
+        st(SL::E0, E0);
+        st(SL::RP, half(rcp_nr(prho)));
+        // V_1 = (e + p/rho)/T - s - |v|^2/(2T) with s = cv ln T + R ln((1 - b rho)/rho)
+        const double w0 = fma(0.5, G.cv, hRiom) - E0;
+        st(SL::W0, parts & ALL ? v1_logs(w0, lnr, lnom, lnT, G) : w0);
+        st(SL::WE, -half(iT));
 #pragma unroll
-    for (int k = 0; k < D; ++k) {
-        st(SL::V + k, v[k]);
-        st(SL::VT + k, v[k] * iT);
-        st(SL::RV + k, m[k]);
+        for (int k = 0; k < D; ++k) {
+            st(SL::V + k, v[k]);
+            st(SL::VT + k, v[k] * iT);
+            st(SL::RV + k, m[k]);
+        }
     }
     return positive(rho) && positive(om) && positive(T) && positive(prho);
 }
@@ -295,20 +304,25 @@ __device__ __forceinline__ Frame<D> face_frame(const double* n) {
 }
 
 // ------------------------------------------------------------ face dissipation
-// F += -1/2 Lambda T^{-1} R Y [[W]]^WENO at the face between nodes l and l + step (Sec. 3.3, eq. HOstable): face state
-// rho = {rho}^ln, v = {v}, p = {rho}^ln/{rho/p}^ln; n, xtf the means of the nodes' metrics and J xi_t; R = R~ S in the
-// frame of the face normal; W = R^T T V at the six stencil nodes, from the entropy variables' jumps between neighbours
-// along the line (JB[c * NJ + jq + o] = half of V_{l+o+1} - V_{l+o}, o = -2 .. 2).  They are halved, and with them W
-// and its reconstructed jump, so Lambda/2 becomes Lambda.
+// -1/2 Lambda T^{-1} R Y [[W]]^WENO at the face between nodes l and r (Sec. 3.3, eq. HOstable): R = R~ S in the frame of
+// the face normal, W = R^T T V at the six stencil nodes.  The state and the scales of a face:
 template <int D>
-__device__ __forceinline__ void face_dissipation(const double* S, int NB, int l, int step, const double* n, double xtf,
-                                                 const Gas& G, const Weno& Wc, const double* JB, int NJ, int jq, double* F,
-                                                 DevStatus* st, int gidx) {
+struct Face {
+    Frame<D> fr;
+    double vr[D];               // {v} in the frame: normal, tangential
+    double c, H;                // sound speed, (E + p)/rho
+    double hm;                  // H less the entropy wave's last entry
+    double sA, sE, sT;          // scales of the acoustic, entropy and shear waves
+    double sAc, Lam;
+};
+// rho = {rho}^ln, v = {v}, p = {rho}^ln/{rho/p}^ln; n, xtf the means of the nodes' metrics and J xi_t
+template <int D>
+__device__ __forceinline__ Face<D> face_state(const double* S, int NB, int l, int r, const double* n, double xtf,
+                                              const Gas& G, DevStatus* st, int gidx) {
     using SL = Slots<D>;
-    constexpr int NC = D + 2;
-    const int r = l + step;
     auto at = [&](int f, int q) { return S[f * NB + q]; };
-    double rho, z;                                          // {rho}^ln; p/rho + a rho
+    Face<D> f;
+    double rho;
     {
         const double al = at(SL::RHO, l), ar = at(SL::RHO, r);
         const double m = al + ar;
@@ -321,7 +335,7 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
         prho = mean_over_logmean((al - ar) * im, at(SL::LNRP, l), at(SL::LNRP, r)) * im;
     }
     const double arho = G.a * rho;
-    z = fma(G.a, rho, prho);
+    const double z = fma(G.a, rho, prho);
     const double om = fma(-G.b, rho, 1.0);
     const double iom = rcp_nr(om);
     const double RT = z * om;
@@ -329,160 +343,202 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
     const double w = fma(-2.0 * arho, om, z);               // (R T - 2 a rho (1 - b rho)^2)/(1 - b rho)
     if (!positive(c2) || !positive(w) || !positive(om)) raise_error(st, ES_ERR_INADMISSIBLE, gidx);
     const double ic = rsqrt_nr(c2);
-    const double c = __dmul_rn(c2, ic);
-    const Frame<D> fr = face_frame<D>(n);
-    const double L = fr.L;
-    double vm[D], vr[D];                                    // velocity, and in the frame: normal, tangential
+    f.c = __dmul_rn(c2, ic);
+    f.fr = face_frame<D>(n);
+    double vm[D];
 #pragma unroll
     for (int k = 0; k < D; ++k) vm[k] = at(SL::V + k, l) + at(SL::V + k, r);
     double v2 = 0.0;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        vr[a] = fr.e[a][0] * vm[0];
+        f.vr[a] = f.fr.e[a][0] * vm[0];
 #pragma unroll
         for (int k = 1; k < D; ++k)
-            if (!(a == 1 && k == 2)) vr[a] = fma(fr.e[a][k], vm[k], vr[a]);
-        v2 = a == 0 ? vr[a] * vr[a] : fma(vr[a], vr[a], v2);
+            if (!(a == 1 && k == 2)) f.vr[a] = fma(f.fr.e[a][k], vm[k], f.vr[a]);
+        v2 = a == 0 ? f.vr[a] * f.vr[a] : fma(f.vr[a], f.vr[a], v2);
     }
-    const double vn = vr[0];
     // H = (E + p)/rho = cv T - a rho + |v|^2/2 + p/rho, cv T = R T/delta
-    const double H = fma(0.5, v2, fma(RT, G.idelta, fma(-G.a, rho, prho)));
-    const double hm = __dmul_rn(c2 * om, G.idelta);                  // H less the entropy wave's last entry
+    f.H = fma(0.5, v2, fma(RT, G.idelta, fma(-G.a, rho, prho)));
+    f.hm = __dmul_rn(c2 * om, G.idelta);
     // the scales: S_acoustic = sqrt(rho T/2)/c, S_entropy = sqrt(rho T) sqrt(delta z/w)/c, S_shear = sqrt(rho T)
     const double rT = rho * (RT * G.iR);
-    const double sT = rT * rsqrt_nr(rT);
-    const double sTc = sT * ic;
-    const double sA = 0.70710678118654752440 * sTc;
+    f.sT = rT * rsqrt_nr(rT);
+    const double sTc = f.sT * ic;
+    f.sA = 0.70710678118654752440 * sTc;
     const double dz = G.delta * z;
-    const double sE = sTc * (dz * rsqrt_nr(dz * w));
-    const double Lam = fma(L, c, fabs(fma(L, vn, xtf)));
-    const double sAc = sA * c;
+    f.sE = sTc * (dz * rsqrt_nr(dz * w));
+    f.Lam = fma(f.fr.L, f.c, fabs(fma(f.fr.L, f.vr[0], xtf)));
+    f.sAc = f.sA * f.c;
+    return f;
+}
 
-    // half the differences of W = R^T T V along the stencil nodes l-2 .. l+3; with A = V_1 + v . V_v + H V_E and
-    // B = V_n + v_n V_E: W_acoustic = S (A -+ c B), W_entropy = S (A - hm V_E), W_shear = S (V_t + v_t V_E)
+// W = R^T T d for one difference d of the entropy variables: with A = d_1 + v . d_v + H d_E and B = d_n + v_n d_E,
+// W_acoustic = S (A -+ c B), W_entropy = S (A - hm d_E), W_shear = S (d_t + v_t d_E).  MASK: the waves wanted
+template <int D>
+__device__ __forceinline__ void project(const Face<D>& f, const double* d, double* W, unsigned mask = ~0u) {
+    constexpr int NC = D + 2;
+    double rv[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        rv[a] = f.fr.e[a][0] * d[1];
+#pragma unroll
+        for (int k = 1; k < D; ++k)
+            if (!(a == 1 && k == 2)) rv[a] = fma(f.fr.e[a][k], d[1 + k], rv[a]);
+    }
+    const double dE = d[NC - 1];
+    double A = fma(f.H, dE, d[0]);
+#pragma unroll
+    for (int a = 0; a < D; ++a) A = fma(f.vr[a], rv[a], A);
+    const double B = fma(f.vr[0], dE, rv[0]);
+    const double sa = f.sA * A;
+    if (mask & 1u) W[0] = fma(-f.sAc, B, sa);
+    if (mask & 2u) W[1] = __dmul_rn(f.sE, fma(-f.hm, dE, A));
+#pragma unroll
+    for (int a = 1; a < D; ++a)
+        if (mask & (2u << a)) W[1 + a] = __dmul_rn(f.sT, fma(f.vr[a], dE, rv[a]));
+    if (mask & (1u << (NC - 1))) W[NC - 1] = fma(f.sAc, B, sa);
+}
+
+// The sign switch takes a plain jump within sign_tol of sum_a |R_am| (|(TV_l)_a| + |(TV_r)_a|), the size of the terms
+// that form W_m, for round-off of zero.  That size lies between the FP32 bounds below (the terms of V_1 and V_E, which
+// dominate it, and those plus a bound on the velocity terms); only a jump between them needs it.
+struct SwitchBounds {
+    float vs, es, qs, vsum, c, tol, H, vc, hm;
+};
+template <int D>
+__device__ __forceinline__ SwitchBounds switch_bounds(const Face<D>& f, const double* S, int NB, int l, int r,
+                                                      const Weno& Wc) {
+    using SL = Slots<D>;
+    auto at = [&](int k, int q) { return abs_f(S[k * NB + q]); };
+    SwitchBounds b;
+    b.vs = at(SL::W0, l) + at(SL::W0, r);
+    b.es = at(SL::WE, l) + at(SL::WE, r);
+    b.qs = b.vsum = 0.0f;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        b.qs += at(SL::VT + k, l) + at(SL::VT + k, r);
+        b.vsum += abs_f(f.vr[k]);
+    }
+    b.c = abs_f(f.c);
+    b.tol = abs_f(Wc.sign_tol) * 1.00001f;
+    b.H = abs_f(f.H);
+    b.vc = abs_f(f.vr[0]) * b.c;
+    b.hm = abs_f(f.hm);
+    return b;
+}
+// is the jump j of wave m zero: 0 no, 1 yes, 2 between the bounds (or out of FP32's range)
+template <int D>
+__device__ __forceinline__ int jump_is_zero(const SwitchBounds& b, const Face<D>& f, int m, double j) {
+    const bool shear = m >= 2 && m <= D;
+    // |last entry of R| >= | |H| - |rest| |, <= |H| + |rest|
+    const float rest = m == 1 ? b.hm : b.vc;
+    const float scale = abs_f(m == 1 ? f.sE : (shear ? f.sT : f.sA)) * b.tol;
+    float lo, hi;
+    if (shear) {
+        lo = scale * ((abs_f(f.vr[m < D + 1 ? m - 1 : 0]) + b.c) * b.es);
+        hi = lo + scale * b.qs;
+    } else {
+        lo = scale * (b.vs + fabsf(b.H - rest) * b.es);
+        hi = scale * (b.vs + (b.H + rest) * b.es + (b.vsum + b.c) * b.qs);
+    }
+    const float ja = abs_f(j);
+    // (factors: truncation and rounding of the FP32 values)
+    if ((ja * 1.0001f < lo * 0.99f && ja > 0.0f) || (__double_as_longlong(j) << 1) == 0) return 1;
+    return ja > hi * 1.001f ? 0 : 2;
+}
+// the size itself
+template <int D>
+__device__ __forceinline__ double jump_size(const Face<D>& f, const double* S, int NB, int l, int r, int m) {
+    using SL = Slots<D>;
+    auto at = [&](int k, int q) { return S[k * NB + q]; };
+    double tv[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        double tl = 0.0, tr = 0.0;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            tl = fma(f.fr.e[a][k], at(SL::VT + k, l), tl);
+            tr = fma(f.fr.e[a][k], at(SL::VT + k, r), tr);
+        }
+        tv[a] = fabs(tl) + fabs(tr);
+    }
+    const double e2 = fabs(at(SL::WE, l)) + fabs(at(SL::WE, r));
+    if (m >= 2 && m <= D)                                   // velocity round-off scales with |v_t| + c
+        return f.sT * fma(fabs(f.vr[m < D + 1 ? m - 1 : 0]) + f.c, e2, tv[m < D + 1 ? m - 1 : 0]);
+    double common = fabs(at(SL::W0, l)) + fabs(at(SL::W0, r));
+#pragma unroll
+    for (int a = 1; a < D; ++a) common = fma(fabs(f.vr[a]), tv[a], common);
+    const double vn = f.vr[0];
+    const double u = m == 0 ? vn - f.c : (m == 1 ? vn : vn + f.c);
+    const double h = m == 0 ? fma(-vn, f.c, f.H) : (m == 1 ? f.H - f.hm : fma(vn, f.c, f.H));
+    return (m == 1 ? f.sE : f.sA) * fma(fabs(u), tv[0], fma(fabs(h), e2, common));
+}
+// Y [[W]]^WENO: kept where the reconstruction's jump has the sign of the plain jump j (a NaN jump is dropped)
+__device__ __forceinline__ double switched(double jw, double j, bool zero) {
+    const bool keep = !zero && (__double2hiint(jw) ^ __double2hiint(j)) >= 0 &&
+                      (__double2hiint(jw) & 0x7fffffff) <= 0x7ff00000;
+    return keep ? jw : 0.0;
+}
+
+// F += the dissipation of the face between nodes l and l + step, from the entropy variables' jumps between neighbours
+// along the line (JB[c * NJ + jq + o] = half of V_{l+o+1} - V_{l+o}, o = -2 .. 2).  They are halved, and with them W
+// and its reconstructed jump, so Lambda/2 becomes Lambda.
+template <int D>
+__device__ __forceinline__ void face_dissipation(const double* S, int NB, int l, int step, const double* n, double xtf,
+                                                 const Gas& G, const Weno& Wc, const double* JB, int NJ, int jq, double* F,
+                                                 DevStatus* st, int gidx) {
+    constexpr int NC = D + 2;
+    const int r = l + step;
+    const Face<D> f = face_state<D>(S, NB, l, r, n, xtf, G, st, gidx);
     double dW[NC][5];
 #pragma unroll
     for (int o = 0; o < 5; ++o) {
-        double d[NC];
+        double d[NC], W[NC];
 #pragma unroll
         for (int m = 0; m < NC; ++m) d[m] = JB[m * NJ + jq + o - 2];
-        double rv[D];
+        project<D>(f, d, W);
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            rv[a] = fr.e[a][0] * d[1];
-#pragma unroll
-            for (int k = 1; k < D; ++k)
-                if (!(a == 1 && k == 2)) rv[a] = fma(fr.e[a][k], d[1 + k], rv[a]);
-        }
-        const double dE = d[NC - 1];
-        double A = fma(H, dE, d[0]);
-#pragma unroll
-        for (int a = 0; a < D; ++a) A = fma(vr[a], rv[a], A);
-        const double B = fma(vn, dE, rv[0]);
-        const double sa = sA * A;
-        dW[0][o] = fma(-sAc, B, sa);
-        dW[1][o] = __dmul_rn(sE, fma(-hm, dE, A));
-#pragma unroll
-        for (int a = 1; a < D; ++a) dW[1 + a][o] = __dmul_rn(sT, fma(vr[a], dE, rv[a]));
-        dW[NC - 1][o] = fma(sAc, B, sa);
+        for (int m = 0; m < NC; ++m) dW[m][o] = W[m];
     }
-
-    // The sign switch takes a plain jump within sign_tol of sum_a |R_am| (|(TV_l)_a| + |(TV_r)_a|), the size of the
-    // terms that form W_m, for round-off of zero.  That size lies between the FP32 bounds below (the terms of V_1 and
-    // V_E, which dominate it, and those plus a bound on the velocity terms); only a jump between them needs it.
     bool zero[NC];
     unsigned open = 0u;
     {
-        const float vs = abs_f(at(SL::W0, l)) + abs_f(at(SL::W0, r));
-        const float es = abs_f(at(SL::WE, l)) + abs_f(at(SL::WE, r));
-        float qs = 0.0f, vsum = 0.0f;
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-            qs += abs_f(at(SL::VT + k, l)) + abs_f(at(SL::VT + k, r));
-            vsum += abs_f(vr[k]);
-        }
-        const float cf = abs_f(c), tol = abs_f(Wc.sign_tol) * 1.00001f;
-        const float Hf = abs_f(H), vc = abs_f(vn) * cf, hf = abs_f(hm);
+        const SwitchBounds b = switch_bounds<D>(f, S, NB, l, r, Wc);
 #pragma unroll
         for (int m = 0; m < NC; ++m) {
-            const double j = dW[m][2];
-            const bool shear = m >= 2 && m <= D;
-            // |last entry of R| >= | |H| - |rest| |, <= |H| + |rest|
-            const float rest = m == 1 ? hf : vc;
-            const float scale = abs_f(m == 1 ? sE : (shear ? sT : sA)) * tol;
-            float lo, hi;
-            if (shear) {
-                lo = scale * ((abs_f(vr[m < D + 1 ? m - 1 : 0]) + cf) * es);
-                hi = lo + scale * qs;
-            } else {
-                lo = scale * (vs + fabsf(Hf - rest) * es);
-                hi = scale * (vs + (Hf + rest) * es + (vsum + cf) * qs);
-            }
-            const float ja = abs_f(j);
-            // (factors: truncation and rounding of the FP32 values)
-            const bool small = ja * 1.0001f < lo * 0.99f && ja > 0.0f;
-            zero[m] = small || (__double_as_longlong(j) << 1) == 0;
-            if (!zero[m] && !(ja > hi * 1.001f)) open |= 1u << m;
+            const int is = jump_is_zero<D>(b, f, m, dW[m][2]);
+            zero[m] = is == 1;
+            open |= is == 2 ? 1u << m : 0u;
         }
     }
-    if (open != 0u) {                                       // between the bounds, or out of FP32's range
-        double tv[D];
+    if (open != 0u) {
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            double tl = 0.0, tr = 0.0;
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-                tl = fma(fr.e[a][k], at(SL::VT + k, l), tl);
-                tr = fma(fr.e[a][k], at(SL::VT + k, r), tr);
-            }
-            tv[a] = fabs(tl) + fabs(tr);
-        }
-        const double e2 = fabs(at(SL::WE, l)) + fabs(at(SL::WE, r));
-        double common = fabs(at(SL::W0, l)) + fabs(at(SL::W0, r));
-#pragma unroll
-        for (int a = 1; a < D; ++a) common = fma(fabs(vr[a]), tv[a], common);
-#pragma unroll
-        for (int m = 0; m < NC; ++m) {
-            double size;
-            if (m >= 2 && m <= D) {                         // velocity round-off scales with |v_t| + c
-                size = sT * fma(fabs(vr[m < D + 1 ? m - 1 : 0]) + c, e2, tv[m < D + 1 ? m - 1 : 0]);
-            } else {
-                const double u = m == 0 ? vn - c : (m == 1 ? vn : vn + c);
-                const double h = m == 0 ? fma(-vn, c, H) : (m == 1 ? H - hm : fma(vn, c, H));
-                size = (m == 1 ? sE : sA) * fma(fabs(u), tv[0], fma(fabs(h), e2, common));
-            }
-            if ((open >> m) & 1u) zero[m] = fabs(dW[m][2]) <= Wc.sign_tol * size;
-        }
+        for (int m = 0; m < NC; ++m)
+            if ((open >> m) & 1u) zero[m] = fabs(dW[m][2]) <= Wc.sign_tol * jump_size<D>(f, S, NB, l, r, m);
     }
     double y[NC];
 #pragma unroll
-    for (int m = 0; m < NC; ++m) {
-        const double jw = weno_jump(dW[m], Wc);
-        // kept where the reconstruction's jump has the sign of the plain jump (a NaN jump is dropped)
-        const bool keep = !zero[m] && (__double2hiint(jw) ^ __double2hiint(dW[m][2])) >= 0 &&
-                          (__double2hiint(jw) & 0x7fffffff) <= 0x7ff00000;
-        y[m] = keep ? jw : 0.0;
-    }
-    const double h = -Lam;
-    const double y0 = __dmul_rn(sA, y[0]), y1 = __dmul_rn(sE, y[1]), y4 = __dmul_rn(sA, y[NC - 1]);
+    for (int m = 0; m < NC; ++m) y[m] = switched(weno_jump(dW[m], Wc), dW[m][2], zero[m]);
+    const double h = -f.Lam, vn = f.vr[0];
+    const double y0 = __dmul_rn(f.sA, y[0]), y1 = __dmul_rn(f.sE, y[1]), y4 = __dmul_rn(f.sA, y[NC - 1]);
     const double i0 = (y0 + y4) + y1;
-    const double qc = c * (y4 - y0);
+    const double qc = f.c * (y4 - y0);
     double in[D];                                            // the momentum increment in the frame
     in[0] = fma(vn, i0, qc);
-    double iE = fma(vn, qc, fma(H, i0, -(hm * y1)));
+    double iE = fma(vn, qc, fma(f.H, i0, -(f.hm * y1)));
 #pragma unroll
     for (int a = 1; a < D; ++a) {
-        const double ys = __dmul_rn(sT, y[1 + a]);
-        in[a] = fma(vr[a], i0, ys);
-        iE = fma(vr[a], ys, iE);
+        const double ys = __dmul_rn(f.sT, y[1 + a]);
+        in[a] = fma(f.vr[a], i0, ys);
+        iE = fma(f.vr[a], ys, iE);
     }
     F[0] = fma(h, i0, F[0]);
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-        double t = fr.e[0][k] * in[0];
+        double t = f.fr.e[0][k] * in[0];
 #pragma unroll
         for (int a = 1; a < D; ++a)
-            if (!(a == 1 && k == 2)) t = fma(fr.e[a][k], in[a], t);
+            if (!(a == 1 && k == 2)) t = fma(f.fr.e[a][k], in[a], t);
         F[1 + k] = fma(h, t, F[1 + k]);
     }
     F[NC - 1] = fma(h, iE, F[NC - 1]);

@@ -368,6 +368,177 @@ stage_kernel_fp64(StageParams P) {
     }
 }
 
+// --------------------------------------------------------- short 1D lines
+// A 1D line with few nodes is one warp's chain of dependent work, whatever its width: each of an SM's four schedulers
+// issues one FP64 warp instruction per 64 cycles, so a tile of 8 nodes whose face phase runs on one warp (about 800
+// instructions from load to store) takes 27 us, and a tile of 254 nodes on one SM 62 us.  Here a tile of 8 nodes is
+// shared by the four warps of a CTA, one per scheduler: the node fields with one logarithm each, then the pairs on one
+// warp beside the entropy variables' jumps on another, then one wave of the faces per warp (two lanes a face, one
+// reconstruction each) beside the EC combination on the fourth, about 300 instructions.
+constexpr int LINE = 8;                       // nodes of a tile
+constexpr int LINE_NB = LINE + 6, LINE_NP = 3 * LINE + 6, LINE_NF = LINE + 1, LINE_NJ = LINE + 5;
+static_assert(LINE_NP <= 32 && 2 * LINE_NF <= 32 && LINE_NB <= 32, "a phase is one pass of a warp");
+
+__global__ void __launch_bounds__(128) stage_line_fp64(StageParams P) {
+    using SL = flux64::Slots<1>;
+    constexpr int XT = SL::COUNT;             // half of J xi_t (the metric is 1)
+    constexpr int NB = LINE_NB;
+    __shared__ double S[(SL::COUNT + 1) * NB];
+    __shared__ double PB[3 * LINE_NP], JB[3 * LINE_NJ];
+    __shared__ double FB[4][3][LINE_NF];      // a wave's dissipation per warp, and the EC flux
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i0 = blockIdx.x * LINE;
+    const int n = P.n1;
+    const double dt = P.dt_dev ? *P.dt_dev : P.dt_host;
+    if (P.mode == 0 && dt == 0.0) return;     // finished run: leave the state untouched
+    const Gas& G = P.gas;
+
+    // ---- A: node fields, a logarithm per warp
+    if (lane < NB) {
+        const int gi = i0 - 3 + lane;
+        const int si = state_index(gi, n, P.bc[0]);
+        double JU[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) JU[c] = P.JUs[size_t(c) * n + si];
+        if ((gi < 0 || gi >= n) && end_mirrored(P.bc[0], gi < 0)) JU[1] = -JU[1];
+        const int parts = warp == 0 ? flux64::LOG_RHO : (warp == 1 ? flux64::LOG_OM | flux64::PLAIN
+                                                         : (warp == 2 ? flux64::LOG_T : flux64::LOG_RP));
+        const bool ok = flux64::node_fields<1>(JU, P.Js[si], G, [&](int f, double v) { S[f * NB + lane] = v; }, parts);
+        if (!ok && warp == 0) raise_error(P.status, ES_ERR_INADMISSIBLE, si);
+        if (warp == 0) {
+            double xd = 0.0;
+            if (P.xdot) {
+                const GhostTerms t = ghost_terms(gi, n, P.bc[0]);
+                xd = t.w[0] * P.xdot[t.idx[0]];
+                if (t.nterm > 1) xd = fma(t.w[1], P.xdot[t.idx[1]], xd);
+            }
+            S[XT * NB + lane] = -0.5 * xd;
+        }
+    }
+    __syncthreads();
+
+    // ---- C: pairs on warp 0; the entropy variables and their jumps on warp 1
+    if (warp == 0 && lane < LINE_NP) {
+        int m, q;
+        if (lane < LINE + 1) { m = 1; q = 2 + lane; }
+        else if (lane < 2 * LINE + 3) { m = 2; q = lane - LINE; }
+        else { m = 3; q = lane - 2 * LINE - 3; }
+        const double one = 1.0;
+        double f[3];
+        flux64::pair_flux<1>(S, NB, q, q + m, &one, S[XT * NB + q] + S[XT * NB + q + m], G, f);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) PB[c * LINE_NP + lane] = f[c];
+    } else if (warp == 1) {
+        if (lane < NB)
+            S[SL::W0 * NB + lane] = flux64::v1_logs(S[SL::W0 * NB + lane], S[SL::LNR * NB + lane],
+                                                    S[SL::LNOM * NB + lane], S[SL::LNT * NB + lane], G);
+        __syncwarp();
+        if (lane < LINE_NJ) {
+            double d[3];
+            flux64::entropy_jump<1>(S, NB, lane, lane + 1, d);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) JB[c * LINE_NJ + lane] = d[c];
+        }
+    }
+    __syncthreads();
+
+    // ---- D: faces q + 1/2, q = 2 .. LINE + 2: wave `warp` of each (two lanes: the reconstructions from the left and from
+    // the right), and on the last warp the 6th-order combination of the pairs
+    double FJ = 0.0;
+    if (warp == 3) {
+        if (lane < LINE_NF) {
+            double F[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int m = 1; m <= 3; ++m) {
+                const int off = m == 1 ? 0 : (m == 2 ? LINE + 1 : 2 * LINE + 3);
+                const double al = ec_alpha(m);
+#pragma unroll
+                for (int s = 0; s < m; ++s)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        F[c] = fma(c == 2 ? 4.0 * al : al, PB[c * LINE_NP + off + lane + m - 1 - s], F[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) FB[3][c][lane] = F[c];
+        }
+    } else if (P.diss) {
+        const int face = lane >> 1 < LINE_NF ? lane >> 1 : LINE_NF - 1;         // (idle lanes repeat the last face)
+        const bool right = lane & 1;
+        const int l = 2 + face;
+        const double one = 1.0;
+        const flux64::Face<1> f =
+            flux64::face_state<1>(S, NB, l, l + 1, &one, S[XT * NB + l] + S[XT * NB + l + 1], G, P.status, 0);
+        double d[5];
+#pragma unroll
+        for (int o = 0; o < 5; ++o) {
+            const double dv[3] = {JB[l + o - 2], JB[LINE_NJ + l + o - 2], JB[2 * LINE_NJ + l + o - 2]};
+            double W[3] = {0.0, 0.0, 0.0};
+            flux64::project<1>(f, dv, W, 1u << warp);
+            d[o] = warp == 0 ? W[0] : (warp == 1 ? W[1] : W[2]);
+        }
+        const double s2 = fma(d[2], d[2], P.weno.eps4);
+        const double sx = right ? d[3] : d[1];
+        double num, den;
+        flux64::weno_side(right ? d[4] : d[0], sx, d[2], right ? d[1] : d[3],
+                          flux64::min_pos(fma(sx, sx, P.weno.eps4), s2), P.weno, num, den);
+        const double part = num * rcp_nr(den);
+        const double other = __shfl_xor_sync(0xffffffffu, part, 1);
+        const double jw = d[2] - (part + other);
+        const flux64::SwitchBounds b = flux64::switch_bounds<1>(f, S, NB, l, l + 1, P.weno);
+        const int is = flux64::jump_is_zero<1>(b, f, warp, d[2]);
+        bool zero = is == 1;
+        if (is == 2) zero = fabs(d[2]) <= P.weno.sign_tol * flux64::jump_size<1>(f, S, NB, l, l + 1, warp);
+        const double y = -f.Lam * ((warp == 1 ? f.sE : f.sA) * flux64::switched(jw, d[2], zero));
+        const double vn = f.vr[0], c = warp == 0 ? -f.c : (warp == 1 ? 0.0 : f.c);
+        if (!right && lane >> 1 < LINE_NF) {
+            FB[warp][0][face] = y;
+            FB[warp][1][face] = f.fr.e[0][0] * ((vn + c) * y);
+            FB[warp][2][face] = (warp == 1 ? f.H - f.hm : fma(vn, c, f.H)) * y;
+        }
+    }
+    __syncthreads();
+
+    // ---- E: divergence and the Shu-Osher combination on warp 0, a face per lane
+    if (warp != 0) return;
+    double F[4] = {0.0, 0.0, 0.0, 0.0};
+    if (lane < LINE_NF) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            F[c] = P.diss ? FB[3][c][lane] + ((FB[0][c][lane] + FB[2][c][lane]) + FB[1][c][lane]) : FB[3][c][lane];
+        // sum_m alpha_m sum of the pairs' mean J xi_t, collected by node
+        const double* X = S + XT * NB + 2 + lane;
+        const double a3 = ec_alpha(3), a2 = ec_alpha(2) + a3, a1 = ec_alpha(1) + a2;
+        FJ = fma(a1, X[0] + X[1], fma(a2, X[-1] + X[2], a3 * (X[-2] + X[3])));
+    }
+    F[3] = FJ;
+    double acc[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = (F[c] - __shfl_down_sync(0xffffffffu, F[c], 1)) * P.inv_dxi[0];
+    const int gi = i0 + lane;
+    if (lane >= LINE || gi >= n) return;
+    if (P.mode == 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) P.JUo[size_t(c) * n + gi] = acc[c];
+        P.Jo[gi] = acc[3];
+        return;
+    }
+    double un[4], us[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        un[c] = c < 3 ? P.JUn[size_t(c) * n + gi] : P.Jn[gi];
+        us[c] = c < 3 ? P.JUs[size_t(c) * n + gi] : P.Js[gi];
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const double v = fma(P.ca, un[c], P.cb * fma(dt, acc[c], us[c]));
+        if (c < 3) P.JUo[size_t(c) * n + gi] = v;
+        else {
+            P.Jo[gi] = v;
+            if (!(v > 0.0)) raise_error(P.status, ES_ERR_MESH, gi);
+        }
+    }
+}
+
 // ----------------------------------------------------------------- launch
 template <int DIM, int BX, int BY, int NT>
 static cudaError_t prepare_tile() {
@@ -386,9 +557,13 @@ static cudaError_t launch_tile(const StageParams& P, cudaStream_t s) {
 
 // 2D shapes: 32 x 8 nodes with 288 threads (= the 32 x 9 faces of xi_2), 25 x 11 with 384
 // (25 x 12 = 300 faces; 8 x 19 = 152 tiles cover 200 x 200 in one wave on 152 SMs), 16 x 16
-// with 288 (272 faces), 32 x 12 with 416 (416 faces; less halo per node), 20 x 10 with 224.  1D: 254 nodes, 256 threads (255 faces, 768 pairs = three passes).
+// with 288 (272 faces), 32 x 12 with 416 (416 faces; less halo per node), 20 x 10 with 224.  1D: by the line's length
+// (launch_stage_fp64).
 cudaError_t stage_prepare_fp64(int dim) {
-    if (dim == 1) return prepare_tile<1, 254, 1, 256>();
+    if (dim == 1) {
+        cudaError_t e1 = prepare_tile<1, 254, 1, 256>();
+        return e1 == cudaSuccess ? prepare_tile<1, 62, 1, 128>() : e1;
+    }
     cudaError_t e = prepare_tile<2, 32, 8, 288>();
     if (e == cudaSuccess) e = prepare_tile<2, 25, 11, 384>();
     if (e == cudaSuccess) e = prepare_tile<2, 16, 16, 288>();
@@ -398,7 +573,19 @@ cudaError_t stage_prepare_fp64(int dim) {
 }
 
 cudaError_t launch_stage_fp64(const StageParams& P, cudaStream_t s) {
-    if (P.dim == 1) return launch_tile<1, 254, 1, 256>(P, s);
+    if (P.dim == 1) {
+        // measured per stage launch (us), 8-node lines / 62-node tiles / 254-node tiles: 200 nodes 16.4 / 28.7 / 61.5,
+        // 1600 20.5 / 28.7 / 62.5, 6400 49.2 / 28.7 / 63.5, 25600 164 / 47.2 / 61.5, 102400 621 / 176 / 172.  A line is
+        // spread over an SM's four schedulers, so it pays while an SM has two of them or fewer (152 SMs x 2 x 8 nodes);
+        // 62-node tiles (faces, pairs and nodes two, six and two full warps of four) while the 254-node ones, which
+        // repeat less of the halo, leave SMs idle
+        if (P.n1 <= 2 * 152 * LINE) {
+            stage_line_fp64<<<(P.n1 + LINE - 1) / LINE, 128, 0, s>>>(P);
+            return cudaGetLastError();
+        }
+        if (P.n1 <= 1 << 16) return launch_tile<1, 62, 1, 128>(P, s);
+        return launch_tile<1, 254, 1, 256>(P, s);
+    }
     switch (P.tile) {
         case 1: return launch_tile<2, 25, 11, 384>(P, s);
         case 2: return launch_tile<2, 16, 16, 288>(P, s);

@@ -23,3 +23,43 @@ def test_table_log_within_two_ulp():
     got, ref = y.cpu().numpy(), np.log(x)
     assert got[x == 1.0][0] == 0.0
     assert np.all(np.abs(got - ref) <= 2.5 * np.spacing(np.abs(ref)))
+
+
+@pytest.mark.parametrize("n", [8, 9, 15, 16, 17, 200, 2432, 2433, 2500, 65536, 65537])
+@pytest.mark.parametrize("bc", ["periodic", "outflow", "reflect", "symmetry_lo"])
+def test_1d_stage_shapes_vs_oracle(n, bc):
+    """The three 1D shapes of the FP64 stage kernel (8-node lines shared by four warps, 62- and 254-node tiles) at the
+    edges of their ranges and of their tiles: the right-hand sides of a rough state with a moving mesh, and an RK stage,
+    against the oracle to 1e-12 of their size, with the EC flux alone too."""
+    import torch
+
+    from oracle import operator as op
+    from oracle import stepper
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    from sides import gpu_setup, oracle_setup
+    x, d = wl.uniform_nodes(n, 0.0, 1.0, bc == "periodic")
+    w = wl.sine_1d(max(n, 8))
+    w.update(bc=(bc,), x=x[None].copy(), dxi=(d,))
+    w["rho"], w["v"], w["p"] = wl.rough_state((n,), 3 + n, 1)
+    xdot = 0.05 * np.sin(2 * np.pi * x + 0.3)[None]
+    if bc != "periodic":
+        xdot[:, [0, -1]] = 0.0
+    for diss in (True, False):
+        sch, _, JU_o, J_o, x_o = oracle_setup(w, dissipation=diss)
+        dU_o, dJ_o = op.rhs(sch, JU_o, J_o, x_o, xdot)
+        ctx, JU, J, xt = gpu_setup(w, dissipation=diss)
+        xd = torch.tensor(xdot, device="cuda")
+        dU, dJ = torch.empty_like(JU), torch.empty_like(J)
+        es.es_rhs(ctx, JU, J, xt, xd, dU, dJ)
+        dt = 0.1 * d
+        U1, J1 = torch.empty_like(JU), torch.empty_like(J)
+        es.es_rk_stage(ctx, 2, dt, JU, J, JU, J, xt, xd, U1, J1)
+        assert es.es_check(ctx) == 0, es.es_last_error(ctx)
+        U1_o, J1_o = stepper.rk_stage(sch, 1, dt, JU_o, J_o, JU_o, J_o, x_o, xdot)
+        for c in range(3):
+            flux = np.abs(JU_o[c]).max() * 4.0 / d                  # the size of a flux difference
+            assert np.abs(dU.cpu().numpy()[c] - dU_o[c]).max() < 1e-12 * flux
+        assert np.abs(dJ.cpu().numpy() - dJ_o).max() < 1e-12 / d
+        assert np.abs(U1.cpu().numpy() - U1_o).max() < 1e-12 * np.abs(U1_o).max()
+        assert np.abs(J1.cpu().numpy() - J1_o).max() < 1e-12 * np.abs(J1_o).max()
