@@ -12,6 +12,7 @@
 #include "es_df.cuh"
 #include "es_device.cuh"
 #include "es_log64.cuh"
+#include "es_mesh64.cuh"
 
 namespace es {
 
@@ -46,7 +47,7 @@ __device__ __forceinline__ double coord_at(const GridParams& g, const double* x,
     return coord_ghost(g.n1, g.n2, g.dim, g.bc[0], g.bc[1], g.period[0], g.period[1], x, gi, gj, comp);
 }
 
-// 6th-order central difference delta_k of coordinate `comp` at node (i, j), divided by dxi_k
+// 6th-order central difference delta_k of coordinate `comp` at node (i, j)
 __device__ __forceinline__ double dcoord(const GridParams& g, const double* x, int i, int j, int comp, int k) {
     double s = 0.0;
 #pragma unroll
@@ -55,35 +56,7 @@ __device__ __forceinline__ double dcoord(const GridParams& g, const double* x, i
         if (k == 0) s += h * (coord_at(g, x, i + m, j, comp) - coord_at(g, x, i - m, j, comp));
         else s += h * (coord_at(g, x, i, j + m, comp) - coord_at(g, x, i, j - m, comp));
     }
-    return s * g.inv_dxi[k];
-}
-
-__device__ __forceinline__ double block_reduce_max(double v) {
-    __shared__ double sh[32];
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    v = threadIdx.x < nw ? sh[threadIdx.x] : 0.0;
-    if (w == 0)
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    __syncthreads();
-    return v;
-}
-
-__device__ __forceinline__ double block_reduce_min(double v) {
-    __shared__ double sh[32];
-    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    v = threadIdx.x < nw ? sh[threadIdx.x] : 1e300;
-    if (w == 0)
-        for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-    __syncthreads();
-    return v;
+    return s;
 }
 
 // state element access: double arrays, or the mixed form's (hi, lo) float planes
@@ -106,10 +79,10 @@ __global__ void k_init_J(GridParams g, const double* x, TS* J) {
     for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
         const int i = id % g.n1, j = id / g.n1;
         if (g.dim == 1) {
-            st_state(J, N, id, dcoord(g, x, i, 0, 0, 0));
+            st_state(J, N, id, dcoord(g, x, i, 0, 0, 0) * g.inv_dxi[0]);
         } else {
-            const double x1 = dcoord(g, x, i, j, 0, 0), x2 = dcoord(g, x, i, j, 0, 1);
-            const double y1 = dcoord(g, x, i, j, 1, 0), y2 = dcoord(g, x, i, j, 1, 1);
+            const double x1 = dcoord(g, x, i, j, 0, 0) * g.inv_dxi[0], x2 = dcoord(g, x, i, j, 0, 1) * g.inv_dxi[1];
+            const double y1 = dcoord(g, x, i, j, 1, 0) * g.inv_dxi[0], y2 = dcoord(g, x, i, j, 1, 1) * g.inv_dxi[1];
             st_state(J, N, id, x1 * y2 - x2 * y1);
         }
     }
@@ -164,10 +137,10 @@ __global__ void k_cfl(GridParams g, Gas G, const TS* JU, const TS* J, const doub
             rhoF[id] = rho;
             GF[id] = div_nr(pnn3, 2.0 * c2);
         }
-        const double c = sqrt(fmax(c2, 0.0));
+        const bool ok = c2 > 0.0;
+        const double c = ok ? c2 * rsqrt_nr(c2) : 0.0;
         const double xd1 = xdot != nullptr ? xdot[id] : 0.0;
         double tot;
-        const bool ok = c2 > 0.0;
         if (g.dim == 1) {
             tot = (fabs(-xd1 + v1) + c) * iJ * g.inv_dxi[0];
             if (t0) {
@@ -177,31 +150,35 @@ __global__ void k_cfl(GridParams g, Gas G, const TS* JU, const TS* J, const doub
                 t0[2 * N + id] = ok ? c * f : 1e300;
             }
         } else {
-            const double xd2 = xdot != nullptr ? xdot[N + id] : 0.0;
+            // 6th-order differences, undivided: with f = 1/(J dxi_1 dxi_2), (a_k, b_k) f is (J dxi_k/dx) / (J dxi_k)
             const double x1 = dcoord(g, x, i, j, 0, 0), x2 = dcoord(g, x, i, j, 0, 1);
             const double y1 = dcoord(g, x, i, j, 1, 0), y2 = dcoord(g, x, i, j, 1, 1);
-            const double a1 = y2, b1 = -x2;          // J dxi_1/dx
-            const double a2 = -y1, b2 = x1;          // J dxi_2/dx
-            const double tx1 = -(xd1 * a1 + xd2 * b1), tx2 = -(xd1 * a2 + xd2 * b2);     // J xi_{k,t}
-            const double n1c = sqrt(a1 * a1 + b1 * b1) * c, n2c = sqrt(a2 * a2 + b2 * b2) * c;
-            tot = (fabs(tx1 + (a1 * v1 + b1 * v2)) + n1c) * iJ * g.inv_dxi[0] +
-                  (fabs(tx2 + (a2 * v1 + b2 * v2)) + n2c) * iJ * g.inv_dxi[1];
+            const double f = iJ * (g.inv_dxi[0] * g.inv_dxi[1]), cf = c * f;
+            const double q1 = fma(y2, y2, x2 * x2), q2 = fma(y1, y1, x1 * x1);
+            const double C1 = q1 > 0.0 ? (q1 * rsqrt_nr(q1)) * cf : 0.0, C2 = q2 > 0.0 ? (q2 * rsqrt_nr(q2)) * cf : 0.0;
+            const double P1 = y2 * f, Q1 = -x2 * f, P2 = -y1 * f, Q2 = x1 * f;
+            const double S1 = fma(P1, v1, Q1 * v2), S2 = fma(P2, v1, Q2 * v2);
+            if (xdot != nullptr) {
+                const double xd2 = xdot[N + id];
+                tot = (fabs(S1 - fma(xd1, P1, xd2 * Q1)) + C1) + (fabs(S2 - fma(xd1, P2, xd2 * Q2)) + C2);
+            } else {
+                tot = (fabs(S1) + C1) + (fabs(S2) + C2);
+            }
             if (t0) {
-                const double f1 = iJ * g.inv_dxi[0], f2 = iJ * g.inv_dxi[1];
-                t0[id] = (a1 * v1 + b1 * v2) * f1;
-                t0[N + id] = a1 * f1;
-                t0[2 * N + id] = b1 * f1;
-                t0[3 * N + id] = ok ? n1c * f1 : 1e300;
-                t1[id] = (a2 * v1 + b2 * v2) * f2;
-                t1[N + id] = a2 * f2;
-                t1[2 * N + id] = b2 * f2;
-                t1[3 * N + id] = ok ? n2c * f2 : 0.0;
+                t0[id] = S1;
+                t0[N + id] = P1;
+                t0[2 * N + id] = Q1;
+                t0[3 * N + id] = ok ? C1 : 1e300;
+                t1[id] = S2;
+                t1[N + id] = P2;
+                t1[2 * N + id] = Q2;
+                t1[3 * N + id] = ok ? C2 : 0.0;
             }
         }
         if (!ok) tot = 1e300;
-        m = fmax(m, tot);
+        m = max_bits(m, tot);
     }
-    m = block_reduce_max(m);
+    block_max_bits<1>(&m);
     if (threadIdx.x == 0) {
         atomic_max_pos(&d->red[slot], m);
         if (set_dt) {                   // k_dt's work, by the last block to finish
@@ -385,99 +362,6 @@ __global__ void k_mon_fields(GridParams g, Gas G, const TS* JU, const TS* J, dou
     }
 }
 
-__device__ __forceinline__ double field_at(const GridParams& g, const double* f, int i, int j) {
-    const int si = state_index(i, g.n1, g.bc[0]);
-    const int sj = g.dim == 2 ? state_index(j, g.n2, g.bc[1]) : 0;
-    return f[sj * g.n1 + si];
-}
-
-// raw monitor terms and their grid maxima
-__global__ void k_mon_terms(GridParams g, MonitorParams mp, const double* rhoF, const double* GF, double* t0,
-                            double* t1, double* t2, DevScalars* d) {
-    const int N = g.n1 * g.n2;
-    double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
-        const int i = id % g.n1, j = id / g.n1;
-        double gr = 0.0, gg = 0.0, lg = 0.0, lr = 0.0;
-        #pragma unroll
-        for (int k = 0; k < 2; ++k) {          // fixed bound: the spacings are indexed by constants
-            if (k >= g.dim) break;
-            const int di = k == 0, dj = k == 1;
-            const double h2 = g.inv_dxi[k];
-            const double rp = field_at(g, rhoF, i + di, j + dj), rm = field_at(g, rhoF, i - di, j - dj);
-            const double r0 = rhoF[id];
-            const double Gp = field_at(g, GF, i + di, j + dj), Gm = field_at(g, GF, i - di, j - dj);
-            const double G0 = GF[id];
-            const double a = (rp - rm) * 0.5 * h2, b = (Gp - Gm) * 0.5 * h2;
-            const double c = (Gp - 2.0 * G0 + Gm) * h2 * h2, e = (rp - 2.0 * r0 + rm) * h2 * h2;
-            gr += a * a;
-            gg += b * b;
-            lg += c * c;
-            lr += e * e;
-        }
-        double v0, v1, v2;
-        if (mp.kind == ES_MONITOR_SMOOTH) {
-            v0 = sqrt(gr);
-            v1 = 0.0;
-            v2 = sqrt(lr);
-        } else {
-            v0 = gr;
-            v1 = mp.kappa >= 2 ? gg : 0.0;
-            v2 = lg;
-        }
-        t0[id] = v0;
-        t1[id] = v1;
-        t2[id] = v2;
-        m0 = fmax(m0, v0);
-        m1 = fmax(m1, v1);
-        m2 = fmax(m2, v2);
-    }
-    m0 = block_reduce_max(m0);
-    m1 = block_reduce_max(m1);
-    m2 = block_reduce_max(m2);
-    if (threadIdx.x == 0) {
-        atomic_max_pos(&d->red[RED_MON0], m0);
-        atomic_max_pos(&d->red[RED_MON1], m1);
-        atomic_max_pos(&d->red[RED_MON2], m2);
-    }
-}
-
-__global__ void k_mon_omega(GridParams g, MonitorParams mp, const double* t0, const double* t1, const double* t2,
-                            const DevScalars* d, double* omega) {
-    const int N = g.n1 * g.n2;
-    const double M0 = __longlong_as_double((long long)d->red[RED_MON0]);
-    const double M1 = __longlong_as_double((long long)d->red[RED_MON1]);
-    const double M2 = __longlong_as_double((long long)d->red[RED_MON2]);
-    const double c0 = M0 > 0.0 ? mp.w0 / M0 : 0.0;
-    const double c1 = M1 > 0.0 ? mp.w1 / M1 : 0.0;
-    const double c2 = M2 > 0.0 ? mp.w2 / M2 : 0.0;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x)
-        omega[id] = sqrt(1.0 + c0 * t0[id] + c1 * t1[id] + c2 * t2[id]);
-}
-
-// low-pass filter: omega_i <- sum_{j in {0,+-1}^d} (1/2)^(|j|_1 + d) omega_{i+j}
-__global__ void k_filter(GridParams g, const double* in, double* out) {
-    const int N = g.n1 * g.n2;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
-        const int i = id % g.n1, j = id / g.n1;
-        double s;
-        if (g.dim == 1) {
-            s = 0.25 * field_at(g, in, i - 1, 0) + 0.5 * in[id] + 0.25 * field_at(g, in, i + 1, 0);
-        } else {
-            s = 0.0;
-            for (int dj = -1; dj <= 1; ++dj) {
-                double row = 0.0;
-                for (int di = -1; di <= 1; ++di) {
-                    const double wgt = (di == 0 ? 0.5 : 0.25);
-                    row += wgt * field_at(g, in, i + di, j + dj);
-                }
-                s += (dj == 0 ? 0.5 : 0.25) * row;
-            }
-        }
-        out[id] = s;
-    }
-}
-
 // Result buffer of the Jacobi iteration so far: x_n before the first sweep, else
 // the buffer the last sweep wrote (sweep k writes buf[(pick + k) % 2]).
 __device__ __forceinline__ const double* jacobi_result(const DevScalars* d, const double* xn, const double* xa,
@@ -494,136 +378,6 @@ __device__ __forceinline__ bool fixed_comp(const GridParams& g, int i, int j, in
     if (g.dim == 2 && g.bc[1] != ES_BC_PERIODIC && (j == 0 || j == g.n2 - 1))
         f = f || !end_mirrored(g.bc[1], j == 0) || c == 1;
     return f;
-}
-
-// One Jacobi sweep of sum_k [w_{k,+} (x_{i+e_k} - x_i) - w_{k,-} (x_i - x_{i-e_k})]/dxi_k^2 = 0
-// from xin into xout; returns this thread's max change
-// One sweep from xin into xout; CHG: returns the largest change; LIMIT: also min-accumulates into *lim the
-// limiter's bound Delta_gamma at every node from the result and x^n = xn (k_limiter's rule and arithmetic, so
-// the last sweep can take the limiter's work)
-template <bool CHG, bool LIMIT>
-__device__ __forceinline__ double jacobi_sweep(const GridParams& g, const double* omega, const double* xin,
-                                              double* xout, const double* xn = nullptr, double* lim = nullptr) {
-    const int N = g.n1 * g.n2;
-    double chg = 0.0, m = 1.0;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
-        const int i = id % g.n1, j = id / g.n1;
-        const double w0 = omega[id];
-        double den = 0.0, num[2] = {0.0, 0.0};
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {     // fixed bounds: num[] stays in registers
-            if (kk >= g.dim) break;
-            const int di = kk == 0, dj = kk == 1;
-            const double ih2 = g.inv_dxi[kk] * g.inv_dxi[kk];
-            const double wp = 0.5 * (w0 + field_at(g, omega, i + di, j + dj)) * ih2;
-            const double wm = 0.5 * (w0 + field_at(g, omega, i - di, j - dj)) * ih2;
-            den += wp + wm;
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-                if (c < g.dim)
-                    num[c] += wp * coord_at(g, xin, i + di, j + dj, c) + wm * coord_at(g, xin, i - di, j - dj, c);
-        }
-        const double iden = rcp_nr(den);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            if (c >= g.dim) break;
-            const double xv = fixed_comp(g, i, j, c) ? xin[c * N + id] : num[c] * iden;
-            if (CHG) chg = fmax(chg, fabs(xv - xin[c * N + id]));
-            xout[c * N + id] = xv;
-            if (LIMIT) {
-                const double x0 = xn[c * N + id];
-                const double dx = xv - x0;
-                const int di = c == 0, dj = c == 1;
-                if (dx < 0.0) m = fmin(m, div_nr(-(x0 - coord_at(g, xn, i - di, j - dj, c)), 2.0 * dx));
-                else if (dx > 0.0) m = fmin(m, div_nr(coord_at(g, xn, i + di, j + dj, c) - x0, 2.0 * dx));
-            }
-        }
-    }
-    if (LIMIT) *lim = m;
-    return chg;
-}
-
-// Sweep k of the iteration.  Sweep k >= 1 reads buf[(pick + k - 1) % 2] and writes
-// buf[(pick + k) % 2]; sweep 0 reads `first` (x_n or the warm start) and writes buf[dst0].  Once
-// the iteration has converged (d->conv) the remaining sweeps return at once.  With `check`, the
-// grid-wide max change goes to red[slot]; if `decide`, the last block to finish compares it with eps.
-__global__ void k_jacobi(GridParams g, const double* omega, const double* first, double* xa, double* xb, int k,
-                         int dst0, DevScalars* d, int check, int slot, int decide, double eps, int limit) {
-    if (d->conv) return;
-    const double* xin;
-    double* xout;
-    if (k == 0) {
-        xin = first;
-        xout = dst0 ? xb : xa;
-    } else {
-        const int src = (d->pick + k - 1) & 1;
-        xin = src ? xb : xa;
-        xout = src ? xa : xb;
-    }
-    double chg = 0.0;
-    if (check) {
-        chg = jacobi_sweep<true, false>(g, omega, xin, xout);
-    } else if (limit) {             // the last sweep without a tolerance: k_limiter's work (first is x^n)
-        double lim = 1.0;
-        jacobi_sweep<false, true>(g, omega, xin, xout, first, &lim);
-        lim = block_reduce_min(lim);
-        if (threadIdx.x == 0) atomic_min_pos(&d->red[RED_GAMMA], lim);
-    } else {
-        jacobi_sweep<false, false>(g, omega, xin, xout);
-    }
-    if (check) {
-        chg = block_reduce_max(chg);
-        if (threadIdx.x == 0) {
-            atomic_max_pos(&d->red[slot], chg);
-            __threadfence();
-            const unsigned int ticket = atomicAdd(&d->done, 1u);
-            if (ticket == gridDim.x - 1) {                 // every block's maximum is in
-                if (decide) {
-                    const double c = __longlong_as_double((long long)atomicAdd(&d->red[slot], 0ULL));
-                    if (c < eps) d->conv = 1;
-                    d->red[slot] = 0ULL;
-                }
-                d->done = 0u;
-            }
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (k > 0 || slot == RED_JAC)) atomicAdd(&d->sweeps, 1);
-}
-
-// The body of a graph while-loop over the sweeps with a tolerance: sweep k = d->sweeps (the
-// same buffers as k_jacobi), and the last block to finish tests the change, counts the sweep
-// and sets the loop's condition: another sweep while not converged and fewer than mu sweeps.
-__global__ void k_jacobi_loop(GridParams g, const double* omega, const double* xn, double* xa, double* xb,
-                              DevScalars* d, double eps, int mu, cudaGraphConditionalHandle h) {
-    if (d->conv || d->sweeps >= mu) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
-        return;
-    }
-    const int k = d->sweeps;
-    const double* xin;
-    double* xout;
-    if (k == 0) {
-        xin = xn;
-        xout = xa;
-    } else {
-        const int src = (d->pick + k - 1) & 1;
-        xin = src ? xb : xa;
-        xout = src ? xa : xb;
-    }
-    double chg = block_reduce_max(jacobi_sweep<true, false>(g, omega, xin, xout));
-    if (threadIdx.x == 0) {
-        atomic_max_pos(&d->red[RED_JAC], chg);
-        __threadfence();
-        const unsigned int ticket = atomicAdd(&d->done, 1u);
-        if (ticket == gridDim.x - 1) {
-            const double c = __longlong_as_double((long long)atomicAdd(&d->red[RED_JAC], 0ULL));
-            if (c < eps) d->conv = 1;
-            d->red[RED_JAC] = 0ULL;
-            d->done = 0u;
-            d->sweeps = k + 1;
-            cudaGraphSetConditional(h, (d->conv == 0 && k + 1 < mu) ? 1u : 0u);
-        }
-    }
 }
 
 // Guarded warm start: the first sweep ran from x_n (into buf[0], change c0 in red[RED_JAC]) and
@@ -644,24 +398,6 @@ __global__ void k_pick(DevScalars* d, int check, double eps, double ratio) {
     }
 }
 
-// Delta_gamma: each node moves at most half of the spacing towards its neighbour (Sec. 4)
-__global__ void k_limiter(GridParams g, const double* xn, const double* xa, const double* xb, DevScalars* d) {
-    const int N = g.n1 * g.n2;
-    const double* xit = jacobi_result(d, xn, xa, xb);
-    double m = 1.0;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
-        const int i = id % g.n1, j = id / g.n1;
-        for (int k = 0; k < g.dim; ++k) {
-            const double dx = xit[k * N + id] - xn[k * N + id];
-            const int di = k == 0, dj = k == 1;
-            if (dx < 0.0) m = fmin(m, div_nr(-(xn[k * N + id] - coord_at(g, xn, i - di, j - dj, k)), 2.0 * dx));
-            else if (dx > 0.0) m = fmin(m, div_nr(coord_at(g, xn, i + di, j + dj, k) - xn[k * N + id], 2.0 * dx));
-        }
-    }
-    m = block_reduce_min(m);
-    if (threadIdx.x == 0) atomic_min_pos(&d->red[RED_GAMMA], m);
-}
-
 __global__ void k_velocity(GridParams g, const double* xn, const double* xa, const double* xb, DevScalars* d,
                            double* xdot, const double* t0, const double* t1, double cfl) {
     const int N = g.n1 * g.n2;
@@ -680,9 +416,9 @@ __global__ void k_velocity(GridParams g, const double* xn, const double* xa, con
                 v2 = f * (xit[N + id] - xn[N + id]);
                 xdot[N + id] = v2;
             }
-            m = fmax(m, cfl_moving_term(t0, t1, size_t(N), size_t(id), g.dim, v1, v2));
+            m = max_bits(m, cfl_moving_term(t0, t1, size_t(N), size_t(id), g.dim, v1, v2));
         }
-        m = block_reduce_max(m);
+        block_max_bits<1>(&m);
         if (threadIdx.x == 0) {
             atomic_max_pos(&d->red[RED_CFL2], m);
             __threadfence();

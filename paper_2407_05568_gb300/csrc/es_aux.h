@@ -18,6 +18,8 @@ struct GridParams {
     float finv[2], fdx[2], finv2[2];
     double dx[2];       // 1 / inv_dxi_k (host-formed, as the kernels formed it)
     float dxh[2], dxl[2];   // dx_k as the unevaluated float sum dxh + dxl
+    double d1sq[2], d2sq[2];    // squares of 1/(2 dxi_k) and 1/dxi_k^2 (the monitor's differences)
+    double ratio;               // (dxi_2/dxi_1)^2 (the sweeps' weights)
 };
 
 inline void grid_floats(GridParams& g) {
@@ -28,7 +30,10 @@ inline void grid_floats(GridParams& g) {
         g.dx[k] = 1.0 / g.inv_dxi[k];
         g.dxh[k] = float(g.dx[k]);
         g.dxl[k] = float(g.dx[k] - double(g.dxh[k]));
+        g.d1sq[k] = 0.25 * g.inv_dxi[k] * g.inv_dxi[k];
+        g.d2sq[k] = g.inv_dxi[k] * g.inv_dxi[k] * g.inv_dxi[k] * g.inv_dxi[k];
     }
+    g.ratio = g.dim == 2 ? (g.inv_dxi[0] / g.inv_dxi[1]) * (g.inv_dxi[0] / g.inv_dxi[1]) : 1.0;
 }
 
 struct MonitorParams {
@@ -128,15 +133,30 @@ __global__ void k_advance(GridParams g, double* x, const double* xdot, DevScalar
 // fxd is written only when xdot is given (its readers take it only then)
 __global__ void k_mesh_f32(GridParams g, const double* __restrict__ x, const double* __restrict__ xdot,
                            float* __restrict__ disp, float* __restrict__ fxd, DevScalars* rst = nullptr);
-__global__ void k_mon_terms(GridParams g, MonitorParams mp, const double* rhoF, const double* GF, double* t0,
-                            double* t1, double* t2, DevScalars* d);
-__global__ void k_mon_omega(GridParams g, MonitorParams mp, const double* t0, const double* t1, const double* t2,
-                            const DevScalars* d, double* omega);
-__global__ void k_filter(GridParams g, const double* in, double* out);
-__global__ void k_jacobi(GridParams g, const double* omega, const double* first, double* xa, double* xb, int k,
-                         int dst0, DevScalars* d, int check, int slot, int decide, double eps, int limit = 0);
-__global__ void k_jacobi_loop(GridParams g, const double* omega, const double* xn, double* xa, double* xb,
-                              DevScalars* d, double eps, int mu, cudaGraphConditionalHandle h);
+void launch_mon_terms(const GridParams& g, const MonitorParams& mp, const double* rhoF, const double* GF, double* t0,
+                      double* t1, double* t2, DevScalars* d, int grid, int block, cudaStream_t s);
+__global__ void k_mon_omega(GridParams g, MonitorParams mp, const double* __restrict__ t0,
+                            const double* __restrict__ t1, const double* __restrict__ t2, const DevScalars* d,
+                            double* __restrict__ omega);
+__global__ void k_filter(GridParams g, const double* __restrict__ in, double* __restrict__ out);
+// the sweeps' normalised weights, written by sweep 0 (2 dim planes of the mesh size)
+struct SweepWeights {
+    double* w[4];
+};
+__global__ void k_jacobi(GridParams g, const double* omega, SweepWeights w, const double* first, double* xa, double* xb,
+                         int k, int dst0, DevScalars* d, int check, int slot, int decide, double eps, int limit = 0);
+__global__ void k_jacobi_loop(GridParams g, const double* omega, SweepWeights w, const double* xn, double* xa,
+                              double* xb, DevScalars* d, double eps, int mu, cudaGraphConditionalHandle h);
+// Small meshes: omega with all filter passes, and all sweeps (no tolerance) with Delta_gamma, in one launch each on tiles
+// in shared memory; false where the mesh is larger than TILE_NODES_PER_SM nodes per SM or the halo does not fit (nothing
+// launched).
+constexpr int TILE_THREADS = 512;
+constexpr int TILE_NODES_PER_SM = 512;
+cudaError_t mesh64_prepare();
+bool launch_filter_tile(const GridParams& g, const MonitorParams& mp, const double* t0, const double* t1,
+                        const double* t2, const DevScalars* d, int passes, double* omega, int nsm, cudaStream_t s);
+bool launch_sweep_tile(const GridParams& g, const double* omega, const double* xn, double* xout, int mu, DevScalars* d,
+                       int nsm, cudaStream_t s);
 __global__ void k_pick(DevScalars* d, int check, double eps, double ratio);
 __global__ void k_limiter(GridParams g, const double* xn, const double* xa, const double* xb, DevScalars* d);
 // cfl > 0: also eq. cfl with the new velocity from the stored terms (t0, t1) into RED_CFL2, and the last block

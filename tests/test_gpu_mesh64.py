@@ -1,0 +1,67 @@
+"""The FP64 mesh redistribution's kernels at the edges of their ranges: the tiles of small meshes (filter passes and sweeps
+in one launch) and the pass-by-pass kernels of larger ones, every boundary condition, ragged sizes and pass counts."""
+import numpy as np
+import pytest
+
+from oracle import stepper
+from paper_2407_05568_gb300 import workloads as wl
+
+from sides import gpu_setup, oracle_setup
+
+pytestmark = pytest.mark.gpu
+
+BCS = {"periodic": ("periodic", "periodic"), "outflow": ("outflow", "outflow"), "walls": ("reflect", "symmetry_lo"),
+       "mixed": ("periodic", "reflect"), "swapped": ("outflow", "periodic")}
+
+
+def _mesh2d(n1, n2, bc, seed):
+    """Density bumps and a moved mesh on [0, 1]^2; periodic directions take a periodic displacement."""
+    x1, d1 = wl.uniform_nodes(n1, 0.0, 1.0, bc[0] == "periodic")
+    x2, d2 = wl.uniform_nodes(n2, 0.0, 1.0, bc[1] == "periodic")
+    X, Y = np.meshgrid(x1, x2)
+    rng = np.random.default_rng(seed)
+    ph = rng.uniform(0.0, 2 * np.pi, 3)
+    bx = np.sin(np.pi * X) if bc[0] != "periodic" else 1.0
+    by = np.sin(np.pi * Y) if bc[1] != "periodic" else 1.0
+    x = np.stack([X + 0.2 * d1 * bx * by * np.sin(2 * np.pi * (X + Y) + ph[0]),
+                  Y + 0.2 * d2 * bx * by * np.cos(2 * np.pi * (X - Y) + ph[1])])
+    rho = 0.6 + 0.25 * np.tanh(8.0 * np.sin(2 * np.pi * (X + 0.6 * Y) + ph[2]))
+    return dict(gas=wl.UNITS_A, dim=2, n=(n2, n1), dxi=(d1, d2), bc=bc, period=(1.0, 1.0), x=x, rho=rho,
+                v=np.stack([0.1 * np.ones_like(X), 0.0 * X]), p=1.0 + 0.05 * np.cos(2 * np.pi * Y), cfl=0.4, moving=True,
+                t_end=1e30)
+
+
+def _compare(w, tol=1e-11):
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    sch, mc, JU_o, J_o, x_o = oracle_setup(w)
+    dt = 1e-3
+    xd_o, sw_o, gam_o = stepper.redistribute(sch, mc, JU_o, J_o, x_o, dt)
+    ctx, JU, J, xt = gpu_setup(w)
+    xd = torch.empty_like(xt)
+    sw, gam = es.es_mesh_redistribute(ctx, JU, J, xt, dt, xd)
+    assert sw == sw_o
+    # x^[mu] - x^n keeps 16 digits of the coordinates, so a few 1e-16 of 1 over the displacements' size
+    size = max(np.abs(xd_o).max(), 1e-3 * min(w["dxi"]) / dt)
+    assert abs(gam - gam_o) <= 1e-10 * gam_o
+    assert np.abs(xd.cpu().numpy() - xd_o).max() <= tol * size
+
+
+@pytest.mark.parametrize("bc", list(BCS))
+@pytest.mark.parametrize("shape,passes,sweeps", [((8, 8), 5, 5), ((9, 31), 1, 1), ((20, 14), 5, 10), ((41, 29), 10, 3),
+                                                 ((61, 33), 11, 2), ((33, 61), 0, 11), ((270, 285), 5, 5),
+                                                 ((290, 271), 2, 4)])
+def test_redistribution_2d(bc, shape, passes, sweeps):
+    w = _mesh2d(*shape, BCS[bc], 7 + shape[0])
+    w["mesh"] = dict(monitor="vdw", alphas=(1200.0, 1200.0, 1200.0), kappa=2, filter_passes=passes, sweeps=sweeps,
+                     eps=0.0)
+    _compare(w)
+
+
+@pytest.mark.parametrize("monitor,kappa,eps", [("smooth", 2, 0.0), ("vdw", 1, 0.0), ("vdw", 2, 0.05)])
+def test_redistribution_monitors_and_tolerance(monitor, kappa, eps):
+    w = _mesh2d(45, 38, BCS["outflow"], 3)
+    w["mesh"] = dict(monitor=monitor, alphas=(20.0, 15.0, 30.0), kappa=kappa, filter_passes=4, sweeps=30,
+                     eps=eps * w["dxi"][0])
+    _compare(w)
