@@ -270,13 +270,17 @@ __device__ __forceinline__ void face_dissipation3_f(const float* S, int NB, int 
     float y[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
-        const float wmin = mr_weno5_f(W[0][m], W[1][m], W[2][m], W[3][m], W[4][m], Wc);
-        const float wplu = mr_weno5_f(W[5][m], W[4][m], W[3][m], W[2][m], W[1][m], Wc);
-        const float jw = wplu - wmin;
-        float j = W[3][m];
-        if (fabsf(j) <= Wc.sign_tol * scl[m]) j = 0.0f;
-        const bool keep = (jw > 0.0f && j > 0.0f) || (jw < 0.0f && j < 0.0f);
-        y[m] = keep ? jw : 0.0f;
+        // a wave whose plain jump is within round-off of zero adds nothing whatever its reconstruction (the shear waves of
+        // a uniform flow, every wave of a constant state)
+        const float j = W[3][m];
+        y[m] = 0.0f;
+        if (!(fabsf(j) <= Wc.sign_tol * scl[m])) {
+            const float wmin = mr_weno5_f(W[0][m], W[1][m], W[2][m], W[3][m], W[4][m], Wc);
+            const float wplu = mr_weno5_f(W[5][m], W[4][m], W[3][m], W[2][m], W[1][m], Wc);
+            const float jw = wplu - wmin;
+            const bool keep = (jw > 0.0f && j > 0.0f) || (jw < 0.0f && j < 0.0f);
+            y[m] = keep ? jw : 0.0f;
+        }
     }
     const float h = -0.5f * Lam;
     const float y0 = sA * y[0], y1 = sE * y[1], y2 = sT * y[2], y3 = sT * y[3], y4 = sA * y[4];

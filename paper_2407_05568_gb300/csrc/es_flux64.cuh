@@ -474,9 +474,8 @@ __device__ __forceinline__ double jump_size(const Face<D>& f, const double* S, i
     return (m == 1 ? f.sE : f.sA) * fma(fabs(u), tv[0], fma(fabs(h), e2, common));
 }
 // Y [[W]]^WENO: kept where the reconstruction's jump has the sign of the plain jump j (a NaN jump is dropped)
-__device__ __forceinline__ double switched(double jw, double j, bool zero) {
-    const bool keep = !zero && (__double2hiint(jw) ^ __double2hiint(j)) >= 0 &&
-                      (__double2hiint(jw) & 0x7fffffff) <= 0x7ff00000;
+__device__ __forceinline__ double switched(double jw, double j) {
+    const bool keep = (__double2hiint(jw) ^ __double2hiint(j)) >= 0 && (__double2hiint(jw) & 0x7fffffff) <= 0x7ff00000;
     return keep ? jw : 0.0;
 }
 
@@ -518,7 +517,12 @@ __device__ __forceinline__ void face_dissipation(const double* S, int NB, int l,
     }
     double y[NC];
 #pragma unroll
-    for (int m = 0; m < NC; ++m) y[m] = switched(weno_jump(dW[m], Wc), dW[m][2], zero[m]);
+    for (int m = 0; m < NC; ++m) {
+        // a wave whose plain jump is zero adds nothing whatever its reconstruction: the shear waves of a uniform flow,
+        // every wave of a constant state
+        y[m] = 0.0;
+        if (!zero[m]) y[m] = switched(weno_jump(dW[m], Wc), dW[m][2]);
+    }
     const double h = -f.Lam, vn = f.vr[0];
     const double y0 = __dmul_rn(f.sA, y[0]), y1 = __dmul_rn(f.sE, y[1]), y4 = __dmul_rn(f.sA, y[NC - 1]);
     const double i0 = (y0 + y4) + y1;

@@ -476,19 +476,22 @@ __global__ void __launch_bounds__(128) stage_line_fp64(StageParams P) {
             flux64::project<1>(f, dv, W, 1u << warp);
             d[o] = warp == 0 ? W[0] : (warp == 1 ? W[1] : W[2]);
         }
-        const double s2 = fma(d[2], d[2], P.weno.eps4);
-        const double sx = right ? d[3] : d[1];
-        double num, den;
-        flux64::weno_side(right ? d[4] : d[0], sx, d[2], right ? d[1] : d[3],
-                          flux64::min_pos(fma(sx, sx, P.weno.eps4), s2), P.weno, num, den);
-        const double part = num * rcp_nr(den);
-        const double other = __shfl_xor_sync(0xffffffffu, part, 1);
-        const double jw = d[2] - (part + other);
         const flux64::SwitchBounds b = flux64::switch_bounds<1>(f, S, NB, l, l + 1, P.weno);
         const int is = flux64::jump_is_zero<1>(b, f, warp, d[2]);
         bool zero = is == 1;
         if (is == 2) zero = fabs(d[2]) <= P.weno.sign_tol * flux64::jump_size<1>(f, S, NB, l, l + 1, warp);
-        const double y = -f.Lam * ((warp == 1 ? f.sE : f.sA) * flux64::switched(jw, d[2], zero));
+        double y = 0.0;
+        if (__any_sync(0xffffffffu, !zero)) {
+            const double s2 = fma(d[2], d[2], P.weno.eps4);
+            const double sx = right ? d[3] : d[1];
+            double num, den;
+            flux64::weno_side(right ? d[4] : d[0], sx, d[2], right ? d[1] : d[3],
+                              flux64::min_pos(fma(sx, sx, P.weno.eps4), s2), P.weno, num, den);
+            const double part = num * rcp_nr(den);
+            const double other = __shfl_xor_sync(0xffffffffu, part, 1);
+            if (!zero)
+                y = -f.Lam * ((warp == 1 ? f.sE : f.sA) * flux64::switched(d[2] - (part + other), d[2]));
+        }
         const double vn = f.vr[0], c = warp == 0 ? -f.c : (warp == 1 ? 0.0 : f.c);
         if (!right && lane >> 1 < LINE_NF) {
             FB[warp][0][face] = y;
