@@ -45,6 +45,7 @@ struct StageParams {
     // float copies of the constants (GB300 converts double -> float at FP64 speed)
     float fgas[9];                // a, b, R, cv, delta, R b, 1/cv, 1/R, 1/delta
     float fweno[8];               // g1, g2, g3, g12, ig22, ig3, eps, sign_tol
+    float fwc[9];                 // h1, h2, q2, q3[4], eps4, sign_tol (2D)
     float finv_dxi[2];
     float fca, fcb, fca_lo, fcb_lo, fcst;
     // mixed form strides: component stride, JU lo-plane offset, J lo-plane offset
@@ -66,6 +67,9 @@ inline void set_float_params(StageParams& P) {
     const double w[8] = {P.weno.g1, P.weno.g2, P.weno.g3, P.weno.g12, P.weno.ig22, P.weno.ig3, P.weno.eps,
                          P.weno.sign_tol};
     for (int k = 0; k < 8; ++k) P.fweno[k] = float(w[k]);
+    const double wc[9] = {P.weno.h1, P.weno.h2, P.weno.q2, P.weno.q3[0], P.weno.q3[1], P.weno.q3[2], P.weno.q3[3],
+                          P.weno.eps4, P.weno.sign_tol};
+    for (int k = 0; k < 9; ++k) P.fwc[k] = float(wc[k]);
     P.finv_dxi[0] = float(P.inv_dxi[0]);
     P.finv_dxi[1] = float(P.inv_dxi[1]);
     P.fca = float(P.ca);
