@@ -1026,7 +1026,6 @@ int es_set_warm_start(es_ctx* c, const uint16_t* w_bf16, const float* bias, int 
     CK(cudaMalloc((void**)&c->nn_b, sizeof(float) * nb), "cudaMalloc");
     CK(cudaMemcpyAsync(c->nn_wbf, w_bf16, sizeof(uint16_t) * nw, cudaMemcpyDeviceToDevice, c->stream), "weight copy");
     CK(cudaMemcpyAsync(c->nn_b, bias, sizeof(float) * nb, cudaMemcpyDeviceToDevice, c->stream), "bias copy");
-    CK(nn_prepare(), "conv kernel attributes");
     CK(cudaStreamSynchronize(c->stream), "sync");
     c->nn_layers = layers;
     c->nn_hidden = hidden;

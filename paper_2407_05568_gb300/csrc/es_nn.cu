@@ -20,158 +20,32 @@ namespace {
 constexpr int TS = 16;            // output tile edge (pixels)
 constexpr int HALO = TS + 2;
 constexpr int MAXC = 32;          // channel limit
-constexpr int WG_THREADS = 288;   // weight-gradient block: 9 * 32 (ci, tap) pairs
 
-// One thread per output pixel with all COUT channels in registers.  The input tile
-// with its halo and the weights (transposed to [ci][tap][co], so one thread reads
-// COUT consecutive floats) sit in shared memory.
-template <int COUT>
-__global__ void __launch_bounds__(TS * TS) k_conv_fwd(const float* __restrict__ in, const float* __restrict__ wf,
-                                                     const float* __restrict__ bias, float* __restrict__ out,
-                                                     int Cin, int H, int W, int act) {
-    extern __shared__ float4 sm4[];
-    float* sm = reinterpret_cast<float*>(sm4);
-    float* ws = sm;                                   // Cin * 9 * COUT
-    float* xs = sm + COUT * Cin * 9;                  // Cin * HALO * HALO
-    const int tx = threadIdx.x % TS, ty = threadIdx.x / TS;
-    const int x0 = blockIdx.x * TS, y0 = blockIdx.y * TS, b = blockIdx.z;
-    const size_t HW = size_t(H) * W;
-    for (int k = threadIdx.x; k < COUT * Cin * 9; k += TS * TS) {
-        const int co = k / (Cin * 9), r = k % (Cin * 9);
-        ws[r * COUT + co] = wf[k];
-    }
-    const float* inb = in + size_t(b) * Cin * HW;
-    for (int k = threadIdx.x; k < Cin * HALO * HALO; k += TS * TS) {
-        const int ci = k / (HALO * HALO), r = k % (HALO * HALO);
-        const int yy = y0 - 1 + r / HALO, xx = x0 - 1 + r % HALO;
-        xs[k] = (yy >= 0 && yy < H && xx >= 0 && xx < W) ? inb[ci * HW + size_t(yy) * W + xx] : 0.0f;
-    }
+// out[o] = sum_s partial[s][o] over the strips: RP_GROUPS threads per output take every RP_GROUPS-th strip, and their sums
+// are added in order (the same order every time)
+constexpr int RP_GROUPS = 16;
+__global__ void __launch_bounds__(32 * RP_GROUPS) k_reduce_partials(const float* __restrict__ partial, int nstrips,
+                                                                    int len, float* grad_w, float* grad_b, int nout) {
+    __shared__ float part[RP_GROUPS][32];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int o = blockIdx.x * 32 + lane;
+    float s = 0.0f;
+    if (o < len)
+#pragma unroll 4
+        for (int k = grp; k < nstrips; k += RP_GROUPS) s += partial[size_t(k) * len + o];
+    part[grp][lane] = s;
     __syncthreads();
-    float acc[COUT];
+    if (grp != 0 || o >= len) return;
+    s = 0.0f;
 #pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[co] = bias ? bias[co] : 0.0f;
-    for (int ci = 0; ci < Cin; ++ci) {
-        const float* xc = xs + ci * HALO * HALO + ty * HALO + tx;
-        const float* wc = ws + ci * 9 * COUT;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const float v = xc[(k / 3) * HALO + k % 3];
-#pragma unroll
-            for (int co = 0; co < COUT; ++co) acc[co] = fmaf(wc[k * COUT + co], v, acc[co]);
-        }
-    }
-    const int x = x0 + tx, y = y0 + ty;
-    if (x < W && y < H) {
-        float* ob = out + size_t(b) * COUT * HW + size_t(y) * W + x;
-#pragma unroll
-        for (int co = 0; co < COUT; ++co) ob[co * HW] = act ? tanhf(acc[co]) : acc[co];
-    }
-}
-
-// Weight and bias gradients of one strip of tiles (a 16-pixel column, `rows` tiles
-// high, one image): thread (group gi, pair q = (ci, tap)) sums g[co](p) in[ci](p + tap)
-// over its share of the strip's pixels for all COUT channels; the groups are summed in
-// shared memory and the strip's partial sums written to partial[strip][...] (reduced
-// over strips, in a fixed order, by k_reduce_partials).
-template <int COUT>
-__global__ void __launch_bounds__(WG_THREADS) k_conv_wgrad(const float* __restrict__ in,
-                                                          const float* __restrict__ g, float* __restrict__ partial,
-                                                          int Cin, int H, int W, int rows) {
-    extern __shared__ float4 sm4[];
-    float* sm = reinterpret_cast<float*>(sm4);
-    float* gs = sm;                                   // TS*TS * COUT, [p][co]
-    float* xs = sm + TS * TS * COUT;                  // Cin * HALO * HALO
-    const int npairs = Cin * 9;
-    const int G = WG_THREADS / npairs;                // pixel groups (Cin divides 32)
-    const int q = threadIdx.x % npairs, gi = threadIdx.x / npairs;
-    const int ci = q / 9, tap = q % 9;
-    const int x0 = blockIdx.x * TS, b = blockIdx.z;
-    const size_t HW = size_t(H) * W;
-    const float* inb = in + size_t(b) * Cin * HW;
-    const float* gb = g + size_t(b) * COUT * HW;
-    float acc[COUT];
-    float accb = 0.0f;                                // bias: threads 0..COUT-1
-#pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[co] = 0.0f;
-    for (int r = 0; r < rows; ++r) {
-        const int y0 = (blockIdx.y * rows + r) * TS;
-        if (y0 >= H) break;
-        __syncthreads();
-        for (int k = threadIdx.x; k < COUT * TS * TS; k += WG_THREADS) {
-            const int co = k / (TS * TS), p = k % (TS * TS);
-            const int yy = y0 + p / TS, xx = x0 + p % TS;
-            gs[p * COUT + co] = (yy < H && xx < W) ? gb[co * HW + size_t(yy) * W + xx] : 0.0f;
-        }
-        for (int k = threadIdx.x; k < Cin * HALO * HALO; k += WG_THREADS) {
-            const int c = k / (HALO * HALO), rr = k % (HALO * HALO);
-            const int yy = y0 - 1 + rr / HALO, xx = x0 - 1 + rr % HALO;
-            xs[k] = (yy >= 0 && yy < H && xx >= 0 && xx < W) ? inb[c * HW + size_t(yy) * W + xx] : 0.0f;
-        }
-        __syncthreads();
-        if (gi < G) {
-            const float* xc = xs + ci * HALO * HALO + (tap / 3) * HALO + tap % 3;
-            for (int p = gi; p < TS * TS; p += G) {
-                const float v = xc[(p / TS) * HALO + p % TS];
-                const float* gp = gs + p * COUT;
-#pragma unroll
-                for (int co = 0; co < COUT; ++co) acc[co] = fmaf(gp[co], v, acc[co]);
-            }
-        }
-        if (threadIdx.x < COUT)
-            for (int p = 0; p < TS * TS; ++p) accb += gs[p * COUT + threadIdx.x];
-    }
-    __syncthreads();
-    // sum the pixel groups: red[gi][co][q]
-    float* red = sm;
-    if (gi < G)
-#pragma unroll
-        for (int co = 0; co < COUT; ++co) red[(gi * COUT + co) * npairs + q] = acc[co];
-    __syncthreads();
-    const int nout = COUT * npairs;
-    const size_t strip = (size_t(b) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    float* part = partial + strip * (nout + COUT);
-    for (int o = threadIdx.x; o < nout; o += WG_THREADS) {
-        float s = 0.0f;
-        for (int k = 0; k < G; ++k) s += red[k * nout + o];
-        part[o] = s;                                  // o = co * Cin * 9 + ci * 9 + tap
-    }
-    if (threadIdx.x < COUT) part[nout + threadIdx.x] = accb;
-}
-
-// out[o] = sum_s partial[s][o] in strip order (deterministic)
-__global__ void k_reduce_partials(const float* partial, int nstrips, int len, float* grad_w, float* grad_b,
-                                  int nout) {
-    for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < len; o += gridDim.x * blockDim.x) {
-        float s = 0.0f;
-        for (int k = 0; k < nstrips; ++k) s += partial[size_t(k) * len + o];
-        if (o < nout) grad_w[o] = s;
-        else grad_b[o - nout] = s;
-    }
-}
-
-__global__ void k_bf16_to_f32(const __nv_bfloat16* w, float* f, size_t n) {
-    for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
-        f[i] = __bfloat162float(w[i]);
+    for (int k = 0; k < RP_GROUPS; ++k) s += part[k][lane];
+    if (o < nout) grad_w[o] = s;
+    else grad_b[o - nout] = s;
 }
 
 __global__ void k_f32_to_bf16(const float* f, __nv_bfloat16* w, size_t n) {
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
         w[i] = __float2bfloat16_rn(f[i]);
-}
-
-// weights of the input-gradient correlation: w'[ci][co][tap] = w[co][ci][8 - tap]
-__global__ void k_flip_weights(const __nv_bfloat16* w, float* wt, int Cin, int Cout) {
-    const int n = Cin * Cout * 9;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int ci = i / (Cout * 9), r = i % (Cout * 9), co = r / 9, k = r % 9;
-        wt[i] = __bfloat162float(w[(co * Cin + ci) * 9 + (8 - k)]);
-    }
-}
-
-// gradient through tanh: g *= 1 - a^2 (a = the layer's output)
-__global__ void k_tanh_back(float* g, const float* a, size_t n) {
-    for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
-        g[i] *= 1.0f - a[i] * a[i];
 }
 
 // loss += mean (pred - target)^2; grad = 2 (pred - target) / n
@@ -360,34 +234,368 @@ __global__ void __launch_bounds__(128) k_conv_fwd_tc(const void* __restrict__ in
     }
 }
 
+// ---- FP32 layers and gradients on the tensor cores.  A float is the exact sum of three bf16 numbers (8 significand bits
+// each), and the weights are bf16: the correlations (forward, and the input gradient's) are three bf16 products per term,
+// the weight gradient, whose operands are both FP32, six (the three of relative size 2^-24 and less are dropped).  On
+// mma.sync the CUDA-core kernels' 22 TFLOP/s no longer bound them.  The tensor cores truncate their FP32 sums, so the
+// leading products are summed over one tap's channels (forward) or 16 pixels (weight gradient) only and added to the
+// result with a rounded FP32 addition; the other products are 2^-8 of these and share one accumulator.  Errors against 64
+// bits are measured in the tests of the layers; they are below the FMA chains' they replace.
+struct Split3 {
+    uint32_t v[3];                 // bf16 pairs: leading, middle, last parts
+};
+__device__ __forceinline__ Split3 split3(float a, float b) {
+    Split3 s;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        s.v[k] = *reinterpret_cast<const uint32_t*>(&h);
+        const float ha = __uint_as_float(s.v[k] << 16), hb = __uint_as_float(s.v[k] & 0xffff0000u);
+        a = isinf(ha) ? 0.0f : a - ha;                       // (an infinity has no remainder)
+        b = isinf(hb) ? 0.0f : b - hb;
+    }
+    return s;
+}
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void ldsm4(uint32_t* r, uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t* r, uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldsm2_t(uint32_t* r, uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
+}
+__device__ __forceinline__ void zero4(float* d) { d[0] = d[1] = d[2] = d[3] = 0.0f; }
+
+// words (bf16 pairs) per staged pixel of C channels: 16-byte rows at a stride of 20 words spread over all banks
+template <int C>
+constexpr int pixel_words() {
+    return C == 32 ? 20 : 4;
+}
+// the three parts of C channels of pixels [n] into planes of n pixels; value(c, p) reads channel c of pixel p
+template <int C, int THREADS, class F>
+__device__ __forceinline__ void stage_split(uint32_t* dst, int n, F value) {
+    constexpr int PW = pixel_words<C>(), G = C == 32 ? 4 : 1;           // groups of 8 channels
+    for (int k = threadIdx.x; k < G * n; k += THREADS) {
+        const int c0 = k / n * 8, p = k % n;
+        float x[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) x[c] = c < C ? value(c0 + c, p) : 0.0f;
+        uint32_t w[3][4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const Split3 s = split3(x[2 * c], x[2 * c + 1]);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) w[q][c] = s.v[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            *reinterpret_cast<uint4*>(dst + (q * n + p) * PW + c0 / 2) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+    }
+}
+
+constexpr int C3_THREADS = 256;
+template <int CIN, int NPAD>
+struct Conv3 {
+    // K = 9 taps of CIN channels, 8 at least (zero weights and inputs fill them up)
+    static constexpr int CP = CIN == 32 ? 32 : 8;
+    static constexpr int K = 9 * CP;                         // 288 or 72
+    static constexpr int KP = (K + 15) / 16 * 16;
+    static constexpr int KSW = KP / 2 + 4;                   // words per weight row: 148 or 44 (16-byte rows, spread banks)
+    static constexpr int PW = pixel_words<CIN>();
+    static constexpr int HP = HALO * HALO;
+    static constexpr size_t SMEM = sizeof(uint32_t) * (size_t(3) * HP * PW + size_t(NPAD) * KSW);
+};
+
+// out = act(bias + w (*) in) for FP32 in and out, or (FLIP) the input gradient's correlation with the flipped, transposed
+// weights w[cin][cout][8 - tap].  A CTA of 8 warps computes 16 x 16 pixels, a warp two rows of them (one m16 tile per
+// row), all channels.
+template <int CIN, int NPAD, bool FLIP>
+__global__ void __launch_bounds__(C3_THREADS, 2) k_conv_fwd_s3(const float* __restrict__ in,
+                                                              const __nv_bfloat16* __restrict__ w,
+                                                              const float* __restrict__ bias, float* __restrict__ out,
+                                                              int Cout, int H, int W, int act) {
+    using CV = Conv3<CIN, NPAD>;
+    constexpr int NT = NPAD / 8, PW = CV::PW, HP = CV::HP, CP = CV::CP;
+    extern __shared__ uint4 sm16[];
+    uint32_t* xs = reinterpret_cast<uint32_t*>(sm16);        // [3][HALO^2][PW]
+    uint32_t* ws = xs + 3 * HP * PW;                         // [NPAD][KSW]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int x0 = blockIdx.x * TS, y0 = blockIdx.y * TS, b = blockIdx.z;
+    const size_t HW = size_t(H) * W;
+    const float* inb = in + size_t(b) * CIN * HW;
+    stage_split<CIN, C3_THREADS>(xs, HP, [&](int c, int p) {
+        const int yy = y0 - 1 + p / HALO, xx = x0 - 1 + p % HALO;
+        return yy >= 0 && yy < H && xx >= 0 && xx < W ? inb[c * HW + size_t(yy) * W + xx] : 0.0f;
+    });
+    for (int idx = tid; idx < NPAD * (CV::KP / 2); idx += C3_THREADS) {
+        const int n = idx / (CV::KP / 2), k0 = 2 * (idx % (CV::KP / 2));
+        uint32_t v = 0u;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int c = (k0 + e) % CP, tap = (k0 + e) / CP;
+            if (n < Cout && c < CIN && tap < 9) {
+                const __nv_bfloat16 q = FLIP ? w[(size_t(c) * Cout + n) * 9 + 8 - tap] : w[(size_t(n) * CIN + c) * 9 + tap];
+                v |= uint32_t(*reinterpret_cast<const uint16_t*>(&q)) << (16 * e);
+            }
+        }
+        ws[n * CV::KSW + k0 / 2] = v;
+    }
+    __syncthreads();
+    // ldmatrix rows: lanes 0..15 the 16 pixels' first 8 channels of a k16 step, lanes 16..31 the next 8 (CP = 8: the next tap's)
+    const uint32_t xa = smem_addr(xs), wa = smem_addr(ws);
+    const int ap = lane & 15, ah = lane >> 4;
+    const int bn = (lane & 7) + ((lane >> 4) << 3), bk = (lane >> 3) & 1;      // weight rows: n, k half
+    float acc[2][NT][4], low[2][NT][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            zero4(acc[mt][nt]);
+            zero4(low[mt][nt]);
+        }
+    constexpr int STEPS = CV::KP / 16, FLUSH = CP == 32 ? 2 : 1;               // k16 steps; steps per rounded addition
+#pragma unroll 1
+    for (int s0 = 0; s0 < STEPS; s0 += FLUSH) {
+        float lead[2][NT][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) zero4(lead[mt][nt]);
+#pragma unroll
+        for (int f = 0; f < FLUSH; ++f) {
+            const int s = s0 + f;
+            uint32_t bf[NT][2];
+            if constexpr (NT == 1) {
+                const uint32_t* r = ws + (lane >> 2) * CV::KSW + s * 8 + (lane & 3);
+                bf[0][0] = r[0];
+                bf[0][1] = r[4];
+            } else {
+#pragma unroll
+                for (int nt = 0; nt < NT; nt += 2) {
+                    uint32_t r[4];
+                    ldsm4(r, wa + 4u * ((nt * 8 + bn) * CV::KSW + s * 8 + bk * 4));
+                    bf[nt][0] = r[0];
+                    bf[nt][1] = r[1];
+                    bf[nt + 1][0] = r[2];
+                    bf[nt + 1][1] = r[3];
+                }
+            }
+            // tap and channel offset of this lane's row (a step past the last tap has zero weights: any pixel will do)
+            const int k = s * 16 + ah * 8;
+            const int tap = min(k / CP, 8), c = k % CP;
+            const int off = ((tap / 3) * HALO + tap % 3 + ap) * PW + c / 2;
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                const uint32_t row = xa + 4u * ((warp * 2 + mt) * HALO * PW + off);
+                uint32_t a[3][4];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) ldsm4(a[q], row + 4u * q * HP * PW);
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) {
+                    mma_bf16_16816(lead[mt][nt], a[0], bf[nt]);
+                    mma_bf16_16816(low[mt][nt], a[1], bf[nt]);
+                    mma_bf16_16816(low[mt][nt], a[2], bf[nt]);
+                }
+            }
+        }
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[mt][nt][e] += lead[mt][nt][e];
+    }
+    const int g = lane >> 2, t = lane & 3;
+    float* ob = out + size_t(b) * Cout * HW;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        const int y = y0 + warp * 2 + mt;
+        if (y >= H) continue;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int x = x0 + g + (e >= 2 ? 8 : 0), co = nt * 8 + 2 * t + (e & 1);
+                if (co < Cout && x < W) {
+                    const float v = acc[mt][nt][e] + low[mt][nt][e] + (bias ? bias[co] : 0.0f);
+                    ob[co * HW + size_t(y) * W + x] = act ? tanhf(v) : v;
+                }
+            }
+    }
+}
+
+// Weight and bias gradients of one strip of tiles (a 16-pixel column, `rows` tiles high, one image): partial[strip] gets
+// sum_p g[co](p) in[ci](p + tap) and sum_p g[co](p) over the strip's pixels (reduced over strips by k_reduce_partials).
+// GEMM per tap: M = Cout, N = Cin, K = pixels, a warp per tap, both operands read from [pixel][channel] planes by transposed
+// ldmatrix, so a tap is a pixel offset.  With tanh the gradient through it, g (1 - a^2), is formed while the tile is staged
+// and written back (each pixel belongs to one tile).
+constexpr int WG_THREADS = 288;   // nine warps: the taps
+template <int CIN, int COUT>
+struct Wgrad {
+    static constexpr int MT = COUT == 32 ? 2 : 1, NT = CIN == 32 ? 4 : 1;
+    static constexpr int PX = pixel_words<CIN>(), PG = pixel_words<COUT>();
+    static constexpr int HP = HALO * HALO, NP = TS * TS;
+    static constexpr size_t SMEM = sizeof(uint32_t) * size_t(3) * (HP * PX + NP * PG);
+};
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(WG_THREADS, 1) k_conv_wgrad_s3(const float* __restrict__ in, float* __restrict__ g,
+                                                                const float* __restrict__ aout,
+                                                                float* __restrict__ partial, int H, int W, int rows) {
+    using WG = Wgrad<CIN, COUT>;
+    constexpr int MT = WG::MT, NT = WG::NT, PX = WG::PX, PG = WG::PG, HP = WG::HP, NP = WG::NP;
+    extern __shared__ uint4 sm16[];
+    uint32_t* xs = reinterpret_cast<uint32_t*>(sm16);        // [3][HALO^2][PX]
+    uint32_t* gs = xs + 3 * HP * PX;                         // [3][TS^2][PG]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int x0 = blockIdx.x * TS, b = blockIdx.z;
+    const size_t HW = size_t(H) * W;
+    const float* inb = in + size_t(b) * CIN * HW;
+    float* gb = g + size_t(b) * COUT * HW;
+    const float* ab = aout ? aout + size_t(b) * COUT * HW : nullptr;
+    float acc[MT][NT][4], low[MT][NT][4], accb[MT][4], lowb[MT][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+        zero4(accb[mt]);
+        zero4(lowb[mt]);
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            zero4(acc[mt][nt]);
+            zero4(low[mt][nt]);
+        }
+    }
+    const int ty = warp / 3, tx = warp % 3;
+    const uint32_t xa = smem_addr(xs), ga = smem_addr(gs);
+    const uint32_t one[2] = {0x3f803f80u, 0x3f803f80u};      // bf16 ones: the bias gradient as a product
+    for (int r = 0; r < rows; ++r) {
+        const int y0 = (blockIdx.y * rows + r) * TS;
+        if (y0 >= H) break;
+        __syncthreads();
+        stage_split<COUT, WG_THREADS>(gs, NP, [&](int c, int p) {
+            const int yy = y0 + p / TS, xx = x0 + p % TS;
+            if (yy >= H || xx >= W) return 0.0f;
+            const size_t o = c * HW + size_t(yy) * W + xx;
+            float v = gb[o];
+            if (ab) {
+                const float a = ab[o];
+                v *= 1.0f - a * a;
+                gb[o] = v;
+            }
+            return v;
+        });
+        stage_split<CIN, WG_THREADS>(xs, HP, [&](int c, int p) {
+            const int yy = y0 - 1 + p / HALO, xx = x0 - 1 + p % HALO;
+            return yy >= 0 && yy < H && xx >= 0 && xx < W ? inb[c * HW + size_t(yy) * W + xx] : 0.0f;
+        });
+        __syncthreads();
+#pragma unroll 1
+        for (int row = 0; row < TS; ++row) {                 // 16 pixels of the sum
+            // A: (m, k) = (co, pixel); ldmatrix rows are pixels of 8 channels: matrices (k 0-7 | k 8-15) x (m 0-7 | m 8-15)
+            uint32_t a[3][MT][4];
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    const int p = row * TS + (lane & 7) + ((lane >> 4) << 3);
+                    if constexpr (COUT == 32) {
+                        ldsm4_t(a[q][mt], ga + 4u * ((q * NP + p) * PG + mt * 8 + ((lane >> 3) & 1) * 4));
+                    } else {                                 // channels 8..15 of the tile are zero
+                        uint32_t h[2];
+                        ldsm2_t(h, ga + 4u * ((q * NP + row * TS + (lane & 15)) * PG));
+                        a[q][mt][0] = h[0];
+                        a[q][mt][2] = h[1];
+                        a[q][mt][1] = a[q][mt][3] = 0u;
+                    }
+                }
+            // B: (k, n) = (pixel + tap, ci)
+            uint32_t bf[3][NT][2];
+            const int pr = (row + ty) * HALO + tx;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                if constexpr (CIN == 32) {
+#pragma unroll
+                    for (int nt = 0; nt < NT; nt += 2) {
+                        uint32_t v[4];
+                        ldsm4_t(v, xa + 4u * ((q * HP + pr + (lane & 15)) * PX + nt * 4 + (lane >> 4) * 4));
+                        bf[q][nt][0] = v[0];
+                        bf[q][nt][1] = v[1];
+                        bf[q][nt + 1][0] = v[2];
+                        bf[q][nt + 1][1] = v[3];
+                    }
+                } else {
+                    ldsm2_t(bf[q][0], xa + 4u * ((q * HP + pr + (lane & 15)) * PX));
+                }
+            }
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) {
+                    float lead[4];
+                    zero4(lead);
+                    mma_bf16_16816(lead, a[0][mt], bf[0][nt]);
+                    mma_bf16_16816(low[mt][nt], a[0][mt], bf[1][nt]);
+                    mma_bf16_16816(low[mt][nt], a[1][mt], bf[0][nt]);
+                    mma_bf16_16816(low[mt][nt], a[1][mt], bf[1][nt]);
+                    mma_bf16_16816(low[mt][nt], a[0][mt], bf[2][nt]);
+                    mma_bf16_16816(low[mt][nt], a[2][mt], bf[0][nt]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[mt][nt][e] += lead[e];
+                }
+                if (warp == 4) {
+                    float lead[4];
+                    zero4(lead);
+                    mma_bf16_16816(lead, a[0][mt], one);
+                    mma_bf16_16816(lowb[mt], a[1][mt], one);
+                    mma_bf16_16816(lowb[mt], a[2][mt], one);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) accb[mt][e] += lead[e];
+                }
+            }
+        }
+    }
+    constexpr int nout = COUT * CIN * 9;
+    const size_t strip = (size_t(b) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    float* part = partial + strip * (nout + COUT);
+    const int gq = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int co = mt * 16 + gq + (e >= 2 ? 8 : 0), ci = nt * 8 + 2 * t + (e & 1);
+                if (co < COUT && ci < CIN) part[(co * CIN + ci) * 9 + warp] = acc[mt][nt][e] + low[mt][nt][e];
+            }
+        if (warp == 4 && t == 0)
+#pragma unroll
+            for (int e = 0; e < 4; e += 2) {
+                const int co = mt * 16 + gq + (e >= 2 ? 8 : 0);
+                if (co < COUT) part[nout + co] = accb[mt][e] + lowb[mt][e];
+            }
+    }
+}
+
 int grid_for(size_t n) {
     const size_t g = (n + 255) / 256;
     return int(g < 4096 ? (g > 0 ? g : 1) : 4096);
 }
 
-size_t fwd_smem(int Cin, int Cout) { return sizeof(float) * (size_t(Cout) * Cin * 9 + size_t(Cin) * HALO * HALO); }
-size_t wgrad_smem(int Cin, int Cout) {
-    const size_t tile = sizeof(float) * (size_t(TS) * TS * Cout + size_t(Cin) * HALO * HALO);
-    const size_t red = sizeof(float) * size_t(WG_THREADS) * Cout;   // G * npairs * COUT = 288 * COUT
-    return tile > red ? tile : red;
-}
-
-template <int COUT>
-cudaError_t fwd_launch(const float* in, const float* wf, const float* bias, float* out, int B, int Cin, int H, int W,
-                       int act, cudaStream_t s) {
-    dim3 grid((W + TS - 1) / TS, (H + TS - 1) / TS, B);
-    k_conv_fwd<COUT><<<grid, TS * TS, fwd_smem(Cin, COUT), s>>>(in, wf, bias, out, Cin, H, W, act);
-    return cudaGetLastError();
-}
-
-// strip height (tiles) so that the weight-gradient grid holds about 4 blocks per SM
+// strip height (tiles) so that the weight-gradient grid holds about 7 blocks per SM (one is resident: with 4 the last of 5
+// waves was a fifth full)
 int strip_rows(int B, int H, int W) {
     int nsm = 152;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const long long gx = (W + TS - 1) / TS, ty = (H + TS - 1) / TS;
-    const long long want = 4LL * nsm;
+    const long long want = 7LL * nsm;
     long long gy = (want + B * gx - 1) / (B * gx);
     if (gy < 1) gy = 1;
     if (gy > ty) gy = ty;
@@ -403,22 +611,58 @@ bool shape_ok(int B, int Cin, int Cout, int H, int W) {
 
 }  // namespace
 
-cudaError_t nn_prepare() {
-    const int f32 = int(fwd_smem(MAXC, 32)), f4 = int(fwd_smem(MAXC, 4)), f2 = int(fwd_smem(MAXC, 2));
-    cudaError_t e = cudaFuncSetAttribute(k_conv_fwd<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, f32);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_fwd<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, f4);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_fwd<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, f2);
-    const int g32 = int(wgrad_smem(MAXC, 32)), g4 = int(wgrad_smem(MAXC, 4)), g2 = int(wgrad_smem(MAXC, 2));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_wgrad<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, g32);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, g4);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_wgrad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, g2);
-    return e;
-}
+namespace {
 
-cudaError_t nn_bf16_to_float(const uint16_t* w, float* f, size_t n, cudaStream_t s) {
-    k_bf16_to_f32<<<grid_for(n), 256, 0, s>>>((const __nv_bfloat16*)w, f, n);
+// the FP32 layers' kernels by their channel counts: f(integral constants Cin, output channels padded to 8 or 32)
+template <int C>
+struct Int {
+    static constexpr int value = C;
+};
+template <class F>
+cudaError_t by_channels(int Cin, int Cout, F f) {
+    const bool wide = Cout > 8;
+    switch (Cin) {
+        case 2: return wide ? f(Int<2>(), Int<32>()) : f(Int<2>(), Int<8>());
+        case 4: return wide ? f(Int<4>(), Int<32>()) : f(Int<4>(), Int<8>());
+        case 32: return wide ? f(Int<32>(), Int<32>()) : f(Int<32>(), Int<8>());
+        default: return cudaErrorInvalidValue;
+    }
+}
+template <bool FLIP>
+cudaError_t conv_s3(const float* in, const uint16_t* w, const float* bias, float* out, int B, int Cin, int Cout, int H,
+                    int W, int act, cudaStream_t s) {
+    return by_channels(Cin, Cout, [&](auto ci, auto np) {
+        constexpr int CIN = decltype(ci)::value, NPAD = decltype(np)::value;
+        const size_t sm = Conv3<CIN, NPAD>::SMEM;
+        const cudaError_t e = cudaFuncSetAttribute(k_conv_fwd_s3<CIN, NPAD, FLIP>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+        if (e != cudaSuccess) return e;
+        const dim3 grid((W + TS - 1) / TS, (H + TS - 1) / TS, B);
+        k_conv_fwd_s3<CIN, NPAD, FLIP><<<grid, C3_THREADS, sm, s>>>(in, (const __nv_bfloat16*)w, bias, out, Cout, H, W, act);
+        return cudaGetLastError();
+    });
+}
+template <int CIN, int COUT>
+cudaError_t wgrad_launch(dim3 grid, const float* in, float* g, const float* aout, float* partial, int H, int W, int rows,
+                         cudaStream_t s) {
+    const size_t sm = Wgrad<CIN, COUT>::SMEM;
+    const cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_s3<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(sm));
+    if (e != cudaSuccess) return e;
+    k_conv_wgrad_s3<CIN, COUT><<<grid, WG_THREADS, sm, s>>>(in, g, aout, partial, H, W, rows);
     return cudaGetLastError();
 }
+template <int CIN>
+cudaError_t wgrad_by_cout(int Cout, dim3 grid, const float* in, float* g, const float* aout, float* partial, int H, int W,
+                          int rows, cudaStream_t s) {
+    switch (Cout) {
+        case 2: return wgrad_launch<CIN, 2>(grid, in, g, aout, partial, H, W, rows, s);
+        case 4: return wgrad_launch<CIN, 4>(grid, in, g, aout, partial, H, W, rows, s);
+        default: return wgrad_launch<CIN, 32>(grid, in, g, aout, partial, H, W, rows, s);
+    }
+}
+
+}  // namespace
 
 template <bool IN_NHWC, bool OUT_NHWC>
 cudaError_t conv_tc_launch(const void* in, const __nv_bfloat16* wb, const float* bias, void* out, int B, int Cin,
@@ -460,16 +704,6 @@ cudaError_t nn_conv_forward_bf16_fmt(const void* in, bool in_nhwc, const uint16_
                     : conv_tc_launch<false, false>(in, wb, bias, out, B, Cin, Cout, H, W, act, s);
 }
 
-cudaError_t nn_conv_forward_f32(const float* in, const float* wf, const float* bias, float* out, int B, int Cin,
-                                int Cout, int H, int W, int act, cudaStream_t s) {
-    switch (Cout) {
-        case 2: return fwd_launch<2>(in, wf, bias, out, B, Cin, H, W, act, s);
-        case 4: return fwd_launch<4>(in, wf, bias, out, B, Cin, H, W, act, s);
-        case 32: return fwd_launch<32>(in, wf, bias, out, B, Cin, H, W, act, s);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
 }  // namespace es
 
 using namespace es;
@@ -490,12 +724,8 @@ int es_nn_conv_forward(const float* in, const uint16_t* w, const float* bias, fl
     if (!in || !w || !out || !workspace || !shape_ok(B, Cin, Cout, H, W)) return ES_ERR_ARG;
     if (workspace_bytes < sizeof(float) * size_t(Cout) * Cin * 9) return ES_ERR_ARG;
     if (in == out) return ES_ERR_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
-    float* wf = (float*)workspace;
-    if (nn_prepare() != cudaSuccess) return ES_ERR_CUDA;
-    if (nn_bf16_to_float(w, wf, size_t(Cout) * Cin * 9, s) != cudaSuccess) return ES_ERR_CUDA;
-    return nn_conv_forward_f32(in, wf, bias, out, B, Cin, Cout, H, W, act_tanh, s) == cudaSuccess ? ES_OK
-                                                                                                : ES_ERR_CUDA;
+    return conv_s3<false>(in, w, bias, out, B, Cin, Cout, H, W, act_tanh, (cudaStream_t)stream) == cudaSuccess ? ES_OK
+                                                                                                              : ES_ERR_CUDA;
 }
 
 int es_nn_conv_forward_bf16(const float* in, const uint16_t* w, const float* bias, float* out, int B, int Cin,
@@ -515,28 +745,19 @@ int es_nn_conv_backward(const float* in, const uint16_t* w, const float* out, fl
     if (workspace_bytes < es_nn_workspace_bytes(B, Cin, Cout, H, W)) return ES_ERR_ARG;
     if (grad_in && (grad_in == grad_out || grad_in == in)) return ES_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (nn_prepare() != cudaSuccess) return ES_ERR_CUDA;
-    const size_t nout_g = size_t(B) * Cout * H * W;
-    if (act_tanh) k_tanh_back<<<grid_for(nout_g), 256, 0, s>>>(grad_out, out, nout_g);
-    float* wt = (float*)workspace;
-    float* partial = wt + size_t(Cout) * Cin * 9;
+    float* partial = (float*)workspace + size_t(Cout) * Cin * 9;
     const int rows = strip_rows(B, H, W);
-    dim3 grid((W + TS - 1) / TS, ((H + TS - 1) / TS + rows - 1) / rows, B);
-    const size_t sm = wgrad_smem(Cin, Cout);
-    switch (Cout) {
-        case 2: k_conv_wgrad<2><<<grid, WG_THREADS, sm, s>>>(in, grad_out, partial, Cin, H, W, rows); break;
-        case 4: k_conv_wgrad<4><<<grid, WG_THREADS, sm, s>>>(in, grad_out, partial, Cin, H, W, rows); break;
-        default: k_conv_wgrad<32><<<grid, WG_THREADS, sm, s>>>(in, grad_out, partial, Cin, H, W, rows); break;
-    }
-    const int nout = Cout * Cin * 9;
-    const int strips = int(grid.x * grid.y * grid.z);
-    k_reduce_partials<<<grid_for(size_t(nout + Cout)), 256, 0, s>>>(partial, strips, nout + Cout, grad_w, grad_b,
-                                                                     nout);
-    if (grad_in) {
-        k_flip_weights<<<grid_for(size_t(nout)), 256, 0, s>>>((const __nv_bfloat16*)w, wt, Cin, Cout);
-        if (nn_conv_forward_f32(grad_out, wt, nullptr, grad_in, B, Cout, Cin, H, W, 0, s) != cudaSuccess)
-            return ES_ERR_CUDA;
-    }
+    const dim3 grid((W + TS - 1) / TS, ((H + TS - 1) / TS + rows - 1) / rows, B);
+    const float* aout = act_tanh ? out : nullptr;            // the gradient through tanh is formed in the same pass
+    const cudaError_t e = Cin == 2   ? wgrad_by_cout<2>(Cout, grid, in, grad_out, aout, partial, H, W, rows, s)
+                          : Cin == 4 ? wgrad_by_cout<4>(Cout, grid, in, grad_out, aout, partial, H, W, rows, s)
+                                     : wgrad_by_cout<32>(Cout, grid, in, grad_out, aout, partial, H, W, rows, s);
+    if (e != cudaSuccess) return ES_ERR_CUDA;
+    const int nout = Cout * Cin * 9, len = nout + Cout;
+    k_reduce_partials<<<(len + 31) / 32, 32 * RP_GROUPS, 0, s>>>(partial, int(grid.x * grid.y * grid.z), len, grad_w, grad_b,
+                                                              nout);
+    if (grad_in && conv_s3<true>(grad_out, w, nullptr, grad_in, B, Cout, Cin, H, W, 0, s) != cudaSuccess)
+        return ES_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? ES_OK : ES_ERR_CUDA;
 }
 

@@ -1,0 +1,45 @@
+"""The FP32 layers on the tensor cores (operands split into bf16 parts): every channel combination, ragged images and
+tiles, against the oracle's correlations, to the rounding of FP32 sums."""
+import numpy as np
+import pytest
+
+from oracle import convnet
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("cin", [2, 4, 32])
+@pytest.mark.parametrize("cout", [2, 4, 32])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 16, 16), (1, 17, 15), (2, 50, 33)])
+def test_forward_and_gradients_vs_oracle(cin, cout, shape):
+    """Sums of n products rounded to FP32 stay within 4e-7 sqrt(n) of the largest result (an FMA chain's random walk, the
+    bound the CUDA-core layers were held to); inputs over several decades."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    B, H, W = shape
+    rng = np.random.default_rng(11 + 100 * cin + cout + H)
+    a = (rng.standard_normal((B, cin, H, W)) * 10.0 ** rng.uniform(-2, 1, (B, cin, 1, 1))).astype(np.float32)
+    w = convnet.bf16_round((rng.standard_normal((cout, cin, 3, 3)) / np.sqrt(9 * cin)).astype(np.float32))
+    wt = torch.tensor(w, dtype=torch.bfloat16, device="cuda")
+    b = rng.standard_normal(cout).astype(np.float32)
+    at = torch.tensor(a, device="cuda")
+    ws = torch.empty(es.es_nn_workspace_bytes(B, cin, cout, H, W) // 4 + 1, dtype=torch.float32, device="cuda")
+    z = convnet.conv3x3(a.astype(np.float64), w, b.astype(np.float64))
+    for act in (False, True):
+        out = torch.empty((B, cout, H, W), dtype=torch.float32, device="cuda")
+        es.es_nn_conv_forward(at, wt, torch.tensor(b, device="cuda"), out, act, ws)
+        got, ref = out.cpu().double().numpy(), np.tanh(z) if act else z
+        assert np.abs(got - ref).max() <= 4e-7 * np.sqrt(9 * cin) * np.abs(z).max()
+        go = rng.standard_normal((B, cout, H, W)).astype(np.float32)
+        g = torch.tensor(go, device="cuda")
+        gin, gw, gb = torch.empty_like(at), torch.empty((cout, cin, 3, 3), device="cuda"), torch.empty(cout, device="cuda")
+        es.es_nn_conv_backward(at, wt, out, g, gin, gw, gb, act, ws)
+        gz = go * (1.0 - np.tanh(z) ** 2) if act else go.astype(np.float64)
+        rw, rb, ra = convnet.conv3x3_backward(a.astype(np.float64), w, gz)
+        # the layer's output enters the gradient through tanh with its own rounding: 4e-7 sqrt(n) of |z| in 1 - a^2
+        back = 8e-7 * np.sqrt(9 * cin) * np.abs(z).max() if act else 0.0
+        assert np.abs(g.cpu().double().numpy() - gz).max() <= (2e-7 + back) * np.abs(go).max()
+        for got, ref, n in ((gw, rw, B * H * W), (gb, rb, B * H * W), (gin, ra, 9 * cout)):
+            scale = np.abs(ref).max() + np.abs(go).max() * (np.abs(a).max() if ref is rw else 1.0)
+            assert np.abs(got.cpu().double().numpy() - ref).max() <= (4e-7 * np.sqrt(n) + back * np.sqrt(n)) * scale
