@@ -434,152 +434,200 @@ __global__ void __launch_bounds__(C3_THREADS, 2) k_conv_fwd_s3(const float* __re
 
 // Weight and bias gradients of one strip of tiles (a 16-pixel column, `rows` tiles high, one image): partial[strip] gets
 // sum_p g[co](p) in[ci](p + tap) and sum_p g[co](p) over the strip's pixels (reduced over strips by k_reduce_partials).
-// GEMM per tap: M = Cout, N = Cin, K = pixels, a warp per tap, both operands read from [pixel][channel] planes by transposed
+// GEMM per tap: M = Cout, N = Cin, K = pixels, both operands read from [pixel][channel] planes by transposed
 // ldmatrix, so a tap is a pixel offset.  With tanh the gradient through it, g (1 - a^2), is formed while the tile is staged
 // and written back (each pixel belongs to one tile).
-constexpr int WG_THREADS = 288;   // nine warps: the taps
+// Tiles are 16 x 8 pixels in two buffers: the next tile's values are loaded into registers before the current tile's
+// products and split into the other buffer after them, so that the loads' latency hides behind the tensor cores.  18 warps
+// (9 taps x 2 halves of 32 output channels) spread over the four schedulers as 5, 5, 4, 4 (with a warp per tap, 3, 2, 2, 2,
+// and 16 x 16 tiles in one buffer: 920 us instead of 487 us for 32 -> 32 channels at 4 x 512^2).
+constexpr int WG_H = 8;           // rows of a tile
 template <int CIN, int COUT>
 struct Wgrad {
     static constexpr int MT = COUT == 32 ? 2 : 1, NT = CIN == 32 ? 4 : 1;
+    static constexpr int THREADS = 32 * 9 * MT;              // a warp per tap and 16 output channels
     static constexpr int PX = pixel_words<CIN>(), PG = pixel_words<COUT>();
-    static constexpr int HP = HALO * HALO, NP = TS * TS;
-    static constexpr size_t SMEM = sizeof(uint32_t) * size_t(3) * (HP * PX + NP * PG);
+    static constexpr int HP = HALO * (WG_H + 2), NP = TS * WG_H;
+    static constexpr int NG = (COUT == 32 ? 4 : 1) * NP, NX = (CIN == 32 ? 4 : 1) * HP;    // groups of 8 channels
+    static constexpr int GI = (NG + THREADS - 1) / THREADS, XI = (NX + THREADS - 1) / THREADS;
+    static constexpr int BUF = 3 * (HP * PX + NP * PG);      // words of a buffer
+    static constexpr size_t SMEM = sizeof(uint32_t) * size_t(2) * BUF;
 };
+// the three parts of 8 channels at word `w` of a plane, planes `plane` words apart
+__device__ __forceinline__ void store_split(uint32_t* w, int plane, const float* x) {
+    uint32_t v[3][4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const Split3 s = split3(x[2 * c], x[2 * c + 1]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q][c] = s.v[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4*>(w + q * plane) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
+}
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(WG_THREADS, 1) k_conv_wgrad_s3(const float* __restrict__ in, float* __restrict__ g,
-                                                                const float* __restrict__ aout,
-                                                                float* __restrict__ partial, int H, int W, int rows) {
+__global__ void __launch_bounds__(Wgrad<CIN, COUT>::THREADS, 1)
+    k_conv_wgrad_s3(const float* __restrict__ in, float* g, const float* __restrict__ aout, float* __restrict__ partial,
+                    int H, int W, int rows) {
     using WG = Wgrad<CIN, COUT>;
-    constexpr int MT = WG::MT, NT = WG::NT, PX = WG::PX, PG = WG::PG, HP = WG::HP, NP = WG::NP;
+    constexpr int NT = WG::NT, PX = WG::PX, PG = WG::PG, HP = WG::HP, NP = WG::NP, TH = WG::THREADS;
     extern __shared__ uint4 sm16[];
-    uint32_t* xs = reinterpret_cast<uint32_t*>(sm16);        // [3][HALO^2][PX]
-    uint32_t* gs = xs + 3 * HP * PX;                         // [3][TS^2][PG]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t* sm = reinterpret_cast<uint32_t*>(sm16);        // two of { [3][HP][PX], [3][NP][PG] }
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tap = warp % 9, mt = warp / 9;
     const int x0 = blockIdx.x * TS, b = blockIdx.z;
+    const int yb = blockIdx.y * rows * TS;
+    const int ye = min(H, yb + rows * TS);                   // the strip's rows
     const size_t HW = size_t(H) * W;
     const float* inb = in + size_t(b) * CIN * HW;
     float* gb = g + size_t(b) * COUT * HW;
     const float* ab = aout ? aout + size_t(b) * COUT * HW : nullptr;
-    float acc[MT][NT][4], low[MT][NT][4], accb[MT][4], lowb[MT][4];
+
+    float gv[WG::GI][8], av[WG::GI][8], xv[WG::XI][8];
+    auto load = [&](int y0) {
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-        zero4(accb[mt]);
-        zero4(lowb[mt]);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            zero4(acc[mt][nt]);
-            zero4(low[mt][nt]);
-        }
-    }
-    const int ty = warp / 3, tx = warp % 3;
-    const uint32_t xa = smem_addr(xs), ga = smem_addr(gs);
-    const uint32_t one[2] = {0x3f803f80u, 0x3f803f80u};      // bf16 ones: the bias gradient as a product
-    for (int r = 0; r < rows; ++r) {
-        const int y0 = (blockIdx.y * rows + r) * TS;
-        if (y0 >= H) break;
-        __syncthreads();
-        stage_split<COUT, WG_THREADS>(gs, NP, [&](int c, int p) {
+        for (int i = 0; i < WG::GI; ++i) {
+            const int k = tid + i * TH, c0 = k / NP * 8, p = k % NP;
             const int yy = y0 + p / TS, xx = x0 + p % TS;
-            if (yy >= H || xx >= W) return 0.0f;
-            const size_t o = c * HW + size_t(yy) * W + xx;
-            float v = gb[o];
-            if (ab) {
-                const float a = ab[o];
-                v *= 1.0f - a * a;
-                gb[o] = v;
+            const bool ok = k < WG::NG && yy < H && xx < W;
+            const size_t o = size_t(yy) * W + xx;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                gv[i][c] = ok && c < COUT ? gb[(c0 + c) * HW + o] : 0.0f;
+                av[i][c] = ok && c < COUT && ab ? ab[(c0 + c) * HW + o] : 0.0f;
             }
-            return v;
-        });
-        stage_split<CIN, WG_THREADS>(xs, HP, [&](int c, int p) {
+        }
+#pragma unroll
+        for (int i = 0; i < WG::XI; ++i) {
+            const int k = tid + i * TH, c0 = k / HP * 8, p = k % HP;
             const int yy = y0 - 1 + p / HALO, xx = x0 - 1 + p % HALO;
-            return yy >= 0 && yy < H && xx >= 0 && xx < W ? inb[c * HW + size_t(yy) * W + xx] : 0.0f;
-        });
-        __syncthreads();
-#pragma unroll 1
-        for (int row = 0; row < TS; ++row) {                 // 16 pixels of the sum
-            // A: (m, k) = (co, pixel); ldmatrix rows are pixels of 8 channels: matrices (k 0-7 | k 8-15) x (m 0-7 | m 8-15)
-            uint32_t a[3][MT][4];
+            const bool ok = k < WG::NX && yy >= 0 && yy < H && xx >= 0 && xx < W;
+            const size_t o = size_t(ok ? yy : 0) * W + (ok ? xx : 0);
 #pragma unroll
-            for (int q = 0; q < 3; ++q)
+            for (int c = 0; c < 8; ++c) xv[i][c] = ok && c < CIN ? inb[(c0 + c) * HW + o] : 0.0f;
+        }
+    };
+    auto store = [&](int y0, uint32_t* buf) {
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    const int p = row * TS + (lane & 7) + ((lane >> 4) << 3);
-                    if constexpr (COUT == 32) {
-                        ldsm4_t(a[q][mt], ga + 4u * ((q * NP + p) * PG + mt * 8 + ((lane >> 3) & 1) * 4));
-                    } else {                                 // channels 8..15 of the tile are zero
-                        uint32_t h[2];
-                        ldsm2_t(h, ga + 4u * ((q * NP + row * TS + (lane & 15)) * PG));
-                        a[q][mt][0] = h[0];
-                        a[q][mt][2] = h[1];
-                        a[q][mt][1] = a[q][mt][3] = 0u;
-                    }
+        for (int i = 0; i < WG::GI; ++i) {
+            const int k = tid + i * TH, c0 = k / NP * 8, p = k % NP;
+            if (k >= WG::NG) break;
+            if (ab) {                                        // the gradient through tanh, kept for the input gradient
+                const int yy = y0 + p / TS, xx = x0 + p % TS;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    gv[i][c] *= 1.0f - av[i][c] * av[i][c];
+                    if (c < COUT && yy < H && xx < W) gb[(c0 + c) * HW + size_t(yy) * W + xx] = gv[i][c];
                 }
-            // B: (k, n) = (pixel + tap, ci)
-            uint32_t bf[3][NT][2];
-            const int pr = (row + ty) * HALO + tx;
+            }
+            store_split(buf + 3 * HP * PX + p * PG + c0 / 2, NP * PG, gv[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < WG::XI; ++i) {
+            const int k = tid + i * TH, c0 = k / HP * 8, p = k % HP;
+            if (k < WG::NX) store_split(buf + p * PX + c0 / 2, HP * PX, xv[i]);
+        }
+    };
+
+    float acc[NT][4], low[NT][4], accb[4], lowb[4];
+    zero4(accb);
+    zero4(lowb);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        zero4(acc[nt]);
+        zero4(low[nt]);
+    }
+    const int ty = tap / 3, tx = tap % 3;
+    const uint32_t one[2] = {0x3f803f80u, 0x3f803f80u};      // bf16 ones: the bias gradient as a product
+    load(yb);
+    store(yb, sm);
+    __syncthreads();
+    int cur = 0;
+    for (int y0 = yb; y0 < ye; y0 += WG_H, cur ^= 1) {
+        const bool more = y0 + WG_H < ye;
+        if (more) load(y0 + WG_H);
+        const uint32_t xa = smem_addr(sm + cur * WG::BUF), ga = xa + 4u * 3 * HP * PX;
+#pragma unroll 1
+        for (int row = 0; row < WG_H; ++row) {               // 16 pixels of the sum
+            // A: (m, k) = (co, pixel); ldmatrix rows are pixels of 8 channels: matrices (k 0-7 | k 8-15) x (m 0-7 | m 8-15)
+            uint32_t a[3][4];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                if constexpr (CIN == 32) {
-#pragma unroll
-                    for (int nt = 0; nt < NT; nt += 2) {
-                        uint32_t v[4];
-                        ldsm4_t(v, xa + 4u * ((q * HP + pr + (lane & 15)) * PX + nt * 4 + (lane >> 4) * 4));
-                        bf[q][nt][0] = v[0];
-                        bf[q][nt][1] = v[1];
-                        bf[q][nt + 1][0] = v[2];
-                        bf[q][nt + 1][1] = v[3];
-                    }
-                } else {
-                    ldsm2_t(bf[q][0], xa + 4u * ((q * HP + pr + (lane & 15)) * PX));
+                if constexpr (COUT == 32) {
+                    const int p = row * TS + (lane & 7) + ((lane >> 4) << 3);
+                    ldsm4_t(a[q], ga + 4u * ((q * NP + p) * PG + mt * 8 + ((lane >> 3) & 1) * 4));
+                } else {                                     // channels 8..15 of the tile are zero
+                    uint32_t h[2];
+                    ldsm2_t(h, ga + 4u * ((q * NP + row * TS + (lane & 15)) * PG));
+                    a[q][0] = h[0];
+                    a[q][2] = h[1];
+                    a[q][1] = a[q][3] = 0u;
                 }
             }
+            // B: (k, n) = (pixel + tap, ci), two n8 tiles at a time
+            const int pr = (row + ty) * HALO + tx;
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
+            for (int n0 = 0; n0 < NT; n0 += 2) {
+                constexpr int NB = NT == 1 ? 1 : 2;
+                uint32_t bf[3][2][2];
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
+                for (int q = 0; q < 3; ++q) {
+                    if constexpr (CIN == 32) {
+                        uint32_t v[4];
+                        ldsm4_t(v, xa + 4u * ((q * HP + pr + (lane & 15)) * PX + n0 * 4 + (lane >> 4) * 4));
+                        bf[q][0][0] = v[0];
+                        bf[q][0][1] = v[1];
+                        bf[q][1][0] = v[2];
+                        bf[q][1][1] = v[3];
+                    } else {
+                        ldsm2_t(bf[q][0], xa + 4u * ((q * HP + pr + (lane & 15)) * PX));
+                    }
+                }
+#pragma unroll
+                for (int n = 0; n < NB; ++n) {
+                    float* l = low[n0 + n];
                     float lead[4];
                     zero4(lead);
-                    mma_bf16_16816(lead, a[0][mt], bf[0][nt]);
-                    mma_bf16_16816(low[mt][nt], a[0][mt], bf[1][nt]);
-                    mma_bf16_16816(low[mt][nt], a[1][mt], bf[0][nt]);
-                    mma_bf16_16816(low[mt][nt], a[1][mt], bf[1][nt]);
-                    mma_bf16_16816(low[mt][nt], a[0][mt], bf[2][nt]);
-                    mma_bf16_16816(low[mt][nt], a[2][mt], bf[0][nt]);
+                    mma_bf16_16816(lead, a[0], bf[0][n]);
+                    mma_bf16_16816(l, a[0], bf[1][n]);
+                    mma_bf16_16816(l, a[1], bf[0][n]);
+                    mma_bf16_16816(l, a[1], bf[1][n]);
+                    mma_bf16_16816(l, a[0], bf[2][n]);
+                    mma_bf16_16816(l, a[2], bf[0][n]);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[mt][nt][e] += lead[e];
+                    for (int e = 0; e < 4; ++e) acc[n0 + n][e] += lead[e];
                 }
-                if (warp == 4) {
-                    float lead[4];
-                    zero4(lead);
-                    mma_bf16_16816(lead, a[0][mt], one);
-                    mma_bf16_16816(lowb[mt], a[1][mt], one);
-                    mma_bf16_16816(lowb[mt], a[2][mt], one);
+            }
+            if (tap == 4) {
+                float lead[4];
+                zero4(lead);
+                mma_bf16_16816(lead, a[0], one);
+                mma_bf16_16816(lowb, a[1], one);
+                mma_bf16_16816(lowb, a[2], one);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) accb[mt][e] += lead[e];
-                }
+                for (int e = 0; e < 4; ++e) accb[e] += lead[e];
             }
         }
+        if (more) store(y0 + WG_H, sm + (cur ^ 1) * WG::BUF);
+        __syncthreads();
     }
     constexpr int nout = COUT * CIN * 9;
     const size_t strip = (size_t(b) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     float* part = partial + strip * (nout + COUT);
     const int gq = lane >> 2, t = lane & 3;
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
+        for (int e = 0; e < 4; ++e) {
+            const int co = mt * 16 + gq + (e >= 2 ? 8 : 0), ci = nt * 8 + 2 * t + (e & 1);
+            if (co < COUT && ci < CIN) part[(co * CIN + ci) * 9 + tap] = acc[nt][e] + low[nt][e];
+        }
+    if (tap == 4 && t == 0)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int co = mt * 16 + gq + (e >= 2 ? 8 : 0), ci = nt * 8 + 2 * t + (e & 1);
-                if (co < COUT && ci < CIN) part[(co * CIN + ci) * 9 + warp] = acc[mt][nt][e] + low[mt][nt][e];
-            }
-        if (warp == 4 && t == 0)
-#pragma unroll
-            for (int e = 0; e < 4; e += 2) {
-                const int co = mt * 16 + gq + (e >= 2 ? 8 : 0);
-                if (co < COUT) part[nout + co] = accb[mt][e] + lowb[mt][e];
-            }
-    }
+        for (int e = 0; e < 4; e += 2) {
+            const int co = mt * 16 + gq + (e >= 2 ? 8 : 0);
+            if (co < COUT) part[nout + co] = accb[e] + lowb[e];
+        }
 }
 
 int grid_for(size_t n) {
@@ -649,7 +697,7 @@ cudaError_t wgrad_launch(dim3 grid, const float* in, float* g, const float* aout
     const cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_s3<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                int(sm));
     if (e != cudaSuccess) return e;
-    k_conv_wgrad_s3<CIN, COUT><<<grid, WG_THREADS, sm, s>>>(in, g, aout, partial, H, W, rows);
+    k_conv_wgrad_s3<CIN, COUT><<<grid, Wgrad<CIN, COUT>::THREADS, sm, s>>>(in, g, aout, partial, H, W, rows);
     return cudaGetLastError();
 }
 template <int CIN>
