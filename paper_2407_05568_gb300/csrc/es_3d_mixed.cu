@@ -4,9 +4,9 @@
 // primitive state rho, v, T of every node carries a low part so that jumps between neighbours
 // keep their digits, the two-point fluxes and MR-WENO5 run in float, and the dissipation works on
 // entropy-variable jumps from the jump decomposition of Sec. 3.1 (eq. jumpV) shared by the faces
-// of a line.  The node fields are computed once per node in double-float arithmetic and stored
-// as floats (with the low parts), and the metrics are the FP64 cross-form metrics of es_3d.cu
-// rounded to float at load.  The right-hand sides are accumulated over the
+// of a line (es_flux32.cuh, D = 3).  The node fields are computed once per node in double-float arithmetic and stored
+// as floats (with the low parts), and the metrics are the cross-form metrics of es_3d.cu formed in double-float and
+// rounded to float.  The right-hand sides are accumulated over the
 // three directions in float and the Shu-Osher combination is done in double-float.
 #include <cuda.h>            // CUtensorMap (the encoder is fetched from the driver at run time)
 #include <cuda_runtime.h>
@@ -17,6 +17,7 @@
 #include "es_bits.cuh"
 #include "es_3d_grid.cuh"
 #include "es_device.cuh"
+#include "es_flux32.cuh"
 #include "es_internal.h"
 #include "es_mesh_f32.h"
 #include "es_mixed_device.cuh"
@@ -33,18 +34,14 @@ using mixed::df_mul;
 using mixed::df_mul_f;
 using mixed::df_recip;
 using mixed::GasF;
-using mixed::inv_log_mean_f;
-using mixed::inv_log_mean_j;
-using mixed::mr_weno5_f;
-using mixed::WenoF;
 
-// float node fields (global planes and shared-memory slots)
+// Float node fields (global planes), in the order of the direction kernels' float4: halves of rho, T, v, v/T, rho v,
+// g = R/(1 - b rho) - a rho/T, a rho/T, E0 = |v|^2/(2T) + 2 a rho/T, rho/p and of the low parts of the double-float rho, T,
+// v (the faces and pairs read means of two nodes, then one addition); 1/(1 - b rho) and 1/T whole.
 enum FieldM {
-    M_RHO, M_V1, M_V2, M_V3, M_T, M_IT, M_OM, M_IOM, M_G, M_RT, M_VT1, M_VT2, M_VT3, M_V2T,
-    M_RV1, M_RV2, M_RV3, M_RP, M_RHOL, M_V1L, M_V2L, M_V3L, M_TL,
-    MF_COUNT,
-    M_NX = MF_COUNT, M_NY, M_NZ, M_XT,
-    MS_COUNT
+    M_RHO, M_T, M_IOM, M_E0, M_V1, M_V2, M_V3, M_G, M_VT1, M_VT2, M_VT3, M_ART, M_RV1, M_RV2, M_RV3, M_RP,
+    M_RHOL, M_TL, M_IT, M_V1L, M_V2L, M_V3L,
+    MF_COUNT
 };
 static_assert(MF_COUNT <= 23, "the float node fields reuse the FP64 node-field buffer");
 
@@ -72,233 +69,40 @@ __global__ void k3_nodes_f(Grid3 g, GasF G, const float* JU, const float* J, flo
         const df Td = df_mul_f(df_add(e, df_mul_f(rho, G.a)), G.icv);
         const float r = rho.hi, Tf = Td.hi;
         const float om = 1.0f - G.b * r;
-        const float iom = 1.0f / om;
-        const float iT = 1.0f / Tf;
-        const float p = r * G.R * Tf * iom - G.a * r * r;
-        if (!(r > 0.0f) || !(om > 0.0f) || !(Tf > 0.0f) || !(p > 0.0f)) raise_error(st, ES_ERR_INADMISSIBLE, id);
-        NF[M_RHO * P + id] = r;
-        NF[M_RHOL * P + id] = rho.lo;
-        NF[M_T * P + id] = Tf;
-        NF[M_TL * P + id] = Td.lo;
+        const float iom = flux32::rcp(om), iT = flux32::rcp(Tf);
+        const float ar = G.a * r;
+        const float prho = G.R * Tf * iom - ar;              // p/rho
+        if (!(r > 0.0f) || !(om > 0.0f) || !(Tf > 0.0f) || !(prho > 0.0f)) raise_error(st, ES_ERR_INADMISSIBLE, id);
+        const float hiT = 0.5f * iT, art = ar * hiT;
+        NF[M_RHO * P + id] = 0.5f * r;
+        NF[M_RHOL * P + id] = 0.5f * rho.lo;
+        NF[M_T * P + id] = 0.5f * Tf;
+        NF[M_TL * P + id] = 0.5f * Td.lo;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            NF[(M_V1 + c) * P + id] = v[c].hi;
-            NF[(M_V1L + c) * P + id] = v[c].lo;
-            NF[(M_VT1 + c) * P + id] = v[c].hi * iT;
-            NF[(M_RV1 + c) * P + id] = m[c].hi;
+            NF[(M_V1 + c) * P + id] = 0.5f * v[c].hi;
+            NF[(M_V1L + c) * P + id] = 0.5f * v[c].lo;
+            NF[(M_VT1 + c) * P + id] = v[c].hi * hiT;
+            NF[(M_RV1 + c) * P + id] = 0.5f * m[c].hi;
         }
         NF[M_IT * P + id] = iT;
-        NF[M_OM * P + id] = om;
         NF[M_IOM * P + id] = iom;
-        NF[M_G * P + id] = G.R * iom - G.a * r * iT;
-        NF[M_RT * P + id] = r * iT;
-        NF[M_V2T * P + id] = 2.0f * ke.hi * iT;
-        NF[M_RP * P + id] = r / p;
+        NF[M_G * P + id] = fmaf(0.5f * G.R, iom, -art);
+        NF[M_ART * P + id] = art;
+        NF[M_E0 * P + id] = fmaf(ke.hi, hiT, 2.0f * art);
+        NF[M_RP * P + id] = 0.5f * flux32::rcp(prho);
     }
 }
 
-// ---------------------------------------------------------------- pair flux
-__device__ __forceinline__ void pair_flux3_f(const float* S, int NB, int l, int r, float nx, float ny, float nz,
-                                             float xt, const GasF& G, float* out) {
-    const float rl = S[M_RHO * NB + l], rr = S[M_RHO * NB + r];
-    const float Tl = S[M_T * NB + l], Tr = S[M_T * NB + r];
-    const float rho_m = 0.5f * (rl + rr);
-    const float T_m = 0.5f * (Tl + Tr);
-    const float iT_m = 0.5f * (S[M_IT * NB + l] + S[M_IT * NB + r]);
-    const float drho = (rl - rr) + (S[M_RHOL * NB + l] - S[M_RHOL * NB + r]);
-    const float ilr = inv_log_mean_j(rl, rr, drho);
-    const float ilT = inv_log_mean_j(Tl, Tr, (Tl - Tr) + (S[M_TL * NB + l] - S[M_TL * NB + r]));
-    const float Pinv = S[M_IOM * NB + l] * S[M_IOM * NB + r];
-    const float iTa = 1.0f / T_m;
-    const float coef = G.Rb * Pinv - G.a * iTa;
-    float D = G.R * ilr + coef - G.a * iTa;
-    if (G.b > 0.0f) D += G.Rb * inv_log_mean_j(S[M_OM * NB + l], S[M_OM * NB + r], -G.b * drho);
-    const float iD = 1.0f / D;
-    const float g_m = 0.5f * (S[M_G * NB + l] + S[M_G * NB + r]);
-    const float rT_m = 0.5f * (S[M_RT * NB + l] + S[M_RT * NB + r]);
-    const float v2T_m = 0.5f * (S[M_V2T * NB + l] + S[M_V2T * NB + r]);
-    float vm[3], vT[3], rv[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        vm[c] = 0.5f * (S[(M_V1 + c) * NB + l] + S[(M_V1 + c) * NB + r]);
-        vT[c] = 0.5f * (S[(M_VT1 + c) * NB + l] + S[(M_VT1 + c) * NB + r]);
-        rv[c] = 0.5f * (S[(M_RV1 + c) * NB + l] + S[(M_RV1 + c) * NB + r]);
-    }
-    const float U1 = (rho_m * coef + g_m) * iD;
-    const float F11 = (rv[0] * coef + g_m * vm[0]) * iD;
-    const float F21 = (rv[1] * coef + g_m * vm[1]) * iD;
-    const float F31 = (rv[2] * coef + g_m * vm[2]) * iD;
-    const float P = rho_m * T_m * g_m;
-    const float B0 = 0.5f * v2T_m - G.cv * T_m * ilT + 2.0f * G.a * rT_m;
-    const float Q1 = xt * U1 + nx * F11 + ny * F21 + nz * F31;
-    const float sv = vT[0] * vm[0] + vT[1] * vm[1] + vT[2] * vm[2];
-    out[0] = Q1;
-    out[1] = vm[0] * Q1 + nx * P;
-    out[2] = vm[1] * Q1 + ny * P;
-    out[3] = vm[2] * Q1 + nz * P;
-    out[4] = (G.a * rT_m * (xt * rho_m + nx * rv[0] + ny * rv[1] + nz * rv[2]) + (sv - B0) * Q1 +
-              P * (nx * vT[0] + ny * vT[1] + nz * vT[2])) /
-             iT_m;
-}
-
-// entropy-variable jump V_j - V_i by eq. jumpV in general units (the 2D form of the mixed
-// kernels with three velocity components)
-__device__ __forceinline__ void entropy_jump3_f(const float* S, int NB, int i, int j, const GasF& G, float* dV) {
-    const float ri = S[M_RHO * NB + i], rj = S[M_RHO * NB + j];
-    const float Ti = S[M_T * NB + i], Tj = S[M_T * NB + j];
-    const float dr = (rj - ri) + (S[M_RHOL * NB + j] - S[M_RHOL * NB + i]);
-    const float dT = (Tj - Ti) + (S[M_TL * NB + j] - S[M_TL * NB + i]);
-    const float iTa = 2.0f / (Ti + Tj);
-    float crho = G.R * inv_log_mean_j(ri, rj, -dr) + G.Rb * S[M_IOM * NB + i] * S[M_IOM * NB + j] - 2.0f * G.a * iTa;
-    if (G.b > 0.0f) crho += G.Rb * inv_log_mean_j(S[M_OM * NB + i], S[M_OM * NB + j], G.b * dr);
-    const float rT = 0.5f * (S[M_RT * NB + i] + S[M_RT * NB + j]);
-    const float v2T = 0.5f * (S[M_V2T * NB + i] + S[M_V2T * NB + j]);
-    const float cT = -G.cv * inv_log_mean_j(Ti, Tj, -dT) + (2.0f * G.a * rT + 0.5f * v2T) * iTa;
-    float kin = 0.0f;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float vi = S[(M_V1 + c) * NB + i], vj = S[(M_V1 + c) * NB + j];
-        const float dv = (vj - vi) + (S[(M_V1L + c) * NB + j] - S[(M_V1L + c) * NB + i]);
-        kin += 0.5f * (vi + vj) * dv;
-        dV[1 + c] = (dv - 0.5f * (S[(M_VT1 + c) * NB + i] + S[(M_VT1 + c) * NB + j]) * dT) * iTa;
-    }
-    dV[0] = dr * crho + dT * cT - kin * iTa;
-    dV[4] = dT * S[M_IT * NB + i] * S[M_IT * NB + j];
-}
-
-// -1/2 Lambda T^{-1} R Y [[W]]^WENO at the face between l and l+1 with the 3D frame (as in the FP64
-// 3D kernel), W measured from node l through the shared neighbour jumps JB (line offset jq)
-__device__ __forceinline__ void face_dissipation3_f(const float* S, int NB, int l, float nx, float ny, float nz,
-                                                    float xtf, const GasF& G, const WenoF& Wc, float* out,
-                                                    DevStatus* st, const float* JB, int NJ, int jq) {
-    const int r = l + 1;
-    const float ilr = inv_log_mean_f(S[M_RHO * NB + l], S[M_RHO * NB + r]);
-    const float rho = 1.0f / ilr;
-    const float ilrp = inv_log_mean_f(S[M_RP * NB + l], S[M_RP * NB + r]);
-    const float p = rho * ilrp;
-    const float om = 1.0f - G.b * rho;
-    const float T = (p + G.a * rho * rho) * om * ilr * G.iR;
-    const float iom = 1.0f / om;
-    const float c2 = (1.0f + G.delta) * G.R * T * iom * iom - 2.0f * G.a * rho;
-    const float dcrit = G.R * T - 2.0f * G.a * rho * om * om;
-    if (!(c2 > 0.0f) || !(dcrit > 0.0f) || !(om > 0.0f)) raise_error(st, ES_ERR_INADMISSIBLE, 0);
-    const float c = sqrtf(c2);
-    const float vm1 = 0.5f * (S[M_V1 * NB + l] + S[M_V1 * NB + r]);
-    const float vm2 = 0.5f * (S[M_V2 * NB + l] + S[M_V2 * NB + r]);
-    const float vm3 = 0.5f * (S[M_V3 * NB + l] + S[M_V3 * NB + r]);
-    const float L = sqrtf(nx * nx + ny * ny + nz * nz);
-    const float r12 = sqrtf(nx * nx + ny * ny);
-    float ct = 1.0f, sn = 0.0f;
-    if (r12 > 1e-12f * L) {                  // below: the rounding of metrics that vanish exactly
-        const float ir = 1.0f / r12;
-        ct = nx * ir;
-        sn = ny * ir;
-    }
-    const float iL = 1.0f / L;
-    const float cp = r12 * iL, sp = nz * iL;
-    const float en[3] = {cp * ct, cp * sn, sp};
-    const float et1[3] = {-sn, ct, 0.0f};
-    const float et2[3] = {-sp * ct, -sp * sn, cp};
-    const float vn = en[0] * vm1 + en[1] * vm2 + en[2] * vm3;
-    const float vt1 = et1[0] * vm1 + et1[1] * vm2;
-    const float vt2 = et2[0] * vm1 + et2[1] * vm2 + et2[2] * vm3;
-    const float E = rho * (G.cv * T - G.a * rho) + 0.5f * rho * (vn * vn + vt1 * vt1 + vt2 * vt2);
-    const float H = (E + p) * ilr;
-    const float mid = H - c2 * om * G.idelta;
-    const float ic2 = 1.0f / c2;
-    const float sA = sqrtf(0.5f * rho * T * ic2);
-    const float sE = sqrtf(G.R * G.delta * rho * T * T * ic2 / dcrit);
-    const float sT = sqrtf(rho * T);
-    const float Lam = fabsf(xtf + L * vn) + L * c;
-    const float Hm = H - vn * c, Hp = H + vn * c;
-
-    // V_j - V_l at nodes l-2 .. l+3 from the neighbour jumps (zero at l)
-    float W[6][5];
-    float cum[5];
-#pragma unroll
-    for (int m = 0; m < 5; ++m) {
-        W[2][m] = 0.0f;
-        cum[m] = 0.0f;
-    }
-#pragma unroll
-    for (int o = 3; o < 6; ++o)
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            cum[m] += JB[m * NJ + jq + (o - 3)];
-            W[o][m] = cum[m];
-        }
-#pragma unroll
-    for (int m = 0; m < 5; ++m) cum[m] = 0.0f;
-#pragma unroll
-    for (int o = 1; o >= 0; --o)
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            cum[m] -= JB[m * NJ + jq + (o - 2)];
-            W[o][m] = cum[m];
-        }
-    float aTV[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int o = 0; o < 6; ++o) {
-        if (o == 2) continue;
-        const float V0 = W[o][0], V4 = W[o][4];
-        const float a1 = W[o][1], a2 = W[o][2], a3 = W[o][3];
-        const float V1 = en[0] * a1 + en[1] * a2 + en[2] * a3;
-        const float V2 = et1[0] * a1 + et1[1] * a2;
-        const float V3 = et2[0] * a1 + et2[1] * a2 + et2[2] * a3;
-        const float base = V0 + vt1 * V2 + vt2 * V3;
-        W[o][0] = sA * (base + (vn - c) * V1 + Hm * V4);
-        W[o][1] = sE * (base + vn * V1 + mid * V4);
-        W[o][2] = sT * (V2 + vt1 * V4);
-        W[o][3] = sT * (V3 + vt2 * V4);
-        W[o][4] = sA * (base + (vn + c) * V1 + Hp * V4);
-        if (o == 3) {
-            aTV[0] = fabsf(V0);
-            aTV[1] = fabsf(V1);
-            aTV[2] = fabsf(V2);
-            aTV[3] = fabsf(V3);
-            aTV[4] = fabsf(V4);
-        }
-    }
-    const float avt1 = fabsf(vt1), avt2 = fabsf(vt2);
-    const float common = aTV[0] + avt1 * aTV[2] + avt2 * aTV[3];
-    float scl[5];
-    scl[0] = sA * (common + fabsf(vn - c) * aTV[1] + fabsf(Hm) * aTV[4]);
-    scl[1] = sE * (common + fabsf(vn) * aTV[1] + fabsf(mid) * aTV[4]);
-    scl[2] = sT * (aTV[2] + (avt1 + c) * aTV[4]);
-    scl[3] = sT * (aTV[3] + (avt2 + c) * aTV[4]);
-    scl[4] = sA * (common + fabsf(vn + c) * aTV[1] + fabsf(Hp) * aTV[4]);
-    float y[5];
-#pragma unroll
-    for (int m = 0; m < 5; ++m) {
-        // a wave whose plain jump is within round-off of zero adds nothing whatever its reconstruction (the shear waves of
-        // a uniform flow, every wave of a constant state)
-        const float j = W[3][m];
-        y[m] = 0.0f;
-        if (!(fabsf(j) <= Wc.sign_tol * scl[m])) {
-            const float wmin = mr_weno5_f(W[0][m], W[1][m], W[2][m], W[3][m], W[4][m], Wc);
-            const float wplu = mr_weno5_f(W[5][m], W[4][m], W[3][m], W[2][m], W[1][m], Wc);
-            const float jw = wplu - wmin;
-            const bool keep = (jw > 0.0f && j > 0.0f) || (jw < 0.0f && j < 0.0f);
-            y[m] = keep ? jw : 0.0f;
-        }
-    }
-    const float h = -0.5f * Lam;
-    const float y0 = sA * y[0], y1 = sE * y[1], y2 = sT * y[2], y3 = sT * y[3], y4 = sA * y[4];
-    const float i0 = y0 + y1 + y4;
-    const float i1 = (vn - c) * y0 + vn * y1 + (vn + c) * y4;
-    const float i2 = vt1 * i0 + y2;
-    const float i3 = vt2 * i0 + y3;
-    const float i4 = Hm * y0 + mid * y1 + vt1 * y2 + vt2 * y3 + Hp * y4;
-    out[0] = h * i0;
-#pragma unroll
-    for (int c3 = 0; c3 < 3; ++c3) out[1 + c3] = h * (en[c3] * i1 + et1[c3] * i2 + et2[c3] * i3);
-    out[4] = h * i4;
-}
-
+// ---------------------------------------------------------------- direction kernels
+// Bound by instruction issue at the occupancy that 96 registers leave (96^3, 32 x 4 pencils: 50 M warp instructions,
+// half of the issue slots busy, the rest waits at the barriers between the phases and on shared memory; DRAM at 20%).
+// With means of unhalved scalar fields, whole values W_j - W_l and exact divisions the three directions took 130, 141 and
+// 159 us at 96^3; on es_flux32.cuh's forms 72, 89 and 87 us.
 struct Dir3FParams {
     Grid3 g;
     GasF gas;
-    WenoF weno;
+    flux32::WenoC weno;
     int diss;
     const float* NF;          // float node fields [MF_COUNT][N]
     const float* NK;          // metrics of this direction [3][M] (float, from k3f_metric)
@@ -315,6 +119,8 @@ struct Dir3FParams {
     DevStatus* status;
 };
 
+// Shared memory of a pencil of W lines: node values that are read together lie in one float4, so that a pair or face takes
+// a node in a few 16-byte loads; the lines' pitch is odd, which spreads them over the banks.
 template <int LB, int W>
 struct PencilF {
     static constexpr int LS = (LB + 6) | 1;
@@ -323,11 +129,70 @@ struct PencilF {
     static constexpr int NP = W * PL;
     static constexpr int NF = W * (LB + 1);
     static constexpr int NJ = W * (LB + 5);
-    static constexpr size_t SMEM = sizeof(float) * (size_t(MS_COUNT) * NB + 5 * NP + 6 * NF + 5 * NJ);
+    // float4: five groups of the node fields and (n, J xi_t), pairs, jumps, faces; float2: the last two node fields;
+    // floats: the fifth components and the faces' J xi_t
+    static constexpr size_t SMEM = sizeof(float) * (size_t(26) * NB + 5 * NP + 5 * NJ + 6 * NF);
     // TMA staging of the node fields of a xi_2 / xi_3 pencil: [MF_COUNT][LB + 6][W] floats, in 128-byte units
     static constexpr int STG = (W * (LB + 6) * MF_COUNT + 31) / 32 * 32;
     static constexpr size_t STG_BYTES = sizeof(float) * size_t(W) * (LB + 6) * MF_COUNT;
 };
+
+struct PencilViews {
+    float4 *a, *b, *c, *d, *l, *n, *pairs, *jumps, *faces;
+    float2* vl;
+    float *pairsE, *jumpsE, *facesE, *facesJ;
+};
+template <class PC>
+__device__ __forceinline__ PencilViews views(float* sm) {
+    PencilViews v;
+    v.a = reinterpret_cast<float4*>(sm);
+    v.b = v.a + PC::NB;
+    v.c = v.b + PC::NB;
+    v.d = v.c + PC::NB;
+    v.l = v.d + PC::NB;
+    v.n = v.l + PC::NB;
+    v.pairs = v.n + PC::NB;
+    v.jumps = v.pairs + PC::NP;
+    v.faces = v.jumps + PC::NJ;
+    v.vl = reinterpret_cast<float2*>(v.faces + PC::NF);
+    v.pairsE = reinterpret_cast<float*>(v.vl + PC::NB);
+    v.jumpsE = v.pairsE + PC::NP;
+    v.facesE = v.jumpsE + PC::NJ;
+    v.facesJ = v.facesE + PC::NF;
+    return v;
+}
+__device__ __forceinline__ flux32::Node<3> node_at(const PencilViews& v, int q) {
+    const float4 a = v.a[q], b = v.b[q], c = v.c[q], d = v.d[q];
+    flux32::Node<3> n;
+    n.rho = a.x;
+    n.T = a.y;
+    n.iom = a.z;
+    n.E0 = a.w;
+    n.v[0] = b.x;
+    n.v[1] = b.y;
+    n.v[2] = b.z;
+    n.g = b.w;
+    n.vT[0] = c.x;
+    n.vT[1] = c.y;
+    n.vT[2] = c.z;
+    n.art = c.w;
+    n.rv[0] = d.x;
+    n.rv[1] = d.y;
+    n.rv[2] = d.z;
+    return n;
+}
+__device__ __forceinline__ flux32::NodeLow<3> low_at(const PencilViews& v, int q) {
+    const float4 l = v.l[q];
+    const float2 w = v.vl[q];
+    flux32::NodeLow<3> n;
+    n.rho = l.x;
+    n.T = l.y;
+    n.iT = l.z;
+    n.v[0] = l.w;
+    n.v[1] = w.x;
+    n.v[2] = w.y;
+    return n;
+}
 
 // ---------------------------------------------------------------- TMA staging
 // The xi_2 and xi_3 kernels run persistent: a CTA takes pencils p, p + gridDim.x, ... and, while it
@@ -378,15 +243,12 @@ template <int K, int LB, int W, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k3_dir_f(const __grid_constant__ Dir3FParams P,
                                                      const __grid_constant__ CUtensorMap tmap) {
     using PC = PencilF<LB, W>;
-    constexpr int LS = PC::LS, NB = PC::NB, NP = PC::NP, NFc = PC::NF, NJ = PC::NJ;
+    constexpr int LS = PC::LS, NFc = PC::NF;
     extern __shared__ __align__(128) float smf[];
     __shared__ __align__(8) unsigned long long bar;
     const bool tma = K != 0 && P.tma;
     float* STG = smf;
-    float* S = smf + (tma ? PC::STG : 0);
-    float* PB = S + MS_COUNT * NB;
-    float* FB = PB + 5 * NP;
-    float* JB = FB + 6 * NFc;
+    const PencilViews pv = views<PC>(smf + (tma ? PC::STG : 0));
     const Grid3& g = P.g;
     const int tid = threadIdx.x;
     const int nk = g.n[K];
@@ -458,18 +320,19 @@ __global__ void __launch_bounds__(NT, MINB) k3_dir_f(const __grid_constant__ Dir
 #pragma unroll
                 for (int f = 0; f < MF_COUNT; ++f) v[f] = P.NF[f * N + id];
             }
-#pragma unroll
-            for (int f = 0; f < MF_COUNT; ++f) S[f * NB + bx] = v[f];
+            pv.a[bx] = make_float4(v[0], v[1], v[2], v[3]);
+            pv.b[bx] = make_float4(v[4], v[5], v[6], v[7]);
+            pv.c[bx] = make_float4(v[8], v[9], v[10], v[11]);
+            pv.d[bx] = make_float4(v[12], v[13], v[14], v[15]);
+            pv.l[bx] = make_float4(v[16], v[17], v[18], v[19]);
+            pv.vl[bx] = make_float2(v[20], v[21]);
             int se = s + 3;
             se = se < 0 ? 0 : (se > nk + 5 ? nk + 5 : se);
             if (K == 0) { j1 = se; j2 = a; j3 = b; }
             else if (K == 1) { j1 = a; j2 = se; j3 = b; }
             else { j1 = a; j2 = b; j3 = se; }
             const size_t mi = (size_t(j3) * M2 + j2) * M1 + j1;
-            const float nx = P.NK[mi], ny = P.NK[M + mi], nz = P.NK[2 * M + mi];
-            S[M_NX * NB + bx] = nx;
-            S[M_NY * NB + bx] = ny;
-            S[M_NZ * NB + bx] = nz;
+            const float nx = 0.5f * P.NK[mi], ny = 0.5f * P.NK[M + mi], nz = 0.5f * P.NK[2 * M + mi];
             float xt = 0.0f;
             if (P.XD) {     // J xi_{k,t} = -xdot . n_k, xdot from the extended mesh (its ghosts: the coordinates' rule)
                 const size_t NE = size_t(M1e) * M2e * M3e;
@@ -479,7 +342,7 @@ __global__ void __launch_bounds__(NT, MINB) k3_dir_f(const __grid_constant__ Dir
                 else e = (size_t(se) * M2e + (b + 3)) * M1e + (a + 3);
                 xt = -(P.XD[e] * nx + P.XD[NE + e] * ny + P.XD[2 * NE + e] * nz);
             }
-            S[M_XT * NB + bx] = xt;
+            pv.n[bx] = make_float4(nx, ny, nz, xt);
         }
         __syncthreads();
         if (tma && tid == 0 && pen + int(gridDim.x) < total) {    // the staging buffer is free: next pencil
@@ -487,73 +350,94 @@ __global__ void __launch_bounds__(NT, MINB) k3_dir_f(const __grid_constant__ Dir
             stage_pencil<K, LB>(STG, &tmap, &bar, stg_bytes, (gp % ngA) * W, gp / ngA, (p % nseg) * LB);
         }
 
-        // ---- C: pair fluxes, and B: neighbour jumps V_{q+1} - V_q, q = 0 .. LB+4 (eq. jumpV)
-        for (int t = tid; t < NP; t += NT) {
-            const int line = t / PC::PL, kk = t % PC::PL;
-            int m, q;
-            if (kk < LB + 1) { m = 1; q = 2 + kk; }
-            else if (kk < 2 * LB + 3) { m = 2; q = 1 + (kk - LB - 1); }
-            else { m = 3; q = kk - 2 * LB - 3; }
+        // ---- B: pair fluxes by their reach m; those with m = 1 also give the neighbour jumps V_{q+1} - V_q,
+        // q = 0 .. LB + 4 (eq. jumpV)
+        constexpr int c1 = W * (LB + 5), c2 = c1 + W * (LB + 2), c3 = c2 + W * (LB + 3);
+        for (int t = tid; t < c3; t += NT) {
+            const int m = t < c1 ? 1 : (t < c2 ? 2 : 3);
+            const int u = m == 1 ? t : (m == 2 ? t - c1 : t - c2);
+            const int line = m == 1 ? u / (LB + 5) : (m == 2 ? u / (LB + 2) : u / (LB + 3));
+            const int pos = u - line * (LB + (m == 1 ? 5 : m));
+            const int q = m == 2 ? pos + 1 : pos;
             const int l = line * LS + q, r = l + m;
-            const float nx = 0.5f * (S[M_NX * NB + l] + S[M_NX * NB + r]);
-            const float ny = 0.5f * (S[M_NY * NB + l] + S[M_NY * NB + r]);
-            const float nz = 0.5f * (S[M_NZ * NB + l] + S[M_NZ * NB + r]);
-            const float xt = 0.5f * (S[M_XT * NB + l] + S[M_XT * NB + r]);
+            const flux32::Node<3> nl = node_at(pv, l), nr = node_at(pv, r);
+            const flux32::PairMeans<3> p = flux32::pair_means<3>(nl, nr, G);
             float f[5];
-            pair_flux3_f(S, NB, l, r, nx, ny, nz, xt, G, f);
-#pragma unroll
-            for (int c = 0; c < 5; ++c) PB[c * NP + t] = f[c];
-        }
-        if (P.diss) {
-            for (int t = tid; t < NJ; t += NT) {
-                const int line = t / (LB + 5), q = t % (LB + 5);
-                const int l = line * LS + q;
-                float dV[5];
-                entropy_jump3_f(S, NB, l, l + 1, G, dV);
-#pragma unroll
-                for (int c = 0; c < 5; ++c) JB[c * NJ + t] = dV[c];
+            if (m == 1) {
+                flux32::entropy_jump<3>(nl, nr, low_at(pv, l), low_at(pv, r), p, f);
+                pv.jumps[u] = make_float4(f[0], f[1], f[2], f[3]);
+                pv.jumpsE[u] = f[4];
+                if (q < 2 || q > LB + 2) continue;
             }
+            const float4 na = pv.n[l], nb = pv.n[r];
+            const float n[3] = {na.x + nb.x, na.y + nb.y, na.z + nb.z};
+            flux32::pair_flux<3>(nl, nr, p, n, na.w + nb.w, f);
+            const int o = line * PC::PL + (m == 1 ? q - 2 : (m == 2 ? LB + 1 : 2 * LB + 3) + pos);
+            pv.pairs[o] = make_float4(f[0], f[1], f[2], f[3]);
+            pv.pairsE[o] = f[4];
         }
         __syncthreads();
 
-        // ---- D: face fluxes
+        // ---- C: face fluxes
         for (int t = tid; t < NFc; t += NT) {
-            const int line = t / (LB + 1), f = t % (LB + 1);
-            const int q = 2 + f;
-            const int pbase = line * PC::PL;
-            const int base = line * LS;
-            float F[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-            float FJ = 0.0f;
-#pragma unroll
-            for (int m = 1; m <= 3; ++m) {
-                const int off = m == 1 ? 0 : (m == 2 ? LB + 1 : 2 * LB + 3);
-                const float al = float(ec_alpha(m));
-                for (int s = 0; s < m; ++s) {
-                    const int qq = q - s;
-                    const int pi = pbase + off + (qq - (3 - m));
-#pragma unroll
-                    for (int c = 0; c < 5; ++c) F[c] += al * PB[c * NP + pi];
-                    FJ += al * 0.5f * (S[M_XT * NB + base + qq] + S[M_XT * NB + base + qq + m]);
-                }
+            const int line = t / (LB + 1);
+            const int q = 2 + t - line * (LB + 1);
+            const int l = line * LS + q, r = l + 1;
+            // the 6th-order combination of the pairs (the energy component is a quarter); pairs of reach m start at
+            // q = 3 - m
+            constexpr float a1 = 1.5f, a2 = -0.3f, a3 = 1.0f / 30.0f;
+            constexpr int o2 = LB, o3 = 2 * LB + 3;
+            float F[5];
+            {
+                const float4* pb = pv.pairs + line * PC::PL + q;
+                const float* pe = pv.pairsE + line * PC::PL + q;
+                const float4 p1 = pb[-2], p2a = pb[o2 - 1], p2b = pb[o2], p3a = pb[o3 - 2], p3b = pb[o3 - 1], p3c = pb[o3];
+                F[0] = fmaf(a1, p1.x, fmaf(a2, p2a.x + p2b.x, a3 * (p3a.x + p3b.x + p3c.x)));
+                F[1] = fmaf(a1, p1.y, fmaf(a2, p2a.y + p2b.y, a3 * (p3a.y + p3b.y + p3c.y)));
+                F[2] = fmaf(a1, p1.z, fmaf(a2, p2a.z + p2b.z, a3 * (p3a.z + p3b.z + p3c.z)));
+                F[3] = fmaf(a1, p1.w, fmaf(a2, p2a.w + p2b.w, a3 * (p3a.w + p3b.w + p3c.w)));
+                F[4] = 4.0f * fmaf(a1, pe[-2], fmaf(a2, pe[o2 - 1] + pe[o2], a3 * (pe[o3 - 2] + pe[o3 - 1] + pe[o3])));
             }
+            const float4 na = pv.n[l], nb = pv.n[r];
+            // sum_m alpha_m sum of the pairs' mean J xi_t, collected by node
+            constexpr float b3 = a3, b2 = a2 + b3, b1 = a1 + b2;
+            pv.facesJ[t] = fmaf(b1, na.w + nb.w, fmaf(b2, pv.n[l - 1].w + pv.n[r + 1].w, b3 * (pv.n[l - 2].w + pv.n[r + 2].w)));
             if (P.diss) {
-                const int l = base + q;
-                const float nx = 0.5f * (S[M_NX * NB + l] + S[M_NX * NB + l + 1]);
-                const float ny = 0.5f * (S[M_NY * NB + l] + S[M_NY * NB + l + 1]);
-                const float nz = 0.5f * (S[M_NZ * NB + l] + S[M_NZ * NB + l + 1]);
-                const float xtf = 0.5f * (S[M_XT * NB + l] + S[M_XT * NB + l + 1]);
-                float d[5];
-                face_dissipation3_f(S, NB, l, nx, ny, nz, xtf, G, P.weno, d, P.status, JB, NJ, line * (LB + 5) + q);
+                const float n[3] = {na.x + nb.x, na.y + nb.y, na.z + nb.z};
+                const float4 vl = pv.b[l], vr = pv.b[r];
+                const float v[3] = {vl.x + vr.x, vl.y + vr.y, vl.z + vr.z};
+                const flux32::Face<3> f =
+                    flux32::face_state<3>(pv.a[l].x, pv.a[r].x, pv.d[l].w, pv.d[r].w, v, n, na.w + nb.w, G, P.status);
+                float w[5][5], sz[5], y[5];
+                const float4* jb = pv.jumps + line * (LB + 5) + q - 2;
+                const float* je = pv.jumpsE + line * (LB + 5) + q - 2;
 #pragma unroll
-                for (int c = 0; c < 5; ++c) F[c] += d[c];
+                for (int o = 0; o < 5; ++o) {
+                    const float4 j = jb[o];
+                    const float d[5] = {j.x, j.y, j.z, j.w, je[o]};
+                    const flux32::Rotated<3> R = flux32::rotate<3>(f, d);
+                    const float sa = f.sA * R.A;
+                    w[0][o] = fmaf(-f.sAc, R.B, sa);
+                    w[1][o] = f.sE * fmaf(-f.hm, d[4], R.A);
+                    w[2][o] = f.sT * fmaf(f.vr[1], d[4], R.rv[1]);
+                    w[3][o] = f.sT * fmaf(f.vr[2], d[4], R.rv[2]);
+                    w[4][o] = fmaf(f.sAc, R.B, sa);
+                    if (o == 2) flux32::term_sizes<3>(f, d, R, sz);
+                }
+                // a wave whose plain jump is round-off adds nothing whatever its reconstruction
+#pragma unroll
+                for (int m = 0; m < 5; ++m) {
+                    const float S = m == 1 ? f.sE : (m == 2 || m == 3 ? f.sT : f.sA);
+                    y[m] = fabsf(w[m][2]) <= P.weno.tol * (S * sz[m]) ? 0.0f : flux32::weno_jump(w[m], P.weno);
+                }
+                flux32::add_increment<3>(f, y, F);
             }
-#pragma unroll
-            for (int c = 0; c < 5; ++c) FB[c * NFc + t] = F[c];
-            FB[5 * NFc + t] = FJ;
+            pv.faces[t] = make_float4(F[0], F[1], F[2], F[3]);
+            pv.facesE[t] = F[4];
         }
         __syncthreads();
 
-        // ---- E: divergence, accumulated in float; the last direction writes double-float results
+        // ---- D: divergence, accumulated in float; the last direction writes double-float results
         const float inv = g.finv[K];
         for (int t = tid; t < W * LB; t += NT) {
             int line, pos;
@@ -588,12 +472,13 @@ __global__ void __launch_bounds__(NT, MINB) k3_dir_f(const __grid_constant__ Dir
                     ul[c] = P.ca != 0.0f ? un[lo + id] : 0.0f;
                 }
             }
-            float acc[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                acc[c] = -(FB[c * NFc + fm + 1] - FB[c * NFc + fm]) * inv;
-                if (!P.first) acc[c] += rh[c];
-            }
+            const float4 fl = pv.faces[fm], fr = pv.faces[fm + 1];
+            const float acc[6] = {fmaf(fl.x - fr.x, inv, rh[0]),
+                                  fmaf(fl.y - fr.y, inv, rh[1]),
+                                  fmaf(fl.z - fr.z, inv, rh[2]),
+                                  fmaf(fl.w - fr.w, inv, rh[3]),
+                                  fmaf(pv.facesE[fm] - pv.facesE[fm + 1], inv, rh[4]),
+                                  fmaf(pv.facesJ[fm] - pv.facesJ[fm + 1], inv, rh[5])};
             if (!P.last) {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) P.RH[c * N + id] = acc[c];
@@ -621,7 +506,7 @@ __global__ void __launch_bounds__(NT, MINB) k3_dir_f(const __grid_constant__ Dir
                 }
             }
         }
-        __syncthreads();                                      // S, PB, FB and JB are refilled next
+        __syncthreads();                                      // the nodes, pairs, jumps and faces are refilled next
     }
 }
 
@@ -648,13 +533,13 @@ static cudaError_t launch_shape(const Dir3FParams& P, const CUtensorMap& map, cu
 }
 
 // pencil shapes of the float kernels: 16 x 16 lines / 288 threads (two CTAs per SM), 32 x 8 / 288,
-// 16 x 8 / 160 (three per SM), 32 x 4 / 160
+// 16 x 8 / 160 (four per SM: 96 registers and, with the TMA staging, 50 KB each), 32 x 4 / 160
 template <int K>
 static cudaError_t prep_dir() {
     cudaError_t e = prep_shape<K, 16, 16, 288, 2>();
     if (e == cudaSuccess) e = prep_shape<K, 32, 8, 288, 2>();
-    if (e == cudaSuccess) e = prep_shape<K, 16, 8, 160, 3>();
-    if (e == cudaSuccess) e = prep_shape<K, 32, 4, 160, 3>();
+    if (e == cudaSuccess) e = prep_shape<K, 16, 8, 160, 4>();
+    if (e == cudaSuccess) e = prep_shape<K, 32, 4, 160, 4>();
     return e;
 }
 
@@ -662,8 +547,8 @@ template <int K>
 static cudaError_t launch_dir(const Dir3FParams& P, const CUtensorMap& map, int shape, cudaStream_t s) {
     switch (shape) {
         case 1: return launch_shape<K, 32, 8, 288, 2>(P, map, s);
-        case 2: return launch_shape<K, 16, 8, 160, 3>(P, map, s);
-        case 3: return launch_shape<K, 32, 4, 160, 3>(P, map, s);
+        case 2: return launch_shape<K, 16, 8, 160, 4>(P, map, s);
+        case 3: return launch_shape<K, 32, 4, 160, 4>(P, map, s);
         default: return launch_shape<K, 16, 16, 288, 2>(P, map, s);
     }
 }
@@ -876,8 +761,8 @@ __global__ void k3_cfl_f(Grid3 g, Gas Gd, const float* NF, const float* J, const
     float mx = 0.0f;
     for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
         const int i1 = int(id % g.n[0]), i2 = int((id / g.n[0]) % g.n[1]), i3 = int(id / (size_t(g.n[0]) * g.n[1]));
-        const float rho = NF[M_RHO * N + id], T = NF[M_T * N + id], iom = NF[M_IOM * N + id];
-        const float v[3] = {NF[M_V1 * N + id], NF[M_V2 * N + id], NF[M_V3 * N + id]};
+        const float rho = 2.0f * NF[M_RHO * N + id], T = 2.0f * NF[M_T * N + id], iom = NF[M_IOM * N + id];
+        const float v[3] = {2.0f * NF[M_V1 * N + id], 2.0f * NF[M_V2 * N + id], 2.0f * NF[M_V3 * N + id]};
         const float c2 = (1.0f + delta) * R * T * (iom * iom) - 2.0f * a * rho;
         const float c = sqrtf(fmaxf(c2, 0.0f));
         const float iJ = 1.0f / J[id];
@@ -1228,19 +1113,6 @@ static GasF gasf(const Gas& g) {
     return G;
 }
 
-static WenoF wenof(const Weno& w) {
-    WenoF W;
-    W.g1 = float(w.g1);
-    W.g2 = float(w.g2);
-    W.g3 = float(w.g3);
-    W.g12 = float(w.g12);
-    W.ig22 = float(w.ig22);
-    W.ig3 = float(w.ig3);
-    W.eps = float(w.eps);
-    W.sign_tol = float(w.sign_tol);
-    return W;
-}
-
 int d3f_metrics(Ctx3* d, const double* xn, const double* xdot, double cst, const double* dt_dev, double dt_host,
                 cudaStream_t s, const Stage3* inc) {
     const int G = d->grid;
@@ -1286,7 +1158,7 @@ int d3f_directions(Ctx3* d, const Stage3& a, DevStatus* st, cudaStream_t s, cuda
     Dir3FParams P;
     P.g = d->g;
     P.gas = gasf(d->gas);
-    P.weno = wenof(d->weno);
+    P.weno = flux32::weno_floats(d->weno);
     P.diss = d->diss;
     P.NF = (const float*)d->NF;
     P.XD = a.xdot ? d->XD : nullptr;          // d3_stage formed it from a.xdot
