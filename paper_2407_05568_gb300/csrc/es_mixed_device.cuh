@@ -669,7 +669,22 @@ __device__ __forceinline__ void stage_tile_mixed(float* smemf, const StageParams
                     FJ += al * 0.5f * (S[fXT * NB + base + qq * step] + S[fXT * NB + base + (qq + m) * step]);
                 }
             }
-            if (P.diss) {
+            bool jump = P.diss;
+            if (DIM == 1 && P.diss) {
+                // between two nodes of equal state no wave has a jump and the dissipation is zero whatever the rest of
+                // the stencil (eq. sign switch): most faces of a tube whose waves have not reached its ends.  The face
+                // state's own check is then the node's.
+                const float* jl = JB + q;
+                jump = jl[0] != 0.0f || jl[TL::NJ] != 0.0f || jl[2 * TL::NJ] != 0.0f;
+                if (!jump) {
+                    const int l = base + q;
+                    const float RT = G.R * S[G_T * NB + l], ar = 2.0f * G.a * S[G_RHO * NB + l];
+                    const float om = S[G_OM * NB + l], iom = S[G_IOM * NB + l];
+                    if (!((1.0f + G.delta) * RT * iom * iom > ar) || !(RT > ar * om * om))
+                        raise_error(P.status, ES_ERR_INADMISSIBLE, 0);
+                }
+            }
+            if (jump) {
                 const int l = base + q * step;
                 const float nx = 0.5f * (S[fN * NB + l] + S[fN * NB + l + step]);
                 const float ny = 0.5f * (S[fNy * NB + l] + S[fNy * NB + l + step]);

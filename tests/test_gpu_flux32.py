@@ -1,10 +1,10 @@
-"""The mixed form's 3D direction kernels (FP32 fluxes on double-float node values) in every pencil shape."""
+"""The mixed form's FP32 fluxes: the 3D direction kernels in every pencil shape, and the 1D tile's faces of equal states."""
 import numpy as np
 import pytest
 
 from oracle import operator as op
 
-from sides import oracle_setup
+from sides import gpu_setup, oracle_setup, to_np
 from test_gpu_3d import _box, _mixed_rhs, _xdot
 
 pytestmark = pytest.mark.gpu
@@ -22,3 +22,28 @@ def test_pencil_shapes_against_oracle(tile, n, periodic):
     h = min(w["dxi"])
     assert np.abs(dU[0].astype(float) - dU_o).sum() < 1e-5 * np.abs(JU_o).sum() / h
     assert np.abs(dJ[0].astype(float) - dJ_o).sum() < 1e-5 * np.abs(J_o).sum() / h
+
+
+@pytest.mark.parametrize("t_over_tc,ok", [(1.2, True), (0.9, False)])
+def test_1d_uniform_state(t_over_tc, ok):
+    """A uniform state at the critical density: every face lies between equal nodes, where the dissipation is zero.  Above
+    the critical temperature the right-hand sides vanish exactly; below it (p > 0, but inside the spinodal) the state is
+    refused as it is between unequal nodes."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    w = wl.sine_1d(300)
+    g = w["gas"]
+    rho = 1.0 / (3.0 * g["b"])
+    T = t_over_tc * 8.0 * g["a"] / (27.0 * g["R"] * g["b"])
+    w["rho"] = np.full_like(w["rho"], rho)
+    w["v"] = np.full_like(w["v"], 0.25)
+    w["p"] = np.full_like(w["p"], rho * g["R"] * T / (1.0 - g["b"] * rho) - g["a"] * rho * rho)
+    assert w["p"].min() > 0.0
+    ctx, JU, J, xt = gpu_setup(w, precision="mixed")
+    dU, dJ = torch.empty_like(JU), torch.empty_like(J)
+    es.es_rhs(ctx, JU, J, xt, None, dU, dJ)
+    assert (es.es_check(ctx) == 0) == ok
+    if ok:
+        assert not to_np(dU).any()
