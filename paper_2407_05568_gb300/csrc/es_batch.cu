@@ -4,7 +4,7 @@
 // longest first) and advances it by `nsteps` full steps -- its own CFL time
 // step (eq. cfl), its own mesh redistribution (Sec. 4: monitor with G, low-pass
 // filter, Jacobi sweeps, limiter, mesh velocity) and the three SSP-RK3 stages,
-// each stage a loop over 254-node chunks of the fused operator -- using only
+// each stage a loop over chunks of the fused operator -- using only
 // __syncthreads between phases.  No CTA ever waits for another, so there is no
 // grid-wide synchronisation and no spin-wait.  The state of all problems is
 // packed component-major: value c of node i of problem p at c * ntot + off_p + i.
@@ -28,12 +28,17 @@ using namespace mixed;
 
 namespace {
 
-// CTA shapes the autotuner chooses from: BT threads, chunks of BT - 2 nodes per stage tile
+// CTA shapes the autotuner chooses from: BT threads, chunks of BT - 6 nodes per stage tile, so that the chunk with its halo
+// is one node per thread and each of its phases one round (with BT - 2, four threads loaded a second node and three formed
+// a second jump while the others waited), 32 warps per SM (64 registers, no spills; at 24 the warps waited for the global
+// loads of the short phases, 57% of the issue slots busy, at 32 71%).  4096 tubes of 200 to 8000 nodes, 10 steps: 42.5 ms
+// with 24 warps, chunks of BT - 2 and the mesh buffers in global memory, 33.4 ms now; bound by instruction issue.
 template <int BT>
 struct BatchShape {
-    static constexpr int BXC = BT - 2;
+    static constexpr int BXC = BT - 6;
     using TB = TileF<1, BXC, 1, BT>;
-    static constexpr int MIN_BLOCKS = BT >= 512 ? 1 : 768 / BT;     // 24 warps per SM (80 registers) below 512
+    static constexpr int MIN_BLOCKS = 1024 / BT;
+    static constexpr int SMEM_FLOATS = int(TB::SMEM / sizeof(float));
 };
 
 __device__ __forceinline__ float block_max_f(float v, float* red) {
@@ -92,8 +97,6 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
         float* t2 = B.work + 4 * ntot + off;
         float* om0 = B.work + 5 * ntot + off;
         float* om1 = B.work + 6 * ntot + off;
-        float* da = B.work + 7 * ntot + off;
-        float* db = B.work + 8 * ntot + off;
         double t = B.tprob[p];
 
         // node i's velocity, sound speed squared (rho, T for the monitor) and 1/J from the state
@@ -162,10 +165,14 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
                 const float c0 = m0 > 0.0f ? B.w0 / m0 : 0.0f;
                 const float c1 = m1 > 0.0f ? B.w1 / m1 : 0.0f;
                 const float c2 = m2 > 0.0f ? B.w2 / m2 : 0.0f;
-                for (int i = tid; i < L; i += BT) om0[i] = sqrtf(1.0f + c0 * t0[i] + c1 * t1[i] + c2 * t2[i]);
+                // the filter's and the sweeps' two buffers lie in the stage tiles' shared memory where they fit (lines of
+                // up to 5218 nodes with 256 threads; the passes are short dependent reads); the sweeps start in the buffer
+                // that the filter left free, and take omega's once the coefficients are formed
+                const bool in_smem = 2 * L <= BatchShape<BT>::SMEM_FLOATS;
+                float* om = in_smem ? smemf : om0;
+                float* ot = in_smem ? smemf + L : om1;
+                for (int i = tid; i < L; i += BT) om[i] = sqrtf(1.0f + c0 * t0[i] + c1 * t1[i] + c2 * t2[i]);
                 __syncthreads();
-                float* om = om0;
-                float* ot = om1;
                 for (int f = 0; f < B.filter_passes; ++f) {
                     for (int i = tid; i < L; i += BT)
                         ot[i] = 0.25f * om[clampi(i - 1, L)] + 0.5f * om[i] + 0.25f * om[clampi(i + 1, L)];
@@ -191,11 +198,11 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
                         ap[i] = a;
                         gc[i] = a * (dxi + d[i + 1] - d[i]) - (1.0f - a) * (dxi + d[i] - d[i - 1]);
                     }
-                    da[i] = 0.0f;
+                    ot[i] = 0.0f;
                 }
                 __syncthreads();
-                const float* din = da;
-                float* dout = db;
+                const float* din = ot;
+                float* dout = om;
                 for (int k = 0; k < B.sweeps; ++k) {
                     for (int i = tid; i < L; i += BT)
                         dout[i] = (i == 0 || i == L - 1)
@@ -203,7 +210,7 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
                                       : gc[i] + ap[i] * din[i + 1] + (1.0f - ap[i]) * din[i - 1];
                     __syncthreads();
                     din = dout;
-                    dout = (dout == da) ? db : da;
+                    dout = (dout == om) ? ot : om;
                 }
                 // limiter: each node moves at most half of its spacing towards its neighbour
                 float g = 1.0f;
@@ -471,7 +478,7 @@ int es_batch_create(es_batch** out, const es_params* p, int nprob, const int* le
         if ((e = cudaMalloc((void**)&b->d_offsets, sizeof(long long) * nprob))) break;
         // state planes: JU 6n, J 2n, S1 6n, S1J 2n, S2 6n, S2J 2n, disp n, xdot n
         if ((e = cudaMalloc((void**)&b->state, sizeof(float) * n * 26))) break;
-        if ((e = cudaMalloc((void**)&b->work, sizeof(float) * n * 9))) break;
+        if ((e = cudaMalloc((void**)&b->work, sizeof(float) * n * 7))) break;
         if ((e = cudaMalloc((void**)&b->tprob, sizeof(double) * nprob))) break;
         if ((e = cudaMalloc((void**)&b->queue, sizeof(int)))) break;
         if ((e = cudaMalloc((void**)&b->status, sizeof(DevStatus)))) break;

@@ -23,7 +23,7 @@ struct BatchParams {
     float* S2J;
     float* disp;                  // x_i - i/(L - 1), [ntot]
     float* xdot;                  // [ntot]
-    float* work;                  // 9 scratch fields of ntot floats (monitor, filter, Jacobi)
+    float* work;                  // 7 scratch fields of ntot floats (monitor, filter, Jacobi)
     double* tprob;                // time of each problem
     int* queue;                   // work counter, zeroed before each launch
     int nsteps;
