@@ -19,10 +19,12 @@
 #include <cuda_runtime.h>
 
 #include "es_3d.h"
+#include "es_3d_filter.cuh"
 #include "es_3d_grid.cuh"
 #include "es_device.cuh"
 #include "es_flux64.cuh"
 #include "es_internal.h"
+#include "es_mesh64.cuh"
 
 namespace es {
 
@@ -32,12 +34,6 @@ constexpr int F3_COUNT = SL3::COUNT;
 constexpr int G_N = F3_COUNT;              // halves of the three metric components, then of J xi_t
 constexpr int G_XT = G_N + 3;
 constexpr int S3_COUNT = G_XT + 1;
-
-// field at a possibly-ghost node, ghosts by copy / wrap (monitor and filter)
-__device__ __forceinline__ double field3(const Grid3& g, const double* f, int i1, int i2, int i3) {
-    return f[idx3(g, state_index(i1, g.n[0], g.bc[0]), state_index(i2, g.n[1], g.bc[1]),
-                  state_index(i3, g.n[2], g.bc[2]))];
-}
 
 // stride of direction k in a [n3][n2][n1] field
 __device__ __forceinline__ size_t stride3(const Grid3& g, int k) {
@@ -70,18 +66,10 @@ __device__ __forceinline__ double nb_coord(const Grid3& g, const double* f, size
     return 2.0 * f[id + (long long)(b - ik) * st] - f[id + (long long)(m - ik) * st];
 }
 
-__device__ __forceinline__ double block_max(double v) {
-    __shared__ double sh[32];
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    v = threadIdx.x < nw ? sh[threadIdx.x] : 0.0;
-    if (w == 0)
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    __syncthreads();
-    return v;
+// sqrt(x), x >= 0 (or NaN): x rsqrt_nr(x) where x is normal and not huge, six FP64 instructions
+__device__ __forceinline__ double sqrt_pos(double x) {
+    const unsigned h = unsigned(__double2hiint(x));
+    return h - 0x03000000u < 0x7a000000u ? x * rsqrt_nr(x) : sqrt(x);
 }
 
 __device__ __forceinline__ double block_min(double v) {
@@ -471,35 +459,39 @@ static cudaError_t dir_launch(const Dir3Params& P, int shape, cudaStream_t s) {
 // ================================================================ CFL (eq. cfl)
 // max_i sum_k (|J xi_{k,t} + n_k . v| + |n_k| c) / (J dxi_k), J xi_{k,t} = -xdot . n_k (eq. VCLCoeff), from the
 // node fields and metrics of x^n; xdot = nullptr is a mesh at rest.  The maximum goes to d->red[slot].
+// Bound by the FP64 pipe: 60 instructions a node (library square roots, FP64 maxima and J xi_t apart from n . v: 95).
 __global__ void k3_cfl(Grid3 g, Gas G, const double* NF, const double* J, const double* NK0, const double* NK1,
                        const double* NK2, const double* xdot, int slot, DevScalars* d) {
     const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
     const size_t M[3] = {size_t(g.n[0] + 6) * g.n[1] * g.n[2], size_t(g.n[0]) * (g.n[1] + 6) * g.n[2],
                          size_t(g.n[0]) * g.n[1] * (g.n[2] + 6)};
     const double* NK[3] = {NK0, NK1, NK2};
+    const double c2f = 2.0 * (1.0 + G.delta) * G.R, a4 = 4.0 * G.a;
     double mx = 0.0;
-    for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
-        const int i1 = int(id % g.n[0]), i2 = int((id / g.n[0]) % g.n[1]), i3 = int(id / (size_t(g.n[0]) * g.n[1]));
+    for (unsigned id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
+        const int i1 = int(id % unsigned(g.n[0])), r12 = int(id / unsigned(g.n[0]));
+        const int i2 = r12 % g.n[1], i3 = r12 / g.n[1];
         // the node fields and metrics are halves
         const double r = NF[SL3::RHO * N + id], hT = NF[SL3::T * N + id], iom = NF[SL3::IOM * N + id];
-        const double v[3] = {NF[SL3::V * N + id], NF[(SL3::V + 1) * N + id], NF[(SL3::V + 2) * N + id]};
-        const double c2 = 2.0 * (1.0 + G.delta) * G.R * hT * (iom * iom) - 4.0 * G.a * r;
-        const double c = sqrt(fmax(c2, 0.0));
-        const double iJ = rcp_nr(J[id]);
-        const double xd[3] = {xdot ? xdot[id] : 0.0, xdot ? xdot[N + id] : 0.0, xdot ? xdot[2 * N + id] : 0.0};
+        double v[3] = {NF[SL3::V * N + id], NF[(SL3::V + 1) * N + id], NF[(SL3::V + 2) * N + id]};
+        if (xdot) {                                           // half the velocity relative to the mesh
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[k] = fma(-0.5, xdot[k * N + id], v[k]);
+        }
+        const double c2 = fma(c2f * hT, iom * iom, -a4 * r);
+        const double hc = c2 > 0.0 ? 0.5 * sqrt_pos(c2) : 0.0;
         double tot = 0.0;
+#pragma unroll
         for (int k = 0; k < 3; ++k) {
             const int m1 = g.n[0] + (k == 0 ? 6 : 0), m2 = g.n[1] + (k == 1 ? 6 : 0);
             const size_t mi = (size_t(i3 + (k == 2 ? 3 : 0)) * m2 + i2 + (k == 1 ? 3 : 0)) * m1 + i1 + (k == 0 ? 3 : 0);
             const double n0 = NK[k][mi], n1 = NK[k][M[k] + mi], n2 = NK[k][2 * M[k] + mi];
-            const double xt = -(xd[0] * n0 + xd[1] * n1 + xd[2] * n2);
-            tot += (fabs(xt + 2.0 * (n0 * v[0] + n1 * v[1] + n2 * v[2])) + sqrt(n0 * n0 + n1 * n1 + n2 * n2) * c) * iJ *
-                   (2.0 * g.inv_dxi[k]);
+            const double nv = fma(n2, v[2], fma(n1, v[1], n0 * v[0])), nn = fma(n2, n2, fma(n1, n1, n0 * n0));
+            tot = fma(fma(sqrt_pos(nn), hc, fabs(nv)), g.inv_dxi[k], tot);
         }
-        if (!(c2 > 0.0)) tot = 1e300;
-        mx = fmax(mx, tot);
+        mx = max_bits(mx, c2 > 0.0 ? 4.0 * tot * rcp_nr(J[id]) : 1e300);
     }
-    mx = block_max(mx);
+    block_max_bits<1>(&mx);
     if (threadIdx.x == 0) atomic_max_pos(&d->red[slot], mx);
 }
 
@@ -529,83 +521,55 @@ __global__ void k3_init_J(Grid3 g, const double* x, double* J) {
 }
 
 // ================================================================ mesh (Sec. 4)
-__global__ void k3_mon_terms(Grid3 g, MonitorParams mp, const double* rhoF, const double* GF, double* t0,
-                             double* t1, double* t2, DevScalars* d) {
-    const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
-    double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-    for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
-        const int i1 = int(id % g.n[0]), i2 = int((id / g.n[0]) % g.n[1]), i3 = int(id / (size_t(g.n[0]) * g.n[1]));
-        double gr = 0.0, gg = 0.0, lg = 0.0, lr = 0.0;
-        const int ii[3] = {i1, i2, i3};
+// squares of the difference quotients' factors per direction: (1/(2 dxi))^2 and (1/dxi^2)^2
+struct MonScale3 {
+    double d1[3], d2[3];
+};
+
+// raw monitor terms (eq. van der Waalsmonitor, or the smooth-test monitor): central first and second differences, whose
+// factors multiply the squares; maxima by their ordered bits.  Bound by the FP64 pipe: about 30 instructions a node for
+// the van der Waals monitor and 45 with the two square roots of the other, where both forms' sums, differences divided
+// one by one and FP64 maxima were 91 (140 us at 96^3).
+template <bool SMOOTH>
+__global__ void k3_mon_terms(Grid3 g, MonScale3 sc, int kappa, const double* rhoF, const double* GF, double* t0, double* t1,
+                             double* t2, DevScalars* d) {
+    const unsigned N = unsigned(g.n[0]) * g.n[1] * g.n[2];
+    double mx[3] = {0.0, 0.0, 0.0};
+    for (unsigned id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
+        const int i1 = int(id % unsigned(g.n[0])), r = int(id / unsigned(g.n[0]));
+        const int ii[3] = {i1, r % g.n[1], r / g.n[1]};
+        const double* f2 = SMOOTH ? rhoF : GF;               // the field of the second differences
+        const double c0 = f2[id];
+        double v0 = 0.0, v1 = 0.0, v2 = 0.0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const double h = g.inv_dxi[k];
             const size_t ip = nb_index(g, id, ii[k], k, 1), im = nb_index(g, id, ii[k], k, -1);
-            const double rp = rhoF[ip], rm = rhoF[im];
-            const double Gp = GF[ip], Gm = GF[im];
-            const double r0 = rhoF[id], G0 = GF[id];
-            const double a = (rp - rm) * 0.5 * h, bb = (Gp - Gm) * 0.5 * h;
-            const double c = (Gp - 2.0 * G0 + Gm) * h * h, e = (rp - 2.0 * r0 + rm) * h * h;
-            gr += a * a;
-            gg += bb * bb;
-            lg += c * c;
-            lr += e * e;
+            const double a = rhoF[ip] - rhoF[im];
+            v0 = fma(sc.d1[k] * a, a, v0);
+            const double fp = f2[ip], fm = f2[im];
+            if (!SMOOTH && kappa >= 2) {
+                const double b = fp - fm;
+                v1 = fma(sc.d1[k] * b, b, v1);
+            }
+            const double c = fma(-2.0, c0, fp) + fm;
+            v2 = fma(sc.d2[k] * c, c, v2);
         }
-        double v0, v1, v2;
-        if (mp.kind == ES_MONITOR_SMOOTH) {
-            v0 = sqrt(gr);
-            v1 = 0.0;
-            v2 = sqrt(lr);
-        } else {
-            v0 = gr;
-            v1 = mp.kappa >= 2 ? gg : 0.0;
-            v2 = lg;
+        if (SMOOTH) {
+            v0 = sqrt_pos(v0);
+            v2 = sqrt_pos(v2);
         }
         t0[id] = v0;
         t1[id] = v1;
         t2[id] = v2;
-        m0 = fmax(m0, v0);
-        m1 = fmax(m1, v1);
-        m2 = fmax(m2, v2);
+        mx[0] = max_bits(mx[0], v0);
+        mx[1] = max_bits(mx[1], v1);
+        mx[2] = max_bits(mx[2], v2);
     }
-    m0 = block_max(m0);
-    m1 = block_max(m1);
-    m2 = block_max(m2);
+    block_max_bits<3>(mx);
     if (threadIdx.x == 0) {
-        atomic_max_pos(&d->red[RED_MON0], m0);
-        atomic_max_pos(&d->red[RED_MON1], m1);
-        atomic_max_pos(&d->red[RED_MON2], m2);
-    }
-}
-
-// omega_i <- sum_{j in {0,+-1}^3} (1/2)^(|j|_1 + 3) omega_{i+j}
-__global__ void k3_filter(Grid3 g, const double* in, double* out) {
-    const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
-    for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
-        const int i1 = int(id % g.n[0]), i2 = int((id / g.n[0]) % g.n[1]), i3 = int(id / (size_t(g.n[0]) * g.n[1]));
-        // offsets of the neighbours along each direction (ghosts by copy / wrap, per direction)
-        long long o1[3], o2[3], o3[3];
-        o1[1] = o2[1] = o3[1] = 0;
-        o1[0] = (long long)nb_index(g, id, i1, 0, -1) - (long long)id;
-        o1[2] = (long long)nb_index(g, id, i1, 0, 1) - (long long)id;
-        o2[0] = (long long)nb_index(g, id, i2, 1, -1) - (long long)id;
-        o2[2] = (long long)nb_index(g, id, i2, 1, 1) - (long long)id;
-        o3[0] = (long long)nb_index(g, id, i3, 2, -1) - (long long)id;
-        o3[2] = (long long)nb_index(g, id, i3, 2, 1) - (long long)id;
-        double s = 0.0;
-#pragma unroll
-        for (int d3 = 0; d3 < 3; ++d3) {
-            double pl = 0.0;
-#pragma unroll
-            for (int d2 = 0; d2 < 3; ++d2) {
-                double row = 0.0;
-#pragma unroll
-                for (int d1 = 0; d1 < 3; ++d1) row += (d1 == 1 ? 0.5 : 0.25) * in[(long long)id + o1[d1] + o2[d2] + o3[d3]];
-                pl += (d2 == 1 ? 0.5 : 0.25) * row;
-            }
-            s += (d3 == 1 ? 0.5 : 0.25) * pl;
-        }
-        out[id] = s;
+        atomic_max_pos(&d->red[RED_MON0], mx[0]);
+        atomic_max_pos(&d->red[RED_MON1], mx[1]);
+        atomic_max_pos(&d->red[RED_MON2], mx[2]);
     }
 }
 
@@ -624,43 +588,72 @@ __device__ __forceinline__ bool fixed3(const Grid3& g, const int* ii, int c) {
     return f;
 }
 
+// The sweeps' normalised weights of a node's neighbours (-xi_1, +xi_1, -xi_2, ...): the first sweep forms them from omega,
+// the others read them.
+struct SweepWeights3 {
+    double* a[6];
+};
+
 // Jacobi sweep k (no warm start in 3D: sweep 0 reads x_n and writes xa, sweep k reads
 // buf[(k - 1) % 2] and writes buf[k % 2]); with `check` the last block to finish compares the
-// grid's max change with eps and latches convergence, after which the remaining sweeps return
-__global__ void k3_jacobi(Grid3 g, const double* omega, const double* xn, double* xa, double* xb, int k,
-                          DevScalars* d, int check, double eps) {
+// grid's max change with eps and latches convergence, after which the remaining sweeps return.
+// A sweep that formed the weights again took 78 FP64 instructions a node (119 us at 96^3, bound by the FP64 pipe); with
+// stored weights it is 18 and the traffic of 12 doubles a node bounds it.
+template <bool FIRST, bool CHG>
+__global__ void k3_jacobi(Grid3 g, const double* omega, SweepWeights3 W, double r2, double r3, const double* xin,
+                          double* xout, DevScalars* d, double eps) {
     if (d->conv) return;
-    const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
-    const double* xin = k == 0 ? xn : (((k - 1) & 1) ? xb : xa);
-    double* xout = (k & 1) ? xb : xa;
+    const unsigned N = unsigned(g.n[0]) * g.n[1] * g.n[2];
+    const int st[3] = {1, g.n[0], g.n[0] * g.n[1]};
     double chg = 0.0;
-    for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
-        const int ii[3] = {int(id % g.n[0]), int((id / g.n[0]) % g.n[1]), int(id / (size_t(g.n[0]) * g.n[1]))};
-        const double w0 = omega[id];
-        double den = 0.0, num[3] = {0.0, 0.0, 0.0};
+    for (unsigned id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
+        const int i1 = int(id % unsigned(g.n[0])), r = int(id / unsigned(g.n[0]));
+        const int ii[3] = {i1, r % g.n[1], r / g.n[1]};
+        double a[6];
+        if (FIRST) {
+            const double w0 = omega[id];
+            double sum = 0.0;
 #pragma unroll
-        for (int kk = 0; kk < 3; ++kk) {
-            const double ih2 = g.inv_dxi[kk] * g.inv_dxi[kk];
-            const double wp = 0.5 * (w0 + omega[nb_index(g, id, ii[kk], kk, 1)]) * ih2;
-            const double wm = 0.5 * (w0 + omega[nb_index(g, id, ii[kk], kk, -1)]) * ih2;
-            den += wp + wm;
+            for (int k = 0; k < 3; ++k)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const double xp = nb_coord(g, xin + c * N, id, ii[kk], kk, 1, c);
-                const double xq = nb_coord(g, xin + c * N, id, ii[kk], kk, -1, c);
-                num[c] += wp * xp + wm * xq;
-            }
+                for (int q = 0; q < 2; ++q) {
+                    const double w = w0 + omega[nb_index(g, id, ii[k], k, 2 * q - 1)];
+                    a[2 * k + q] = k == 0 ? w : w * (k == 1 ? r2 : r3);
+                }
+            sum = ((a[0] + a[1]) + (a[2] + a[3])) + (a[4] + a[5]);
+            const double is = rcp_nr(sum);
+            // the first is 1 less the others: their sum is 1 to one rounding and a sweep adds no drift to the coordinates
+#pragma unroll
+            for (int m = 1; m < 6; ++m) a[m] *= is;
+            a[0] = 1.0 - ((a[1] + (a[2] + a[3])) + (a[4] + a[5]));
+#pragma unroll
+            for (int m = 0; m < 6; ++m) W.a[m][id] = a[m];
+        } else {
+#pragma unroll
+            for (int m = 0; m < 6; ++m) a[m] = W.a[m][id];
         }
-        const double iden = rcp_nr(den);
+        const bool in = inside3(g, ii[0], ii[1], ii[2], 1);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double xv = fixed3(g, ii, c) ? xin[c * N + id] : num[c] * iden;
-            chg = fmax(chg, fabs(xv - xin[c * N + id]));
-            xout[c * N + id] = xv;
+            const double* x = xin + size_t(c) * N;
+            double v = 0.0;
+            if (in) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    v = fma(a[2 * k + 1], x[id + st[k]], k == 0 ? a[0] * x[id - 1] : fma(a[2 * k], x[id - st[k]], v));
+            } else if (fixed3(g, ii, c)) {
+                v = x[id];
+            } else {
+                for (int k = 0; k < 3; ++k)
+                    v = fma(a[2 * k + 1], nb_coord(g, x, id, ii[k], k, 1, c),
+                            fma(a[2 * k], nb_coord(g, x, id, ii[k], k, -1, c), v));
+            }
+            if (CHG) chg = max_bits(chg, fabs(v - x[id]));
+            xout[size_t(c) * N + id] = v;
         }
     }
-    if (check) {
-        chg = block_max(chg);
+    if (CHG) {
+        block_max_bits<1>(&chg);
         if (threadIdx.x == 0) {
             atomic_max_pos(&d->red[RED_JAC], chg);
             __threadfence();
@@ -676,20 +669,25 @@ __global__ void k3_jacobi(Grid3 g, const double* omega, const double* xn, double
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&d->sweeps, 1);
 }
 
-// Delta_gamma over all nodes and directions (Sec. 4)
+// Delta_gamma over all nodes and directions (Sec. 4): the spacing to the neighbour that a node moves towards over twice its
+// displacement; the division only where it lowers the minimum so far (a node that moves less than half of its spacing, as
+// nearly all do, is three FP64 instructions a direction)
 __global__ void k3_limiter(Grid3 g, const double* xn, const double* xa, const double* xb, DevScalars* d) {
-    const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
+    const unsigned N = unsigned(g.n[0]) * g.n[1] * g.n[2];
     const double* xit = d->sweeps == 0 ? xn : (((d->sweeps - 1) & 1) ? xb : xa);
     double m = 1.0;
-    for (size_t id = blockIdx.x * size_t(blockDim.x) + threadIdx.x; id < N; id += size_t(gridDim.x) * blockDim.x) {
-        const int ii[3] = {int(id % g.n[0]), int((id / g.n[0]) % g.n[1]), int(id / (size_t(g.n[0]) * g.n[1]))};
+    for (unsigned id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
+        const int i1 = int(id % unsigned(g.n[0])), r = int(id / unsigned(g.n[0]));
+        const int ii[3] = {i1, r % g.n[1], r / g.n[1]};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const double dx = xit[k * N + id] - xn[k * N + id];
-            if (dx < 0.0)
-                m = fmin(m, div_nr(-(xn[k * N + id] - nb_coord(g, xn + k * N, id, ii[k], k, -1, k)), 2.0 * dx));
-            else if (dx > 0.0)
-                m = fmin(m, div_nr(nb_coord(g, xn + k * N, id, ii[k], k, 1, k) - xn[k * N + id], 2.0 * dx));
+            const double* x = xn + size_t(k) * N;
+            const double x0 = x[id], dx = xit[size_t(k) * N + id] - x0;
+            if (__double_as_longlong(dx) << 1 == 0) continue;                        // +-0
+            const bool back = __double2hiint(dx) < 0;
+            const double xb1 = nb_coord(g, x, id, ii[k], k, back ? -1 : 1, k);
+            const double gap = back ? x0 - xb1 : xb1 - x0, two = 2.0 * fabs(dx);
+            if (gap < m * two) m = fmin(m, div_nr(gap, two));
         }
     }
     m = block_min(m);
@@ -845,21 +843,42 @@ int d3_mesh(Ctx3* d, const void* JU, const void* J, const double* xn, double* xd
     grid_floats(flat);
     int n = 0;
     launch_mon_fields(flat, d->gas, JU, J, d->rhoF, d->GF, false, G, s);
-    k3_mon_terms<<<G, 256, 0, s>>>(d->g, d->mon, d->rhoF, d->GF, d->t0, d->t1, d->t2, dv);
+    MonScale3 sc;
+    for (int k = 0; k < 3; ++k) {
+        const double h = d->g.inv_dxi[k];
+        sc.d1[k] = 0.25 * h * h;
+        sc.d2[k] = (h * h) * (h * h);
+    }
+    if (d->mon.kind == ES_MONITOR_SMOOTH)
+        k3_mon_terms<true><<<G, 256, 0, s>>>(d->g, sc, d->mon.kappa, d->rhoF, d->GF, d->t0, d->t1, d->t2, dv);
+    else
+        k3_mon_terms<false><<<G, 256, 0, s>>>(d->g, sc, d->mon.kappa, d->rhoF, d->GF, d->t0, d->t1, d->t2, dv);
     k_mon_omega<<<G, 256, 0, s>>>(flat, d->mon, d->t0, d->t1, d->t2, dv, d->om0);
     n += 3;
     double* om = d->om0;
     double* other = d->om1;
     for (int k = 0; k < d->filter_passes; ++k) {
-        k3_filter<<<G, 256, 0, s>>>(d->g, om, other);
+        launch_filter3(d->g, om, other, s);
         ++n;
         double* t = om;
         om = other;
         other = t;
     }
-    const int check = d->eps > 0.0;
+    // the monitor's fields and the filter's other buffer are free: the sweeps' weights
+    const SweepWeights3 W = {{d->t0, d->t1, d->t2, d->rhoF, d->GF, other}};
+    const double h1 = d->g.inv_dxi[0], h2 = d->g.inv_dxi[1], h3 = d->g.inv_dxi[2];
+    const double r2 = (h2 / h1) * (h2 / h1), r3 = (h3 / h1) * (h3 / h1);
+    const bool check = d->eps > 0.0;
     for (int k = 0; k < d->sweeps; ++k) {
-        k3_jacobi<<<G, 256, 0, s>>>(d->g, om, xn, d->xa, d->xb, k, dv, check, d->eps);
+        const double* xin = k == 0 ? xn : ((k & 1) ? d->xa : d->xb);
+        double* xout = (k & 1) ? d->xb : d->xa;
+        if (k == 0) {
+            if (check) k3_jacobi<true, true><<<G, 256, 0, s>>>(d->g, om, W, r2, r3, xin, xout, dv, d->eps);
+            else k3_jacobi<true, false><<<G, 256, 0, s>>>(d->g, om, W, r2, r3, xin, xout, dv, d->eps);
+        } else {
+            if (check) k3_jacobi<false, true><<<G, 256, 0, s>>>(d->g, om, W, r2, r3, xin, xout, dv, d->eps);
+            else k3_jacobi<false, false><<<G, 256, 0, s>>>(d->g, om, W, r2, r3, xin, xout, dv, d->eps);
+        }
         ++n;
     }
     k3_limiter<<<G, 256, 0, s>>>(d->g, xn, d->xa, d->xb, dv);

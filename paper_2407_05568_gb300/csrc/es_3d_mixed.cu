@@ -15,6 +15,7 @@
 
 #include "es_3d.h"
 #include "es_bits.cuh"
+#include "es_3d_filter.cuh"
 #include "es_3d_grid.cuh"
 #include "es_device.cuh"
 #include "es_flux32.cuh"
@@ -891,36 +892,6 @@ __global__ void k3f_mon_terms(Grid3 g, MonitorParams mp, const float* rhoF, cons
     }
 }
 
-// omega_i <- sum_{j in {0,+-1}^3} (1/2)^(|j|_1 + 3) omega_{i+j} (Sec. 4's low-pass filter)
-__global__ void k3f_filter(Grid3 g, const float* in, float* out) {
-    const int N = g.n[0] * g.n[1] * g.n[2];
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
-        int ii[3];
-        split3(g, id, ii);
-        int o1[3], o2[3], o3[3];
-        o1[1] = o2[1] = o3[1] = 0;
-        o1[0] = nb3(g, id, ii[0], 0, -1) - id;
-        o1[2] = nb3(g, id, ii[0], 0, 1) - id;
-        o2[0] = nb3(g, id, ii[1], 1, -1) - id;
-        o2[2] = nb3(g, id, ii[1], 1, 1) - id;
-        o3[0] = nb3(g, id, ii[2], 2, -1) - id;
-        o3[2] = nb3(g, id, ii[2], 2, 1) - id;
-        float s = 0.0f;
-#pragma unroll
-        for (int d3 = 0; d3 < 3; ++d3) {
-            float pl = 0.0f;
-#pragma unroll
-            for (int d2 = 0; d2 < 3; ++d2) {
-                const int b = id + o2[d2] + o3[d3];
-                const float row = 0.25f * in[b + o1[0]] + 0.5f * in[b] + 0.25f * in[b + o1[2]];
-                pl += (d2 == 1 ? 0.5f : 0.25f) * row;
-            }
-            s += (d3 == 1 ? 0.5f : 0.25f) * pl;
-        }
-        out[id] = s;
-    }
-}
-
 // the sweep coefficients of every node: a_nb for the six neighbours ([6][N], order -xi_1, +xi_1,
 // -xi_2, ...) and g ([3][N]); zero at fixed nodes
 __global__ void k3f_coeffs(Grid3 g, const float* om, const float* XEh, const float* XEl, float* A, float* Gc) {
@@ -1230,7 +1201,7 @@ int d3f_mesh(Ctx3* d, const void* JU, const void* J, const double* xn, double* x
     k_mon_omega_f<<<G, 256, 0, s>>>(flat, d->mon, t0, t1, t2, dv, om);
     n += 3;
     for (int k = 0; k < d->filter_passes; ++k) {
-        k3f_filter<<<G, 256, 0, s>>>(d->g, om, other);
+        launch_filter3(d->g, om, other, s);
         ++n;
         float* t = om;
         om = other;
