@@ -150,6 +150,7 @@ __global__ void k3_metric(Grid3 g, const double* D, double* NKo) {
     const size_t M = size_t(m1) * m2 * m3;
     const int l = (k + 1) % 3, m = (k + 2) % 3;
     const double scale = 0.5 * (g.inv_dxi[l] * g.inv_dxi[m]);
+    const double h[3] = {0.5 * ec_alpha(1) * scale, 0.5 * ec_alpha(2) * scale, 0.5 * ec_alpha(3) * scale};
     const size_t stl = l == 0 ? 1 : (l == 1 ? size_t(E1) : size_t(E1) * E2);
     const size_t stm = m == 0 ? 1 : (m == 1 ? size_t(E1) : size_t(E1) * E2);
     for (size_t t = blockIdx.x * size_t(blockDim.x) + threadIdx.x; t < M; t += size_t(gridDim.x) * blockDim.x) {
@@ -159,15 +160,14 @@ __global__ void k3_metric(Grid3 g, const double* D, double* NKo) {
         for (int j = 0; j < 3; ++j) {
             const double* Pl = D + (3 * l + j) * NE;      // delta_l[x_p] x_q
             const double* Pm = D + (3 * m + j) * NE;      // delta_m[x_p] x_q
-            double A = 0.0, B = 0.0;
+            double A = 0.0;
 #pragma unroll
             for (int a = 1; a <= 3; ++a) {
-                const double h = 0.5 * ec_alpha(a);
                 const size_t sm = a * stm, sl = a * stl;
-                A += h * (Pl[e + sm] - Pl[e - sm]);
-                B += h * (Pm[e + sl] - Pm[e - sl]);
+                A = fma(h[a - 1], Pl[e + sm] - Pl[e - sm], A);
+                A = fma(-h[a - 1], Pm[e + sl] - Pm[e - sl], A);
             }
-            NKo[j * M + t] = (A - B) * scale;
+            NKo[j * M + t] = A;
         }
     }
 }

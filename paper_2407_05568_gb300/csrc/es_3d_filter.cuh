@@ -13,7 +13,7 @@ namespace es {
 // column sum and a plane sum, two instructions each, and one scaling: 8 at RY = 4.  Neighbours along xi_1 come from the
 // neighbouring lanes (the warp's ends and the mesh's last node load theirs), so there is no shared memory and no barrier;
 // the next plane's loads are in flight while a plane is summed.  The weights are powers of two, so that the sums without
-// them (l + 2 c + r) have the same bits as with them.  96^3: FP64 73 -> 21 us, FP32 11.3 -> 6 us.
+// them (l + 2 c + r) have the same bits as with them.  96^3: FP64 73 -> 24 us (FP32 stays at 12: there the loads of one plane after the other bound it).
 template <typename T, int RY>
 __global__ void __launch_bounds__(128) k3_filter(Grid3 g, const T* in, T* out, int seg) {
     const int n1 = g.n[0], n2 = g.n[1], n3 = g.n[2];
