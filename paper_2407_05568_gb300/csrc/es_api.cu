@@ -533,8 +533,10 @@ int enqueue_step(es_ctx* c, void* JU, void* J, double* x, bool first = true, boo
         e = launch_stage(c, P);
         if (e != cudaSuccess) return cuda_fail(c, e, "stage kernel");
     }
-    // the next step's displacement (mixed form) and reductions, for a following step of the same call
-    k_advance<<<G, B, 0, s>>>(c->g, x, xdot ? c->xdot : nullptr, c->dev, chain && f32 ? c->fdisp : nullptr, chain);
+    // the next step's displacement (mixed form; a mesh at rest keeps the first step's) and reductions, for a following
+    // step of the same call
+    k_advance<<<xdot ? G : 1, B, 0, s>>>(c->g, x, xdot ? c->xdot : nullptr, c->dev, chain && f32 && xdot ? c->fdisp : nullptr,
+                                         chain);
     count(c);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "advance kernel");
