@@ -8,12 +8,14 @@ namespace es {
 
 // omega_i <- sum_{j in {0,+-1}^3} (1/2)^(|j|_1 + 3) omega_{i+j} (Sec. 4), ghosts by copy / wrap.
 // The filter is the product of three (1/4, 1/2, 1/4) sums.  Read node by node it is 27 products (in FP64, 48 instructions on
-// the FP64 pipe, which bound it: 73 us at 96^3); here the sums are shared: a warp takes 32 nodes along xi_1 and RY lines,
+// the FP64 pipe, which bound it: 77 us at 96^3); here the sums are shared: a warp takes 32 nodes along xi_1 and RY lines,
 // and marches along xi_3 keeping the last two planes' partial sums, so a node costs the row sums of (RY + 2)/RY lines, a
-// column sum and a plane sum, two instructions each, and one scaling: 8 at RY = 4.  Neighbours along xi_1 come from the
-// neighbouring lanes (the warp's ends and the mesh's last node load theirs), so there is no shared memory and no barrier;
-// the next plane's loads are in flight while a plane is summed.  The weights are powers of two, so that the sums without
-// them (l + 2 c + r) have the same bits as with them.  96^3: FP64 73 -> 24 us (FP32 stays at 12: there the loads of one plane after the other bound it).
+// column sum and a plane sum, two instructions each, and one scaling: 9 at RY = 2, 8 at RY = 4 (and the segments' ends).
+// Neighbours along xi_1 come from the neighbouring lanes (the warp's ends and the mesh's last node load theirs), so there is
+// no shared memory and no barrier; the next plane's loads are in flight while a plane is summed.  The weights are powers of
+// two, so that the sums without them (l + 2 c + r) have the same bits as with them.  96^3: FP64 77 -> 25 us, FP32 12.4 ->
+// 10.3.  (Four passes at a time on 16^3 tiles in shared memory, FP32: 9.7 us a pass, bound by the nine shared loads a node,
+// and no better on larger meshes.)
 template <typename T, int RY>
 __global__ void __launch_bounds__(128) k3_filter(Grid3 g, const T* in, T* out, int seg) {
     const int n1 = g.n[0], n2 = g.n[1], n3 = g.n[2];
@@ -64,17 +66,25 @@ __global__ void __launch_bounds__(128) k3_filter(Grid3 g, const T* in, T* out, i
     }
 }
 
-// segments along xi_3: short enough for two warps on each of the 608 schedulers, at least 4 planes (each segment sums two
-// planes more), at most 32
-template <typename T>
-inline void launch_filter3(const Grid3& g, const T* in, T* out, cudaStream_t s) {
-    constexpr int RY = 4;
+// Lines per warp and planes per segment.  A warp's planes follow one another, 1.1 us each (FP32; a load's latency), so on
+// meshes of up to 2^21 nodes short segments and two lines keep the launch short although they sum more planes and rows
+// twice: four warps on each of the 608 schedulers where the mesh gives them, at least 2 planes.  96^3: 24.6 us (FP64) and
+// 10.3 us (FP32, 12.4 node by node), with four lines and 1216 warps 26.2 and 12.4; 40^3: 10.3 and 6.2 us (12.4 and 6.1 node
+// by node), 14.4 and 10.3.  Above, four lines in segments of 4 to 12 planes: 200^3 172 and 41 us (two lines 190 and 43, node
+// by node 625 and 78).
+template <typename T, int RY>
+inline void launch_filter3(const Grid3& g, const T* in, T* out, int target, int lo, cudaStream_t s) {
     const int cols = (g.n[0] + 31) / 32 * ((g.n[1] + RY - 1) / RY);
-    const int parts = (1216 + cols - 1) / cols;
+    const int parts = (target + cols - 1) / cols;
     int seg = (g.n[2] + parts - 1) / parts;
-    seg = seg < 4 ? 4 : (seg > 32 ? 32 : seg);
+    seg = seg < lo ? lo : (seg > 12 ? 12 : seg);
     const int warps = cols * ((g.n[2] + seg - 1) / seg);
     k3_filter<T, RY><<<(warps + 3) / 4, 128, 0, s>>>(g, in, out, seg);
+}
+template <typename T>
+inline void launch_filter3(const Grid3& g, const T* in, T* out, cudaStream_t s) {
+    if (size_t(g.n[0]) * g.n[1] * g.n[2] <= (size_t(1) << 21)) launch_filter3<T, 2>(g, in, out, 2432, 2, s);
+    else launch_filter3<T, 4>(g, in, out, 1216, 4, s);
 }
 
 }  // namespace es

@@ -71,7 +71,7 @@ def test_redistribution_monitors_and_tolerance(monitor, kappa, eps):
 @pytest.mark.parametrize("shape,passes,sweeps,monitor", [((33, 9, 14), 3, 2, "vdw"), ((32, 12, 8), 2, 3, "smooth"),
                                                          ((65, 8, 37), 1, 1, "vdw"), ((8, 31, 9), 5, 4, "smooth")])
 def test_redistribution_3d(bc, shape, passes, sweeps, monitor):
-    """The filter's warps of 32 nodes by four lines and segments of planes at their edges (one node over, whole, one
+    """The filter's warps of 32 nodes by two lines and segments of planes at their edges (one node over, whole, one
     short), and the sweeps with stored weights, every boundary."""
     from test_gpu_3d import _box
     w = _box(*shape, bc == "periodic", amp=0.0 if bc == "walls" else 0.2 / max(shape))
