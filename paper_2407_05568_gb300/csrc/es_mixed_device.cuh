@@ -629,7 +629,9 @@ __device__ __forceinline__ void stage_tile_mixed(float* smemf, const StageParams
         }
         if (P.diss) {
             // neighbour jumps V_{q+1} - V_q, q = 0 .. LB+4 along each line (eq. jumpV)
-            for (int t = tid; t < nlines * (LB + 5); t += NT) {
+            // (in a 1D tile whose pairs leave enough threads, the warps after the pairs')
+            constexpr int JOFF = DIM == 1 && (TL::NP + 31) / 32 * 32 + TL::NJ <= NT ? (TL::NP + 31) / 32 * 32 : 0;
+            for (int t = JOFF ? (tid + NT - JOFF) % NT : tid; t < nlines * (LB + 5); t += NT) {
                 const int line = t / (LB + 5), q = t % (LB + 5);
                 const int base = k == 0 ? (DIM == 2 ? (3 + line) * GX : 0) : 3 + line;
                 const int l = base + q * step;

@@ -414,8 +414,14 @@ cudaError_t launch_tile_f(const StageParams& P, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-constexpr int LINE_BX = 254, LINE_NT = 256;
+// 1D tiles: 254 nodes, a node per thread, or 58 with the same 256 threads, one thread per pair or jump, for lines that the
+// smaller tiles cover in one wave of two CTAs per SM: there a stage is the length of one tile's dependent phases, which
+// take three rounds of pairs and two of jumps with 254 nodes.  Stages of 40 to 17632 nodes, launch to launch: 8.3 -> 6.3 us,
+// the same bits; a second wave would bring the short tile to 8.3, where the other stays up to 30000 nodes.
+constexpr int LINE_BX = 254, SHORT_BX = 58, LINE_NT = 256;
 using LineTile = TileF<1, LINE_BX, 1, LINE_NT>;
+using ShortTile = TileF<1, SHORT_BX, 1, LINE_NT>;
+constexpr int SHORT_MAX = SHORT_BX * 2 * 152;
 
 }  // namespace
 
@@ -427,7 +433,7 @@ using LineTile = TileF<1, LINE_BX, 1, LINE_NT>;
 cudaError_t stage_prepare_mixed(int dim) {
     if (dim == 1)
         return cudaFuncSetAttribute(stage_kernel_mixed1<LINE_BX, LINE_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(LineTile::SMEM));
+                                    int(LineTile::SMEM));      // (the short tile's 11 KB need no attribute)
     cudaError_t e = prepare_tile_f<20, 8, 384, true>();
     if (e == cudaSuccess) e = prepare_tile_f<25, 6, 192>();
     if (e == cudaSuccess) e = prepare_tile_f<20, 8, 192>();
@@ -438,7 +444,10 @@ cudaError_t stage_prepare_mixed(int dim) {
 
 cudaError_t launch_stage_mixed(const StageParams& P, cudaStream_t s) {
     if (P.dim == 1) {
-        stage_kernel_mixed1<LINE_BX, LINE_NT><<<(P.n1 + LINE_BX - 1) / LINE_BX, LINE_NT, LineTile::SMEM, s>>>(P);
+        if (P.n1 <= SHORT_MAX)
+            stage_kernel_mixed1<SHORT_BX, LINE_NT><<<(P.n1 + SHORT_BX - 1) / SHORT_BX, LINE_NT, ShortTile::SMEM, s>>>(P);
+        else
+            stage_kernel_mixed1<LINE_BX, LINE_NT><<<(P.n1 + LINE_BX - 1) / LINE_BX, LINE_NT, LineTile::SMEM, s>>>(P);
         return cudaGetLastError();
     }
     switch (P.tile) {

@@ -69,3 +69,29 @@ def test_3d_filter_passes(n, periodic, passes):
     _, gam = es.es_mesh_redistribute(ctx, JU, J, xt, 1e-3, xd)
     assert abs(gam - gam_o) <= 2e-5 * gam_o
     assert np.abs(xd.cpu().numpy() - xd_o).max() <= 2e-5 * np.abs(xd_o).max()
+
+
+@pytest.mark.parametrize("n", [8, 57, 58, 59, 116, 117, 254, 255, 17632, 17633])
+@pytest.mark.parametrize("bc", ["periodic", "outflow"])
+def test_1d_tiles_against_oracle(n, bc):
+    """The two 1D tiles (58 and 254 nodes) at their edges and at the size where one takes over from the other: right-hand
+    sides of a rough state on a moving mesh within 1e-5 of the flux scale, the bound of the form's other right-hand sides."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    x, d = wl.uniform_nodes(n, 0.0, 1.0, bc == "periodic")
+    w = wl.sine_1d(max(n, 8))
+    w.update(bc=(bc,), x=x[None].copy(), dxi=(d,))
+    w["rho"], w["v"], w["p"] = wl.rough_state((n,), 3 + n, 1)
+    xdot = 0.05 * np.sin(2 * np.pi * x + 0.3)[None]
+    if bc != "periodic":
+        xdot[:, [0, -1]] = 0.0
+    sch, _, JU_o, J_o, x_o = oracle_setup(w)
+    dU_o, dJ_o = op.rhs(sch, JU_o, J_o, x_o, xdot)
+    ctx, JU, J, xt = gpu_setup(w, precision="mixed")
+    dU, dJ = torch.empty_like(JU), torch.empty_like(J)
+    es.es_rhs(ctx, JU, J, xt, torch.tensor(xdot, device="cuda"), dU, dJ)
+    assert es.es_check(ctx) == 0, es.es_last_error(ctx)
+    assert np.abs(to_np(dU) - dU_o).sum() < 1e-5 * np.abs(JU_o).sum() / d
+    assert np.abs(to_np(dJ) - dJ_o).sum() < 1e-5 * np.abs(J_o).sum() / d
