@@ -32,13 +32,16 @@ namespace {
 // is one node per thread and each of its phases one round (with BT - 2, four threads loaded a second node and three formed
 // a second jump while the others waited), 32 warps per SM (64 registers, no spills; at 24 the warps waited for the global
 // loads of the short phases, 57% of the issue slots busy, at 32 71%).  4096 tubes of 200 to 8000 nodes, 10 steps: 42.5 ms
-// with 24 warps, chunks of BT - 2 and the mesh buffers in global memory, 33.4 ms now; bound by instruction issue.
+// with 24 warps, chunks of BT - 2 and the mesh buffers in global memory, 31.9 ms now; bound by instruction issue.
 template <int BT>
 struct BatchShape {
     static constexpr int BXC = BT - 6;
-    using TB = TileF<1, BXC, 1, BT>;
+    using TB = TileF<BXC, BT>;
     static constexpr int MIN_BLOCKS = 1024 / BT;
-    static constexpr int SMEM_FLOATS = int(TB::SMEM / sizeof(float));
+    // four CTAs of 256 threads leave 57 KB each: 42 KB for the mesh passes' buffers, which a stage tile takes 34 KB of
+    static constexpr int SMEM_FLOATS = 41 * BT;
+    static constexpr size_t SMEM = sizeof(float) * SMEM_FLOATS;
+    static_assert(TB::SMEM <= SMEM, "the stage tile fits");
 };
 
 __device__ __forceinline__ float block_max_f(float v, float* red) {
@@ -166,7 +169,7 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
                 const float c1 = m1 > 0.0f ? B.w1 / m1 : 0.0f;
                 const float c2 = m2 > 0.0f ? B.w2 / m2 : 0.0f;
                 // the filter's and the sweeps' two buffers lie in the stage tiles' shared memory where they fit (lines of
-                // up to 5218 nodes with 256 threads; the passes are short dependent reads); the sweeps start in the buffer
+                // up to 5248 nodes with 256 threads; the passes are short dependent reads); the sweeps start in the buffer
                 // that the filter left free, and take omega's once the coefficients are formed
                 const bool in_smem = 2 * L <= BatchShape<BT>::SMEM_FLOATS;
                 float* om = in_smem ? smemf : om0;
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
                 P.fJUo = (st == 0 ? B.S1 : (st == 1 ? B.S2 : B.JU)) + off;
                 P.fJo = (st == 0 ? B.S1J : (st == 1 ? B.S2J : B.J)) + off;
                 for (int c0 = 0; c0 < L; c0 += BXC) {
-                    stage_tile_mixed<1, BXC, 1, BT>(smemf, P, c0, 0, dtf, G, W);
+                    stage_tile_mixed<BXC, BT>(smemf, P, c0, dtf, G, W);
                     __syncthreads();
                 }
             }
@@ -280,13 +283,13 @@ __global__ void __launch_bounds__(BT, BatchShape<BT>::MIN_BLOCKS) batch_kernel(B
 template <int BT>
 cudaError_t prepare_shape() {
     return cudaFuncSetAttribute(batch_kernel<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(BatchShape<BT>::TB::SMEM));
+                                int(BatchShape<BT>::SMEM));
 }
 
 template <int BT>
 int blocks_per_sm_shape() {
     int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<BT>, BT, BatchShape<BT>::TB::SMEM);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<BT>, BT, BatchShape<BT>::SMEM);
     return nb;
 }
 
@@ -295,7 +298,7 @@ int blocks_per_sm_shape() {
 const int BATCH_SHAPES[BATCH_NSHAPES] = {128, 256, 512};
 
 size_t batch_smem_bytes(int bt) {
-    return bt == 128 ? BatchShape<128>::TB::SMEM : bt == 512 ? BatchShape<512>::TB::SMEM : BatchShape<256>::TB::SMEM;
+    return bt == 128 ? BatchShape<128>::SMEM : bt == 512 ? BatchShape<512>::SMEM : BatchShape<256>::SMEM;
 }
 
 cudaError_t batch_prepare() {
@@ -307,9 +310,9 @@ cudaError_t batch_prepare() {
 
 cudaError_t batch_launch(const BatchParams& B, int grid, int bt, cudaStream_t s) {
     switch (bt) {
-        case 128: batch_kernel<128><<<grid, 128, BatchShape<128>::TB::SMEM, s>>>(B); break;
-        case 512: batch_kernel<512><<<grid, 512, BatchShape<512>::TB::SMEM, s>>>(B); break;
-        case 256: batch_kernel<256><<<grid, 256, BatchShape<256>::TB::SMEM, s>>>(B); break;
+        case 128: batch_kernel<128><<<grid, 128, BatchShape<128>::SMEM, s>>>(B); break;
+        case 512: batch_kernel<512><<<grid, 512, BatchShape<512>::SMEM, s>>>(B); break;
+        case 256: batch_kernel<256><<<grid, 256, BatchShape<256>::SMEM, s>>>(B); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -1,6 +1,6 @@
-// es_mixed_device.cuh -- device functions of the mixed-precision form (FP32 pipe,
-// double-float state and primitive jumps), shared by the tiled stage kernel and
-// the batched persistent kernel.  See es_stage_mixed.cu for the design.
+// es_mixed_device.cuh -- device functions of the mixed-precision form (FP32 pipe, double-float state and primitive jumps) in
+// 1D, shared by the tiled stage kernel and the batched persistent kernel (see es_stage_mixed.cu for the design), and the
+// displacement at a node in 1D and 2D.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -12,33 +12,24 @@ namespace es {
 namespace mixed {
 
 enum FieldF {
-    G_RHO, G_V1, G_V2, G_T, G_IT, G_OM, G_IOM, G_G, G_RT, G_VT1, G_VT2, G_V2T, G_RV1, G_RV2, G_RP,
-    G_RHOL, G_V1L, G_V2L, G_TL,   // low parts of rho, v, T (double-float)
-    G_N1X, G_N1Y, G_XT1, G_N2X, G_N2Y, G_XT2,
+    G_RHO, G_V1, G_T, G_IT, G_OM, G_IOM, G_G, G_RT, G_VT1, G_V2T, G_RV1, G_RP,
+    G_RHOL, G_V1L, G_TL,          // low parts of rho, v, T (double-float)
+    G_N1X, G_XT1,
     G_COUNT
 };
 
-template <int DIM, int BX, int BY, int NT>
+template <int BX, int NT>
 struct TileF {
-    static constexpr int GX = BX + 6;
-    static constexpr int GY = DIM == 2 ? BY + 6 : 1;
-    static constexpr int NB = GX * GY;
-    static constexpr int NC = DIM + 2;
-    static constexpr int NP1 = (DIM == 2 ? BY : 1) * (3 * BX + 6);
-    static constexpr int NP2 = DIM == 2 ? BX * (3 * BY + 6) : 0;
-    static constexpr int NP = NP1 > NP2 ? NP1 : NP2;
-    static constexpr int NF1 = (DIM == 2 ? BY : 1) * (BX + 1);
-    static constexpr int NF2 = DIM == 2 ? BX * (BY + 1) : 0;
-    static constexpr int NF = NF1 > NF2 ? NF1 : NF2;
-    static constexpr int PAIR_FLOATS = (NP * NC > 4 * NB) ? NP * NC : 4 * NB;
-    // entropy-variable jumps between neighbours along each line (box positions q, q + 1), shared
-    // by the faces whose stencils contain them
-    static constexpr int NJ1 = (DIM == 2 ? BY : 1) * (BX + 5);
-    static constexpr int NJ2 = DIM == 2 ? BX * (BY + 5) : 0;
-    static constexpr int NJ = NJ1 > NJ2 ? NJ1 : NJ2;
+    static constexpr int NB = BX + 6;
+    static constexpr int NC = 3;
+    static constexpr int NP = 3 * BX + 6;
+    static constexpr int NF = BX + 1;
+    static constexpr int PAIR_FLOATS = NP * NC;            // also holds the displacement and the mesh velocity
+    // entropy-variable jumps between neighbours (box positions q, q + 1), shared by the faces whose stencils contain them
+    static constexpr int NJ = BX + 5;
     static constexpr size_t SMEM =
         sizeof(float) * (size_t(G_COUNT) * NB + PAIR_FLOATS + NF * (NC + 1) + size_t(NJ) * NC);
-    static_assert(NT >= BX * (DIM == 2 ? BY : 1) && NT % 32 == 0, "threads cover the tile");
+    static_assert(NT >= BX && NT % 32 == 0 && PAIR_FLOATS >= 2 * NB, "threads cover the tile");
 };
 
 struct GasF {
@@ -93,9 +84,8 @@ __device__ __forceinline__ float mr_weno5_f(float wm2, float wm1, float w0, floa
     return (w1 * p1 + w2 * p2 + w3 * p3) / (w1 + w2 + w3);
 }
 
-template <int DIM>
-__device__ __forceinline__ void pair_flux_f(const float* S, int NB, int l, int r, float nx, float ny, float xt,
-                                            const GasF& G, float* out) {
+__device__ __forceinline__ void pair_flux_f(const float* S, int NB, int l, int r, float nx, float xt, const GasF& G,
+                                            float* out) {
     const float rl = S[G_RHO * NB + l], rr = S[G_RHO * NB + r];
     const float Tl = S[G_T * NB + l], Tr = S[G_T * NB + r];
     const float rho_m = 0.5f * (rl + rr);
@@ -121,24 +111,11 @@ __device__ __forceinline__ void pair_flux_f(const float* S, int NB, int l, int r
     const float P = rho_m * T_m * g_m;
     const float B0 = 0.5f * v2T_m - G.cv * T_m * ilT + 2.0f * G.a * rT_m;
     const float iiT = 1.0f / iT_m;
-    if (DIM == 1) {
-        const float Q1 = xt * U1 + nx * F11;
-        const float sv = vT1 * vm1;
-        out[0] = Q1;
-        out[1] = vm1 * Q1 + nx * P;
-        out[2] = (G.a * rT_m * (xt * rho_m + nx * rv1) + (sv - B0) * Q1 + P * nx * vT1) * iiT;
-    } else {
-        const float vm2 = 0.5f * (S[G_V2 * NB + l] + S[G_V2 * NB + r]);
-        const float vT2 = 0.5f * (S[G_VT2 * NB + l] + S[G_VT2 * NB + r]);
-        const float rv2 = 0.5f * (S[G_RV2 * NB + l] + S[G_RV2 * NB + r]);
-        const float F21 = (rv2 * coef + g_m * vm2) * iD;
-        const float Q1 = xt * U1 + nx * F11 + ny * F21;
-        const float sv = vT1 * vm1 + vT2 * vm2;
-        out[0] = Q1;
-        out[1] = vm1 * Q1 + nx * P;
-        out[2] = vm2 * Q1 + ny * P;
-        out[3] = (G.a * rT_m * (xt * rho_m + nx * rv1 + ny * rv2) + (sv - B0) * Q1 + P * (nx * vT1 + ny * vT2)) * iiT;
-    }
+    const float Q1 = xt * U1 + nx * F11;
+    const float sv = vT1 * vm1;
+    out[0] = Q1;
+    out[1] = vm1 * Q1 + nx * P;
+    out[2] = (G.a * rT_m * (xt * rho_m + nx * rv1) + (sv - B0) * Q1 + P * nx * vT1) * iiT;
 }
 
 // Entropy-variable jump V_j - V_i written as the jump decomposition of Sec. 3.1
@@ -146,7 +123,6 @@ __device__ __forceinline__ void pair_flux_f(const float* S, int NB, int l, int r
 //   [[V_1]] = [[rho]] (R/{rho}^ln + R b/{1-b rho}^ln + R b/Pi - 2a/{T})
 //           + [[T]] (-c_v/{T}^ln + (2a {rho/T} + {|v|^2/T}/2)/{T}) - sum_m {v_m}[[v_m]]/{T}
 //   [[V_{1+m}]] = ([[v_m]] - {v_m/T}[[T]])/{T},   [[V_E]] = [[T]]/(T_i T_j)
-template <int DIM>
 __device__ __forceinline__ void entropy_jump(const float* S, int NB, int i, int j, const GasF& G, float* dV) {
     const float ri = S[G_RHO * NB + i], rj = S[G_RHO * NB + j];
     const float Ti = S[G_T * NB + i], Tj = S[G_T * NB + j];
@@ -163,27 +139,20 @@ __device__ __forceinline__ void entropy_jump(const float* S, int NB, int i, int 
     const float dv1 = (v1j - v1i) + (S[G_V1L * NB + j] - S[G_V1L * NB + i]);
     float kin = 0.5f * (v1i + v1j) * dv1;
     dV[1] = (dv1 - 0.5f * (S[G_VT1 * NB + i] + S[G_VT1 * NB + j]) * dT) * iTa;
-    if (DIM == 2) {
-        const float v2i = S[G_V2 * NB + i], v2j = S[G_V2 * NB + j];
-        const float dv2 = (v2j - v2i) + (S[G_V2L * NB + j] - S[G_V2L * NB + i]);
-        kin += 0.5f * (v2i + v2j) * dv2;
-        dV[2] = (dv2 - 0.5f * (S[G_VT2 * NB + i] + S[G_VT2 * NB + j]) * dT) * iTa;
-    }
     dV[0] = dr * crho + dT * cT - kin * iTa;
-    dV[DIM + 1] = dT * S[G_IT * NB + i] * S[G_IT * NB + j];
+    dV[2] = dT * S[G_IT * NB + i] * S[G_IT * NB + j];
 }
 
-// the face state of eq. HOstable's dissipation: log-mean density and pressure ratio, T, c, the rotation
-// (cos, sin) of the face normal of length L, normal / tangential velocity, and the scalings of R^T T
+// the face state of eq. HOstable's dissipation: log-mean density and pressure ratio, T, c, the sign of the face normal of
+// length L, normal velocity, and the scalings of R^T T
 struct FaceF {
-    float rho, c, cs, sn, L, vn, vt, H, mid, sA, sE, sT, Lam, Hm, Hp;
+    float c, cs, vn, mid, sA, sE, Lam, Hm, Hp;
 };
 
-template <int DIM>
-__device__ __forceinline__ FaceF face_state_f(const float* S, int NB, int l, int step, float nx, float ny, float xtf,
-                                              const GasF& G, DevStatus* st) {
+__device__ __forceinline__ FaceF face_state_f(const float* S, int NB, int l, float nx, float xtf, const GasF& G,
+                                              DevStatus* st) {
     FaceF f;
-    const int r = l + step;
+    const int r = l + 1;
     const float ilr = inv_log_mean_f(S[G_RHO * NB + l], S[G_RHO * NB + r]);
     const float rho = 1.0f / ilr;
     const float ilrp = inv_log_mean_f(S[G_RP * NB + l], S[G_RP * NB + r]);
@@ -196,261 +165,110 @@ __device__ __forceinline__ FaceF face_state_f(const float* S, int NB, int l, int
     if (!(c2 > 0.0f) || !(dcrit > 0.0f) || !(om > 0.0f)) raise_error(st, ES_ERR_INADMISSIBLE, 0);
     const float c = sqrtf(c2);
     const float vm1 = 0.5f * (S[G_V1 * NB + l] + S[G_V1 * NB + r]);
-    float cs = 1.0f, sn = 0.0f, L = 1.0f, vn = vm1, vt = 0.0f;
-    if (DIM == 2) {
-        const float vm2 = 0.5f * (S[G_V2 * NB + l] + S[G_V2 * NB + r]);
-        L = sqrtf(nx * nx + ny * ny);
-        const float iL = 1.0f / L;
-        cs = nx * iL;
-        sn = ny * iL;
-        vn = cs * vm1 + sn * vm2;
-        vt = -sn * vm1 + cs * vm2;
-    } else {
-        L = fabsf(nx);
-        cs = nx > 0.0f ? 1.0f : -1.0f;
-        vn = cs * vm1;
-    }
-    const float E = rho * (G.cv * T - G.a * rho) + 0.5f * rho * (vn * vn + vt * vt);
+    const float L = fabsf(nx);
+    const float cs = nx > 0.0f ? 1.0f : -1.0f;
+    const float vn = cs * vm1;
+    const float E = rho * (G.cv * T - G.a * rho) + 0.5f * rho * (vn * vn);
     const float H = (E + p) * ilr;
-    f.rho = rho;
     f.c = c;
     f.cs = cs;
-    f.sn = sn;
-    f.L = L;
     f.vn = vn;
-    f.vt = vt;
-    f.H = H;
     f.mid = H - c2 * om * G.idelta;
     const float ic2 = 1.0f / c2;
     f.sA = sqrtf(0.5f * rho * T * ic2);
     f.sE = sqrtf(G.R * G.delta * rho * T * T * ic2 / dcrit);
-    f.sT = sqrtf(rho * T);
     f.Lam = fabsf(xtf + L * vn) + L * c;
     f.Hm = H - vn * c;
     f.Hp = H + vn * c;
     return f;
 }
 
-template <int DIM>
-__device__ __forceinline__ void face_dissipation_f(const float* S, int NB, int l, int step, float nx, float ny,
-                                                   float xtf, const GasF& G, const WenoF& Wc, float* out,
-                                                   DevStatus* st, const float* JB, int NJ, int jq) {
-    const FaceF fs = face_state_f<DIM>(S, NB, l, step, nx, ny, xtf, G, st);
-    const float c = fs.c, cs = fs.cs, sn = fs.sn, vn = fs.vn, vt = fs.vt, mid = fs.mid;
-    const float sA = fs.sA, sE = fs.sE, sT = fs.sT, Lam = fs.Lam, Hm = fs.Hm, Hp = fs.Hp;
+__device__ __forceinline__ void face_dissipation_f(const float* S, int NB, int l, float nx, float xtf, const GasF& G,
+                                                   const WenoF& Wc, float* out, DevStatus* st, const float* JB, int NJ,
+                                                   int jq) {
+    const FaceF fs = face_state_f(S, NB, l, nx, xtf, G, st);
+    const float c = fs.c, cs = fs.cs, vn = fs.vn, mid = fs.mid;
+    const float sA = fs.sA, sE = fs.sE, Lam = fs.Lam, Hm = fs.Hm, Hp = fs.Hp;
 
     // W_j - W_l = R^T T (V_j - V_l) at nodes l-2 .. l+3 (zero at l itself); V_j - V_l is the sum
     // of the neighbour jumps between them (JB[c][jq + q] = V_{q+1} - V_q along the line, the
     // face's left node at jq + 0)
-    float W[6][DIM + 2];
-    float aTV[DIM + 2];
-    float cum[DIM + 2];
+    float W[6][3];
+    float aTV[3];
+    float cum[3];
 #pragma unroll
-    for (int m = 0; m < DIM + 2; ++m) {
+    for (int m = 0; m < 3; ++m) {
         W[2][m] = 0.0f;
         cum[m] = 0.0f;
     }
 #pragma unroll
     for (int o = 3; o < 6; ++o)
 #pragma unroll
-        for (int m = 0; m < DIM + 2; ++m) {
+        for (int m = 0; m < 3; ++m) {
             cum[m] += JB[m * NJ + jq + (o - 3)];
             W[o][m] = cum[m];
         }
 #pragma unroll
-    for (int m = 0; m < DIM + 2; ++m) cum[m] = 0.0f;
+    for (int m = 0; m < 3; ++m) cum[m] = 0.0f;
 #pragma unroll
     for (int o = 1; o >= 0; --o)
 #pragma unroll
-        for (int m = 0; m < DIM + 2; ++m) {
+        for (int m = 0; m < 3; ++m) {
             cum[m] -= JB[m * NJ + jq + (o - 2)];
             W[o][m] = cum[m];
         }
 #pragma unroll
     for (int o = 0; o < 6; ++o) {
         if (o == 2) continue;
-        float dV[DIM + 2];
+        float dV[3];
 #pragma unroll
-        for (int m = 0; m < DIM + 2; ++m) dV[m] = W[o][m];
-        if (DIM == 1) {
-            const float V0 = dV[0], V1 = cs * dV[1], V2 = dV[2];
-            W[o][0] = sA * (V0 + (vn - c) * V1 + Hm * V2);
-            W[o][1] = sE * (V0 + vn * V1 + mid * V2);
-            W[o][2] = sA * (V0 + (vn + c) * V1 + Hp * V2);
-            if (o == 3) {
-                aTV[0] = fabsf(V0);
-                aTV[1] = fabsf(V1);
-                aTV[2] = fabsf(V2);
-            }
-        } else {
-            const float V0 = dV[0];
-            const float V1 = cs * dV[1] + sn * dV[2], V2 = -sn * dV[1] + cs * dV[2], V3 = dV[3];
-            const float base = V0 + vt * V2;
-            W[o][0] = sA * (base + (vn - c) * V1 + Hm * V3);
-            W[o][1] = sE * (base + vn * V1 + mid * V3);
-            W[o][2] = sT * (V2 + vt * V3);
-            W[o][3] = sA * (base + (vn + c) * V1 + Hp * V3);
-            if (o == 3) {
-                aTV[0] = fabsf(V0);
-                aTV[1] = fabsf(V1);
-                aTV[2] = fabsf(V2);
-                aTV[3] = fabsf(V3);
-            }
-        }
-    }
-    float scl[DIM + 2];
-    if (DIM == 1) {
-        scl[0] = sA * (aTV[0] + fabsf(vn - c) * aTV[1] + fabsf(Hm) * aTV[2]);
-        scl[1] = sE * (aTV[0] + fabsf(vn) * aTV[1] + fabsf(mid) * aTV[2]);
-        scl[2] = sA * (aTV[0] + fabsf(vn + c) * aTV[1] + fabsf(Hp) * aTV[2]);
-    } else {
-        const float avt = fabsf(vt);
-        scl[0] = sA * (aTV[0] + fabsf(vn - c) * aTV[1] + avt * aTV[2] + fabsf(Hm) * aTV[3]);
-        scl[1] = sE * (aTV[0] + fabsf(vn) * aTV[1] + avt * aTV[2] + fabsf(mid) * aTV[3]);
-        scl[2] = sT * (aTV[2] + (avt + c) * aTV[3]);     // velocity round-off scales with |v_t| + c
-        scl[3] = sA * (aTV[0] + fabsf(vn + c) * aTV[1] + avt * aTV[2] + fabsf(Hp) * aTV[3]);
-    }
-    float y[DIM + 2];
-#pragma unroll
-    for (int m = 0; m < DIM + 2; ++m) {
-        // a wave whose plain jump is within round-off of zero adds nothing whatever its reconstruction (the shear waves of
-        // a uniform flow, every wave of a constant state); in 1D, where the batched form's results are compared bit for
-        // bit over many steps, the reconstruction stays in line (the branch changes which products the compiler fuses)
-        float j = W[3][m];
-        if (fabsf(j) <= Wc.sign_tol * scl[m]) j = 0.0f;
-        y[m] = 0.0f;
-        if (DIM == 1 || j != 0.0f) {
-            const float wmin = mr_weno5_f(W[0][m], W[1][m], W[2][m], W[3][m], W[4][m], Wc);
-            const float wplu = mr_weno5_f(W[5][m], W[4][m], W[3][m], W[2][m], W[1][m], Wc);
-            const float jw = wplu - wmin;
-            const bool keep = (jw > 0.0f && j > 0.0f) || (jw < 0.0f && j < 0.0f);
-            y[m] = keep ? jw : 0.0f;
-        }
-    }
-    const float h = -0.5f * Lam;
-    if (DIM == 1) {
-        const float y0 = sA * y[0], y1 = sE * y[1], y2 = sA * y[2];
-        out[0] = h * (y0 + y1 + y2);
-        out[1] = h * cs * ((vn - c) * y0 + vn * y1 + (vn + c) * y2);
-        out[2] = h * (Hm * y0 + mid * y1 + Hp * y2);
-    } else {
-        const float y0 = sA * y[0], y1 = sE * y[1], y2 = sT * y[2], y3 = sA * y[3];
-        const float i0 = y0 + y1 + y3;
-        const float i1 = (vn - c) * y0 + vn * y1 + (vn + c) * y3;
-        const float i2 = vt * i0 + y2;
-        const float i3 = Hm * y0 + mid * y1 + vt * y2 + Hp * y3;
-        out[0] = h * i0;
-        out[1] = h * (cs * i1 - sn * i2);
-        out[2] = h * (sn * i1 + cs * i2);
-        out[3] = h * i3;
-    }
-}
-
-// face_dissipation_f in 2D shared by the two lanes (2 p, 2 p + 1) of a warp: both form the face state, lane
-// half = 0 the characteristic components 0 and 1 (the acoustic wave u - c and the entropy wave), half = 1
-// components 2 and 3 (the shear wave and u + c), each its own reconstructions and sign switch, and the two
-// exchange their y values; every lane of the warp must call it (a lane without a face passes a valid one and
-// drops the result).  The same arithmetic per component as face_dissipation_f; twice the lanes per face.
-__device__ __forceinline__ void face_dissipation_split_f(const float* S, int NB, int l, int step, float nx, float ny,
-                                                         float xtf, const GasF& G, const WenoF& Wc, float* out,
-                                                         DevStatus* st, const float* JB, int NJ, int jq, int half) {
-    const FaceF fs = face_state_f<2>(S, NB, l, step, nx, ny, xtf, G, st);
-    const float c = fs.c, cs = fs.cs, sn = fs.sn, vn = fs.vn, vt = fs.vt, mid = fs.mid;
-    const float sA = fs.sA, sE = fs.sE, sT = fs.sT, Lam = fs.Lam, Hm = fs.Hm, Hp = fs.Hp;
-    const bool h0 = half == 0;
-    // rows of R^T T for this lane's components: a = 0 or 2, b = 1 or 3; component 2 is sT (V2 + vt V3), the
-    // others s (base + B V1 + D V3)
-    const float s_a = h0 ? sA : sT, B_a = h0 ? vn - c : 0.0f, D_a = h0 ? Hm : vt;
-    const float s_b = h0 ? sE : sA, B_b = h0 ? vn : vn + c, D_b = h0 ? mid : Hp;
-    float Wa[6], Wb[6];
-    float aTV[4];
-    Wa[2] = 0.0f;
-    Wb[2] = 0.0f;
-    float cum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    float Vn[6][4];
-#pragma unroll
-    for (int o = 3; o < 6; ++o)
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            cum[m] += JB[m * NJ + jq + (o - 3)];
-            Vn[o][m] = cum[m];
-        }
-#pragma unroll
-    for (int m = 0; m < 4; ++m) cum[m] = 0.0f;
-#pragma unroll
-    for (int o = 1; o >= 0; --o)
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            cum[m] -= JB[m * NJ + jq + (o - 2)];
-            Vn[o][m] = cum[m];
-        }
-#pragma unroll
-    for (int o = 0; o < 6; ++o) {
-        if (o == 2) continue;
-        const float V0 = Vn[o][0];
-        const float V1 = cs * Vn[o][1] + sn * Vn[o][2], V2 = -sn * Vn[o][1] + cs * Vn[o][2], V3 = Vn[o][3];
-        const float base = V0 + vt * V2;
-        Wa[o] = s_a * ((h0 ? base : V2) + B_a * V1 + D_a * V3);
-        Wb[o] = s_b * (base + B_b * V1 + D_b * V3);
+        for (int m = 0; m < 3; ++m) dV[m] = W[o][m];
+        const float V0 = dV[0], V1 = cs * dV[1], V2 = dV[2];
+        W[o][0] = sA * (V0 + (vn - c) * V1 + Hm * V2);
+        W[o][1] = sE * (V0 + vn * V1 + mid * V2);
+        W[o][2] = sA * (V0 + (vn + c) * V1 + Hp * V2);
         if (o == 3) {
             aTV[0] = fabsf(V0);
             aTV[1] = fabsf(V1);
             aTV[2] = fabsf(V2);
-            aTV[3] = fabsf(V3);
         }
     }
-    const float avt = fabsf(vt);
-    const float scl_a = h0 ? sA * (aTV[0] + fabsf(vn - c) * aTV[1] + avt * aTV[2] + fabsf(Hm) * aTV[3])
-                           : sT * (aTV[2] + (avt + c) * aTV[3]);
-    const float scl_b = s_b * (aTV[0] + fabsf(B_b) * aTV[1] + avt * aTV[2] + fabsf(D_b) * aTV[3]);
-    float ya = 0.0f, yb = 0.0f;
-    if (!(fabsf(Wa[3]) <= Wc.sign_tol * scl_a)) {
-        const float wmin = mr_weno5_f(Wa[0], Wa[1], Wa[2], Wa[3], Wa[4], Wc);
-        const float wplu = mr_weno5_f(Wa[5], Wa[4], Wa[3], Wa[2], Wa[1], Wc);
-        const float jw = wplu - wmin, j = Wa[3];
+    float scl[3];
+    scl[0] = sA * (aTV[0] + fabsf(vn - c) * aTV[1] + fabsf(Hm) * aTV[2]);
+    scl[1] = sE * (aTV[0] + fabsf(vn) * aTV[1] + fabsf(mid) * aTV[2]);
+    scl[2] = sA * (aTV[0] + fabsf(vn + c) * aTV[1] + fabsf(Hp) * aTV[2]);
+    float y[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        // (no test for a zero wave here: its branch would change which products the compiler fuses, and the batched form's
+        // results over many steps with it)
+        float j = W[3][m];
+        if (fabsf(j) <= Wc.sign_tol * scl[m]) j = 0.0f;
+        const float wmin = mr_weno5_f(W[0][m], W[1][m], W[2][m], W[3][m], W[4][m], Wc);
+        const float wplu = mr_weno5_f(W[5][m], W[4][m], W[3][m], W[2][m], W[1][m], Wc);
+        const float jw = wplu - wmin;
         const bool keep = (jw > 0.0f && j > 0.0f) || (jw < 0.0f && j < 0.0f);
-        ya = keep ? jw : 0.0f;
+        y[m] = keep ? jw : 0.0f;
     }
-    if (!(fabsf(Wb[3]) <= Wc.sign_tol * scl_b)) {
-        const float wmin = mr_weno5_f(Wb[0], Wb[1], Wb[2], Wb[3], Wb[4], Wc);
-        const float wplu = mr_weno5_f(Wb[5], Wb[4], Wb[3], Wb[2], Wb[1], Wc);
-        const float jw = wplu - wmin, j = Wb[3];
-        const bool keep = (jw > 0.0f && j > 0.0f) || (jw < 0.0f && j < 0.0f);
-        yb = keep ? jw : 0.0f;
-    }
-    const float oa = __shfl_xor_sync(0xffffffffu, ya, 1);
-    const float ob = __shfl_xor_sync(0xffffffffu, yb, 1);
-    const float y[4] = {h0 ? ya : oa, h0 ? yb : ob, h0 ? oa : ya, h0 ? ob : yb};
     const float h = -0.5f * Lam;
-    const float y0 = sA * y[0], y1 = sE * y[1], y2 = sT * y[2], y3 = sA * y[3];
-    const float i0 = y0 + y1 + y3;
-    const float i1 = (vn - c) * y0 + vn * y1 + (vn + c) * y3;
-    const float i2 = vt * i0 + y2;
-    const float i3 = Hm * y0 + mid * y1 + vt * y2 + Hp * y3;
-    out[0] = h * i0;
-    out[1] = h * (cs * i1 - sn * i2);
-    out[2] = h * (sn * i1 + cs * i2);
-    out[3] = h * i3;
+    const float y0 = sA * y[0], y1 = sE * y[1], y2 = sA * y[2];
+    out[0] = h * (y0 + y1 + y2);
+    out[1] = h * cs * ((vn - c) * y0 + vn * y1 + (vn + c) * y2);
+    out[2] = h * (Hm * y0 + mid * y1 + Hp * y2);
 }
 
-template <int DIM>
-__device__ __forceinline__ void load_node_f(float* S, int NB, int b, const StageParams& P, const GasF& G, int gi,
-                                            int gj) {
-    const int si = state_index(gi, P.n1, P.bc[0]);
-    const int sj = DIM == 2 ? state_index(gj, P.n2, P.bc[1]) : 0;
-    const int idx = sj * P.n1 + si;
+__device__ __forceinline__ void load_node_f(float* S, int NB, int b, const StageParams& P, const GasF& G, int gi) {
+    const int idx = state_index(gi, P.n1, P.bc[0]);
     const size_t N = P.fcs;                                 // component stride
     const size_t LO = P.fps;                                // offset of the lo plane of JU
     // primitive state in double-float arithmetic
     const df iJ = df_recip({P.fJs[idx], P.fJs[P.fpsJ + idx]});
     const df rho = df_mul({P.fJUs[idx], P.fJUs[LO + idx]}, iJ);
     const df m1 = df_mul({P.fJUs[N + idx], P.fJUs[LO + N + idx]}, iJ);
-    const df m2 = DIM == 2 ? df_mul({P.fJUs[2 * N + idx], P.fJUs[LO + 2 * N + idx]}, iJ) : df{0.0f, 0.0f};
-    const df E = df_mul({P.fJUs[(DIM + 1) * N + idx], P.fJUs[LO + (DIM + 1) * N + idx]}, iJ);
+    const df E = df_mul({P.fJUs[2 * N + idx], P.fJUs[LO + 2 * N + idx]}, iJ);
     const df irho = df_recip(rho);
     const df v1 = df_mul(m1, irho);
-    const df v2 = DIM == 2 ? df_mul(m2, irho) : df{0.0f, 0.0f};
-    const df ke = df_mul_f(df_add(df_mul(v1, v1), df_mul(v2, v2)), 0.5f);
+    const df ke = df_mul_f(df_mul(v1, v1), 0.5f);
     // T = (E/rho - |v|^2/2 + a rho) / cv
     const df e = df_add(df_mul(E, irho), {-ke.hi, -ke.lo});
     const df Td = df_mul_f(df_add(e, df_mul_f(rho, G.a)), G.icv);
@@ -465,8 +283,6 @@ __device__ __forceinline__ void load_node_f(float* S, int NB, int b, const Stage
     S[G_RHOL * NB + b] = rho.lo;
     S[G_V1 * NB + b] = v1.hi;
     S[G_V1L * NB + b] = v1.lo;
-    S[G_V2 * NB + b] = v2.hi;
-    S[G_V2L * NB + b] = v2.lo;
     S[G_T * NB + b] = T;
     S[G_TL * NB + b] = Td.lo;
     S[G_IT * NB + b] = iT;
@@ -475,10 +291,8 @@ __device__ __forceinline__ void load_node_f(float* S, int NB, int b, const Stage
     S[G_G * NB + b] = G.R * iom - G.a * r * iT;
     S[G_RT * NB + b] = r * iT;
     S[G_VT1 * NB + b] = v1.hi * iT;
-    S[G_VT2 * NB + b] = v2.hi * iT;
     S[G_V2T * NB + b] = 2.0f * ke.hi * iT;
     S[G_RV1 * NB + b] = m1.hi;
-    S[G_RV2 * NB + b] = m2.hi;
     S[G_RP * NB + b] = r / p;
 }
 
@@ -521,208 +335,114 @@ __device__ __forceinline__ void stage_disp(const StageParams& P, int gi, int gj,
 }
 
 
-// One tile of the fused operator + RK stage (mixed form): the box of the tile at
-// (i0, j0) is staged in shared memory S / PB / FB (TileF layout), then pair
-// fluxes, face fluxes, divergence and the RK combination follow.  Called by the
-// tiled kernel (one tile per CTA) and by the batched kernel (a loop over the
-// chunks of one problem per CTA).
-// SPLIT (2D): two lanes per face in the face phase (face_dissipation_split_f), for tiles with twice the threads
-template <int DIM, int BX, int BY, int NT, bool SPLIT = false>
-__device__ __forceinline__ void stage_tile_mixed(float* smemf, const StageParams& P, int i0, int j0, float dt,
-                                                 const GasF& G, const WenoF& Wc) {
-    static_assert(!SPLIT || DIM == 2, "the split face phase is written for 2D");
-    using TL = TileF<DIM, BX, BY, NT>;
-    constexpr int GX = TL::GX, NB = TL::NB, NC = TL::NC;
+// One tile of the fused operator + RK stage in 1D (mixed form): the tile at i0 is staged with its halo in shared memory
+// S / PB / FB / JB (TileF layout), then pair fluxes, face fluxes, divergence and the RK combination follow.  Called by the
+// tiled kernel (one tile per CTA) and by the batched kernel (a loop over the chunks of one problem per CTA).
+template <int BX, int NT>
+__device__ __forceinline__ void stage_tile_mixed(float* smemf, const StageParams& P, int i0, float dt, const GasF& G,
+                                                 const WenoF& Wc) {
+    using TL = TileF<BX, NT>;
+    constexpr int NB = TL::NB, NC = TL::NC;
     float* S = smemf;
     float* PB = smemf + G_COUNT * NB;
     float* FB = PB + TL::PAIR_FLOATS;
     float* JB = FB + TL::NF * (NC + 1);
     const int tid = threadIdx.x;
     const float cdt = P.fcst * dt;
-    const float idx1 = P.finv_dxi[0], idx2 = P.finv_dxi[1];
-    float* XS = PB;
-    float* XD = PB + 2 * NB;
     for (int b = tid; b < NB; b += NT) {
-        const int ii = b % GX, jj = b / GX;
-        const int gi = i0 - 3 + ii, gj = j0 - 3 + jj;
+        const int gi = i0 - 3 + b;
         float ds[2], xd[2];
-        stage_disp<DIM>(P, gi, DIM == 2 ? gj : 0, cdt, ds, xd);
-        XS[b] = ds[0];
-        XD[b] = xd[0];
-        if (DIM == 2) {
-            XS[NB + b] = ds[1];
-            XD[NB + b] = xd[1];
-        }
-        const bool in_x = ii >= 3 && ii < 3 + BX;
-        const bool in_y = DIM == 1 || (jj >= 3 && jj < 3 + BY);
-        if (in_x || in_y) load_node_f<DIM>(S, NB, b, P, G, gi, gj);
-    }
-    __syncthreads();
-    for (int b = tid; b < NB; b += NT) {
-        const int ii = b % GX, jj = b / GX;
-        if (DIM == 1) {
-            S[G_N1X * NB + b] = 1.0f;
-            S[G_N1Y * NB + b] = 0.0f;
-            S[G_XT1 * NB + b] = -XD[b];
-        } else {
-            if (jj >= 3 && jj < 3 + BY) {        // J dxi_1/dx = (1 + d2[d_y]/dxi_2, -d2[d_x]/dxi_2)
-                float dy = 0.0f, dx = 0.0f;
-#pragma unroll
-                for (int m = 1; m <= 3; ++m) {
-                    const float h = 0.5f * float(ec_alpha(m));
-                    dx += h * (XS[b + m * GX] - XS[b - m * GX]);
-                    dy += h * (XS[NB + b + m * GX] - XS[NB + b - m * GX]);
-                }
-                const float nx = 1.0f + dy * idx2, ny = -dx * idx2;
-                S[G_N1X * NB + b] = nx;
-                S[G_N1Y * NB + b] = ny;
-                S[G_XT1 * NB + b] = -(XD[b] * nx + XD[NB + b] * ny);
-            }
-            if (ii >= 3 && ii < 3 + BX) {        // J dxi_2/dx = (-d1[d_y]/dxi_1, 1 + d1[d_x]/dxi_1)
-                float dy = 0.0f, dx = 0.0f;
-#pragma unroll
-                for (int m = 1; m <= 3; ++m) {
-                    const float h = 0.5f * float(ec_alpha(m));
-                    dx += h * (XS[b + m] - XS[b - m]);
-                    dy += h * (XS[NB + b + m] - XS[NB + b - m]);
-                }
-                const float nx = -dy * idx1, ny = 1.0f + dx * idx1;
-                S[G_N2X * NB + b] = nx;
-                S[G_N2Y * NB + b] = ny;
-                S[G_XT2 * NB + b] = -(XD[b] * nx + XD[NB + b] * ny);
-            }
-        }
+        stage_disp<1>(P, gi, 0, cdt, ds, xd);
+        load_node_f(S, NB, b, P, G, gi);
+        S[G_N1X * NB + b] = 1.0f;
+        S[G_XT1 * NB + b] = -xd[0];
     }
     __syncthreads();
 
+    for (int t = tid; t < TL::NP; t += NT) {
+        int m, q;
+        if (t < BX + 1) { m = 1; q = 2 + t; }
+        else if (t < 2 * BX + 3) { m = 2; q = 1 + (t - BX - 1); }
+        else { m = 3; q = t - 2 * BX - 3; }
+        const int l = q, r = l + m;
+        const float nx = 0.5f * (S[G_N1X * NB + l] + S[G_N1X * NB + r]);
+        const float xt = 0.5f * (S[G_XT1 * NB + l] + S[G_XT1 * NB + r]);
+        float f[NC];
+        pair_flux_f(S, NB, l, r, nx, xt, G, f);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) PB[c * TL::NP + t] = f[c];
+    }
+    if (P.diss) {
+        // neighbour jumps V_{q+1} - V_q, q = 0 .. BX+4 (eq. jumpV); in a tile whose pairs leave enough threads, on the
+        // warps after the pairs'
+        constexpr int JOFF = (TL::NP + 31) / 32 * 32 + TL::NJ <= NT ? (TL::NP + 31) / 32 * 32 : 0;
+        for (int t = JOFF ? (tid + NT - JOFF) % NT : tid; t < TL::NJ; t += NT) {
+            float dV[NC];
+            entropy_jump(S, NB, t, t + 1, G, dV);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) JB[c * TL::NJ + t] = dV[c];
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < TL::NF; t += NT) {
+        const int q = 2 + t;
+        float F[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) F[c] = 0.0f;
+        float FJ = 0.0f;
+#pragma unroll
+        for (int m = 1; m <= 3; ++m) {
+            const int off = m == 1 ? 0 : (m == 2 ? BX + 1 : 2 * BX + 3);
+            const float al = float(ec_alpha(m));
+            for (int s = 0; s < m; ++s) {
+                const int qq = q - s;
+                const int pi = off + (qq - (3 - m));
+#pragma unroll
+                for (int c = 0; c < NC; ++c) F[c] += al * PB[c * TL::NP + pi];
+                FJ += al * 0.5f * (S[G_XT1 * NB + qq] + S[G_XT1 * NB + qq + m]);
+            }
+        }
+        bool jump = P.diss;
+        if (P.diss) {
+            // between two nodes of equal state no wave has a jump and the dissipation is zero whatever the rest of
+            // the stencil (eq. sign switch): most faces of a tube whose waves have not reached its ends.  The face
+            // state's own check is then the node's.
+            const float* jl = JB + q;
+            jump = jl[0] != 0.0f || jl[TL::NJ] != 0.0f || jl[2 * TL::NJ] != 0.0f;
+            if (!jump) {
+                const float RT = G.R * S[G_T * NB + q], ar = 2.0f * G.a * S[G_RHO * NB + q];
+                const float om = S[G_OM * NB + q], iom = S[G_IOM * NB + q];
+                if (!((1.0f + G.delta) * RT * iom * iom > ar) || !(RT > ar * om * om))
+                    raise_error(P.status, ES_ERR_INADMISSIBLE, 0);
+            }
+        }
+        if (jump) {
+            const float nx = 0.5f * (S[G_N1X * NB + q] + S[G_N1X * NB + q + 1]);
+            const float xtf = 0.5f * (S[G_XT1 * NB + q] + S[G_XT1 * NB + q + 1]);
+            float d[NC];
+            face_dissipation_f(S, NB, q, nx, xtf, G, Wc, d, P.status, JB, TL::NJ, q);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) F[c] += d[c];
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) FB[c * TL::NF + t] = F[c];
+        FB[NC * TL::NF + t] = FJ;
+    }
+    __syncthreads();
     float acc[NC + 1];
 #pragma unroll
     for (int c = 0; c <= NC; ++c) acc[c] = 0.0f;
-    const int tx = tid % BX, ty = tid / BX;
-
-    // one copy of the direction pipeline for both directions (unrolled, the kernel's code was twice the size
-    // and its warps stalled on instruction fetch); the line lengths and strides are then run-time values
-#pragma unroll 1
-    for (int k = 0; k < DIM; ++k) {
-        const int nlines = k == 0 ? (DIM == 2 ? BY : 1) : BX;
-        const int LB = k == 0 ? BX : BY;
-        const int per_line = 3 * LB + 6;
-        const int step = k == 0 ? 1 : GX;
-        const int fN = k == 0 ? G_N1X : G_N2X;
-        const int fNy = k == 0 ? G_N1Y : G_N2Y;
-        const int fXT = k == 0 ? G_XT1 : G_XT2;
-        for (int t = tid; t < nlines * per_line; t += NT) {
-            const int line = t / per_line, kk = t % per_line;
-            int m, q;
-            if (kk < LB + 1) { m = 1; q = 2 + kk; }
-            else if (kk < 2 * LB + 3) { m = 2; q = 1 + (kk - LB - 1); }
-            else { m = 3; q = kk - 2 * LB - 3; }
-            const int base = k == 0 ? (DIM == 2 ? (3 + line) * GX : 0) : 3 + line;
-            const int l = base + q * step, r = l + m * step;
-            const float nx = 0.5f * (S[fN * NB + l] + S[fN * NB + r]);
-            const float ny = 0.5f * (S[fNy * NB + l] + S[fNy * NB + r]);
-            const float xt = 0.5f * (S[fXT * NB + l] + S[fXT * NB + r]);
-            float f[NC];
-            pair_flux_f<DIM>(S, NB, l, r, nx, ny, xt, G, f);
+    if (tid < BX) {
+        const float inv = P.finv_dxi[0];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) PB[c * TL::NP + t] = f[c];
-        }
-        if (P.diss) {
-            // neighbour jumps V_{q+1} - V_q, q = 0 .. LB+4 along each line (eq. jumpV)
-            // (in a 1D tile whose pairs leave enough threads, the warps after the pairs')
-            constexpr int JOFF = DIM == 1 && (TL::NP + 31) / 32 * 32 + TL::NJ <= NT ? (TL::NP + 31) / 32 * 32 : 0;
-            for (int t = JOFF ? (tid + NT - JOFF) % NT : tid; t < nlines * (LB + 5); t += NT) {
-                const int line = t / (LB + 5), q = t % (LB + 5);
-                const int base = k == 0 ? (DIM == 2 ? (3 + line) * GX : 0) : 3 + line;
-                const int l = base + q * step;
-                float dV[NC];
-                entropy_jump<DIM>(S, NB, l, l + step, G, dV);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) JB[c * TL::NJ + t] = dV[c];
-            }
-        }
-        __syncthreads();
-        const int nfaces = nlines * (LB + 1);
-        const int lane = tid & 31;
-        // SPLIT: lanes (2 p, 2 p + 1) share face p; the trip count is uniform per warp (the halves exchange
-        // values), and a lane past the last face works on the last face and stores nothing
-        for (int ub = SPLIT ? tid - lane : tid; ub < (SPLIT ? 2 * nfaces : nfaces); ub += NT) {
-            const int u = SPLIT ? ub + lane : ub;
-            const bool active = !SPLIT || u < 2 * nfaces;
-            const int t = SPLIT ? (active ? (u >> 1) : nfaces - 1) : u;
-            const int half = SPLIT ? (u & 1) : 0;
-            const int line = t / (LB + 1), f = t % (LB + 1);
-            const int q = 2 + f;
-            const int pbase = line * per_line;
-            float F[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) F[c] = 0.0f;
-            float FJ = 0.0f;
-            const int base = k == 0 ? (DIM == 2 ? (3 + line) * GX : 0) : 3 + line;
-#pragma unroll
-            for (int m = 1; m <= 3; ++m) {
-                const int off = m == 1 ? 0 : (m == 2 ? LB + 1 : 2 * LB + 3);
-                const float al = float(ec_alpha(m));
-                for (int s = 0; s < m; ++s) {
-                    const int qq = q - s;
-                    const int pi = pbase + off + (qq - (3 - m));
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) F[c] += al * PB[c * TL::NP + pi];
-                    FJ += al * 0.5f * (S[fXT * NB + base + qq * step] + S[fXT * NB + base + (qq + m) * step]);
-                }
-            }
-            bool jump = P.diss;
-            if (DIM == 1 && P.diss) {
-                // between two nodes of equal state no wave has a jump and the dissipation is zero whatever the rest of
-                // the stencil (eq. sign switch): most faces of a tube whose waves have not reached its ends.  The face
-                // state's own check is then the node's.
-                const float* jl = JB + q;
-                jump = jl[0] != 0.0f || jl[TL::NJ] != 0.0f || jl[2 * TL::NJ] != 0.0f;
-                if (!jump) {
-                    const int l = base + q;
-                    const float RT = G.R * S[G_T * NB + l], ar = 2.0f * G.a * S[G_RHO * NB + l];
-                    const float om = S[G_OM * NB + l], iom = S[G_IOM * NB + l];
-                    if (!((1.0f + G.delta) * RT * iom * iom > ar) || !(RT > ar * om * om))
-                        raise_error(P.status, ES_ERR_INADMISSIBLE, 0);
-                }
-            }
-            if (jump) {
-                const int l = base + q * step;
-                const float nx = 0.5f * (S[fN * NB + l] + S[fN * NB + l + step]);
-                const float ny = 0.5f * (S[fNy * NB + l] + S[fNy * NB + l + step]);
-                const float xtf = 0.5f * (S[fXT * NB + l] + S[fXT * NB + l + step]);
-                float d[NC];
-                if constexpr (SPLIT)
-                    face_dissipation_split_f(S, NB, l, step, nx, ny, xtf, G, Wc, d, P.status, JB, TL::NJ,
-                                             line * (LB + 5) + q, half);
-                else
-                    face_dissipation_f<DIM>(S, NB, l, step, nx, ny, xtf, G, Wc, d, P.status, JB, TL::NJ,
-                                            line * (LB + 5) + q);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) F[c] += d[c];
-            }
-            if (active && half == 0) {
-#pragma unroll
-                for (int c = 0; c < NC; ++c) FB[c * TL::NF + t] = F[c];
-                FB[NC * TL::NF + t] = FJ;
-            }
-        }
-        __syncthreads();
-        if (tid < BX * (DIM == 2 ? BY : 1)) {
-            const int line = k == 0 ? ty : tx;
-            const int pos = k == 0 ? tx : ty;
-            const int fm = line * (LB + 1) + pos;
-            const float inv = k == 0 ? idx1 : idx2;
-#pragma unroll
-            for (int c = 0; c <= NC; ++c) acc[c] -= (FB[c * TL::NF + fm + 1] - FB[c * TL::NF + fm]) * inv;
-        }
-        __syncthreads();
+        for (int c = 0; c <= NC; ++c) acc[c] -= (FB[c * TL::NF + tid + 1] - FB[c * TL::NF + tid]) * inv;
     }
+    __syncthreads();
 
-    const int gi = i0 + tx, gj = j0 + ty;
-    if (tid < BX * (DIM == 2 ? BY : 1) && gi < P.n1 && (DIM == 1 || gj < P.n2)) {
+    const int gi = i0 + tid;
+    if (tid < BX && gi < P.n1) {
         const size_t N = P.fcs;
-        const size_t idx = size_t(DIM == 2 ? gj : 0) * P.n1 + gi;
+        const size_t idx = size_t(gi);
         const size_t LO = P.fps;
         if (P.mode == 1) {
 #pragma unroll

@@ -14,8 +14,9 @@
 //     and an FP32 mesh velocity, converted from the FP64 mesh once per step, so
 //     the metric differences delta_k[x] = dxi_k e_k + delta_k[d] lose no digits;
 //   * logarithmic means are taken per pair from the relative jump
-//     f = (a_l - a_r)/(a_l + a_r) (series for |f| < 0.05, log1p otherwise), which
-//     is accurate to FP32 rounding of the result even for nearly equal states;
+//     f = (a_l - a_r)/(a_l + a_r) (a series for |f| < 0.2 in 2D and 3D, es_flux32.cuh,
+//     and 0.05 in 1D, the logarithm otherwise), which is accurate to FP32 rounding of
+//     the result even for nearly equal states;
 //   * the entropy variables never appear as absolute values (V_1 is O(c_v) =
 //     O(200) and its jumps are O(h)): the dissipation works on the jumps
 //     V_j - V_i written exactly as the jump decomposition of Sec. 3.1
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(NT, 2) stage_kernel_mixed1(StageParams P) {
     extern __shared__ float smemf[];
     const double dtd = P.dt_dev ? *P.dt_dev : P.dt_host;
     if (P.mode == 0 && dtd == 0.0) return;
-    stage_tile_mixed<1, BX, 1, NT>(smemf, P, blockIdx.x * BX, 0, float(dtd), gas_f(P), weno_f(P));
+    stage_tile_mixed<BX, NT>(smemf, P, blockIdx.x * BX, float(dtd), gas_f(P), weno_f(P));
 }
 
 template <int BX, int BY, int NT, bool SPLIT = false>
@@ -419,8 +420,8 @@ cudaError_t launch_tile_f(const StageParams& P, cudaStream_t s) {
 // take three rounds of pairs and two of jumps with 254 nodes.  Stages of 40 to 17632 nodes, launch to launch: 8.3 -> 6.3 us,
 // the same bits; a second wave would bring the short tile to 8.3, where the other stays up to 30000 nodes.
 constexpr int LINE_BX = 254, SHORT_BX = 58, LINE_NT = 256;
-using LineTile = TileF<1, LINE_BX, 1, LINE_NT>;
-using ShortTile = TileF<1, SHORT_BX, 1, LINE_NT>;
+using LineTile = TileF<LINE_BX, LINE_NT>;
+using ShortTile = TileF<SHORT_BX, LINE_NT>;
 constexpr int SHORT_MAX = SHORT_BX * 2 * 152;
 
 }  // namespace
