@@ -485,8 +485,7 @@ int enqueue_step(es_ctx* c, void* JU, void* J, double* x, bool first = true, boo
             count(c);
         }
         if (!c->p.moving) {         // on a moving mesh the monitor kernel takes eq. cfl (with_dt = 2 below)
-            k_cfl_f<<<G, B, 0, s>>>(c->g, gas_f32(c->gas), (const float*)JU, (const float*)J, c->fdisp, nullptr,
-                                    RED_CFL, c->dev);
+            launch_cfl_f(c->g, gas_f32(c->gas), (const float*)JU, (const float*)J, c->fdisp, nullptr, RED_CFL, c->dev, G, B, s);
             count(c);
         }
     } else {
@@ -884,8 +883,8 @@ int es_cfl_dt(es_ctx* c, const void* JU, const void* J, const double* x, const d
         count(c, n);
     } else if (mesh_on_fp32(c)) {
         k_mesh_f32<<<c->grid1d, c->block1d, 0, c->stream>>>(c->g, x, xdot, c->fdisp, c->fxd);
-        k_cfl_f<<<c->grid1d, c->block1d, 0, c->stream>>>(c->g, gas_f32(c->gas), (const float*)JU, (const float*)J,
-                                                   c->fdisp, xdot ? c->fxd : nullptr, slot, c->dev);
+        launch_cfl_f(c->g, gas_f32(c->gas), (const float*)JU, (const float*)J, c->fdisp, xdot ? c->fxd : nullptr, slot, c->dev,
+                     c->grid1d, c->block1d, c->stream);
         count(c, 2);
     } else {
         enqueue_cfl(c, JU, J, x, xdot, slot);

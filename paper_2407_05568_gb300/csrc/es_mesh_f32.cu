@@ -257,10 +257,12 @@ __device__ __forceinline__ float cfl_node_f(const GridParams& g, const GasF32& G
 }  // namespace
 
 // eq. cfl on the FP32 pipe: the maximum over the nodes of cfl_node_f goes to d->red[slot]; vel = nullptr
-// is a mesh at rest.  Bound by the latency of a node's 34 loads: five blocks per SM (48 registers; with 94 there were
-// 2.6 and a quarter of the issue slots busy).  1024 x 1024: 38 -> 31 us.
-__global__ void __launch_bounds__(256, 5) k_cfl_f(GridParams g, GasF32 G, const float* JU, const float* J, const float* disp, const float* vel,
-                        int slot, DevScalars* d) {
+// is a mesh at rest.  Bound by the latency of a node's 34 loads.  Two register limits: meshes whose blocks are at most 256
+// threads (among them all of more than 512 nodes per SM) take five blocks per SM (48 registers; with 94 there were 2.6 and a
+// quarter of the issue slots busy: 38 -> 31 us at 1024 x 1024); between, a block of up to 512 threads has an SM to itself.
+template <int NT, int NB>
+__global__ void __launch_bounds__(NT, NB) k_cfl_f(GridParams g, GasF32 G, const float* JU, const float* J,
+                                                  const float* disp, const float* vel, int slot, DevScalars* d) {
     const int N = g.n1 * g.n2;
     float m = 0.0f;
     for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < N; id += gridDim.x * blockDim.x) {
@@ -270,6 +272,12 @@ __global__ void __launch_bounds__(256, 5) k_cfl_f(GridParams g, GasF32 G, const 
     }
     m = block_max_f32(m);
     if (threadIdx.x == 0) atomic_max_pos(&d->red[slot], double(m));
+}
+
+void launch_cfl_f(const GridParams& g, const GasF32& G, const float* JU, const float* J, const float* disp,
+                  const float* vel, int slot, DevScalars* d, int grid, int block, cudaStream_t s) {
+    if (block <= 256) k_cfl_f<256, 5><<<grid, block, 0, s>>>(g, G, JU, J, disp, vel, slot, d);
+    else k_cfl_f<512, 1><<<grid, block, 0, s>>>(g, G, JU, J, disp, vel, slot, d);
 }
 
 // density and G = nu^3 p_nunu|_s / (2 c^2) at a node from the (hi, lo) state planes, in double-float

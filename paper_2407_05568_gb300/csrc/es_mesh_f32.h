@@ -27,8 +27,8 @@ inline GasF32 gas_f32(const Gas& g) {
 
 // JU, J: the mixed form's (hi, lo) float planes; disp: the FP32 displacement [dim][N]
 // vel (nullable): the float mesh velocity; slot: RED_CFL (mesh at rest) or RED_CFL2 (with the step's velocity)
-__global__ void k_cfl_f(GridParams g, GasF32 G, const float* JU, const float* J, const float* disp, const float* vel,
-                        int slot, DevScalars* d);
+void launch_cfl_f(const GridParams& g, const GasF32& G, const float* JU, const float* J, const float* disp,
+                  const float* vel, int slot, DevScalars* d, int grid, int block, cudaStream_t s);
 // rhoF, GF: 2 N floats each, (hi, lo) planes of the density and the fundamental derivative
 __global__ void k_mon_fields_f(GridParams g, GasF32 G, const float* JU, const float* J, float* rhoF, float* GF);
 // monitor terms over tiles of MON_NT threads (k_mon_f, 32 x 8 or 30 x 6 nodes, chosen by the mesh size)

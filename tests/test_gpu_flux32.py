@@ -95,3 +95,19 @@ def test_1d_tiles_against_oracle(n, bc):
     assert es.es_check(ctx) == 0, es.es_last_error(ctx)
     assert np.abs(to_np(dU) - dU_o).sum() < 1e-5 * np.abs(JU_o).sum() / d
     assert np.abs(to_np(dJ) - dJ_o).sum() < 1e-5 * np.abs(J_o).sum() / d
+
+
+@pytest.mark.parametrize("n", [200, 239, 256, 278, 280, 300])
+def test_2d_cfl_blocks(n):
+    """The mixed form's CFL kernel with blocks of up to 256 threads, of up to 512 (one per SM: 196 to 278 squared nodes on 152
+    SMs) and of 256 again: the time step of a smooth state on a fixed mesh within 1e-5 of the FP64 form's, and steps run."""
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    w = wl.sine_2d(n)
+    dts = []
+    for prec in ("fp64", "mixed"):
+        ctx, JU, J, x = es.setup_workload(w, prec)
+        dts.append(es.es_cfl_dt(ctx, JU, J, x, None))
+        es.es_steps(ctx, JU, J, x, 2, 1e30)
+        assert es.es_check(ctx) == 0, es.es_last_error(ctx)
+    assert abs(dts[1] - dts[0]) <= 1e-5 * dts[0]
