@@ -3,6 +3,8 @@
 // loss and the Adam update.  The network maps the filtered monitor, the
 // fundamental derivative and the current mesh (Sec. 4) to the displacement that
 // starts the Jacobi iteration; the plain iteration always finishes the solve.
+// The FP32 layers run on the tensor cores with their operands split into three bf16
+// parts (k_conv_fwd_s3, k_conv_wgrad_s3), the inference path on bf16 operands.
 //
 // Layout: activations [B][C][H][W] float; weights [Cout][Cin][3][3] (bf16 in the
 // C ABI, float inside the context); cross-correlation with zero padding:

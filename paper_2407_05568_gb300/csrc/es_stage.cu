@@ -598,14 +598,4 @@ cudaError_t launch_stage_fp64(const StageParams& P, cudaStream_t s) {
     }
 }
 
-void stage_tile_shape(bool mixed, int k, int* bx, int* by, int* nt) {
-    static const int fp64[STAGE_NTILES][3] = {{32, 8, 288}, {25, 11, 384}, {16, 16, 288}, {32, 12, 416},
-                                              {20, 10, 224}};
-    static const int f32[STAGE_NTILES][3] = {{32, 8, 288}, {25, 6, 192}, {20, 8, 192}, {32, 16, 544}, {16, 8, 160}};
-    const int(*t)[3] = mixed ? f32 : fp64;
-    *bx = t[k][0];
-    *by = t[k][1];
-    *nt = t[k][2];
-}
-
 }  // namespace es
