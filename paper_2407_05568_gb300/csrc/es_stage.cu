@@ -560,8 +560,14 @@ static cudaError_t launch_tile(const StageParams& P, cudaStream_t s) {
 
 // 2D shapes: 32 x 8 nodes with 288 threads (= the 32 x 9 faces of xi_2), 25 x 11 with 384
 // (25 x 12 = 300 faces; 8 x 19 = 152 tiles cover 200 x 200 in one wave on 152 SMs), 16 x 16
-// with 288 (272 faces), 32 x 12 with 416 (416 faces; less halo per node), 20 x 10 with 224.  1D: by the line's length
-// (launch_stage_fp64).
+// with 288 (272 faces), 32 x 12 with 416 (416 faces; less halo per node), 20 x 10 with 224.  A mesh that 20 x 10 tiles
+// cover in one wave has five shapes of its own, 64 to 200 nodes: a launch there is the time of one tile on its SM's FP64
+// pipe, so the smallest tile whose tiles the SMs can hold wins (a
+// Riemann stage, us: 64 x 64 74 with 8 x 8 nodes against 137 with 20 x 10, 120 x 120 83 with 12 x 8 against 139, 140 x 140
+// 114 with 20 x 8 against 138; the shapes of larger meshes take at least the last).  Above one wave 20 x 10 nodes and less
+// cost more halo than they balance (170 x 170: 166 us in one wave; 200 x 200: 192 against 176 with 25 x 11).
+// All shapes give the same bits.  1D: by the line's length (launch_stage_fp64).
+static bool small_mesh(const StageParams& P) { return (P.n1 + 19) / 20 * ((P.n2 + 9) / 10) <= 152; }
 cudaError_t stage_prepare_fp64(int dim) {
     if (dim == 1) {
         cudaError_t e1 = prepare_tile<1, 254, 1, 256>();
@@ -572,6 +578,10 @@ cudaError_t stage_prepare_fp64(int dim) {
     if (e == cudaSuccess) e = prepare_tile<2, 16, 16, 288>();
     if (e == cudaSuccess) e = prepare_tile<2, 32, 12, 416>();
     if (e == cudaSuccess) e = prepare_tile<2, 20, 10, 224>();
+    if (e == cudaSuccess) e = prepare_tile<2, 8, 8, 128>();
+    if (e == cudaSuccess) e = prepare_tile<2, 12, 8, 128>();
+    if (e == cudaSuccess) e = prepare_tile<2, 16, 8, 160>();
+    if (e == cudaSuccess) e = prepare_tile<2, 20, 8, 192>();
     return e;
 }
 
@@ -588,6 +598,15 @@ cudaError_t launch_stage_fp64(const StageParams& P, cudaStream_t s) {
         }
         if (P.n1 <= 1 << 16) return launch_tile<1, 62, 1, 128>(P, s);
         return launch_tile<1, 254, 1, 256>(P, s);
+    }
+    if (small_mesh(P)) {
+        switch (P.tile) {
+            case 1: return launch_tile<2, 12, 8, 128>(P, s);
+            case 2: return launch_tile<2, 16, 8, 160>(P, s);
+            case 3: return launch_tile<2, 20, 8, 192>(P, s);
+            case 4: return launch_tile<2, 20, 10, 224>(P, s);
+            default: return launch_tile<2, 8, 8, 128>(P, s);
+        }
     }
     switch (P.tile) {
         case 1: return launch_tile<2, 25, 11, 384>(P, s);

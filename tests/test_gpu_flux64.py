@@ -63,3 +63,42 @@ def test_1d_stage_shapes_vs_oracle(n, bc):
         assert np.abs(dJ.cpu().numpy() - dJ_o).max() < 1e-12 / d
         assert np.abs(U1.cpu().numpy() - U1_o).max() < 1e-12 * np.abs(U1_o).max()
         assert np.abs(J1.cpu().numpy() - J1_o).max() < 1e-12 * np.abs(J1_o).max()
+
+
+@pytest.mark.parametrize("n1,n2", [(8, 8), (9, 17), (41, 23), (200, 100), (300, 101)])
+@pytest.mark.parametrize("bc", [("periodic", "outflow"), ("reflect", "symmetry_lo")])
+def test_2d_small_mesh_shapes(n1, n2, bc):
+    """The five shapes of meshes that one wave covers (8 x 8 to 20 x 10 nodes), whole and ragged, and the first size past it:
+    right-hand sides of a rough state against the oracle to 1e-12 of a flux difference, the same bits from every shape."""
+    import torch
+
+    from oracle import operator as op
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    from sides import oracle_setup
+    x1, d1 = wl.uniform_nodes(n1, 0.0, 1.0, bc[0] == "periodic")
+    x2, d2 = wl.uniform_nodes(n2, 0.0, 1.0, bc[1] == "periodic")
+    X, Y = np.meshgrid(x1, x2)
+    w = wl.sine_2d(16)
+    w.update(bc=bc, x=np.stack([X, Y]), dxi=(d1, d2), n=(n2, n1))
+    w["rho"], w["v"], w["p"] = wl.rough_state((n2, n1), 3 + n1, 2)
+    sch, _, JU_o, J_o, x_o = oracle_setup(w)
+    dU_o, dJ_o = op.rhs(sch, JU_o, J_o, x_o, np.zeros_like(x_o))
+    outs = []
+    for tile in (1, 2, 3, 4, 5):
+        ctx = es.es_create(es.make_params(w, tile=tile))
+        xt = torch.tensor(np.ascontiguousarray(w["x"]), device="cuda")
+        J = torch.empty((n2, n1), dtype=torch.float64, device="cuda")
+        es.es_init_mesh(ctx, xt, J)
+        JU = torch.empty((4, n2, n1), dtype=torch.float64, device="cuda")
+        es.es_prim_to_cons(ctx, torch.tensor(w["rho"], device="cuda"), torch.tensor(w["v"], device="cuda"),
+                           torch.tensor(w["p"], device="cuda"), J, JU)
+        dU, dJ = torch.empty_like(JU), torch.empty_like(J)
+        es.es_rhs(ctx, JU, J, xt, None, dU, dJ)
+        assert es.es_check(ctx) == 0, es.es_last_error(ctx)
+        outs.append((dU.cpu().numpy(), dJ.cpu().numpy()))
+    for c in range(4):
+        flux = np.abs(JU_o[c]).max() * 4.0 / min(d1, d2)
+        assert np.abs(outs[0][0][c] - dU_o[c]).max() < 1e-12 * flux
+    for o in outs[1:]:
+        assert np.array_equal(o[0], outs[0][0]) and np.array_equal(o[1], outs[0][1])
