@@ -244,7 +244,7 @@ int es_time_stage(es_ctx* ctx, const void* JU, const void* J, const double* x, i
 int es_selftest_division(const double* a, const double* b, double* q, double* r, int64_t n, void* stream);
 
 /* Self-test of the library's FP64 logarithm (the node fields of the FP64 operator take their logarithms from a
- * table and a short series): y[i] = ln x[i] for device arrays of n positive doubles, within 2 ulp, on `stream`
+ * table and a short series): y[i] = ln x[i] for device arrays of n positive doubles, within 1 ulp, on `stream`
  * (asynchronous; ES_ERR_ARG for null arrays or n <= 0, ES_ERR_CUDA if the launch fails). */
 int es_selftest_log(const double* x, double* y, int64_t n, void* stream);
 
