@@ -686,8 +686,8 @@ __global__ void k3_limiter(Grid3 g, const double* xn, const double* xa, const do
             if (__double_as_longlong(dx) << 1 == 0) continue;                        // +-0
             const bool back = __double2hiint(dx) < 0;
             const double xb1 = nb_coord(g, x, id, ii[k], k, back ? -1 : 1, k);
-            const double gap = back ? x0 - xb1 : xb1 - x0, two = 2.0 * fabs(dx);
-            if (gap < m * two) m = fmin(m, div_nr(gap, two));
+            const double gap = back ? x0 - xb1 : xb1 - x0, a = fabs(dx);
+            if (gap < m * (LIMIT_TEST * a)) m = fmin(m, div_nr(gap, 2.0 * a));
         }
     }
     m = block_min(m);

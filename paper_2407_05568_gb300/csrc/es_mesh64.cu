@@ -180,14 +180,16 @@ __device__ __forceinline__ double coord_beside(const GridParams& g, const double
 
 // The limiter's bound at one node and component: it moves by dx; `room`, the spacing towards the neighbour it moves to.
 // gamma = min(gamma, room/(2 |dx|)) over the grid: the quotient is formed, and the grid's minimum lowered, only where it
-// is below what the grid has reached so far (m; reading an older, larger value only costs the quotient).
+// can be below what the grid has reached so far (m; reading an older, larger value only costs the quotient).  The test is
+// against the bound enlarged by 2^-50: m t is rounded, and where that gives `room` itself the quotient can still be an ulp
+// below m, so that the test would let the order of the nodes decide between quotients that close.
 __device__ __forceinline__ double grid_limit(const DevScalars* d) {
     return __longlong_as_double((long long)__ldcg(&d->red[RED_GAMMA]));
 }
 __device__ __forceinline__ double limit_by(double m, double dx, double room, DevScalars* d) {
-    const double t = 2.0 * fabs(dx);
-    if (room < m * t) {
-        const double q = div_nr(room, t);
+    const double a = fabs(dx);
+    if (room < m * (LIMIT_TEST * a)) {
+        const double q = div_nr(room, 2.0 * a);
         if (q < m) {
             atomic_min_pos(&d->red[RED_GAMMA], q);
             m = q;

@@ -1,9 +1,12 @@
 // es_mesh64.cuh -- maxima of non-negative doubles by their ordered bits (comparisons of doubles and
-// fmax/fmin take the FP64 pipe), for the FP64 mesh and time-step kernels.
+// fmax/fmin take the FP64 pipe), for the FP64 mesh and time-step kernels, and the limiter's test.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace es {
+
+// 2 (1 + 2^-50): the limiter forms room/(2 |dx|) where room < m (LIMIT_TEST |dx|)
+constexpr double LIMIT_TEST = 2.0 + 0x1p-49;
 
 // max(a, b), a >= 0, b >= 0 or NaN (a NaN is passed over, as fmax does)
 __device__ __forceinline__ double max_bits(double a, double b) {

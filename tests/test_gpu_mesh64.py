@@ -81,3 +81,39 @@ def test_redistribution_3d(bc, shape, passes, sweeps, monitor):
     w["mesh"] = dict(monitor=monitor, alphas=(1200.0, 1200.0, 1200.0), kappa=2, filter_passes=passes, sweeps=sweeps,
                      eps=0.0)
     _compare(w)
+
+
+@pytest.mark.parametrize("n", [76000, 380000])
+def test_limiter_is_the_least_quotient(n):
+    """Delta_gamma is the least of the nodes' quotients room/(2 |dx|), bit for bit, also where many differ by single ulps:
+    the same 1D pattern of spacings in every binade from 2^-900 to 2^1000 (one launch of tiles; sweep by sweep), its scale
+    varied a little, so that the blocks' quotients are equal but for rounding."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    rng = np.random.default_rng(4)
+    blocks, P = 1900, n // 1900
+    w = wl.riemann_1d("RP1", n)
+    rho = np.tile(rng.uniform(0.3, 1.2, P), blocks)
+    w.update(rho=rho, v=np.zeros((1, n)), p=np.full(n, 2.0), bc=("outflow",))
+    w["mesh"] = dict(w["mesh"], filter_passes=0, sweeps=1, eps=0.0)
+    ctx, JU, J, _ = gpu_setup(w)
+    xo = torch.empty((1, n), dtype=torch.float64, device="cuda")
+    xd = torch.empty_like(xo)
+    q, r = torch.empty_like(xo[0]), torch.empty_like(xo[0])
+    for _ in range(500):
+        cuts = rng.uniform(0.0, 1.0, 10)                              # a few wide spacings
+        at = np.sort(np.concatenate([cuts, rng.choice(cuts, P - 10) + 1e-4 * rng.uniform(size=P - 10)]))
+        s = 1.0 + 0.04 * rng.uniform(size=blocks)
+        x = (np.ldexp(s, np.arange(blocks) - 900)[:, None] * (1.05 + 0.8 * at)[None, :]).reshape(1, n)
+        xt = torch.tensor(x, device="cuda")
+        _, gam = es.es_mesh_redistribute(ctx, JU, J, xt, 1.0, xd)
+        es.es_mesh_solve(ctx, JU, J, xt, None, xo)
+        dx = (xo - xt)[0]
+        right = torch.cat([xt[0, 1:], xt[0, -1:]]) - xt[0]
+        left = xt[0] - torch.cat([xt[0, :1], xt[0, :-1]])
+        two = torch.where(dx == 0, 1.0, 2.0 * dx.abs())
+        es.es_selftest_division(torch.where(dx < 0, left, right), two, q, r)       # the kernels' quotient
+        least = float(torch.where(dx == 0, 1.0, q).min())
+        assert 0.0 < least < 1.0
+        assert gam == least
