@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(C3_THREADS, 2) k_conv_fwd_s3(const float* __re
                     bf[nt + 1][1] = r[3];
                 }
             }
-            // tap and channel offset of this lane's row (a step past the last tap has zero weights: any pixel will do)
+            // tap and channel offset of this lane's row (past the last tap: any pixel, its fragments are zeroed below)
             const int k = s * 16 + ah * 8;
             const int tap = min(k / CP, 8), c = k % CP;
             const int off = ((tap / 3) * HALO + tap % 3 + ap) * PW + c / 2;
@@ -399,7 +399,10 @@ __global__ void __launch_bounds__(C3_THREADS, 2) k_conv_fwd_s3(const float* __re
                 const uint32_t row = xa + 4u * ((warp * 2 + mt) * HALO * PW + off);
                 uint32_t a[3][4];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) ldsm4(a[q], row + 4u * q * HP * PW);
+                for (int q = 0; q < 3; ++q) {
+                    ldsm4(a[q], row + 4u * q * HP * PW);
+                    if (CV::K % 16 && s == STEPS - 1) a[q][2] = a[q][3] = 0u;      // past the last tap (0 x infinity is NaN)
+                }
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) {
                     mma_bf16_16816(lead[mt][nt], a[0], bf[nt]);

@@ -43,3 +43,37 @@ def test_forward_and_gradients_vs_oracle(cin, cout, shape):
         for got, ref, n in ((gw, rw, B * H * W), (gb, rb, B * H * W), (gin, ra, 9 * cout)):
             scale = np.abs(ref).max() + np.abs(go).max() * (np.abs(a).max() if ref is rw else 1.0)
             assert np.abs(got.cpu().double().numpy() - ref).max() <= (4e-7 * np.sqrt(n) + back * np.sqrt(n)) * scale
+
+
+@pytest.mark.parametrize("cin", [2, 4, 32])
+@pytest.mark.parametrize("cout", [2, 32])
+def test_forward_infinite_and_nan_inputs(cin, cout):
+    """An infinite input reaches the nine outputs whose taps read it as an infinity of the product's sign (tanh: +-1), a NaN
+    as a NaN, and every other output as if they were zero."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    B, H, W = 2, 21, 35
+    rng = np.random.default_rng(5 + cin + cout)
+    a = rng.standard_normal((B, cin, H, W)).astype(np.float32)
+    w = convnet.bf16_round((rng.standard_normal((cout, cin, 3, 3)) / np.sqrt(9 * cin)).astype(np.float32))
+    assert (w != 0.0).all()
+    zero = a.copy()
+    spots = [(0, 0, 10, 14, np.inf), (0, cin - 1, 16, 24, -np.inf), (1, 1, 5, 5, np.nan), (1, 0, 15, 16, np.inf)]
+    for b, c, y, x, v in spots:
+        a[b, c, y, x], zero[b, c, y, x] = v, 0.0
+    z = convnet.conv3x3(zero.astype(np.float64), w)
+    size = np.abs(z).max()
+    for b, c, y, x, v in spots:
+        z[b, :, y - 1:y + 2, x - 1:x + 2] = (v * w[:, c, ::-1, ::-1]).reshape(cout, 3, 3)
+    wt = torch.tensor(w, dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(es.es_nn_workspace_bytes(B, cin, cout, H, W) // 4 + 1, dtype=torch.float32, device="cuda")
+    bias = torch.zeros(cout, device="cuda")
+    for act in (False, True):
+        out = torch.empty((B, cout, H, W), dtype=torch.float32, device="cuda")
+        es.es_nn_conv_forward(torch.tensor(a, device="cuda"), wt, bias, out, act, ws)
+        got, ref = out.cpu().double().numpy(), np.tanh(z) if act else z
+        fin = np.isfinite(ref)
+        assert np.array_equal(np.isnan(got), np.isnan(ref))
+        assert np.array_equal(got[np.isinf(ref)], ref[np.isinf(ref)])
+        assert np.abs(got[fin] - ref[fin]).max() <= 4e-7 * np.sqrt(9 * cin) * size
