@@ -458,6 +458,9 @@ struct Wgrad {
     static constexpr int BUF = 3 * (HP * PX + NP * PG);      // words of a buffer
     static constexpr size_t SMEM = sizeof(uint32_t) * size_t(2) * BUF;
 };
+// a sum and its correction products: beside an infinite sum they are products of an infinity with the other operand's
+// low parts, which may be zero (NaN)
+__device__ __forceinline__ float with_low(float sum, float low) { return isinf(sum) ? sum : sum + low; }
 // the three parts of 8 channels at word `w` of a plane, planes `plane` words apart
 __device__ __forceinline__ void store_split(uint32_t* w, int plane, const float* x) {
     uint32_t v[3][4];
@@ -625,13 +628,13 @@ __global__ void __launch_bounds__(Wgrad<CIN, COUT>::THREADS, 1)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int co = mt * 16 + gq + (e >= 2 ? 8 : 0), ci = nt * 8 + 2 * t + (e & 1);
-            if (co < COUT && ci < CIN) part[(co * CIN + ci) * 9 + tap] = acc[nt][e] + low[nt][e];
+            if (co < COUT && ci < CIN) part[(co * CIN + ci) * 9 + tap] = with_low(acc[nt][e], low[nt][e]);
         }
     if (tap == 4 && t == 0)
 #pragma unroll
         for (int e = 0; e < 4; e += 2) {
             const int co = mt * 16 + gq + (e >= 2 ? 8 : 0);
-            if (co < COUT) part[nout + co] = accb[e] + lowb[e];
+            if (co < COUT) part[nout + co] = with_low(accb[e], lowb[e]);
         }
 }
 

@@ -77,3 +77,37 @@ def test_forward_infinite_and_nan_inputs(cin, cout):
         assert np.array_equal(np.isnan(got), np.isnan(ref))
         assert np.array_equal(got[np.isinf(ref)], ref[np.isinf(ref)])
         assert np.abs(got[fin] - ref[fin]).max() <= 4e-7 * np.sqrt(9 * cin) * size
+
+
+@pytest.mark.parametrize("cin", [2, 32])
+@pytest.mark.parametrize("cout", [4, 32])
+@pytest.mark.parametrize("where", ["input", "gradient"])
+def test_weight_gradient_of_an_infinity(cin, cout, where):
+    """One infinite value of the input, or of the output's gradient, away from the edges: the weight gradients that it
+    enters are infinities of the product's sign, and the others stay finite and as accurate as without it."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    B, H, W, b, y, x, c = 1, 40, 37, 0, 18, 14, 1
+    rng = np.random.default_rng(9 + cin + cout)
+    a = rng.standard_normal((B, cin, H, W)).astype(np.float32)
+    go = rng.standard_normal((B, cout, H, W)).astype(np.float32)
+    w = convnet.bf16_round(rng.standard_normal((cout, cin, 3, 3)).astype(np.float32))
+    a0, g0 = a.copy(), go.copy()
+    (a0 if where == "input" else g0)[b, c, y, x] = 0.0
+    (a if where == "input" else go)[b, c, y, x] = np.inf
+    rw, rb, _ = convnet.conv3x3_backward(a0.astype(np.float64), w, g0.astype(np.float64))
+    size = np.abs(rw).max()
+    if where == "input":                                 # w[co][c][tap] takes g[co] at (y, x) less the tap
+        rw[:, c] = np.inf * np.sign(go[b, :, y - 1:y + 2, x - 1:x + 2][:, ::-1, ::-1])
+    else:
+        rw[c] = np.inf * np.sign(a[b, :, y - 1:y + 2, x - 1:x + 2])
+        rb[c] = np.inf
+    at, g = torch.tensor(a, device="cuda"), torch.tensor(go, device="cuda")
+    ws = torch.empty(es.es_nn_workspace_bytes(B, cin, cout, H, W) // 4 + 1, dtype=torch.float32, device="cuda")
+    gw, gb = torch.empty((cout, cin, 3, 3), device="cuda"), torch.empty(cout, device="cuda")
+    es.es_nn_conv_backward(at, torch.tensor(w, dtype=torch.bfloat16, device="cuda"), None, g, None, gw, gb, False, ws)
+    for got, ref in ((gw.cpu().double().numpy(), rw), (gb.cpu().double().numpy(), rb)):
+        fin = np.isfinite(ref)
+        assert np.array_equal(got[~fin], ref[~fin])
+        assert np.abs(got[fin] - ref[fin]).max() <= 4e-7 * np.sqrt(B * H * W) * (size + 1.0)
