@@ -246,15 +246,18 @@ __global__ void __launch_bounds__(128) k_conv_fwd_tc(const void* __restrict__ in
 struct Split3 {
     uint32_t v[3];                 // bf16 pairs: leading, middle, last parts
 };
+// The first two parts are cut to the finite bf16 range: a finite value that would round past it keeps its sum, and an
+// infinity (or a NaN) leaves itself as the last part.
 __device__ __forceinline__ Split3 split3(float a, float b) {
+    constexpr float MAX = 3.38953139e38f;                    // the largest bf16
     Split3 s;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        const float x = k < 2 ? fminf(fmaxf(a, -MAX), MAX) : a, y = k < 2 ? fminf(fmaxf(b, -MAX), MAX) : b;
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
         s.v[k] = *reinterpret_cast<const uint32_t*>(&h);
-        const float ha = __uint_as_float(s.v[k] << 16), hb = __uint_as_float(s.v[k] & 0xffff0000u);
-        a = isinf(ha) ? 0.0f : a - ha;                       // (an infinity has no remainder)
-        b = isinf(hb) ? 0.0f : b - hb;
+        a -= __uint_as_float(s.v[k] << 16);
+        b -= __uint_as_float(s.v[k] & 0xffff0000u);
     }
     return s;
 }

@@ -111,3 +111,22 @@ def test_weight_gradient_of_an_infinity(cin, cout, where):
         fin = np.isfinite(ref)
         assert np.array_equal(got[~fin], ref[~fin])
         assert np.abs(got[fin] - ref[fin]).max() <= 4e-7 * np.sqrt(B * H * W) * (size + 1.0)
+
+
+def test_forward_of_the_largest_floats():
+    """Finite inputs that round to infinity in bf16 (above 3.39e38): the layer's output is their exact product."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    big = np.array([3.4028234e38, -3.4e38, 3.3961e38], np.float32)
+    a = np.zeros((1, 4, 9, 9), np.float32)
+    a[0, 2, 4, [1, 4, 7]] = big
+    w = np.zeros((2, 4, 3, 3), np.float32)
+    w[0, 2, 1, 1], w[1, 2, 1, 1] = 0.25, -0.5
+    out = torch.empty((1, 2, 9, 9), dtype=torch.float32, device="cuda")
+    ws = torch.empty(es.es_nn_workspace_bytes(1, 4, 2, 9, 9) // 4 + 1, dtype=torch.float32, device="cuda")
+    es.es_nn_conv_forward(torch.tensor(a, device="cuda"), torch.tensor(w, dtype=torch.bfloat16, device="cuda"),
+                          torch.zeros(2, device="cuda"), out, False, ws)
+    got = out.cpu().numpy()[0, :, 4, [1, 4, 7]]
+    ref = np.stack([0.25 * big, -0.5 * big], 1)
+    assert np.all(np.abs(got.astype(np.float64) - ref) <= 2.0 ** -22 * np.abs(ref))
