@@ -23,24 +23,45 @@ constexpr int TS = 16;            // output tile edge (pixels)
 constexpr int HALO = TS + 2;
 constexpr int MAXC = 32;          // channel limit
 
+// a sum and its correction products: beside an infinite sum they are products of an infinity with the other operand's
+// low parts, which may be zero (NaN)
+__device__ __forceinline__ float with_low(float sum, float low) { return isinf(sum) ? sum : sum + low; }
+// the same in place: what the sum's rounding leaves stays in `low`
+__device__ __forceinline__ void take_low(float& sum, float& low) {
+    const float s = with_low(sum, low);
+    low += sum - s;
+    sum = s;
+}
+// sum + v with the rounding error collected in `low` (D. E. Knuth, TAOCP 2, 4.2.2)
+__device__ __forceinline__ void add_comp(float& sum, float& low, float v) {
+    const float s = sum + v, b = s - sum;
+    low += (sum - (s - b)) + (v - b);
+    sum = s;
+}
+
 // out[o] = sum_s partial[s][o] over the strips: RP_GROUPS threads per output take every RP_GROUPS-th strip, and their sums
-// are added in order (the same order every time)
+// are added in order (the same order every time), with the rounding errors: a long image has a thousand strips
 constexpr int RP_GROUPS = 16;
 __global__ void __launch_bounds__(32 * RP_GROUPS) k_reduce_partials(const float* __restrict__ partial, int nstrips,
                                                                     int len, float* grad_w, float* grad_b, int nout) {
-    __shared__ float part[RP_GROUPS][32];
+    __shared__ float part[2][RP_GROUPS][32];
     const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const int o = blockIdx.x * 32 + lane;
-    float s = 0.0f;
+    float s = 0.0f, c = 0.0f;
     if (o < len)
 #pragma unroll 4
-        for (int k = grp; k < nstrips; k += RP_GROUPS) s += partial[size_t(k) * len + o];
-    part[grp][lane] = s;
+        for (int k = grp; k < nstrips; k += RP_GROUPS) add_comp(s, c, partial[size_t(k) * len + o]);
+    part[0][grp][lane] = s;
+    part[1][grp][lane] = c;
     __syncthreads();
     if (grp != 0 || o >= len) return;
-    s = 0.0f;
+    s = c = 0.0f;
 #pragma unroll
-    for (int k = 0; k < RP_GROUPS; ++k) s += part[k][lane];
+    for (int k = 0; k < RP_GROUPS; ++k) {
+        add_comp(s, c, part[0][k][lane]);
+        c += part[1][k][lane];
+    }
+    s = with_low(s, c);
     if (o < nout) grad_w[o] = s;
     else grad_b[o - nout] = s;
 }
@@ -241,8 +262,8 @@ __global__ void __launch_bounds__(128) k_conv_fwd_tc(const void* __restrict__ in
 // the weight gradient, whose operands are both FP32, six (the three of relative size 2^-24 and less are dropped).  On
 // mma.sync the CUDA-core kernels' 22 TFLOP/s no longer bound them.  The tensor cores truncate their FP32 sums, so the
 // leading products are summed over one tap's channels (forward) or 16 pixels (weight gradient) only and added to the
-// result with a rounded FP32 addition; the other products are 2^-8 of these and share one accumulator.  Errors against 64
-// bits are measured in the tests of the layers; they are below the FMA chains' they replace.
+// result with a rounded FP32 addition; the other products are 2^-8 of these and share one accumulator, over 64 rows at most
+// in the weight gradient.
 struct Split3 {
     uint32_t v[3];                 // bf16 pairs: leading, middle, last parts
 };
@@ -461,9 +482,6 @@ struct Wgrad {
     static constexpr int BUF = 3 * (HP * PX + NP * PG);      // words of a buffer
     static constexpr size_t SMEM = sizeof(uint32_t) * size_t(2) * BUF;
 };
-// a sum and its correction products: beside an infinite sum they are products of an infinity with the other operand's
-// low parts, which may be zero (NaN)
-__device__ __forceinline__ float with_low(float sum, float low) { return isinf(sum) ? sum : sum + low; }
 // the three parts of 8 channels at word `w` of a plane, planes `plane` words apart
 __device__ __forceinline__ void store_split(uint32_t* w, int plane, const float* x) {
     uint32_t v[3][4];
@@ -476,7 +494,10 @@ __device__ __forceinline__ void store_split(uint32_t* w, int plane, const float*
 #pragma unroll
     for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4*>(w + q * plane) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
 }
-template <int CIN, int COUT>
+// LONG: strips of more than 64 rows, where the truncated sums of the correction products (2^-8 of the others) are taken into
+// the rounded ones every 64 rows.  (A kernel of its own: the code spills eleven more words, 3% of a training step whose
+// strips are shorter.)
+template <int CIN, int COUT, bool LONG>
 __global__ void __launch_bounds__(Wgrad<CIN, COUT>::THREADS, 1)
     k_conv_wgrad_s3(const float* __restrict__ in, float* g, const float* __restrict__ aout, float* __restrict__ partial,
                     int H, int W, int rows) {
@@ -556,6 +577,14 @@ __global__ void __launch_bounds__(Wgrad<CIN, COUT>::THREADS, 1)
     int cur = 0;
     for (int y0 = yb; y0 < ye; y0 += WG_H, cur ^= 1) {
         const bool more = y0 + WG_H < ye;
+        if (LONG && (y0 & 63) == 0) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) take_low(acc[nt][e], low[nt][e]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) take_low(accb[e], lowb[e]);
+        }
         if (more) load(y0 + WG_H);
         const uint32_t xa = smem_addr(sm + cur * WG::BUF), ga = xa + 4u * 3 * HP * PX;
 #pragma unroll 1
@@ -701,15 +730,21 @@ cudaError_t conv_s3(const float* in, const uint16_t* w, const float* bias, float
         return cudaGetLastError();
     });
 }
+template <int CIN, int COUT, bool LONG>
+cudaError_t wgrad_launch_as(dim3 grid, const float* in, float* g, const float* aout, float* partial, int H, int W, int rows,
+                            cudaStream_t s) {
+    const size_t sm = Wgrad<CIN, COUT>::SMEM;
+    const cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_s3<CIN, COUT, LONG>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+    if (e != cudaSuccess) return e;
+    k_conv_wgrad_s3<CIN, COUT, LONG><<<grid, Wgrad<CIN, COUT>::THREADS, sm, s>>>(in, g, aout, partial, H, W, rows);
+    return cudaGetLastError();
+}
 template <int CIN, int COUT>
 cudaError_t wgrad_launch(dim3 grid, const float* in, float* g, const float* aout, float* partial, int H, int W, int rows,
                          cudaStream_t s) {
-    const size_t sm = Wgrad<CIN, COUT>::SMEM;
-    const cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_s3<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(sm));
-    if (e != cudaSuccess) return e;
-    k_conv_wgrad_s3<CIN, COUT><<<grid, Wgrad<CIN, COUT>::THREADS, sm, s>>>(in, g, aout, partial, H, W, rows);
-    return cudaGetLastError();
+    return rows * TS > 64 ? wgrad_launch_as<CIN, COUT, true>(grid, in, g, aout, partial, H, W, rows, s)
+                          : wgrad_launch_as<CIN, COUT, false>(grid, in, g, aout, partial, H, W, rows, s);
 }
 template <int CIN>
 cudaError_t wgrad_by_cout(int Cout, dim3 grid, const float* in, float* g, const float* aout, float* partial, int H, int W,

@@ -130,3 +130,49 @@ def test_forward_of_the_largest_floats():
     got = out.cpu().numpy()[0, :, 4, [1, 4, 7]]
     ref = np.stack([0.25 * big, -0.5 * big], 1)
     assert np.all(np.abs(got.astype(np.float64) - ref) <= 2.0 ** -22 * np.abs(ref))
+
+
+@pytest.mark.parametrize("shape", [(4, 512, 512), (3, 700, 530)])
+def test_weight_gradient_of_long_strips(shape):
+    """Strips of four 16-row tiles, whose two buffers are refilled several times (the training size, and a ragged image),
+    against float64.  With R the root of the sum of squared products, about 150 rounded additions of partial sums of size R
+    leave a random walk of 2^-24 sqrt(150) R = 7e-7 R; a dropped third part of one operand would leave 4e-6 R."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    B, H, W = shape
+    gen = torch.Generator(device="cuda").manual_seed(H)
+    a = torch.randn((B, 32, H, W), generator=gen, device="cuda")
+    g = torch.randn((B, 32, H, W), generator=gen, device="cuda")
+    w = torch.zeros((32, 32, 3, 3), dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(es.es_nn_workspace_bytes(B, 32, 32, H, W) // 4 + 1, dtype=torch.float32, device="cuda")
+    gw, gb = torch.empty((32, 32, 3, 3), device="cuda"), torch.empty(32, device="cuda")
+    es.es_nn_conv_backward(a, w, None, g, None, gw, gb, False, ws)
+    rw, r2 = torch.zeros((32, 32, 3, 3), dtype=torch.float64, device="cuda"), torch.zeros((32, 32, 3, 3), device="cuda")
+    for b in range(B):
+        ap, gd = torch.nn.functional.pad(a[b], (1, 1, 1, 1)), g[b].double().reshape(32, -1)
+        for t in range(9):
+            x = ap[:, t // 3:t // 3 + H, t % 3:t % 3 + W].reshape(32, -1)
+            rw[:, :, t // 3, t % 3] += gd @ x.double().T
+            r2[:, :, t // 3, t % 3] += (g[b].reshape(32, -1) ** 2) @ (x ** 2).T
+    assert float(((gw.double() - rw).abs() / r2.sqrt()).max()) <= 2e-6
+    rb = g.double().sum((0, 2, 3))
+    assert float((gb.double() - rb).abs().max()) <= 2e-6 * (B * H * W) ** 0.5
+
+
+def test_weight_gradient_of_a_tall_image():
+    """A strip as tall as the image, 4096 rows: every product is (1 + d)(1 + e), whose leading parts are ones and sum
+    exactly, so that the error is that of the correction products' sum.  Added to the rounded sum every 64 rows they leave
+    the random walk of 64 half ulps, 2^-25 sqrt(64) = 2.4e-7, twice that at most."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    H, W = 4096, 16 * 1064                                       # as many strips as the grid takes: one per column
+    x, g = np.float32(1.0037841), np.float32(1.0034173)
+    a = torch.full((1, 2, H, W), float(x), device="cuda")
+    go = torch.full((1, 2, H, W), float(g), device="cuda")
+    ws = torch.empty(es.es_nn_workspace_bytes(1, 2, 2, H, W) // 4 + 1, dtype=torch.float32, device="cuda")
+    gw, gb = torch.empty((2, 2, 3, 3), device="cuda"), torch.empty(2, device="cuda")
+    es.es_nn_conv_backward(a, torch.zeros((2, 2, 3, 3), dtype=torch.bfloat16, device="cuda"), None, go, None, gw, gb, False, ws)
+    assert abs(float(gw[1, 0, 1, 1]) / (float(x) * float(g) * H * W) - 1.0) <= 4.8e-7
+    assert abs(float(gb[1]) / (float(g) * H * W) - 1.0) <= 4.8e-7
