@@ -8,14 +8,14 @@ namespace es {
 
 // omega_i <- sum_{j in {0,+-1}^3} (1/2)^(|j|_1 + 3) omega_{i+j} (Sec. 4), ghosts by copy / wrap.
 // The filter is the product of three (1/4, 1/2, 1/4) sums.  Read node by node it is 27 products (in FP64, 48 instructions on
-// the FP64 pipe, which bound it: 77 us at 96^3); here the sums are shared: a warp takes 32 nodes along xi_1 and RY lines,
+// the FP64 pipe, which bound it: 72 us at 96^3); here the sums are shared: a warp takes 32 nodes along xi_1 and RY lines,
 // and marches along xi_3 keeping the last two planes' partial sums, so a node costs the row sums of (RY + 2)/RY lines, a
 // column sum and a plane sum, two instructions each, and one scaling: 9 at RY = 2, 8 at RY = 4 (and the segments' ends).
 // Neighbours along xi_1 come from the neighbouring lanes (the warp's ends and the mesh's last node load theirs), so there is
 // no shared memory and no barrier; the next plane's loads are in flight while a plane is summed.  The weights are powers of
-// two, so that the sums without them (l + 2 c + r) have the same bits as with them.  96^3: FP64 77 -> 25 us, FP32 12.4 ->
-// 10.3.  (Four passes at a time on 16^3 tiles in shared memory, FP32: 9.7 us a pass, bound by the nine shared loads a node,
-// and no better on larger meshes.)
+// two, so that the sums without them (l + 2 c + r) have the same bits as with them.  A pass within a step at 96^3: FP64 72 ->
+// 17 us, FP32 9.8 -> 8.6.  (Four passes at a time on 16^3 tiles in shared memory, FP32: 9.7 us a pass, bound by the nine
+// shared loads a node, and no better on larger meshes.)
 template <typename T, int RY>
 __global__ void __launch_bounds__(128) k3_filter(Grid3 g, const T* in, T* out, int seg) {
     const int n1 = g.n[0], n2 = g.n[1], n3 = g.n[2];
@@ -66,12 +66,35 @@ __global__ void __launch_bounds__(128) k3_filter(Grid3 g, const T* in, T* out, i
     }
 }
 
-// Lines per warp and planes per segment.  A warp's planes follow one another, 1.1 us each (FP32; a load's latency), so on
-// meshes of up to 2^21 nodes short segments and two lines keep the launch short although they sum more planes and rows
-// twice: four warps on each of the 608 schedulers where the mesh gives them, at least 2 planes.  96^3: 24.6 us (FP64) and
-// 10.3 us (FP32, 12.4 node by node), with four lines and 1216 warps 26.2 and 12.4; 40^3: 10.3 and 6.2 us (12.4 and 6.1 node
-// by node), 14.4 and 10.3.  Above, four lines in segments of 4 to 12 planes: 200^3 172 and 41 us (two lines 190 and 43, node
-// by node 625 and 78).
+// Node by node, the same sums: 27 loads in flight at once.  On a small mesh a pass is the length of one thread's chain, and
+// here it is one load's latency.
+template <typename T>
+__global__ void __launch_bounds__(128) k3_filter_nodes(Grid3 g, const T* __restrict__ in, T* __restrict__ out) {
+    const int n1 = g.n[0], n2 = g.n[1], n12 = n1 * n2;
+    const int id = blockIdx.x * 128 + threadIdx.x;
+    if (id >= n12 * g.n[2]) return;
+    const int r12 = id / n1, i = id - r12 * n1, k = r12 / n2, j = r12 - k * n2;
+    const int xm = state_index(i - 1, n1, g.bc[0]) - i, xp = state_index(i + 1, n1, g.bc[0]) - i;
+    const int y[3] = {(state_index(j - 1, n2, g.bc[1]) - j) * n1, 0, (state_index(j + 1, n2, g.bc[1]) - j) * n1};
+    const int z[3] = {(state_index(k - 1, g.n[2], g.bc[2]) - k) * n12, 0, (state_index(k + 1, g.n[2], g.bc[2]) - k) * n12};
+    T c[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        T r[3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            const T* v = in + (id + y[p] + z[q]);
+            r[p] = fma(T(2), v[0], v[xm]) + v[xp];
+        }
+        c[q] = fma(T(2), r[1], r[0]) + r[2];
+    }
+    out[id] = (fma(T(2), c[1], c[0]) + c[2]) * T(1.0 / 64.0);
+}
+
+// Lines per warp and planes per segment.  A warp's planes follow one another (a load's latency each), so on meshes of up to
+// 2^21 nodes short segments and two lines keep the launch short although they sum more planes and rows twice: four warps on
+// each of the 608 schedulers where the mesh gives them, at least 2 planes.  Above, four lines in segments of 4 to 12 planes:
+// 200^3 172 and 41 us (two lines 190 and 43).
 template <typename T, int RY>
 inline void launch_filter3(const Grid3& g, const T* in, T* out, int target, int lo, cudaStream_t s) {
     const int cols = (g.n[0] + 31) / 32 * ((g.n[1] + RY - 1) / RY);
@@ -81,9 +104,14 @@ inline void launch_filter3(const Grid3& g, const T* in, T* out, int target, int 
     const int warps = cols * ((g.n[2] + seg - 1) / seg);
     k3_filter<T, RY><<<(warps + 3) / 4, 128, 0, s>>>(g, in, out, seg);
 }
+// Meshes that the node-by-node kernel filters faster, a pass within a step in us, it / the marching one: FP32 24^3 1.9 / 4.5,
+// 48^3 2.2 / 4.5, 64^3 3.8 / 5.0, 80^3 5.8 / 6.9, 96^3 8.6 / 8.6; FP64 24^3 2.8 / 6.1, 44^3 6.6 / 7.3, 48^3 7.7 / 7.3.
 template <typename T>
 inline void launch_filter3(const Grid3& g, const T* in, T* out, cudaStream_t s) {
-    if (size_t(g.n[0]) * g.n[1] * g.n[2] <= (size_t(1) << 21)) launch_filter3<T, 2>(g, in, out, 2432, 2, s);
+    const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
+    if (N <= (sizeof(T) == 4 ? size_t(1) << 19 : size_t(100000)))
+        k3_filter_nodes<<<int((N + 127) / 128), 128, 0, s>>>(g, in, out);
+    else if (N <= (size_t(1) << 21)) launch_filter3<T, 2>(g, in, out, 2432, 2, s);
     else launch_filter3<T, 4>(g, in, out, 1216, 4, s);
 }
 
