@@ -148,10 +148,9 @@ __global__ void k_jacobi(GridParams g, const double* omega, SweepWeights w, cons
 __global__ void k_jacobi_loop(GridParams g, const double* omega, SweepWeights w, const double* xn, double* xa,
                               double* xb, DevScalars* d, double eps, int mu, cudaGraphConditionalHandle h);
 // Small meshes: omega with all filter passes, and all sweeps (no tolerance) with Delta_gamma, in one launch each on tiles
-// in shared memory; false where the mesh is larger than TILE_NODES_PER_SM nodes per SM or the halo does not fit (nothing
-// launched).
+// in shared memory; false where the passes one by one are as fast (tile_shape) or the halo does not fit (nothing launched).
 constexpr int TILE_THREADS = 512;
-constexpr int TILE_NODES_PER_SM = 512;
+constexpr int TILE_NODES_PER_SM = 512;      // (2D)
 cudaError_t mesh64_prepare();
 bool launch_filter_tile(const GridParams& g, const MonitorParams& mp, const double* t0, const double* t1,
                         const double* t2, const DevScalars* d, int passes, double* omega, int nsm, cudaStream_t s);

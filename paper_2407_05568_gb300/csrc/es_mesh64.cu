@@ -552,23 +552,36 @@ __global__ void __launch_bounds__(TILE_THREADS) k_sweep_tile(GridParams g, const
     if (threadIdx.x == 0 && blockIdx.x == 0) d->sweeps = mu;
 }
 
-// The tile of a small mesh: 20 nodes wide in 2D (32 in 1D), and as tall as lets the tiles fill the SMs once.  False:
-// the mesh is not small, or the passes' halo does not pay or fit.
-bool tile_shape(const GridParams& g, int halo, int nsm, size_t doubles_per_node, int* bx, int* by, size_t* smem) {
-    const long long N = (long long)g.n1 * g.n2;
-    if (halo < 1 || N > (long long)nsm * TILE_NODES_PER_SM) return false;
+// The tile of a small mesh: 20 nodes wide in 2D (32 in 1D), and as tall as lets the tiles fill the SMs once.  False: the
+// passes one by one are as fast, or the halo does not fit.  Steps with all `halo` passes (or sweeps) in one launch / pass by
+// pass, us:
+//   1D, filter: 100 nodes and 5 passes 68 / 73, 64 passes 109 / 153; 14592 nodes (three tiles per SM) 124 / 126, 171 / 208;
+//     16000 116 / 113, 200 / 197; 77000 316 / 298, 577 / 402.
+//   1D, sweeps: 100 nodes and 5 sweeps 69 / 75, 64 99 / 194; 9728 (two tiles per SM) one sweep 110 / 109, 5 112 / 118; 14592 two
+//     126 / 124; 19456 (four per SM) 3 155 / 154, 5 157 / 159, 64 228 / 286; 24320 5 162 / 160, 10 169 / 170, 64 262 / 282; 28000 10
+//     171 / 173; 32000 10 177 / 173.
+//   2D, filter: 64 x 64 and 5 passes 248 / 254; 200 x 200 547 / 554; 270 x 280 1044 / 1059, 10 passes 1062 / 1084; 9000 x 8 1066 /
+//     1084.
+//   2D, sweeps: a tile forms the weights and the first sweeps of its halo again.  Tiles of 140 nodes (200 x 100) 10 sweeps 380 / 384;
+//     280 (200 x 200) 5 sweeps 555 / 557, 8 565 / 564, 10 574 / 572; 340 (215 x 215) 5 744 / 745, 8 755 / 753; 400 (230 x 230) 5
+//     814 / 812; 560 (270 x 280) one 1047 / 1045, 5 1061 / 1057; three tiles per SM (9000 x 8) 8 1093 / 1089.
+// (Halos of more than 10 nodes in 2D and 64 in 1D were not measured.)
+bool tile_shape(const GridParams& g, int halo, bool sweeps, int nsm, size_t doubles_per_node, int* bx, int* by, size_t* smem) {
+    if (halo < 1) return false;
     if (g.dim == 1) {
         *bx = 32;
         *by = 1;
-        if (halo > 64) return false;
+        const int per_sm = !sweeps ? 3 : (halo >= 10 ? 6 : (halo >= 5 ? 4 : 2));
+        if (halo > 64 || (g.n1 + *bx - 1) / *bx > per_sm * nsm) return false;
     } else {
         *bx = 20;
         const int ntx = (g.n1 + *bx - 1) / *bx;
         const int rows = nsm / ntx > 0 ? nsm / ntx : 1;      // tiles per column
         int b = (g.n2 + rows - 1) / rows;
         if (b < 4) b = 4;
-        if (halo > 10) return false;
         *by = b;
+        if (halo > 10 || (long long)g.n1 * g.n2 > (long long)nsm * TILE_NODES_PER_SM) return false;
+        if (sweeps && (ntx > nsm || *bx * b > 340 || *bx * b * halo > 2000)) return false;
     }
     const size_t box = size_t(*bx + 2 * halo) * (g.dim == 2 ? *by + 2 * halo : 1);
     *smem = sizeof(double) * box * doubles_per_node;
@@ -590,7 +603,7 @@ bool launch_filter_tile(const GridParams& g, const MonitorParams& mp, const doub
                         const double* t2, const DevScalars* d, int passes, double* omega, int nsm, cudaStream_t s) {
     int bx, by;
     size_t sm;
-    if (!tile_shape(g, passes, nsm, 2, &bx, &by, &sm)) return false;
+    if (!tile_shape(g, passes, false, nsm, 2, &bx, &by, &sm)) return false;
     k_filter_tile<<<tiles(g, bx, by), TILE_THREADS, sm, s>>>(g, mp, t0, t1, t2, d, passes, bx, by, omega);
     return true;
 }
@@ -599,7 +612,7 @@ bool launch_sweep_tile(const GridParams& g, const double* omega, const double* x
                        int nsm, cudaStream_t s) {
     int bx, by;
     size_t sm;
-    if (!tile_shape(g, mu, nsm, g.dim == 2 ? 9 : 5, &bx, &by, &sm)) return false;
+    if (!tile_shape(g, mu, true, nsm, g.dim == 2 ? 9 : 5, &bx, &by, &sm)) return false;
     k_sweep_tile<<<tiles(g, bx, by), TILE_THREADS, sm, s>>>(g, omega, xn, xout, mu, bx, by, d);
     return true;
 }

@@ -145,3 +145,31 @@ def test_3d_filter_kernels(shape, bc, precision):
     tol = 1e-11 if precision == "fp64" else 2e-5                     # the bounds of the forms' other redistributions
     assert abs(gam - gam_o) <= 10 * tol * gam_o
     assert np.abs(xd.cpu().numpy() - xd_o).max() <= tol * max(np.abs(xd_o).max(), 1e-3 * min(w["dxi"]) / 1e-3)
+
+
+@pytest.mark.parametrize("bc", ["periodic", "outflow", "reflect", "symmetry_lo"])
+@pytest.mark.parametrize("n,passes,sweeps", [(8, 64, 64), (9, 5, 3), (33, 64, 10), (100, 1, 1), (100, 65, 65), (511, 20, 64),
+                                             (9728, 5, 4), (9729, 5, 4), (14592, 5, 5), (14593, 64, 5), (19456, 5, 9),
+                                             (19457, 5, 9), (29184, 2, 10), (29185, 2, 10)])
+def test_redistribution_1d(n, passes, sweeps, bc):
+    """The line's tiles (filter passes, and sweeps, in one launch) and the pass-by-pass kernels at the edges of their ranges,
+    periodic lines shorter than the halo among them.  A rough state: its second differences are of the size of their factors, so
+    that their rounding stays that of the state.  The coordinates, of size 1, are rounded once a sweep; Delta_gamma divides
+    such differences by a node's displacement, of a spacing's size."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    x, d = wl.uniform_nodes(n, 0.0, 1.0, bc == "periodic")
+    w = wl.sine_1d(max(n, 8))
+    w.update(bc=(bc,), x=x[None].copy(), dxi=(d,), moving=True)
+    w["rho"], w["v"], w["p"] = wl.rough_state((n,), 5 + n, 1)
+    w["mesh"] = dict(monitor="vdw", alphas=(1200.0, 1200.0, 1200.0), kappa=2, filter_passes=passes, sweeps=sweeps, eps=0.0)
+    sch, mc, JU_o, J_o, x_o = oracle_setup(w)
+    dt = 1e-3
+    xd_o, sw_o, gam_o = stepper.redistribute(sch, mc, JU_o, J_o, x_o, dt)
+    ctx, JU, J, xt = gpu_setup(w)
+    xd = torch.empty_like(xt)
+    sw, gam = es.es_mesh_redistribute(ctx, JU, J, xt, dt, xd)
+    assert sw == sw_o
+    assert abs(gam - gam_o) <= 1e-14 * (4 + sweeps) * n * gam_o
+    assert np.abs(xd.cpu().numpy() - xd_o).max() * dt <= 1e-15 * (4 + sweeps)
