@@ -113,7 +113,7 @@ typedef struct es_params {
     int    tile;            /* stage tile shape: 0 = chosen by es_autotune (run by the first es_steps
                                if not called before); k = 1 .. ES_NTILES: shape k of the precision's
                                2D table (FP64: 32x8, 25x11, 16x16, 32x12, 20x10 nodes, on meshes that 20x10
-                               nodes cover with at most 152 tiles 8x8, 12x8, 16x8, 20x8, 20x10; mixed: 20x8 with
+                               nodes cover with one tile per SM at most 8x8, 12x8, 16x8, 20x8, 20x10; mixed: 20x8 with
                                two lanes per face, 25x6, 20x8, 20x14 with two lanes per face, 16x8); in 3D the
                                direction kernels' pencils, FP64:
                                1 = 16 nodes x 16 lines, 2 = 16 x 8, 3 = 16 x 4, 4 = 32 x 4; mixed:

@@ -152,9 +152,9 @@ cudaError_t launch_stage(es_ctx* c, const StageParams& P) {
     if (c->mixed) {
         StageParams Q = P;
         set_float_params(Q);
-        return launch_stage_mixed(Q, c->s_enq);
+        return launch_stage_mixed(Q, c->nsm, c->s_enq);
     }
-    return launch_stage_fp64(P, c->s_enq);
+    return launch_stage_fp64(P, c->nsm, c->s_enq);
 }
 
 const double RK_A[3] = {0.0, 0.75, 1.0 / 3.0};

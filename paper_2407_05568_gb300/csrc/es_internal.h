@@ -85,8 +85,9 @@ inline void set_float_params(StageParams& P) {
     }
 }
 
-cudaError_t launch_stage_fp64(const StageParams& P, cudaStream_t s);
-cudaError_t launch_stage_mixed(const StageParams& P, cudaStream_t s);
+// nsm: the SMs of the device, for the choice of the shape
+cudaError_t launch_stage_fp64(const StageParams& P, int nsm, cudaStream_t s);
+cudaError_t launch_stage_mixed(const StageParams& P, int nsm, cudaStream_t s);
 // 2D tile shapes of the stage kernels; the autotuner times each on the caller's problem
 constexpr int STAGE_NTILES = 5;
 // set the kernels' shared-memory attributes (call outside any stream capture)

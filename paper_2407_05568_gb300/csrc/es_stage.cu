@@ -567,7 +567,7 @@ static cudaError_t launch_tile(const StageParams& P, cudaStream_t s) {
 // 114 with 20 x 8 against 138; the shapes of larger meshes take at least the last).  Above one wave 20 x 10 nodes and less
 // cost more halo than they balance (170 x 170: 166 us in one wave; 200 x 200: 192 against 176 with 25 x 11).
 // All shapes give the same bits.  1D: by the line's length (launch_stage_fp64).
-static bool small_mesh(const StageParams& P) { return (P.n1 + 19) / 20 * ((P.n2 + 9) / 10) <= 152; }
+static bool small_mesh(const StageParams& P, int nsm) { return (P.n1 + 19) / 20 * ((P.n2 + 9) / 10) <= nsm; }
 cudaError_t stage_prepare_fp64(int dim) {
     if (dim == 1) {
         cudaError_t e1 = prepare_tile<1, 254, 1, 256>();
@@ -585,21 +585,21 @@ cudaError_t stage_prepare_fp64(int dim) {
     return e;
 }
 
-cudaError_t launch_stage_fp64(const StageParams& P, cudaStream_t s) {
+cudaError_t launch_stage_fp64(const StageParams& P, int nsm, cudaStream_t s) {
     if (P.dim == 1) {
         // measured per stage launch (us), 8-node lines / 62-node tiles / 254-node tiles: 200 nodes 16.4 / 28.7 / 61.5,
         // 1600 20.5 / 28.7 / 62.5, 6400 49.2 / 28.7 / 63.5, 25600 164 / 47.2 / 61.5, 102400 621 / 176 / 172.  A line is
         // spread over an SM's four schedulers, so it pays while an SM has two of them or fewer (152 SMs x 2 x 8 nodes);
         // 62-node tiles (faces, pairs and nodes two, six and two full warps of four) while the 254-node ones, which
         // repeat less of the halo, leave SMs idle
-        if (P.n1 <= 2 * 152 * LINE) {
+        if (P.n1 <= 2 * nsm * LINE) {
             stage_line_fp64<<<(P.n1 + LINE - 1) / LINE, 128, 0, s>>>(P);
             return cudaGetLastError();
         }
-        if (P.n1 <= 1 << 16) return launch_tile<1, 62, 1, 128>(P, s);
+        if ((long long)P.n1 * 152 <= 65536LL * nsm) return launch_tile<1, 62, 1, 128>(P, s);     // (431 nodes per SM)
         return launch_tile<1, 254, 1, 256>(P, s);
     }
-    if (small_mesh(P)) {
+    if (small_mesh(P, nsm)) {
         switch (P.tile) {
             case 1: return launch_tile<2, 12, 8, 128>(P, s);
             case 2: return launch_tile<2, 16, 8, 160>(P, s);

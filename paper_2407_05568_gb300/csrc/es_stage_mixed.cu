@@ -422,7 +422,6 @@ cudaError_t launch_tile_f(const StageParams& P, cudaStream_t s) {
 constexpr int LINE_BX = 254, SHORT_BX = 58, LINE_NT = 256;
 using LineTile = TileF<LINE_BX, LINE_NT>;
 using ShortTile = TileF<SHORT_BX, LINE_NT>;
-constexpr int SHORT_MAX = SHORT_BX * 2 * 152;
 
 }  // namespace
 
@@ -443,9 +442,9 @@ cudaError_t stage_prepare_mixed(int dim) {
     return e;
 }
 
-cudaError_t launch_stage_mixed(const StageParams& P, cudaStream_t s) {
+cudaError_t launch_stage_mixed(const StageParams& P, int nsm, cudaStream_t s) {
     if (P.dim == 1) {
-        if (P.n1 <= SHORT_MAX)
+        if (P.n1 <= 2 * nsm * SHORT_BX)
             stage_kernel_mixed1<SHORT_BX, LINE_NT><<<(P.n1 + SHORT_BX - 1) / SHORT_BX, LINE_NT, ShortTile::SMEM, s>>>(P);
         else
             stage_kernel_mixed1<LINE_BX, LINE_NT><<<(P.n1 + LINE_BX - 1) / LINE_BX, LINE_NT, LineTile::SMEM, s>>>(P);

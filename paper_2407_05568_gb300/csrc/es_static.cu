@@ -34,18 +34,20 @@ __device__ __align__(256) double g_static_scratch[SCRATCH_DOUBLES];
 std::mutex g_setup_mutex;
 double* g_scratch_ptr[MAX_DEVICES];
 int g_prepared[MAX_DEVICES][3];            // stage kernel attributes set, per dim
+int g_nsm[MAX_DEVICES];
 
 // Device address of the scratch array on the current device (looked up once
 // per device with that device current), and the stage kernel's shared-memory
 // attribute for this dimension.  Under lazy module loading the symbol lookup is
 // also what loads this library's modules, and with them the array.
-int setup_current_device(int dim, double** out) {
+int setup_current_device(int dim, double** out, int* nsm) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return ES_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g_setup_mutex);
     if (!g_scratch_ptr[dev]) {
         void* ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return ES_ERR_CUDA;
+        if (cudaDeviceGetAttribute(&g_nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return ES_ERR_CUDA;
         g_scratch_ptr[dev] = static_cast<double*>(ptr);
     }
     if (!g_prepared[dev][dim]) {
@@ -53,6 +55,7 @@ int setup_current_device(int dim, double** out) {
         g_prepared[dev][dim] = 1;
     }
     *out = g_scratch_ptr[dev];
+    *nsm = g_nsm[dev];
     return ES_OK;
 }
 
@@ -80,7 +83,8 @@ extern "C" int es_rk3_step_static(const es_params* p, double dt, double* JU, dou
                                   const double* xdot, void* stream) {
     if (!params_ok(p) || !JU || !J || !x || !(dt >= 0.0)) return ES_ERR_ARG;
     double* scratch = nullptr;
-    int rc = setup_current_device(p->dim, &scratch);
+    int nsm = 0;
+    int rc = setup_current_device(p->dim, &scratch, &nsm);
     if (rc != ES_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DevStatus* status = reinterpret_cast<DevStatus*>(scratch);
@@ -145,7 +149,7 @@ extern "C" int es_rk3_step_static(const es_params* p, double dt, double* JU, dou
         P.Js = srcJ[st];
         P.JUo = dstU[st];
         P.Jo = dstJ[st];
-        if (launch_stage_fp64(P, s) != cudaSuccess) return ES_ERR_CUDA;
+        if (launch_stage_fp64(P, nsm, s) != cudaSuccess) return ES_ERR_CUDA;
     }
     DevStatus host_status = {0, 0};
     if (cudaMemcpyAsync(&host_status, status, sizeof(DevStatus), cudaMemcpyDeviceToHost, s) != cudaSuccess)
