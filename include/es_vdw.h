@@ -334,9 +334,11 @@ int es_mesh_stats(es_ctx* ctx, int64_t* sweeps_total, int64_t* solves, int64_t* 
  *             when act_tanh, which needs `out`), writes grad_w = dL/dw and
  *             grad_b = dL/db (summed over the batch, in a fixed order) and, if
  *             grad_in is non-null, grad_in = dL/d(in).
- * workspace: device scratch of at least es_nn_workspace_bytes(B, Cin, Cout, H, W)
- * bytes (forward needs only Cout*Cin*9 floats).  Returns ES_ERR_ARG for bad
- * shapes, null pointers or aliasing outputs. */
+ * workspace: device scratch of at least es_nn_workspace_bytes(B, Cin, Cout, H, W) bytes (0: unsupported shape): the
+ * backward call's partial weight and bias gradients.  es_nn_conv_forward uses none, and still asks for a workspace of
+ * Cout*Cin*9 floats, as it did when it kept the weights as floats there.  Returns ES_ERR_ARG for bad shapes, null
+ * pointers or aliasing outputs.
+ */
 size_t es_nn_workspace_bytes(int B, int Cin, int Cout, int H, int W);
 /* Forward layer on the tensor cores (the warm start's inference path): the same
  * correlation with the layer input rounded to bf16 (round to nearest even), bf16

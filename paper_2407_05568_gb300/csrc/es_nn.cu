@@ -6,8 +6,7 @@
 // The FP32 layers run on the tensor cores with their operands split into three bf16
 // parts (k_conv_fwd_s3, k_conv_wgrad_s3), the inference path on bf16 operands.
 //
-// Layout: activations [B][C][H][W] float; weights [Cout][Cin][3][3] (bf16 in the
-// C ABI, float inside the context); cross-correlation with zero padding:
+// Layout: activations [B][C][H][W] float; weights [Cout][Cin][3][3] bf16; cross-correlation with zero padding:
 //   out[co](y, x) = bias[co] + sum_{ci, dy, dx} w[co][ci][dy+1][dx+1] in[ci](y+dy, x+dx).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -810,7 +809,7 @@ size_t es_nn_workspace_bytes(int B, int Cin, int Cout, int H, int W) {
     const size_t gx = (W + TS - 1) / TS, gy = ((H + TS - 1) / TS + rows - 1) / rows;
     const size_t strips = size_t(B) * gx * gy;
     const size_t len = size_t(Cout) * Cin * 9 + Cout;
-    return sizeof(float) * (size_t(Cout) * Cin * 9 + strips * len);
+    return sizeof(float) * strips * len;
 }
 
 int es_nn_conv_forward(const float* in, const uint16_t* w, const float* bias, float* out, int B, int Cin, int Cout,
@@ -839,7 +838,7 @@ int es_nn_conv_backward(const float* in, const uint16_t* w, const float* out, fl
     if (workspace_bytes < es_nn_workspace_bytes(B, Cin, Cout, H, W)) return ES_ERR_ARG;
     if (grad_in && (grad_in == grad_out || grad_in == in)) return ES_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    float* partial = (float*)workspace + size_t(Cout) * Cin * 9;
+    float* partial = (float*)workspace;
     const int rows = strip_rows(B, H, W);
     const dim3 grid((W + TS - 1) / TS, ((H + TS - 1) / TS + rows - 1) / rows, B);
     const float* aout = act_tanh ? out : nullptr;            // the gradient through tanh is formed in the same pass

@@ -89,3 +89,9 @@ def test_null_context_rejected(L):
     assert L.es_steps(None, None, None, None, 1, ctypes.c_double(1.0)) == es.ES_ERR_ARG
     assert L.es_launch_count(None) == 0
     assert L.es_batch_check(None) == es.ES_ERR_ARG
+
+
+@pytest.mark.parametrize("B,Cin,Cout,H,W,strips", [(1, 4, 32, 16, 16, 1), (2, 32, 32, 17, 16, 4), (1, 2, 2, 1, 33, 3)])
+def test_nn_workspace_is_the_partial_gradients(L, B, Cin, Cout, H, W, strips):
+    """One set of weight and bias gradients for every strip of tiles, and nothing else."""
+    assert L.es_nn_workspace_bytes(B, Cin, Cout, H, W) == 4 * strips * (Cout * Cin * 9 + Cout)

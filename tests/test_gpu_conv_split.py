@@ -176,3 +176,26 @@ def test_weight_gradient_of_a_tall_image():
     es.es_nn_conv_backward(a, torch.zeros((2, 2, 3, 3), dtype=torch.bfloat16, device="cuda"), None, go, None, gw, gb, False, ws)
     assert abs(float(gw[1, 0, 1, 1]) / (float(x) * float(g) * H * W) - 1.0) <= 4.8e-7
     assert abs(float(gb[1]) / (float(g) * H * W) - 1.0) <= 4.8e-7
+
+
+@pytest.mark.parametrize("cin,cout,shape", [(4, 32, (1, 16, 16)), (32, 32, (2, 50, 33)), (32, 2, (1, 64, 64))])
+def test_backward_stays_in_its_workspace(cin, cout, shape):
+    """The backward call with exactly the bytes that es_nn_workspace_bytes asks for: nothing behind them is written, and the
+    gradients are those of a call with a larger workspace."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    B, H, W = shape
+    gen = torch.Generator(device="cuda").manual_seed(cin + cout)
+    a = torch.randn((B, cin, H, W), generator=gen, device="cuda")
+    g = torch.randn((B, cout, H, W), generator=gen, device="cuda")
+    w = torch.randn((cout, cin, 3, 3), generator=gen, device="cuda").to(torch.bfloat16)
+    n = es.es_nn_workspace_bytes(B, cin, cout, H, W) // 4
+    whole = torch.full((n + 4096,), 7.0, device="cuda")
+    got = []
+    for ws in (whole[:n], torch.empty(2 * n, device="cuda")):
+        gw, gb, gin = torch.empty((cout, cin, 3, 3), device="cuda"), torch.empty(cout, device="cuda"), torch.empty_like(a)
+        es.es_nn_conv_backward(a, w, None, g.clone(), gin, gw, gb, False, ws)
+        got.append((gw, gb, gin))
+    assert bool((whole[n:] == 7.0).all())
+    assert all(torch.equal(p, q) for p, q in zip(*got))
