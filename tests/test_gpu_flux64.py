@@ -122,3 +122,103 @@ def test_2d_small_mesh_shapes(n1, n2, bc):
         assert np.abs(outs[0][0][c] - dU_o[c]).max() < 1e-12 * flux
     for o in outs[1:]:
         assert np.array_equal(o[0], outs[0][0]) and np.array_equal(o[1], outs[0][1])
+
+
+def _large_mesh(case):
+    """Meshes that 20 x 10 tiles cover with more than 152 tiles: the five shapes of large meshes."""
+    from paper_2407_05568_gb300 import workloads as wl
+    from test_gpu_parity import _ragged_riemann
+    if case == "riemann":
+        w = _ragged_riemann(230, 170, seed=6)
+        w["xdot"] = np.zeros_like(w["x"])
+        return w
+    if case == "wavy":
+        w = wl.sine_2d(188)
+        X, Y = w["x"]
+        w["x"], w["xdot"] = wl.wavy_mesh_2d(X, Y), wl.mesh_velocity_2d(X, Y)
+        w["rho"], w["v"], w["p"] = wl.rough_state(X.shape, 11, 2)
+        return w
+    x1, d1 = wl.uniform_nodes(201, 0.0, 1.0, False)
+    x2, d2 = wl.uniform_nodes(183, 0.0, 1.0, False)
+    X, Y = np.meshgrid(x1, x2)
+    w = wl.sine_2d(16)
+    w.update(bc=("symmetry_lo", "reflect"), x=np.stack([X, Y]), dxi=(d1, d2), n=(183, 201))
+    w["rho"], w["v"], w["p"] = wl.rough_state((183, 201), 5, 2)
+    w["xdot"] = 0.05 * np.stack([np.sin(np.pi * X) * np.cos(np.pi * Y), np.sin(np.pi * Y) * np.cos(np.pi * X)])
+    w["xdot"][0][:, [0, -1]] = w["xdot"][1][[0, -1]] = 0.0
+    w["xdot"][1][:, -1] = 0.0
+    return w
+
+
+@pytest.mark.parametrize("dissipation", [True, False])
+@pytest.mark.parametrize("case", ["riemann", "wavy", "walls"])
+def test_2d_large_mesh_shapes(case, dissipation):
+    """The five shapes of large 2D meshes (among them 32 x 12 nodes, whose directions follow one another): right-hand sides
+    and an RK stage with curved metrics and a mesh velocity, the same bits from every shape, and the first against the oracle
+    (the bounds of the other parity tests)."""
+    import torch
+
+    from oracle import operator as op
+    from oracle import stepper
+    from paper_2407_05568_gb300 import es
+    from sides import gpu_setup, oracle_setup, rel_l1
+    w = _large_mesh(case)
+    assert -(-w["n"][1] // 20) * -(-w["n"][0] // 10) > 152
+    sch, _, JU_o, J_o, x_o = oracle_setup(w, dissipation=dissipation)
+    dU_o, dJ_o = op.rhs(sch, JU_o, J_o, x_o, w["xdot"])
+    dt = 0.1 * min(w["dxi"])
+    U1_o, J1_o = stepper.rk_stage(sch, 1, dt, JU_o, J_o, JU_o, J_o, x_o, w["xdot"])
+    _, JU, J, xt = gpu_setup(w, dissipation=dissipation)
+    xd = torch.tensor(np.ascontiguousarray(w["xdot"]), dtype=torch.float64, device="cuda")
+    outs = []
+    for tile in (1, 2, 3, 4, 5):
+        ctx = es.es_create(es.make_params(w, dissipation=dissipation, tile=tile))
+        out = [torch.empty_like(a) for a in (JU, J, JU, J)]
+        es.es_rhs(ctx, JU, J, xt, xd, out[0], out[1])
+        es.es_rk_stage(ctx, 2, dt, JU, J, JU, J, xt, xd, out[2], out[3])
+        assert es.es_check(ctx) == 0, es.es_last_error(ctx)
+        outs.append(out)
+    for out in outs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(out, outs[0]))
+    dU, dJ, U1, J1 = [a.cpu().numpy() for a in outs[0]]
+    h = min(w["dxi"])
+    assert np.abs(dU - dU_o).sum() < 1e-12 * np.abs(JU_o).sum() / h
+    assert np.abs(dJ - dJ_o).sum() < 1e-12 * np.abs(J_o).sum() / h
+    assert rel_l1(U1, U1_o) < 1e-12 and rel_l1(J1, J1_o) < 1e-12
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("shape", [(200,), (3000,), (40, 36), (230, 170)])
+def test_nan_state_is_reported_and_stays_local(shape, precision):
+    """A NaN in the density or the energy of one node: the state is refused, and right-hand sides out of the stencil's reach
+    (three nodes along each direction) are those without it."""
+    import torch
+
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    from sides import gpu_setup
+    w = wl.sine_1d(shape[0]) if len(shape) == 1 else wl.sine_2d(16)
+    if len(shape) == 2:
+        x1, d1 = wl.uniform_nodes(shape[1], 0.0, 1.0, True)
+        x2, d2 = wl.uniform_nodes(shape[0], 0.0, 1.0, True)
+        w.update(x=np.stack(np.meshgrid(x1, x2)), dxi=(d1, d2), n=shape)
+    w["rho"], w["v"], w["p"] = wl.rough_state(shape, 7, len(shape))
+    ctx, JU, J, xt = gpu_setup(w, precision=precision)
+    clean = [torch.empty_like(JU), torch.empty_like(J)]
+    es.es_rhs(ctx, JU, J, xt, None, *clean)
+    assert es.es_check(ctx) == 0
+    at = tuple(s // 3 for s in shape)
+    far = np.ones(shape, bool)
+    for k in range(len(shape)):
+        cut = list(at)
+        cut[k] = slice(at[k] - 3, at[k] + 4)
+        far[tuple(cut)] = False
+    far = torch.tensor(far, device="cuda")
+    for c in (0, len(shape) + 1):
+        bad = JU.clone()
+        (bad if precision == "fp64" else bad[0])[(c,) + at] = float("nan")
+        dU, dJ = torch.empty_like(JU), torch.empty_like(J)
+        es.es_rhs(ctx, bad, J, xt, None, dU, dJ)
+        assert es.es_check(ctx) == es.ES_ERR_INADMISSIBLE
+        assert torch.equal(dU[..., far], clean[0][..., far])
+        assert bool(torch.isnan(dU[(..., c) + at] if precision == "fp64" else dU[(0, c) + at]).all())
