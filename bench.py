@@ -565,7 +565,7 @@ def measure_precision_sweep(args, dev, cases=None):
         for prec in ("fp64", "mixed"):
             rho, steps, ms, tile = run_to_end(w, prec, dev, dt_fixed=dt_fixed)
             res[prec] = rho
-            bx, by, _ = TILES[prec][tile] if w["dim"] == 2 else (254, 1, 256)
+            (bx, by, _), _ = stage_shape(prec, w["x"].shape[:0:-1], tile, sm_count())
             row[prec] = {"l1_vs_exact": float(np.abs(rho - exact).mean()), "steps": steps, "ms": ms,
                          "cell_updates_per_s": nodes * 3 * (steps - 1) / (ms * 1e-3) if ms > 0 else None,
                          "tile": f"{bx}x{by}"}
@@ -794,13 +794,38 @@ def pin(a):
     return t.numpy()
 
 
-# (nodes along xi_1, along xi_2, threads) of each tile shape; the mixed 384- and 320-thread shapes give two lanes
-# to each face
+# (nodes along xi_1, along xi_2, threads) of each 2D tile shape (es_params.tile); the mixed 384- and 608-thread shapes give
+# two lanes to each face.  An FP64 mesh that 20 x 10 nodes cover with one tile per SM at most has shapes of its own.
 TILES = {"fp64": {1: (32, 8, 288), 2: (25, 11, 384), 3: (16, 16, 288), 4: (32, 12, 416), 5: (20, 10, 224)},
+         "fp64 small": {1: (8, 8, 128), 2: (12, 8, 128), 3: (16, 8, 160), 4: (20, 8, 192), 5: (20, 10, 224)},
          "mixed": {1: (20, 8, 384), 2: (25, 6, 192), 3: (20, 8, 192), 4: (20, 14, 608), 5: (16, 8, 160)}}
+
+
+def stage_shape(precision, n, tile, nsm):
+    """(nodes along xi_1, along xi_2, threads) of the stage kernel's tile on a mesh of n = (n1,) or (n1, n2) nodes, on a
+    device of nsm SMs, and the kernel's name: the library's rules (launch_stage_fp64, launch_stage_mixed)."""
+    if len(n) == 1:
+        if precision == "mixed":
+            bx = 58 if n[0] <= 2 * nsm * 58 else 254
+            return (bx, 1, 256), f"stage_kernel_mixed1<{bx},256>"
+        if n[0] <= 2 * nsm * 8:
+            return (8, 1, 128), "stage_line_fp64"
+        bx, nt = (62, 128) if n[0] * 152 <= 65536 * nsm else (254, 256)
+        return (bx, 1, nt), f"stage_kernel_fp64<1,{bx},1,{nt}>"
+    small = precision == "fp64" and -(-n[0] // 20) * -(-n[1] // 10) <= nsm
+    bx, by, nt = TILES["fp64 small" if small else precision][tile]
+    name = f"stage_kernel_fp64<2,{bx},{by},{nt}>" if precision == "fp64" else f"stage_kernel_mixed2<{bx},{by},{nt}>"
+    return (bx, by, nt), name
+
+
+def sm_count():
+    import torch
+    return torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+
+
 # dram__bytes_read.sum + dram__bytes_write.sum per launch at 200 x 200, from one ncu capture of each
 # kernel as it is now (a kernel changed since its capture has no entry); other sizes were not captured
-TRAFFIC_200 = {"stage_kernel_fp64<2,25,11,384>": 3032064 + 0}
+TRAFFIC_200 = {"stage_kernel_fp64<2,25,11,384>": 2352384 + 0}
 
 
 def stage_roofline(es, ctx, JU, J, x, stream, w, nodes, precision, tile):
@@ -818,12 +843,12 @@ def stage_roofline(es, ctx, JU, J, x, stream, w, nodes, precision, tile):
     peak = f64 if precision == "fp64" else f32
     nominal = perfmodel.fp64_peak_tflops(peaks) if precision == "fp64" else perfmodel.fp32_peak_tflops(peaks)
     achieved = flops / (ms * 1e-3) / 1e12
-    bx, by, nt = TILES[precision][tile]
-    kname = ("stage_kernel_fp64" if precision == "fp64" else "stage_kernel_mixed") + f"<2,{bx},{by},{nt}>"
+    (bx, by, nt), kname = stage_shape(precision, w["x"].shape[:0:-1], tile, sm_count())
     return {"bound": "alu", "kernel": kname, "tile": f"{bx}x{by}/{nt}",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": TRAFFIC_200.get(kname) if nodes == 200 * 200 else None, "launch_ms": ms,
             "flops_per_launch": flops,
+            "flops_counted": "the plain evaluation's (perfmodel); the kernel shares and folds operations and does fewer",
             "peak_source": ("measured in this run: es_selftest_peaks, FMA chains on every SM, best of 5 launches "
                             f"({'FP64' if precision == 'fp64' else 'FP32'}); of measured"),
             "nominal_peak": nominal}
