@@ -12,7 +12,8 @@
 //   * the logarithms come from a table (es_log64.cuh), and the differences of the entropy variables that every face's
 //     reconstruction starts from are formed once per pair of neighbours.
 // Every product that feeds an addition is written as fma() or __dmul_rn(), so that the compiler has no choice of which
-// product to fuse and every tile shape gives the same bits.
+// product to fuse and the tile shapes of a kernel give the same bits.  (The 1D line shared by four warps, es_stage.cu, adds
+// a face's waves in another order than face_dissipation.)
 // Instructions on the FP64 pipe at a 2D pair: 140 before this form, 78 now; at a 2D face: about 1000 and 600.
 #pragma once
 #include <cuda_runtime.h>
@@ -442,8 +443,12 @@ __device__ __forceinline__ int jump_is_zero(const SwitchBounds& b, const Face<D>
         hi = scale * (b.vs + (b.H + rest) * b.es + (b.vsum + b.c) * b.qs);
     }
     const float ja = abs_f(j);
-    // (factors: truncation and rounding of the FP32 values)
-    if ((ja * 1.0001f < lo * 0.99f && ja > 0.0f) || (__double_as_longlong(j) << 1) == 0) return 1;
+    // (factors: truncation and rounding of the FP32 values; bounds that leave FP32's range, in units of extreme size, decide
+    // nothing)
+    if ((__double_as_longlong(j) << 1) == 0) return 1;
+    if (b.tol == 0.0f) return 0;
+    if (!(hi < 1e38f) || hi < 1e-30f) return 2;
+    if (ja * 1.0001f < lo * 0.99f) return 1;
     return ja > hi * 1.001f ? 0 : 2;
 }
 // the size itself

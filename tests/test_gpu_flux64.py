@@ -222,3 +222,38 @@ def test_nan_state_is_reported_and_stays_local(shape, precision):
         assert es.es_check(ctx) == es.ES_ERR_INADMISSIBLE
         assert torch.equal(dU[..., far], clean[0][..., far])
         assert bool(torch.isnan(dU[(..., c) + at] if precision == "fp64" else dU[(0, c) + at]).all())
+
+
+@pytest.mark.parametrize("power", [-90, 90])
+@pytest.mark.parametrize("shape", [(64,), (200, 24), (9, 10, 11)])
+def test_units_of_extreme_size(shape, power):
+    """A flow in units in which velocities are 2^+-90 times the usual ones (energies leave the range of FP32, in whose bounds the
+    sign switch decides the clear cases): right-hand sides against the oracle to 1e-12 of a flux difference."""
+    import torch
+
+    from oracle import operator as op
+    from paper_2407_05568_gb300 import es
+    from paper_2407_05568_gb300 import workloads as wl
+    from sides import gpu_setup, oracle_setup
+    dim, u = len(shape), 2.0 ** power
+    if dim == 3:
+        from test_gpu_3d import _box
+        w = _box(*shape[::-1], True, amp=0.005)
+    else:
+        w = wl.sine_1d(shape[0]) if dim == 1 else wl.sine_2d(16)
+        if dim == 2:
+            x1, d1 = wl.uniform_nodes(shape[1], 0.0, 1.0, True)
+            x2, d2 = wl.uniform_nodes(shape[0], 0.0, 1.0, True)
+            w.update(x=np.stack(np.meshgrid(x1, x2)), dxi=(d1, d2), n=shape)
+    w["rho"], w["v"], w["p"] = wl.rough_state(shape, 7, dim)
+    g = w["gas"]
+    w.update(gas=dict(a=g["a"] * u * u, b=g["b"], R=g["R"] * u * u, cv=g["cv"] * u * u), v=w["v"] * u, p=w["p"] * u * u)
+    sch, _, JU_o, J_o, x_o = oracle_setup(w)
+    dU_o, _ = op.rhs(sch, JU_o, J_o, x_o, np.zeros_like(x_o))
+    ctx, JU, J, xt = gpu_setup(w)
+    dU, dJ = torch.empty_like(JU), torch.empty_like(J)
+    es.es_rhs(ctx, JU, J, xt, None, dU, dJ)
+    assert es.es_check(ctx) == 0, es.es_last_error(ctx)
+    for c in range(dim + 2):
+        flux = np.abs(JU_o[c]).max() * u * 4.0 / min(w["dxi"])
+        assert np.abs(dU[c].cpu().numpy() - dU_o[c]).max() < 1e-12 * flux
