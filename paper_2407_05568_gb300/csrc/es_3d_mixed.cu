@@ -98,8 +98,8 @@ __global__ void k3_nodes_f(Grid3 g, GasF G, const float* JU, const float* J, flo
 }
 
 // ---------------------------------------------------------------- direction kernels
-// Bound by instruction issue at the occupancy that 96 registers leave (96^3, 32 x 4 pencils: 50 M warp instructions,
-// half of the issue slots busy, the rest waits at the barriers between the phases and on shared memory; DRAM at 20%).
+// Bound by instruction issue at the occupancy that 96 registers leave (96^3, 32 x 4 pencils: 61 to 63 M warp instructions,
+// 54 to 62% of the issue slots busy, the rest waits at the barriers between the phases and on shared memory; DRAM at 20%).
 // With means of unhalved scalar fields, whole values W_j - W_l and exact divisions the three directions took 130, 141 and
 // 159 us at 96^3; on es_flux32.cuh's forms 72, 89 and 87 us.
 struct Dir3FParams {

@@ -5,7 +5,7 @@
 // node in 2D before this form), so, as in the FP64 form: nodes keep HALF of every field that a face reads as the mean of
 // its two nodes, quantities are formed in the products that the formulas need, the jump of the entropy variables takes
 // the means of the pair flux between the same nodes, and MR-WENO5 works on halved differences.  Reciprocals and
-// reciprocal square roots are the hardware's approximations (1 and 2 ulp).
+// reciprocal square roots are the hardware's approximations (1 and 2 ulp; subnormal arguments count as zero).
 #pragma once
 #include <cuda_runtime.h>
 

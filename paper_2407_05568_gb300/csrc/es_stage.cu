@@ -566,7 +566,8 @@ static cudaError_t launch_tile(const StageParams& P, cudaStream_t s) {
 // Riemann stage, us: 64 x 64 74 with 8 x 8 nodes against 137 with 20 x 10, 120 x 120 83 with 12 x 8 against 139, 140 x 140
 // 114 with 20 x 8 against 138; the shapes of larger meshes take at least the last).  Above one wave 20 x 10 nodes and less
 // cost more halo than they balance (170 x 170: 166 us in one wave; 200 x 200: 192 against 176 with 25 x 11).
-// All shapes give the same bits.  1D: by the line's length (launch_stage_fp64).
+// All 2D shapes give the same bits.  1D: by the line's length (launch_stage_fp64); the 62- and 254-node tiles give the same
+// bits, the 8-node line adds the waves of a face in another order.
 static bool small_mesh(const StageParams& P, int nsm) { return (P.n1 + 19) / 20 * ((P.n2 + 9) / 10) <= nsm; }
 cudaError_t stage_prepare_fp64(int dim) {
     if (dim == 1) {

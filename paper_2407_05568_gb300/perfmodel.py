@@ -50,7 +50,8 @@ def mesh_bytes_per_node(precision, filter_passes, sweeps):
 
     FP64 form, in 8-byte words: monitor fields (JU, J -> rho, G) 7, monitor terms (rho, G -> three terms) 5,
     omega 4, each filter pass 2, each Jacobi sweep (omega, x -> x) 5, the limiter inside the last sweep (x^n) 2,
-    velocity (x^n, x^mu -> xdot) 6.
+    velocity (x^n, x^mu -> xdot) 6.  (The kernels store the sweeps' four weights and read them in place of omega:
+    three words more a sweep, which save FP64 instructions and are not counted as compulsory.)
     Mixed form, in bytes: the FP32 displacement from x (16 + 8), the fused monitor on the (hi, lo) state
     (40 + 12), omega and all filter passes in one tile kernel (12 + 4), all Jacobi sweeps and the limiter in
     one tile kernel (omega, d -> d: 4 + 8 + 8; the limiter reads the sweeps' own values), velocity (d, d^mu ->
