@@ -858,7 +858,7 @@ int d3_mesh(Ctx3* d, const void* JU, const void* J, const double* xn, double* xd
     double* om = d->om0;
     double* other = d->om1;
     for (int k = 0; k < d->filter_passes; ++k) {
-        launch_filter3(d->g, om, other, s);
+        launch_filter3(d->g, om, other, d->nsm, s);
         ++n;
         double* t = om;
         om = other;

@@ -28,6 +28,7 @@ struct Ctx3 {
     int filter_passes, sweeps;
     double eps;
     int grid;                 // blocks of the grid-stride kernels
+    int nsm;                  // SMs of the device
     int shape;                // pencil shape of the direction kernels (D3_NSHAPES of them, see es_3d.cu)
     size_t N;                 // nodes
     size_t NE;                // nodes of the grid extended by 3 ghosts in every direction

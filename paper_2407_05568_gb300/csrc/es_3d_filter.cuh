@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(128) k3_filter_nodes(Grid3 g, const T* __restr
 }
 
 // Lines per warp and planes per segment.  A warp's planes follow one another (a load's latency each), so on meshes of up to
-// 2^21 nodes short segments and two lines keep the launch short although they sum more planes and rows twice: four warps on
-// each of the 608 schedulers where the mesh gives them, at least 2 planes.  Above, four lines in segments of 4 to 12 planes:
+// 2^21 nodes short segments and two lines keep the launch short although they sum more planes and rows twice: 16 warps on
+// each SM where the mesh gives them, at least 2 planes.  Above, four lines in segments of 4 to 12 planes:
 // 200^3 172 and 41 us (two lines 190 and 43).
 template <typename T, int RY>
 inline void launch_filter3(const Grid3& g, const T* in, T* out, int target, int lo, cudaStream_t s) {
@@ -107,12 +107,12 @@ inline void launch_filter3(const Grid3& g, const T* in, T* out, int target, int 
 // Meshes that the node-by-node kernel filters faster, a pass within a step in us, it / the marching one: FP32 24^3 1.9 / 4.5,
 // 48^3 2.2 / 4.5, 64^3 3.8 / 5.0, 80^3 5.8 / 6.9, 96^3 8.6 / 8.6; FP64 24^3 2.8 / 6.1, 44^3 6.6 / 7.3, 48^3 7.7 / 7.3.
 template <typename T>
-inline void launch_filter3(const Grid3& g, const T* in, T* out, cudaStream_t s) {
+inline void launch_filter3(const Grid3& g, const T* in, T* out, int nsm, cudaStream_t s) {
     const size_t N = size_t(g.n[0]) * g.n[1] * g.n[2];
     if (N <= (sizeof(T) == 4 ? size_t(1) << 19 : size_t(100000)))
         k3_filter_nodes<<<int((N + 127) / 128), 128, 0, s>>>(g, in, out);
-    else if (N <= (size_t(1) << 21)) launch_filter3<T, 2>(g, in, out, 2432, 2, s);
-    else launch_filter3<T, 4>(g, in, out, 1216, 4, s);
+    else if (N <= (size_t(1) << 21)) launch_filter3<T, 2>(g, in, out, 16 * nsm, 2, s);
+    else launch_filter3<T, 4>(g, in, out, 8 * nsm, 4, s);
 }
 
 }  // namespace es

@@ -1214,7 +1214,7 @@ int d3f_mesh(Ctx3* d, const void* JU, const void* J, const double* xn, double* x
     k_mon_omega_f<<<G, 256, 0, s>>>(flat, d->mon, t0, t1, t2, dv, om);
     n += 3;
     for (int k = 0; k < d->filter_passes; ++k) {
-        launch_filter3(d->g, om, other, s);
+        launch_filter3(d->g, om, other, d->nsm, s);
         ++n;
         float* t = om;
         om = other;

@@ -738,6 +738,7 @@ int es_create(es_ctx** out, const es_params* p, void* stream) {
         d->eps = p->jacobi_eps;
         const size_t blocks = (c->N + 255) / 256;             // 256-thread grid-stride kernels
         d->grid = (int)(blocks < size_t(nsm) * 8 ? blocks : size_t(nsm) * 8);
+        d->nsm = nsm;
         // tile 0: chosen by es_autotune; mixed tiles D3_NSHAPES + k: shape k with plain loads (no TMA staging)
         d->shape = p->tile >= 1 ? (p->tile - 1) % D3_NSHAPES : 0;
         d->no_tma = p->tile > D3_NSHAPES;
