@@ -446,8 +446,7 @@ __device__ __forceinline__ int jump_is_zero(const SwitchBounds& b, const Face<D>
     // (factors: truncation and rounding of the FP32 values; bounds that leave FP32's range, in units of extreme size, decide
     // nothing)
     if ((__double_as_longlong(j) << 1) == 0) return 1;
-    if (b.tol == 0.0f) return 0;
-    if (!(hi < 1e38f) || hi < 1e-30f) return 2;
+    if (__float_as_uint(hi) - 0x0da24260u >= 0x7e967699u - 0x0da24260u) return b.tol == 0.0f ? 0 : 2;   // not in [1e-30, 1e38)
     if (ja * 1.0001f < lo * 0.99f) return 1;
     return ja > hi * 1.001f ? 0 : 2;
 }
