@@ -6,8 +6,8 @@
 // table's -ln c are sums of a multiple of 2^-42 and a small rest, so that e ln 2 - ln c is exact but for the rests, which
 // join the series: one rounding of the result's size is left (a face takes the difference of two logarithms over as
 // little as 1/50 of their size, so that their last bit is the flux's sixth).  Beside 1 (c = 1, e = 0) the result is the
-// series alone, so small logarithms keep their relative accuracy.  13 instructions on the FP64 pipe (the exponent's double
-// is put together on the integer and FP32 pipes) against about 27 of the library's log(): four logarithms at each of a
+// series alone, so small logarithms keep their relative accuracy.  12 instructions on the FP64 pipe (the exponent's double and
+// the rests are put together on the integer and FP32 pipes) against about 27 of the library's log(): four logarithms at each of a
 // tile's nodes, halo included, were 7% of the 2D stage's FP64 instructions.
 // Checked against the logarithm in more than 64 bits on the GPU (es_selftest_log): within 1 ulp.
 #pragma once
@@ -59,7 +59,8 @@ constexpr DD LN2 = ln(2.0);
 constexpr double LN2_HI = coarse(LN2.h), LN2_LO = rest(LN2);
 
 struct Table {
-    double c[128], hi[128], lo[128];     // c ~ 1/m and -ln c
+    double c[128], hi[128];              // c ~ 1/m and -ln c
+    float lo[128];
 };
 constexpr Table make_table() {
     Table t{};
@@ -69,7 +70,7 @@ constexpr Table make_table() {
         t.c[i] = one ? 1.0 : 1.0 / m;
         const DD y = one ? DD{0.0, 0.0} : ln(t.c[i]);
         t.hi[i] = -coarse(y.h);
-        t.lo[i] = -rest(y);
+        t.lo[i] = float(-rest(y));
     }
     return t;
 }
@@ -96,7 +97,7 @@ __device__ __forceinline__ double log_tab(double x) {
     p = fma(r, p, -0.5);
     const double de = bits::widen(float(e));
     const double base = fma(de, log64::LN2_HI, __ldg(&log64::TABLE.hi[i]));       // exact
-    const double low = fma(de, log64::LN2_LO, __ldg(&log64::TABLE.lo[i]));
+    const double low = bits::widen(fmaf(float(e), float(log64::LN2_LO), __ldg(&log64::TABLE.lo[i])));   // (2^-43: FP32 will do)
     return base + (r + fma(r * r, p, low));
 }
 
